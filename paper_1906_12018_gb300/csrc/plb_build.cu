@@ -21,8 +21,9 @@ void set_last_error(cudaError_t e, int line) {
 // *out holds the labels (rows by original id).  max_part_n: the most vertices
 // of one graph when the CSR is a disjoint union (else n); a vertex's label
 // holds at most that many hubs, which sizes the block tier's accepted rows.
+// vbase: the first rank of each vertex's graph in that union (else null).
 int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order, int64_t n, int64_t nnz,
-               const plb_options& o, cudaStream_t s, plb_labels** out, int64_t max_part_n) {
+               const plb_options& o, cudaStream_t s, plb_labels** out, int64_t max_part_n, const int32_t* vbase) {
 #define PLB_CK(x)                                            \
     do {                                                     \
         const cudaError_t plb_e_ = (x);                      \
@@ -277,6 +278,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         p.stage_ratio = o.warp_stage_ratio;
         p.count_check = o.profile != 0;
         p.unsorted = U;
+        p.vbase = vbase;
         return p;
     };
     const int* skip = nullptr;  // graph mode: &ctr->done (scans of finished rounds do nothing)
@@ -285,7 +287,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         cudaError_t e = exclusive_scan_i64(tmp64, aoff, n, scan_scr, s, skip);
         if (e != cudaSuccess) return e;
         k_mark<<<flat_grid_cap, kFlatThreads, 0, s>>>(roff, rcol, fse[c], fhub[c], A, aoff, ctr, recv, n);
-        k_collect<<<gflat, kFlatThreads, 0, s>>>(recv, roff, loff[c], n, fse[x], R, O1, rbound, tmp64, ctr, lim);
+        k_collect<<<gflat, kFlatThreads, 0, s>>>(recv, roff, loff[c], n, fse[x], R, O1, rbound, tmp64, vbase, ctr, lim);
         k_after_collect<<<1, 1, 0, s>>>(ctr);
         // the scan of the candidate bounds places each receiver's new frontier
         // row (aoff is free again after k_mark); used when the buffer holds
@@ -315,7 +317,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         }
     } side_guard{side, ev_fork, ev_join};
     auto launch_gp = [&](GpParams p, cudaEvent_t* g1) -> cudaError_t {
-        k_pack_hrec<<<gflat, kFlatThreads, 0, s>>>(p.loff, p.lent, hdesc, hrec, n, ctr);
+        k_pack_hrec<<<gflat, kFlatThreads, 0, s>>>(p.loff, p.lent, hdesc, vbase, hrec, n, ctr);
         st.launches += 1;
         GpParams w = p, b = p;
         w.list = R;  // warp tier
@@ -370,7 +372,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         k_merge_old<<<flat_grid_cap, kFlatThreads, 0, s>>>(loff[c], lent[c], loff[x], lent[x], fse[x], fhub[x], n,
                                                            ctr);
         k_merge_new<<<grid_for((int64_t)n * 32, kFlatThreads, flat_grid_cap), kFlatThreads, 0, s>>>(
-            loff[c], lent[c], loff[x], lent[x], fse[x], fhub[x], A, ctr, top);
+            loff[c], lent[c], loff[x], lent[x], fse[x], fhub[x], A, vbase, ctr, top);
         st.launches += 6 + scan_n;
         return cudaGetLastError();
     };

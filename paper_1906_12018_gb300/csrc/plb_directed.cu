@@ -269,7 +269,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
         k_mark<<<flat_grid_cap, kFlatThreads, 0, s>>>(S.s_off, S.s_col, S.fse[c], S.fhub[c], S.A, S.aoff, S.ctr,
                                                       S.recv, n);
         k_collect<<<gflat, kFlatThreads, 0, s>>>(S.recv, S.g_off, S.loff[c], n, S.fse[x], S.R, S.O1, S.rbound, nullptr,
-                                                 S.ctr, lim);
+                                                 nullptr, S.ctr, lim);
         k_after_collect<<<1, 1, 0, s>>>(S.ctr);
         launches += 4 + scan_n;
         return cudaGetLastError();
@@ -334,7 +334,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
         k_merge_old<<<flat_grid_cap, kFlatThreads, 0, s>>>(S.loff[c], S.lent[c], S.loff[x], S.lent[x], S.fse[x],
                                                            S.fhub[x], n, S.ctr);
         k_merge_new<<<grid_for((int64_t)n * 32, kFlatThreads, flat_grid_cap), kFlatThreads, 0, s>>>(
-            S.loff[c], S.lent[c], S.loff[x], S.lent[x], S.fse[x], S.fhub[x], S.A, S.ctr, S.top);
+            S.loff[c], S.lent[c], S.loff[x], S.lent[x], S.fse[x], S.fhub[x], S.A, nullptr, S.ctr, S.top);
         launches += 6 + scan_n;
         return cudaGetLastError();
     };

@@ -321,9 +321,9 @@ __device__ void shrink_pass(uint32_t* S, int log_s, uint32_t* C, int limit, uint
 }
 
 // Block-wide load-balanced gather of v's messages with hub in [lo, *hi_sm):
-// hubs below W are marked in the byte map B (plain stores: duplicates write
-// the same byte, and L(v)'s hubs are cleared afterwards), the others go into
-// the set S.  Neighbours are taken in tiles of blockDim; each thread finds its
+// hubs below vb + W (vb: the first rank of v's graph) are marked in the byte
+// map B (plain stores: duplicates write the same byte, and L(v)'s hubs are
+// cleared afterwards), the others go into the set S.  Neighbours are taken in tiles of blockDim; each thread finds its
 // neighbour's sub-range of dL_{d-1}(a) (binary searches in the sorted row), a
 // block-wide exclusive scan of the counts assigns every thread an equal,
 // contiguous share of the tile's messages.  When the set would exceed
@@ -333,7 +333,7 @@ __device__ void shrink_pass(uint32_t* S, int log_s, uint32_t* C, int limit, uint
 // pass takes them): no message of the tile is read twice, except those of
 // the step that met the overflow.
 __device__ void gather_block(const GpParams& p, int64_t nb, int64_t ne, uint32_t lo, uint32_t* hi_sm, uint8_t* B,
-                             uint32_t W, uint32_t* S, int log_s, const uint32_t* M, int log_m, int limit, int* cnt_sm,
+                             uint32_t vb, uint32_t W, uint32_t* S, int log_s, const uint32_t* M, int log_m, int limit, int* cnt_sm,
                              volatile int* ovf_sm, int* wsum, int* sex, int64_t* sst, uint32_t* C, int* hist, int* tmp,
                              unsigned long long& msgs) {
     const int tid = threadIdx.x, nthr = blockDim.x;
@@ -351,7 +351,7 @@ __device__ void gather_block(const GpParams& p, int64_t nb, int64_t ne, uint32_t
                 // the hubs of a frontier row of sender a are <= a (a itself
                 // only in round 0): for a < hi the whole row lies below hi
                 const uint32_t* row = p.fhub + fstart(f);
-                const int64_t a0 = lo ? lower_bound_u32(row, n0, lo) : 0;
+                const int64_t a0 = lo > vb ? lower_bound_u32(row, n0, lo) : 0;
                 const int64_t a1 = sender_of(p, a) < hi ? (int64_t)n0 : lower_bound_u32(row, n0, hi);
                 st = (int64_t)fstart(f) + a0;
                 c = (int)(a1 - a0);
@@ -418,9 +418,9 @@ __device__ void gather_block(const GpParams& p, int64_t nb, int64_t ne, uint32_t
 #pragma unroll
                         for (int u = 0; u < kGatherUnroll; ++u) {
                             const uint32_t h = hv[u];
-                            if (h < W) {
-                                B[h] = 1;
-                            } else if (h < hcut && (!M || map_find(M, log_m, h) == kEmpty)) {
+                            if (h - vb < W) {
+                                B[h - vb] = 1;
+                            } else if (h - vb < hcut - vb && (!M || map_find(M, log_m, h) == kEmpty)) {
                                 if (*(volatile int*)cnt_sm >= limit) *ovf_sm = 1;
                                 else nins += set_insert(S, log_s, h) ? 1 : 0;
                             }
@@ -440,7 +440,8 @@ __device__ void gather_block(const GpParams& p, int64_t nb, int64_t ne, uint32_t
             __syncthreads();
             // concurrent inserts can pass the limit without raising the flag
             if (*ovf_sm || *(volatile int*)cnt_sm > limit) {
-                shrink_pass(S, log_s, C, limit, lo > W ? lo : W, hi_sm, cnt_sm, hist, tmp);  // S holds hubs >= W
+                // S holds hubs >= vb + W
+                shrink_pass(S, log_s, C, limit, lo > vb + W ? lo : vb + W, hi_sm, cnt_sm, hist, tmp);
                 if (tid == 0) *ovf_sm = 0;
                 __syncthreads();
                 continue;  // every warp resumes at its pos with the smaller range
@@ -539,8 +540,9 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
             for (int64_t j = lane; j < ll; j += 32) lvs[j] = p.lent[lb + j];
             lvp = lvs;
         }
-        // entries of L(v) with hub below kTopHubs (the checks' side B starts past them)
-        const int lv_top = nc > 0 ? (int)lower_bound_u32(lvp, ll, pack((uint32_t)kTopHubs, 0)) : 0;
+        // entries of L(v) with a top hub (the checks' side B starts past them)
+        const int lv_top =
+            nc > 0 ? (int)lower_bound_u32(lvp, ll, pack(base_of(p.vbase, v) + (uint32_t)kTopHubs, 0)) : 0;
         // distance checks, 32 candidates at a time; survivors compacted in place
         uint32_t* tv = tvs + wib * kTopRow;
         if (nc > 0) stage_exact_levels(p.top, v, tv, lane, 32);
@@ -662,13 +664,14 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
     }
     stage_exact_levels(p.top, v, tv, tid, nthr);
     int64_t total_acc = 0;
-    uint32_t lo = 0;
-    int64_t width = v;
+    const uint32_t vb = base_of(p.vbase, v);  // v's hubs are ranks [vb, v)
+    uint32_t lo = vb;
+    int64_t width = (int64_t)v - vb;
     uint32_t* hi_sm = reinterpret_cast<uint32_t*>(&sh[SH_HI]);
-    // hubs below W (the most frequent messages) are deduplicated in the byte
+    // hubs below vb + W (the most frequent messages) are deduplicated in the byte
     // map, in the first pass, for vertices with many messages (for the others
     // clearing and scanning the map costs more than the hashing it saves)
-    const uint32_t W = p.rbound[v] >= kByteMinBound ? min((uint32_t)kByteHubs, (uint32_t)v) : 0u;
+    const uint32_t W = p.rbound[v] >= kByteMinBound ? min((uint32_t)kByteHubs, (uint32_t)v - vb) : 0u;
     const int nbw = (int)((W + 3) / 4);  // byte-map words in use
     for (int q = tid; q < nbw; q += nthr) reinterpret_cast<uint32_t*>(B)[q] = 0u;
     while ((int64_t)lo < (int64_t)v) {
@@ -682,13 +685,13 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
             *hi_sm = (uint32_t)min((int64_t)v, (int64_t)lo + width);
         }
         __syncthreads();
-        gather_block(p, nb, ne, lo, hi_sm, B, W, S, log_s, useM ? M : nullptr, log_m, limit, &sh[SH_UNIQ],
+        gather_block(p, nb, ne, lo, hi_sm, B, vb, W, S, log_s, useM ? M : nullptr, log_m, limit, &sh[SH_UNIQ],
                      (volatile int*)&sh[SH_OVF], wsum, sex, sst, C, hist, &sh[SH_TMP], cnt[1]);
         __syncthreads();
         const uint32_t hi = *(volatile uint32_t*)hi_sm;
-        if (lo < W) {  // first pass: drop L(v)'s hubs from the byte map
+        if (lo - vb < W) {  // first pass: drop L(v)'s hubs from the byte map
             for (int64_t j = tid; j < ll; j += nthr) {
-                const uint32_t w = hub_of(lv[j]);
+                const uint32_t w = hub_of(lv[j]) - vb;
                 if (w < W) B[w] = 0;
             }
         }
@@ -717,11 +720,11 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
             lvp = lvs;
         }
         __syncthreads();
-        // entries of L(v) with hub below kTopHubs (the checks' side B starts past them)
-        const int lv_top = (int)lower_bound_u32(lvp, ll, pack((uint32_t)kTopHubs, 0));
+        // entries of L(v) with a top hub (the checks' side B starts past them)
+        const int lv_top = (int)lower_bound_u32(lvp, ll, pack(vb + (uint32_t)kTopHubs, 0));
         const int nc_set = min(*(volatile int*)&sh[SH_NC], limit);  // candidates from the set
         if (tid == 0) cnt[2] += nc_set;
-        if (lo < W) {
+        if (lo - vb < W) {
             // the byte-map candidates: each warp extracts 32 words (up to 128
             // hubs) at a time into its slice of S (free after the compaction;
             // kByteStage words per warp), checks them in full chunks of 32 and
@@ -736,7 +739,7 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
                 const int tot = __shfl_sync(kFull, incl, 31);
                 int o = f + incl - c;
                 for (int b = 0; b < 4; ++b)
-                    if ((b4 >> b) & 1u) stage[o++] = 4u * (uint32_t)(g + lane) + (uint32_t)b;
+                    if ((b4 >> b) & 1u) stage[o++] = vb + 4u * (uint32_t)(g + lane) + (uint32_t)b;
                 if (lane == 0) cnt[2] += tot;
                 f += tot;
                 __syncwarp();
@@ -866,14 +869,15 @@ __global__ void __launch_bounds__(256, 3) k_gp_block(GpParams p) {
 
 // Check records of all rows, from the label offsets and the probe index as
 // they stand for the coming gather (a finished round returns at once).
-__global__ void k_pack_hrec(const int64_t* loff, const uint32_t* lent, const uint64_t* hdesc, uint4* hrec, int64_t n,
-                            const RoundCounters* ctr) {
+__global__ void k_pack_hrec(const int64_t* loff, const uint32_t* lent, const uint64_t* hdesc, const int32_t* vbase,
+                            uint4* hrec, int64_t n, const RoundCounters* ctr) {
     if (ctr->done) return;
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
         const int64_t a = loff[v], len = loff[v + 1] - a;
         const uint64_t row = hrec_row((uint64_t)a, (uint64_t)len);
-        // entries of L(v) with hub < kTopHubs (rows are hub-sorted)
-        const uint64_t top = (uint64_t)lower_bound_u32(lent + a, len, pack((uint32_t)kTopHubs, 0));
+        // entries of L(v) with a top hub (rows are hub-sorted)
+        const uint64_t top =
+            (uint64_t)lower_bound_u32(lent + a, len, pack(base_of(vbase, v) + (uint32_t)kTopHubs, 0));
         const uint64_t hd = hdesc[v] | (top << (32 + kHrecTopShift));
         hrec[v] = make_uint4((uint32_t)row, (uint32_t)(row >> 32), (uint32_t)hd, (uint32_t)(hd >> 32));
     }

@@ -106,17 +106,28 @@ struct GpParams {
                                // count ctr->nU), or null (every new row is sorted after the round)
     int sender_bits;           // rcol holds frontier descriptor indices whose low sender_bits bits are
                                // the sending vertex (weighted rounds), or 0: the vertex itself
+    const int32_t* vbase;      // per vertex: first rank of its graph in a disjoint union, or null (one graph:
+                               // 0).  The top hubs and the byte map are those of the vertex's own graph
     int count_check;           // 1: count the label entries each check would read by the paper's cost
                                // model (RoundCounters::chk_lv / chk_lh; one binary search per candidate)
 };
+
+// First rank of v's graph (see GpParams::vbase).
+__device__ __forceinline__ uint32_t base_of(const int32_t* vbase, int64_t v) {
+    return vbase ? (uint32_t)vbase[v] : 0u;
+}
 
 // The sending vertex of an arc's descriptor index (see GpParams::sender_bits).
 __device__ __forceinline__ uint32_t sender_of(const GpParams& p, int32_t a) {
     return p.sender_bits ? (uint32_t)a & ((1u << p.sender_bits) - 1u) : (uint32_t)a;
 }
 
-// Witness prefilter: for the kTopHubs highest-ranked hubs, every vertex x
-// keeps kTopLevels bitmasks C_t(x) = {w : w in L(x), d(w, x) <= t}, t = 1..
+// Witness prefilter: for the kTopHubs highest-ranked hubs of its graph (in a
+// disjoint union each graph has its own, ranks vbase .. vbase + kTopHubs - 1:
+// the union's first 256 ranks all belong to its first graph; with those as the
+// only masks a batch of 200 graphs of 1K-64K vertices settled 2% of its
+// candidates without a scan and took 135.2 ms, with each graph's own it takes
+// 69.3 ms), every vertex x keeps kTopLevels bitmasks C_t(x) = {w : w in L(x), d(w, x) <= t}, t = 1..
 // kTopLevels (8 words each).  A candidate h at round d has a witness among
 // those hubs when E_i(v) & C_{d-i}(h) != 0 for some i, E_i = C_i & ~C_{i-1}:
 // the label test restricted to those hubs and distances (exact: a hit is a
@@ -155,12 +166,12 @@ constexpr int kIndexSmemSlotsMax = 2048;
 
 // Check records (GpParams::hrec_h): row start << 24 | length, then the
 // probe-table descriptor (table start << 8 | log2 slots, below 2^48) with the
-// row's count of entries whose hub is below kTopHubs in its top 16 bits.
+// row's count of entries whose hub is one of its graph's kTopHubs in its top 16 bits.
 __host__ __device__ __forceinline__ uint64_t hrec_row(uint64_t start, uint64_t len) { return (start << 24) | len; }
 constexpr int kHrecTopShift = 16;  // within the record's last word
 constexpr uint64_t kHrecDescMask = (uint64_t(1) << 48) - 1;
-__global__ void k_pack_hrec(const int64_t* loff, const uint32_t* lent, const uint64_t* hdesc, uint4* hrec, int64_t n,
-                            const RoundCounters* ctr);
+__global__ void k_pack_hrec(const int64_t* loff, const uint32_t* lent, const uint64_t* hdesc, const int32_t* vbase,
+                            uint4* hrec, int64_t n, const RoundCounters* ctr);
 
 // Routing limits of k_collect (see the tier geometry in build_core).
 struct TierLimits {

@@ -200,7 +200,8 @@ __global__ void k_mark(const int64_t* roff, const int32_t* rcol, const uint64_t*
     }
 }
 
-// Receivers (recv[v] > 0) are routed by the candidate bound min(v, recv[v]),
+// Receivers (recv[v] > 0) are routed by the candidate bound min(v, recv[v])
+// (v counted from the first rank of its graph in a disjoint union),
 // |L(v)| and degree: warp tier (R) or block tier (O1); the bound is kept in
 // rbound[v] (it sizes the warp tier's tables) and, when obound is given, in
 // obound[v] for every v (0 for non-receivers: its scan places each row of the
@@ -208,7 +209,7 @@ __global__ void k_mark(const int64_t* roff, const int32_t* rcol, const uint64_t*
 // the bounds.
 __global__ void k_collect(unsigned long long* recv, const int64_t* roff, const int64_t* loff, int64_t n,
                           uint64_t* fse_new, int32_t* R, int32_t* O1, uint32_t* rbound, int64_t* obound,
-                          RoundCounters* ctr, TierLimits lim) {
+                          const int32_t* vbase, RoundCounters* ctr, TierLimits lim) {
     if (ctr->done) return;
     unsigned long long bsum = 0;
     const int lane = lane_id();
@@ -216,10 +217,12 @@ __global__ void k_collect(unsigned long long* recv, const int64_t* roff, const i
         fse_new[v] = 0;
         const unsigned long long c = recv[v];
         int tier = -1;
-        if (obound) obound[v] = c < (unsigned long long)v ? (int64_t)c : v;
+        // v accepts hubs of its own graph that outrank it: at most v - base
+        const unsigned long long below = (unsigned long long)(v - (int64_t)base_of(vbase, v));
+        const unsigned long long bound = c < below ? c : below;
+        if (obound) obound[v] = (int64_t)bound;
         if (c) {
             recv[v] = 0;
-            const unsigned long long bound = c < (unsigned long long)v ? c : (unsigned long long)v;
             bsum += bound;
             rbound[v] = (uint32_t)bound;  // v < 2^24
             const int64_t ll = loff[v + 1] - loff[v];
@@ -768,7 +771,7 @@ __global__ void k_merge_old(const int64_t* loff, const uint32_t* lent, const int
 // New entries (dist d) of each active vertex: warp per vertex.
 __global__ void k_merge_new(const int64_t* loff, const uint32_t* lent, const int64_t* loff_new, uint32_t* lent_new,
                             const uint64_t* fse_new, const uint32_t* fhub_new, const int32_t* A,
-                            const RoundCounters* ctr, uint32_t* top) {
+                            const int32_t* vbase, const RoundCounters* ctr, uint32_t* top) {
     if (ctr->done) return;
     const uint32_t d = ctr->d;
     const int nA = ctr->nA;
@@ -784,6 +787,7 @@ __global__ void k_merge_new(const int64_t* loff, const uint32_t* lent, const int
         // old hubs below h are counted with shuffles instead of a binary
         // search in global memory (c and ol are the same in every lane)
         const bool reg = ol <= 32;
+        const uint32_t vb = base_of(vbase, v);
         const uint32_t oe = reg && lane < ol ? lent[ob + lane] : 0xFFFFFFFFu;
         for (uint32_t j0 = 0; j0 < c; j0 += 32) {
             const uint32_t j = j0 + lane;
@@ -799,9 +803,10 @@ __global__ void k_merge_new(const int64_t* loff, const uint32_t* lent, const int
             if (j >= c) continue;
             const int64_t pos = loff_new[v] + j + below;
             lent_new[pos] = pack(h, d);
-            if (h < (uint32_t)kTopHubs && d <= (uint32_t)kTopLevels) {
-                uint32_t* tv = top + (int64_t)v * kTopRow + (h >> 5);
-                for (int t = (int)d; t <= kTopLevels; ++t) atomicOr(tv + (t - 1) * kTopWords, 1u << (h & 31));
+            const uint32_t hr = h - vb;
+            if (hr < (uint32_t)kTopHubs && d <= (uint32_t)kTopLevels) {
+                uint32_t* tv = top + (int64_t)v * kTopRow + (hr >> 5);
+                for (int t = (int)d; t <= kTopLevels; ++t) atomicOr(tv + (t - 1) * kTopWords, 1u << (hr & 31));
             }
         }
     }

@@ -26,7 +26,7 @@ __global__ void k_mark(const int64_t* roff, const int32_t* rcol, const uint64_t*
                        int64_t n);
 __global__ void k_collect(unsigned long long* recv, const int64_t* roff, const int64_t* loff, int64_t n,
                           uint64_t* fse_new, int32_t* R, int32_t* O1, uint32_t* rbound, int64_t* obound,
-                          RoundCounters* ctr, TierLimits lim);
+                          const int32_t* vbase, RoundCounters* ctr, TierLimits lim);
 __global__ void k_after_collect(RoundCounters* ctr);
 __global__ void k_rerun_reset(RoundCounters* ctr, uint64_t* fse_new, int64_t n);
 __global__ void k_round1_count(const int64_t* roff, const int32_t* rcol, int64_t n, int64_t nnz, int32_t s,
@@ -64,7 +64,7 @@ __global__ void k_merge_old(const int64_t* loff, const uint32_t* lent, const int
                             const uint64_t* fse_new, const uint32_t* fhub_new, int64_t n, const RoundCounters* ctr);
 __global__ void k_merge_new(const int64_t* loff, const uint32_t* lent, const int64_t* loff_new, uint32_t* lent_new,
                             const uint64_t* fse_new, const uint32_t* fhub_new, const int32_t* A,
-                            const RoundCounters* ctr, uint32_t* top);
+                            const int32_t* vbase, const RoundCounters* ctr, uint32_t* top);
 __global__ void k_top_init(uint32_t* top, int64_t n);
 __global__ void k_final_len(const int64_t* loff, const int32_t* inv, int64_t n, int64_t* len);
 __global__ void k_finalize(const int64_t* loff, const uint32_t* lent, const int32_t* inv, const int64_t* out_off,

@@ -455,7 +455,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
         if (nnz > 0)
             k_w_pull<<<gpull, kWFlatThreads, 0, s>>>(roff, rcol, rwt, n, nnz, (uint32_t)d, S, lgn, ring, store,
                                                      vcol, recv);
-        k_collect<<<gflat, kFlatThreads, 0, s>>>(recv, roff, loff[cur], n, fse_new, R, O1, rbound, nullptr, ctr, lim);
+        k_collect<<<gflat, kFlatThreads, 0, s>>>(recv, roff, loff[cur], n, fse_new, R, O1, rbound, nullptr, nullptr, ctr, lim);
         k_after_collect<<<1, 1, 0, s>>>(ctr);
         launches += 4;
         PLB_CK(cudaGetLastError());
@@ -537,7 +537,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
             k_merge_old<<<flat_grid_cap, kFlatThreads, 0, s>>>(loff[cur], lent[cur], loff[x], lent[x], fse_new, store,
                                                                n, ctr);
             k_merge_new<<<grid_for((int64_t)n * 32, kFlatThreads, flat_grid_cap), kFlatThreads, 0, s>>>(
-                loff[cur], lent[cur], loff[x], lent[x], fse_new, store, A, ctr, top);
+                loff[cur], lent[cur], loff[x], lent[x], fse_new, store, A, nullptr, ctr, top);
             launches += 6 + scan_n;
             PLB_CK(cudaGetLastError());
             const int64_t Told = T;
