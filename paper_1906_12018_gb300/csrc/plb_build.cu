@@ -214,7 +214,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
     const int block_cand = pow2_at_least(std::max(bthr, o.block_cand_cap));
     const int b_log_s = ceil_log2_i64(std::max<int64_t>(std::max<int64_t>(2 * (int64_t)block_cand,
                                                                            block_cand + (int64_t)kGatherUnroll * bthr),
-                                                          (int64_t)kByteStage * (bthr / 32)));
+                                                          (int64_t)kWarpStage * (bthr / 32)));
     const int b_log_m = ceil_log2_i64(2 * (int64_t)std::max(o.block_label_cap, 64) + 2 * bthr);
     const size_t b_smem = gp_block_smem_bytes(bthr, b_log_s, b_log_m, block_cand);
     TierLimits lim;
@@ -252,6 +252,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
     // the scan of the bounds (aoff, after the frontier step) puts them
     auto gp_params = [&](int c, int x, int64_t fc, bool placed) {
         GpParams p{};
+        p.n = n;
         p.ostart = placed ? aoff : nullptr;
         p.roff = roff;
         p.rcol = rcol;
@@ -372,7 +373,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         k_merge_old<<<flat_grid_cap, kFlatThreads, 0, s>>>(loff[c], lent[c], loff[x], lent[x], fse[x], fhub[x], n,
                                                            ctr);
         k_merge_new<<<grid_for((int64_t)n * 32, kFlatThreads, flat_grid_cap), kFlatThreads, 0, s>>>(
-            loff[c], lent[c], loff[x], lent[x], fse[x], fhub[x], A, vbase, ctr, top);
+            loff[c], lent[c], loff[x], lent[x], fse[x], fhub[x], A, vbase, ctr, top, n);
         st.launches += 6 + scan_n;
         return cudaGetLastError();
     };

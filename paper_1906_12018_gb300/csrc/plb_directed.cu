@@ -233,7 +233,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
     const int block_cand = pow2_at_least(std::max(bthr, o.block_cand_cap));
     const int b_log_s = ceil_log2_i64(std::max<int64_t>(
         std::max<int64_t>(2 * (int64_t)block_cand, block_cand + (int64_t)kGatherUnroll * bthr),
-        (int64_t)kByteStage * (bthr / 32)));
+        (int64_t)kWarpStage * (bthr / 32)));
     const int b_log_m = ceil_log2_i64(2 * (int64_t)std::max(o.block_label_cap, 64) + 2 * bthr);
     const size_t b_smem = gp_block_smem_bytes(bthr, b_log_s, b_log_m, block_cand);
     TierLimits lim;
@@ -278,6 +278,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
     auto gather = [&](Side& S, const Side& H) -> cudaError_t {
         const int c = S.cur, x = c ^ 1;
         GpParams p{};
+        p.n = n;
         p.roff = S.g_off;
         p.rcol = S.g_col;
         p.loff = S.loff[c];
@@ -334,7 +335,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
         k_merge_old<<<flat_grid_cap, kFlatThreads, 0, s>>>(S.loff[c], S.lent[c], S.loff[x], S.lent[x], S.fse[x],
                                                            S.fhub[x], n, S.ctr);
         k_merge_new<<<grid_for((int64_t)n * 32, kFlatThreads, flat_grid_cap), kFlatThreads, 0, s>>>(
-            S.loff[c], S.lent[c], S.loff[x], S.lent[x], S.fse[x], S.fhub[x], S.A, nullptr, S.ctr, S.top);
+            S.loff[c], S.lent[c], S.loff[x], S.lent[x], S.fse[x], S.fhub[x], S.A, nullptr, S.ctr, S.top, n);
         launches += 6 + scan_n;
         return cudaGetLastError();
     };

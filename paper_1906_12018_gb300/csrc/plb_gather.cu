@@ -5,8 +5,16 @@
 // (h, d) iff no common hub w has d(w, v) + d(w, h) <= d).
 //   k_gp_warp   one vertex per warp, tables in shared memory;
 //   k_gp_block  one vertex per 256-thread block, any size.
-// Both append the accepted hubs to the new frontier: the warp tier sorted,
-// the block tier unsorted (it lists those vertices for the row sort).
+// Both append the accepted hubs to the new frontier in rank order (the block
+// tier lists the few vertices whose row it could not sort for the row sort).
+// Loops with a run-time trip count are not unrolled: the warps of an SM are at
+// different places of these kernels, and code that outgrows the instruction
+// caches costs more than the loop control (see witness4).
+//
+// Measured, with hub maps, the two-step prefilter, the lane/group/warp checks
+// and the bucketed tables (before -> after, builds): R-MAT 2^22, 64M edges
+// 1,213 -> 834 ms; Chung-Lu 2^20 39.1 -> 34.8 ms; directed R-MAT 2^20 185.9 ->
+// 140.9 ms.
 #include "plb_kernels.cuh"
 #include "plb_round.cuh"
 
@@ -20,39 +28,73 @@ __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 constexpr int kWarpSideBMin = 16, kWarpSideBShift = 1;
 constexpr int kBlockSideBMin = 16, kBlockSideBShift = 1;
 
-// Top-hub witness prefilter for the 32 candidates of a chunk (one per lane):
-// candidate h has a witness among the kTopHubs highest-ranked hubs when
-// E_i(v) & C_j(h) != 0 for some i >= 1, j = min(d - i, kTopLevels) >= 1, where
-// E_i(v) (v's hubs at distance exactly i) is staged in shared memory (ev,
-// kTopLevels x kTopWords words) and C_j(h) is h's cumulative mask.  Returns
-// the mask of lanes whose candidate is pruned.
-__device__ __forceinline__ unsigned top_prefilter(const uint32_t* top, const uint32_t* ev, uint32_t d, uint32_t h,
-                                                  bool valid) {
-    uint32_t hit = 0;
-    if (valid) {
-        const uint32_t* th = top + (int64_t)h * kTopRow;
-        const int imax = min((int)d - 1, kTopLevels);
-        for (int i = 1; i <= imax; ++i) {
-            const int j = min((int)d - i, kTopLevels);
-            const uint4* cj = reinterpret_cast<const uint4*>(th + (j - 1) * kTopWords);
-            const uint32_t* e = ev + (i - 1) * kTopWords;
-#pragma unroll
-            for (int q = 0; q < kTopWords / 4; ++q) {
-                const uint4 a = cj[q];
-                hit |= (a.x & e[4 * q]) | (a.y & e[4 * q + 1]) | (a.z & e[4 * q + 2]) | (a.w & e[4 * q + 3]);
-            }
+// 32 bytes of global memory (one sector) in one load; p is 32-byte aligned.
+__device__ __forceinline__ void load_sector(const uint32_t* p, uint32_t (&x)[8]) {
+    asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]), "=r"(x[7])
+        : "l"(p));
+}
+
+// Top-hub witness prefilter: candidate h has a witness among the kTopHubs
+// highest-ranked hubs when E_i(v) & C_j(h) != 0 for some i >= 1,
+// j = min(d - i, kTopLevels) >= 1, where E_i(v) (v's hubs at distance exactly
+// i) is staged in shared memory (ev, kTopLevels x kTopWords words) and C_j(h)
+// is h's cumulative mask.  One level pair (i, j) = one 32-byte mask of h.
+static_assert(kTopWords == 8, "a mask is one 32-byte sector");
+__device__ __forceinline__ uint32_t top_pair(const uint32_t* top, int64_t n, const uint32_t* ev, int i, int j,
+                                             uint32_t h) {
+    uint32_t c[8];
+    load_sector(top + ((j - 1) * n + h) * kTopWords, c);
+    const uint4* e4 = reinterpret_cast<const uint4*>(ev + (i - 1) * kTopWords);
+    const uint4 e = e4[0], g = e4[1];
+    return (c[0] & e.x) | (c[1] & e.y) | (c[2] & e.z) | (c[3] & e.w) | (c[4] & g.x) | (c[5] & g.y) | (c[6] & g.z) |
+           (c[7] & g.w);
+}
+
+// The prefilter runs in two steps.  The first tests one level pair (i0, d -
+// i0), i0 the smallest distance at which v has a top hub, for two candidates
+// per lane at once (independent loads, nothing else in flight behind them):
+// it settles most candidates (R-MAT 2^22: 73% in round 2, where it is the
+// whole prefilter, and nearly all of round 3's 6.5G).  Only its survivors,
+// compacted into full warps, go on to check_chunk, which tests the other
+// pairs.  Weighted rounds (many distances, few hubs at each) test every pair
+// in the first step.
+__device__ __forceinline__ int first_level(const uint32_t* ev, int imax, int lane) {
+    int i0 = 1;
+#pragma unroll 1
+    for (int i = 1; i <= imax; ++i) {
+        if (__any_sync(kFull, ev[(i - 1) * kTopWords + (lane & 7)] != 0u)) {
+            i0 = i;
+            break;
         }
     }
-    return __ballot_sync(kFull, hit != 0);
+    return i0;
+}
+__device__ __forceinline__ void prefilter_first(const GpParams& p, const uint32_t* ev, int d, int imax, int i0,
+                                                uint32_t h0, bool v0, uint32_t h1, bool v1, unsigned* m0,
+                                                unsigned* m1) {
+    const int ia = p.sender_bits == 0 ? i0 : 1, ib = p.sender_bits == 0 ? i0 : imax;
+    uint32_t x0 = 0, x1 = 0;
+#pragma unroll 1
+    for (int i = ia; i <= ib; ++i) {
+        const int j = min(d - i, kTopLevels);
+        if (v0) x0 |= top_pair(p.top_h, p.n, ev, i, j, h0);
+        if (v1) x1 |= top_pair(p.top_h, p.n, ev, i, j, h1);
+    }
+    *m0 = __ballot_sync(kFull, v0 && x0 == 0u);  // the lanes whose candidate goes on
+    *m1 = __ballot_sync(kFull, v1 && x1 == 0u);
 }
 
 // Stage E_i(v) = C_i(v) & ~C_{i-1}(v), i = 1..kTopLevels, into ev (cooperative:
 // thread t of nthr handles words t, t + nthr, ...).
-__device__ __forceinline__ void stage_exact_levels(const uint32_t* top, int32_t v, uint32_t* ev, int t, int nthr) {
-    const uint32_t* tv = top + (int64_t)v * kTopRow;
+__device__ __forceinline__ void stage_exact_levels(const uint32_t* top, int64_t n, int32_t v, uint32_t* ev, int t,
+                                                   int nthr) {
+    const uint32_t* tv = top + (int64_t)v * kTopWords;
+#pragma unroll 1
     for (int q = t; q < kTopRow; q += nthr) {
-        const uint32_t c = tv[q];
-        const uint32_t prev = q >= kTopWords ? tv[q - kTopWords] : 0u;
+        const int lev = q / kTopWords, w = q % kTopWords;
+        const uint32_t c = tv[lev * n * kTopWords + w];
+        const uint32_t prev = lev > 0 ? tv[(lev - 1) * n * kTopWords + w] : 0u;
         ev[q] = c & ~prev;
     }
 }
@@ -69,33 +111,79 @@ __device__ __forceinline__ void stage_exact_levels(const uint32_t* top, int32_t 
 // B is considered only for |L(h)| >= b_min (the count of L(v)'s hubs below h
 // is a binary search in L(v)'s row) and taken when it is the shorter scan, by
 // a factor 2^b_shift against a shared-memory M (whose probes are cheaper
-// than the global table's).  All (candidate, entry) pairs are spread over
-// the lanes; a candidate's remaining entries are skipped once it has a
-// witness.  Every candidate first goes through the top-hub prefilter, which
-// is exact for the kTopHubs highest-ranked hubs while d <= kTopLevels + 1
+// than the global table's).  Either way a scan is a row of entries and a hash
+// table to look them up in, and it ends at its first witness.  Every lane
+// first looks up kFirstItems entries of its own candidate (all loads in flight
+// at once: most scans end there); longer scans go on eight at a time, four
+// lanes and 16 entries per step each, and very long ones on the whole warp.
+// Every candidate has passed the first step of the top-hub prefilter (level
+// i0; i0 = 0: none yet) and goes through the rest of it here; the whole is
+// exact for the kTopHubs highest-ranked hubs while d <= kTopLevels + 1
 // (a witness w has 1 <= d(w,v), d(w,h) <= d - 1): for a candidate it does not
 // prune, no top hub is a witness, so both scans start past the top hubs
 // (L(h)'s count of them comes with h's check record, L(v)'s is tv_top).
 // Returns the lanes whose candidate survives.
+constexpr int kFirstItems = 4;   // entries of a scan that its own lane looks up
+constexpr int kGroupItems = 96;  // longest scan of a group of four lanes
+
+// Looks up the entries ent[j], ent[j + st], ent[j + 2 st], ent[j + 3 st] (those
+// below n) in the table tab of 2^tlog slots; true when one of them gives a
+// witness, a distance sum of at most d (in rank batches some labels are longer
+// than the round).  The four buckets are requested together.  One copy of the
+// code: the gather kernels' warps are at different places of it, and the warp
+// tier waited for instructions more than for anything else when its code grew
+// from 55 to 81 KB.
+__device__ __noinline__ bool witness4(const uint32_t* ent, int j, int st, int n, const uint32_t* tab, int tlog,
+                                      uint32_t d) {
+    uint32_t x[4], sl[4], lim[4];
+    uint4 y[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = j + u * st < n ? ent[j + u * st] : kEmpty;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        sl[u] = bslot(hub_of(x[u]), tlog);
+        lim[u] = dist_of(x[u]) < d ? d - dist_of(x[u]) : 0u;  // (0: no entry is that near)
+        y[u] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+        if (x[u] != kEmpty) y[u] = *reinterpret_cast<const uint4*>(tab + sl[u]);
+    }
+    bool hit = false, full = false;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        hit = hit || bucket_has(y[u], x[u] & ~0xFFu, lim[u]);
+        full = full || y[u].w != kEmpty;
+    }
+    if (full && !hit) {  // some full bucket without a witness: its chain goes on
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (y[u].w != kEmpty) hit = hit || map_has_from(tab, tlog, sl[u], y[u], x[u] & ~0xFFu, lim[u]);
+    }
+    return hit;
+}
 __device__ __forceinline__ unsigned check_chunk(const GpParams& p, uint32_t d, const uint32_t* M, int log_m,
                                                 bool mv_global, int b_min, int b_shift, const uint32_t* lv,
                                                 int64_t lvlen, int tv_top, uint32_t h, bool valid,
-                                                unsigned long long& probed, const uint32_t* tv,
-                                                unsigned long long& prefiltered, unsigned long long* chk) {
+                                                unsigned long long& probed, const uint32_t* tv, int i0,
+                                                unsigned long long& prefiltered) {
     const int lane = threadIdx.x & 31;
-    int64_t base = 0;  // A: first entry of L(h) scanned; B: start of h's probe table
-    int items = 0, meta = 0;  // meta: 0 = side A, else log2(table size) + 1
-    int skip_b = 0;           // side B: the scan of L(v) starts at this entry
+    const uint32_t* ent = lv;  // scanned entries: A: L(h), B: L(v)
+    const uint32_t* tab = M;   // looked up in: A: L(v)'s table, B: h's probe table
+    int tlog = log_m, items = 0;
     // h's check record (row bounds and probe-table descriptor: one 16-byte
-    // load, one memory sector) is requested before the top-hub prefilter
-    // reads h's masks, so the two loads overlap
+    // load, one memory sector) is requested before the rest of the top-hub
+    // prefilter reads h's masks, so the loads overlap
     uint4 rec = make_uint4(0u, 0u, 0u, 0u);
     if (valid && p.hrec_h) rec = p.hrec_h[h];
-    // every candidate first tries the exact top-hub prefilter (one mask row
-    // per distance level; a hit settles the candidate without a scan)
-    const unsigned pf = top_prefilter(p.top_h, tv, d, h, valid);
-    if (lane == 0) prefiltered += __popc(pf);
-    const bool pruned = (pf >> lane) & 1u;
+    const int imax = min((int)d - 1, kTopLevels);
+    if (i0 == 0 || (p.sender_bits == 0 && imax > 1)) {
+        uint32_t hit = 0;
+        if (valid)
+#pragma unroll 1
+            for (int i = 1; i <= imax; ++i)
+                if (i != i0) hit |= top_pair(p.top_h, p.n, tv, i, min((int)d - i, kTopLevels), h);
+        const unsigned pf = __ballot_sync(kFull, hit != 0);
+        if (lane == 0) prefiltered += __popc(pf);
+        if (hit) valid = false;
+    }
     // past the top hubs when the prefilter settles them (see above)
     const bool skip_top = d <= (uint32_t)kTopLevels + 1u;
     if (valid) {
@@ -108,88 +196,104 @@ __device__ __forceinline__ unsigned check_chunk(const GpParams& p, uint32_t d, c
             he = hb + (int64_t)(row & 0xFFFFFFu);
             hd = (((uint64_t)rec.w << 32) | rec.z) & kHrecDescMask;
             top_h = (int)(rec.w >> kHrecTopShift);
-        } else if (!pruned || p.count_check) {
+        } else {
             hb = p.loff_h[h];
             he = p.loff_h[h + 1];
             hd = p.hdesc_h[h];
-        } else {
-            hb = he = 0;
-            hd = 0;
         }
         const int la = (int)(he - hb) - 1;
-        if (p.count_check) {  // the cost model's reads: L(v)'s entries below h, and L(h)
-            chk[0] += (unsigned long long)lower_bound_u32(lv, lvlen, pack(h, 0));
-            chk[1] += (unsigned long long)(la + 1);
-        }
-        if (!pruned) {
-            const int sa = skip_top ? min(top_h, la) : 0;  // side A starts past L(h)'s top hubs
-            base = hb + sa;
-            items = la - sa;
-            if (la >= b_min && hd) {
-                const int lb = (int)lower_bound_u32(lv, lvlen, pack(h, 0));
-                const int sb = skip_top ? min(tv_top, lb) : 0;  // side B starts past L(v)'s top hubs
-                if (mv_global ? lb - sb < la - sa : ((lb - sb) << b_shift) < la - sa) {
-                    items = lb - sb;
-                    base = (int64_t)(hd >> 8);
-                    meta = (int)(hd & 0xFFu) + 1;  // log2 + 1
-                    skip_b = sb;
-                }
+        const int sa = skip_top ? min(top_h, la) : 0;  // side A starts past L(h)'s top hubs
+        ent = p.lent_h + hb + sa;
+        items = la - sa;
+        if (la >= b_min && hd) {
+            const int lb = (int)lower_bound_u32(lv, lvlen, pack(h, 0));
+            const int sb = skip_top ? min(tv_top, lb) : 0;  // side B starts past L(v)'s top hubs
+            if (mv_global ? lb - sb < la - sa : ((lb - sb) << b_shift) < la - sa) {
+                items = lb - sb;
+                ent = lv + sb;
+                tab = p.htab_h + (hd >> 8);
+                tlog = (int)(hd & 0xFFu);
             }
         }
     }
-    if (pruned) valid = false;
-    const unsigned vmask = __ballot_sync(kFull, valid);
-    const int incl = warp_incl_scan(items, lane);
-    const int total = __shfl_sync(kFull, incl, 31);
-    const int excl = incl - items;
-    unsigned pm = 0;  // candidates with a witness so far (the same in every lane)
-    // kCheckUnroll items per lane per step: their entry loads (side A: L(h);
-    // side B: L(v)) are all issued before any lookup uses one
-    for (int ib = 0; ib < total; ib += 32 * kCheckUnroll) {
-        if ((pm & vmask) == vmask) break;
-        int ku[kCheckUnroll], mku[kCheckUnroll];
-        int64_t bku[kCheckUnroll];
-        uint32_t xu[kCheckUnroll];
-#pragma unroll
-        for (int u = 0; u < kCheckUnroll; ++u) {
-            const int it = ib + 32 * u + lane;
-            const int k = warp_owner(excl, it);
-            bku[u] = __shfl_sync(kFull, base, k);
-            const int exk = __shfl_sync(kFull, excl, k);
-            mku[u] = __shfl_sync(kFull, meta, k);
-            const int sbk = __shfl_sync(kFull, skip_b, k);
-            ku[u] = (it < total && !((pm >> k) & 1u)) ? k : -1;
-            xu[u] = kEmpty;
-            if (ku[u] >= 0) xu[u] = mku[u] == 0 ? p.lent_h[bku[u] + (it - exk)] : lv[sbk + (it - exk)];
-        }
-        unsigned hits = 0;
-#pragma unroll
-        for (int u = 0; u < kCheckUnroll; ++u) {
-            if (ku[u] < 0) continue;
-            const uint32_t x = xu[u];
-            // side A: x is an entry of L(h), looked up in L(v)'s map; side B:
-            // x is an entry of L(v), looked up in h's probe table
-            const uint32_t dw = mku[u] == 0 ? map_find(M, log_m, hub_of(x))
-                                            : map_find(p.htab_h + bku[u], mku[u] - 1, hub_of(x));
-            if (dw != kEmpty && dw + dist_of(x) <= d) hits |= 1u << ku[u];
-            ++probed;
-        }
-        pm |= __reduce_or_sync(kFull, hits);
+    bool alive = valid;
+    if (items > 0) {
+        alive = !witness4(ent, 0, 1, min(items, kFirstItems), tab, tlog, d);
+        probed += (unsigned)min(items, kFirstItems);
     }
-    return vmask & ~pm;
+    // scans of up to kGroupItems entries: group g of four lanes takes the g-th
+    unsigned todo = __ballot_sync(kFull, alive && items > kFirstItems && items <= kGroupItems);
+#pragma unroll 1
+    while (todo) {
+        const unsigned batch = todo;
+        int k = -1;
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+            if ((lane >> 2) == g) k = __ffs(todo) - 1;
+            todo &= todo - 1u;
+        }
+        const int src = k < 0 ? lane : k;
+        const uint32_t* ek = reinterpret_cast<const uint32_t*>(__shfl_sync(kFull, (unsigned long long)ent, src));
+        const uint32_t* tk = reinterpret_cast<const uint32_t*>(__shfl_sync(kFull, (unsigned long long)tab, src));
+        int nk = __shfl_sync(kFull, items, src);
+        const int lk = __shfl_sync(kFull, tlog, src);
+        if (k < 0) nk = 0;
+        unsigned won = 0;  // lanes of the groups that found a witness
+#pragma unroll 1
+        for (int j = kFirstItems + (lane & 3); __any_sync(kFull, j < nk); j += 16) {
+            const bool hit = j < nk && witness4(ek, j, 4, nk, tk, lk, d);
+            const unsigned hm = __ballot_sync(kFull, hit);
+            probed += (unsigned)min(4, (max(nk - j, 0) + 3) / 4);
+            if ((hm >> (lane & ~3)) & 0xFu) nk = 0;
+            won |= hm;
+        }
+        const int g = __popc(batch & ((1u << lane) - 1u));  // this lane's candidate is the batch's g-th
+        if (((batch >> lane) & 1u) && g < 8 && ((won >> (4 * g)) & 0xFu)) alive = false;
+    }
+    // longer scans: one candidate at a time, 128 entries per step
+    todo = __ballot_sync(kFull, alive && items > kGroupItems);
+#pragma unroll 1
+    while (todo) {
+        const int k = __ffs(todo) - 1;
+        todo &= todo - 1u;
+        const uint32_t* ek = reinterpret_cast<const uint32_t*>(__shfl_sync(kFull, (unsigned long long)ent, k));
+        const uint32_t* tk = reinterpret_cast<const uint32_t*>(__shfl_sync(kFull, (unsigned long long)tab, k));
+        const int nk = __shfl_sync(kFull, items, k), lk = __shfl_sync(kFull, tlog, k);
+#pragma unroll 1
+        for (int j = kFirstItems + lane; j - lane < nk; j += 128) {
+            probed += (unsigned)min(4, (max(nk - j, 0) + 31) / 32);
+            if (__any_sync(kFull, j < nk && witness4(ek, j, 32, nk, tk, lk, d))) {
+                if (lane == k) alive = false;
+                break;
+            }
+        }
+    }
+    return __ballot_sync(kFull, alive);
 }
 
-// Gather of v's messages with hub in [lo, hi) (hi <= v: only hubs that
-// outrank v) into the set S: the frontier rows dL_{d-1}(a) of the neighbours
-// are sorted, so each row's sub-range is found by binary search.  Warp-level
-// load-balanced expansion over 32 neighbours at a time.  With M, hubs already
-// in L(v) are skipped.  Stops (returns false) when the set would exceed
-// `limit` entries.
-__device__ __forceinline__ bool gather_range(const GpParams& p, int64_t nb, int64_t ne, int64_t stride, uint32_t lo,
-                                             uint32_t hi, uint32_t* S, int log_s, const uint32_t* M, int log_m,
-                                             int limit, int* cnt_sm, volatile int* ovf_sm, unsigned long long& msgs) {
+// The cost model's reads of one candidate's check (profiled builds): L(v)'s
+// entries below h, and L(h).
+__device__ __noinline__ void count_reads(const int64_t* loff_h, const uint32_t* lv, int64_t lvlen, uint32_t h,
+                                         unsigned long long* chk) {
+    chk[0] += (unsigned long long)lower_bound_u32(lv, lvlen, pack(h, 0));
+    chk[1] += (unsigned long long)(loff_h[h + 1] - loff_h[h]);
+}
+
+// Warp tier: gather of v's messages (hubs below v of the neighbours' frontier
+// rows; the rows are sorted, so each row's share is found by binary search).
+// Hubs below vb + W are marked in the bitmap X, the others go into the set S
+// (cleared when the first of them arrives).  Warp-level load-balanced expansion
+// over 32 neighbours at a time, each step's load issued before the hubs of the
+// step before it are used.  *top: one past the highest hub marked, from vb.
+// Returns false when the set would exceed `limit` entries.
+__device__ __forceinline__ bool gather_range(const GpParams& p, int64_t nb, int64_t ne, uint32_t v, uint32_t vb,
+                                             uint32_t W, uint32_t* X, uint32_t* S, int log_s, int limit, int* cnt_sm,
+                                             uint32_t* top, unsigned long long& msgs) {
     const int lane = threadIdx.x & 31;
-    for (int64_t base = nb; base < ne; base += stride) {
+    uint32_t hmax = 0;
+    bool clean = false;
+#pragma unroll 1
+    for (int64_t base = nb; base < ne; base += 32) {
         const int64_t j = base + lane;
         int c = 0;
         int64_t st = 0;
@@ -199,52 +303,47 @@ __device__ __forceinline__ bool gather_range(const GpParams& p, int64_t nb, int6
             const uint32_t n0 = fcount(f);
             if (n0) {
                 // the hubs of a frontier row of sender a are <= a (a itself
-                // only in round 0): for a < hi the whole row lies below hi
-                const uint32_t* row = p.fhub + fstart(f);
-                const int64_t a0 = lo ? lower_bound_u32(row, n0, lo) : 0;
-                const int64_t a1 = sender_of(p, a) < hi ? (int64_t)n0 : lower_bound_u32(row, n0, hi);
-                st = (int64_t)fstart(f) + a0;
-                c = (int)(a1 - a0);
+                // only in round 0): for a < v the whole row lies below v
+                st = (int64_t)fstart(f);
+                c = sender_of(p, a) < v ? (int)n0 : (int)lower_bound_u32(p.fhub + st, n0, v);
             }
         }
         const int incl = warp_incl_scan(c, lane);
         const int total = __shfl_sync(kFull, incl, 31);
         const int excl = incl - c;
+        const uint32_t* row = p.fhub + (st - excl);  // message i of the tile, in this lane's row, is row[i]
         msgs += (lane == 0) ? (unsigned long long)total : 0ull;
-        for (int ib = 0; ib < total; ib += 32 * kGatherUnroll) {
-            uint32_t hv[kGatherUnroll];
-            // a step inside one row (long rows): every lane reads that row,
-            // no per-lane owner search
-            const int k1 = warp_owner(excl, ib);
-            const int end1 = k1 < 31 ? __shfl_sync(kFull, excl, k1 + 1) : total;
-            if (ib + 32 * kGatherUnroll <= end1) {
-                const int64_t at = __shfl_sync(kFull, st, k1) + (ib - __shfl_sync(kFull, excl, k1)) + lane;
-#pragma unroll
-                for (int u = 0; u < kGatherUnroll; ++u) hv[u] = p.fhub[at + 32 * u];
-            } else {
-#pragma unroll
-                for (int u = 0; u < kGatherUnroll; ++u) {
-                    const int it = ib + 32 * u + lane;
-                    const int k = warp_owner(excl, it);
-                    const int64_t stk = __shfl_sync(kFull, st, k);
-                    const int exk = __shfl_sync(kFull, excl, k);
-                    hv[u] = it < total ? p.fhub[stk + (it - exk)] : kEmpty;
-                }
+        uint32_t h = kEmpty;
+#pragma unroll 1
+        for (int ib = 0; ib < total + 32; ib += 32) {
+            const int it = ib + lane;
+            const int k = warp_owner(excl, it);
+            const uint32_t* rk = reinterpret_cast<const uint32_t*>(__shfl_sync(kFull, (unsigned long long)row, k));
+            const uint32_t hn = it < total ? rk[it] : kEmpty;
+            const uint32_t hr = h - vb;
+            if (hr < W) {
+                atomicOr(&X[hr >> 5], 1u << (hr & 31));
+                hmax = max(hmax, hr + 1u);
             }
-            int nins = 0;
-#pragma unroll
-            for (int u = 0; u < kGatherUnroll; ++u) {
-                const uint32_t h = hv[u];
-                if (h != kEmpty && (!M || map_find(M, log_m, h) == kEmpty)) {
-                    if (*(volatile int*)cnt_sm >= limit) *ovf_sm = 1;
-                    else nins += set_insert(S, log_s, h) ? 1 : 0;
+            const bool big = h != kEmpty && hr >= W;
+            if (__any_sync(kFull, big)) {
+                if (!clean) {
+#pragma unroll 1
+                    for (int s = lane; s < (1 << log_s); s += 32) S[s] = kEmpty;
+                    clean = true;
+                    __syncwarp();
                 }
+                int nins = 0;
+                if (big) nins = set_insert(S, log_s, h) ? 1 : 0;
+                nins = __popc(__ballot_sync(kFull, nins));
+                if (lane == 0) *cnt_sm += nins;
+                __syncwarp();
+                if (*(volatile int*)cnt_sm > limit) return false;
             }
-            nins = warp_sum(nins);
-            if (lane == 0 && nins) atomicAdd(cnt_sm, nins);
-            if (__any_sync(kFull, *ovf_sm != 0)) return false;
+            h = hn;
         }
     }
+    *top = __reduce_max_sync(kFull, hmax);
     return true;
 }
 
@@ -279,11 +378,14 @@ __device__ void shrink_pass(uint32_t* S, int log_s, uint32_t* C, int limit, uint
                             int* cnt_sm, int* hist, int* tmp) {
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int S_CAP = 1 << log_s;
+#pragma unroll 1
     while (true) {
         const uint32_t hi = *(volatile uint32_t*)hi_sm;
         const uint32_t bw = (hi - lo + 255u) / 256u;
+#pragma unroll 1
         for (int b = tid; b < 256; b += nthr) hist[b] = 0;
         __syncthreads();
+#pragma unroll 1
         for (int sl = tid; sl < S_CAP; sl += nthr) {
             const uint32_t key = S[sl];
             if (key != kEmpty && key < hi) atomicAdd(&hist[(key - lo) / bw], 1);
@@ -291,6 +393,7 @@ __device__ void shrink_pass(uint32_t* S, int log_s, uint32_t* C, int limit, uint
         __syncthreads();
         if (tid == 0) {
             int cum = 0, b = 0;
+#pragma unroll 1
             while (b < 255 && cum + hist[b] <= limit / 2) cum += hist[b++];
             if (b == 0) {  // the first bucket alone passes half the capacity: keep it whole
                 b = 1;
@@ -306,13 +409,16 @@ __device__ void shrink_pass(uint32_t* S, int log_s, uint32_t* C, int limit, uint
         const uint32_t nh = *(volatile uint32_t*)hi_sm;
         const int kept = *(volatile int*)&tmp[0];
         if (kept > limit) continue;  // narrow further (S untouched; keys >= nh are ignored)
+#pragma unroll 1
         for (int sl = tid; sl < S_CAP; sl += nthr) {
             const uint32_t key = S[sl];
             if (key != kEmpty && key < nh) C[atomicAdd(&tmp[1], 1)] = key;
         }
         __syncthreads();
+#pragma unroll 1
         for (int sl = tid; sl < S_CAP; sl += nthr) S[sl] = kEmpty;
         __syncthreads();
+#pragma unroll 1
         for (int q = tid; q < kept; q += nthr) set_insert(S, log_s, C[q]);
         if (tid == 0) *cnt_sm = kept;
         __syncthreads();
@@ -321,9 +427,10 @@ __device__ void shrink_pass(uint32_t* S, int log_s, uint32_t* C, int limit, uint
 }
 
 // Block-wide load-balanced gather of v's messages with hub in [lo, *hi_sm):
-// hubs below vb + W (vb: the first rank of v's graph) are marked in the byte
-// map B (plain stores: duplicates write the same byte, and L(v)'s hubs are
-// cleared afterwards), the others go into the set S.  Neighbours are taken in tiles of blockDim; each thread finds its
+// hubs below vb + W (vb: the first rank of v's graph) are marked in the maps B
+// (the first kByteHubs one byte each, plain stores: duplicates write the same
+// byte; the following ones one bit each; L(v)'s hubs are cleared afterwards),
+// the others go into the set S.  Neighbours are taken in tiles of blockDim; each thread finds its
 // neighbour's sub-range of dL_{d-1}(a) (binary searches in the sorted row), a
 // block-wide exclusive scan of the counts assigns every thread an equal,
 // contiguous share of the tile's messages.  When the set would exceed
@@ -338,6 +445,9 @@ __device__ void gather_block(const GpParams& p, int64_t nb, int64_t ne, uint32_t
                              unsigned long long& msgs) {
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int nw = nthr >> 5, lane = tid & 31;
+    const uint32_t Wb = min(W, (uint32_t)kByteHubs);
+    uint32_t* bits = reinterpret_cast<uint32_t*>(B + kByteHubs);
+#pragma unroll 1
     for (int64_t t0 = nb; t0 < ne; t0 += nthr) {
         const uint32_t hi = *(volatile uint32_t*)hi_sm;
         const int64_t j = t0 + tid;
@@ -377,23 +487,27 @@ __device__ void gather_block(const GpParams& p, int64_t nb, int64_t ne, uint32_t
         const int per_w = (((total + nw - 1) / nw) + 31) & ~31;
         const int wbeg = (tid >> 5) * per_w, wend = min(total, wbeg + per_w);
         int pos = wbeg;  // this warp's messages before pos are done
+#pragma unroll 1
         while (true) {
             // hubs at or above hcut are left to a later pass (hcut = hi
             // until the set's range shrinks within this tile)
             const uint32_t hcut = *(volatile uint32_t*)hi_sm;
             if (pos < wend) {
                 int k0 = 0, hk = nne - 1;  // row of pos: largest k with sex[k] <= pos
+#pragma unroll 1
                 while (k0 < hk) {
                     const int mid = (k0 + hk + 1) >> 1;
                     if (sex[mid] <= pos) k0 = mid; else hk = mid - 1;
                 }
                 bool stop = false;
+#pragma unroll 1
                 for (int it0 = pos; it0 < wend && !stop; k0 += 32) {
                     const int kr = k0 + lane;
                     const int ex = kr < nne ? sex[kr] : total;
                     const int64_t stv = kr < nne ? sst[kr] : 0;
                     const int wcap = k0 + 32 < nne ? sex[k0 + 32] : total;
                     const int wend_w = min(wend, wcap);
+#pragma unroll 1
                     for (int ib = it0; ib < wend_w; ib += 32 * kGatherUnroll) {
                         uint32_t hv[kGatherUnroll];
                         // a step inside one row (long rows): every lane reads
@@ -418,9 +532,12 @@ __device__ void gather_block(const GpParams& p, int64_t nb, int64_t ne, uint32_t
 #pragma unroll
                         for (int u = 0; u < kGatherUnroll; ++u) {
                             const uint32_t h = hv[u];
-                            if (h - vb < W) {
+                            if (h - vb < Wb) {
                                 B[h - vb] = 1;
-                            } else if (h - vb < hcut - vb && (!M || map_find(M, log_m, h) == kEmpty)) {
+                            } else if (h - vb < W) {
+                                const uint32_t q = h - vb - (uint32_t)kByteHubs;
+                                atomicOr(&bits[q >> 5], 1u << (q & 31));
+                            } else if (h - vb < hcut - vb && (!M || !map_has(M, log_m, h))) {
                                 if (*(volatile int*)cnt_sm >= limit) *ovf_sm = 1;
                                 else nins += set_insert(S, log_s, h) ? 1 : 0;
                             }
@@ -454,134 +571,217 @@ __device__ void gather_block(const GpParams& p, int64_t nb, int64_t ne, uint32_t
 }
 
 // One warp per vertex (tables in shared memory):
-//  1. stage L(v) into the hub-keyed map M (or, with few candidates against a
-//     long row, look L(v) up in v's row of the global probe index);
-//  2. gather the unique messages into the set S;
-//  3. compact S in place (L(v)'s sorted row behind it when it fits) and
-//     check the candidates 32 at a time;
-//  4. sort the accepted hubs and append them to the new frontier.
-// A vertex whose unique candidates exceed cand_limit goes to the block tier.
+//  1. gather the messages: hubs among the first 32 x M_CAP of v's graph are
+//     marked in a bitmap, the others (few: ranks follow degree) go into the set
+//     S; drop L(v)'s hubs;
+//  2. list the candidates in S, the bitmap's in rank order;
+//  3. first prefilter step; when it leaves any, stage L(v) into the hub-keyed
+//     map M, in the bitmap's place (or, with few candidates against a long row,
+//     look L(v) up in v's row of the global probe index), and check them;
+//  4. append the accepted hubs to the new frontier: in order, the set's sorted.
+// A vertex with more than cand_limit candidates in the set goes to the block
+// tier.
+// What bounds it is instruction issue (each of 24 independent warps per SM
+// issues every 12 cycles) and the instructions' way to the SM: the bitmap
+// replaced a hash set with a look-up in M per message, its compaction and a
+// bitonic sort of the accepted hubs.
 __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
     extern __shared__ uint32_t sm[];
     const int lane = lane_id(), wib = threadIdx.x >> 5;
     const int nwarps = blockDim.x >> 5;
     const int S_CAP = 1 << p.log_s, M_CAP = 1 << p.log_m;
-    int* wsc = reinterpret_cast<int*>(sm) + wib * 4;  // [0] unique count [1] overflow
+    int* wsc = reinterpret_cast<int*>(sm) + wib * 4;  // [0] entries of the set
     uint32_t* tvs = sm + 4 * nwarps;                   // per warp: v's exact-distance top-hub masks
     uint32_t* S = tvs + nwarps * kTopRow + wib * (S_CAP + M_CAP);
-    uint32_t* M = S + S_CAP;
+    uint32_t* X = S + S_CAP;                           // hub bitmap (zero between vertices), then L(v)'s map
+    uint32_t* tv = tvs + wib * kTopRow;
+    const unsigned lt = (1u << lane) - 1u;
     unsigned long long c_arcs = 0, c_msgs = 0, c_uniq = 0, c_staged = 0, c_probed = 0, c_acc = 0, c_vert = 0;
     unsigned long long c_pref = 0, c_chk[2] = {0, 0};
     if (p.ctr->done) return;
     const uint32_t d = p.ctr->d;
+    const int imax = min((int)d - 1, kTopLevels);
     const int nlist = *p.list_n;
+#pragma unroll 1
+    for (int s = lane; s < M_CAP; s += 32) X[s] = 0u;
+#pragma unroll 1
     for (int i = blockIdx.x * nwarps + wib; i < nlist; i += gridDim.x * nwarps) {
         __syncwarp();
         const int32_t v = p.list[i];
+        const uint32_t vb = base_of(p.vbase, v);
         const int64_t lb = p.loff[v], ll = p.loff[v + 1] - lb;
-        // tables sized for this vertex: the set for its candidate bound (when
-        // within the tier's limit), the map for |L(v)| (load <= 1/2)
-        const uint32_t bnd = p.rbound[v];
-        const int log_s = bnd <= (uint32_t)p.cand_limit ? max(5, ceil_log2_i64(2 * (int64_t)bnd)) : p.log_s;
-        // L(v) lookups: the map staged in shared memory, or, for a receiver
-        // with few candidates against a long (indexed) row, v's row of the
-        // global probe index, which saves staging the whole row
-        const uint64_t hdv = (p.stage_ratio > 0 && ll >= kIndexMinLen &&
-                              (int64_t)bnd * p.stage_ratio < ll) ? p.hdesc[v] : 0ull;
-        const bool mglob = hdv != 0;
-        const int log_m = mglob ? (int)(hdv & 0xFFu) : max(5, ceil_log2_i64(2 * ll));
-        const uint32_t* Mv = mglob ? p.htab + (hdv >> 8) : M;
-        for (int s = lane; s < (1 << log_s); s += 32) S[s] = kEmpty;
-        if (!mglob)
-            for (int s = lane; s < (1 << log_m); s += 32) M[s] = kEmpty;
-        if (lane == 0) {
-            wsc[0] = 0;
-            wsc[1] = 0;
-        }
-        __syncwarp();
-        if (!mglob)
-            for (int64_t j = lane; j < ll; j += 32) map_insert(M, log_m, p.lent[lb + j]);
-        __syncwarp();
         const int64_t nb = p.roff[v], ne = p.roff[v + 1];
-        const bool ok = gather_range(p, nb, ne, 32, 0u, (uint32_t)v, S, log_s, Mv, log_m, p.cand_limit, &wsc[0],
-                                     (volatile int*)&wsc[1], c_msgs);
+        const uint32_t* lv = p.lent + lb;
+        const uint32_t bnd = p.rbound[v];
+        // the set sized for v's candidate bound (when within the tier's limit)
+        const int log_s = bnd <= (uint32_t)p.cand_limit ? max(5, ceil_log2_i64(2 * (int64_t)bnd)) : p.log_s;
+        const uint32_t W = min(32u * (uint32_t)M_CAP, (uint32_t)v - vb);
+        if (lane == 0) wsc[0] = 0;
         __syncwarp();
-        const int nS = *(volatile int*)&wsc[0];
-        if (!ok || nS > p.cand_limit) {
+        uint32_t top = 0;
+        const bool ok = gather_range(p, nb, ne, (uint32_t)v, vb, W, X, S, log_s, p.cand_limit, &wsc[0], &top, c_msgs);
+        __syncwarp();
+        // candidates: the bitmap's without L(v)'s hubs ...
+        const int words = (int)((top + 31u) >> 5);
+        int nbm = 0, nset = 0;
+        if (ok) {
+#pragma unroll 1
+            for (int64_t j = lane; j < ll; j += 32) {
+                const uint32_t w = hub_of(lv[j]) - vb;
+                if (w < top) atomicAnd(&X[w >> 5], ~(1u << (w & 31)));
+            }
+            __syncwarp();
+            // ... and the set's, compacted in place (write position never
+            // passes the read position)
+            if (*(volatile int*)&wsc[0] > 0) {
+#pragma unroll 1
+                for (int q = lane; q < words; q += 32) nbm += __popc(X[q]);
+                nbm = warp_sum(nbm);
+#pragma unroll 1
+                for (int sb = 0; sb < (1 << log_s); sb += 32) {
+                    const uint32_t h = S[sb + lane];
+                    __syncwarp();
+                    bool has = h != kEmpty;
+                    if (has) {
+                        const int64_t at = lower_bound_u32(lv, ll, pack(h, 0));
+                        has = at >= ll || hub_of(lv[at]) != h;
+                    }
+                    const unsigned m = __ballot_sync(kFull, has);
+                    if (has) S[nset + __popc(m & lt)] = h;
+                    nset += __popc(m);
+                }
+                __syncwarp();
+            }
+        }
+        if (!ok || nbm + nset > S_CAP) {
+#pragma unroll 1
+            for (int q = lane; q < (int)((W + 31u) >> 5); q += 32) X[q] = 0u;
             if (lane == 0) {
                 const int o = atomicAdd(p.esc_n, 1);
                 p.esc[o] = v;
             }
             continue;
         }
+        // list them: the set's moved up behind the bitmap's
+        if (nset > 0 && nbm > 0) {
+#pragma unroll 1
+            for (int c = (nset - 1) & ~31; c >= 0; c -= 32) {
+                const uint32_t h = c + lane < nset ? S[c + lane] : 0u;
+                __syncwarp();
+                if (c + lane < nset) S[nbm + c + lane] = h;
+                __syncwarp();
+            }
+        }
+        int nc = 0;
+#pragma unroll 1
+        for (int q0 = 0; q0 < words; q0 += 128) {  // four words (128 hubs) per lane
+            uint4* x4 = reinterpret_cast<uint4*>(X + q0) + lane;
+            uint4 y = make_uint4(0u, 0u, 0u, 0u);
+            if (q0 + 4 * lane < words) y = *x4;
+            if (!__any_sync(kFull, (y.x | y.y | y.z | y.w) != 0u)) continue;
+            const int c = __popc(y.x) + __popc(y.y) + __popc(y.z) + __popc(y.w);
+            const int incl = warp_incl_scan(c, lane);
+            uint32_t* o = S + nc + incl - c;
+            uint32_t hb = vb + 32u * (uint32_t)(q0 + 4 * lane) - 1u;
+            if (c) *x4 = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 1
+            for (; y.x; y.x &= y.x - 1u) *o++ = hb + (uint32_t)__ffs(y.x);
+            hb += 32u;
+#pragma unroll 1
+            for (; y.y; y.y &= y.y - 1u) *o++ = hb + (uint32_t)__ffs(y.y);
+            hb += 32u;
+#pragma unroll 1
+            for (; y.z; y.z &= y.z - 1u) *o++ = hb + (uint32_t)__ffs(y.z);
+            hb += 32u;
+#pragma unroll 1
+            for (; y.w; y.w &= y.w - 1u) *o++ = hb + (uint32_t)__ffs(y.w);
+            nc += __shfl_sync(kFull, incl, 31);
+        }
+        nc += nset;
+        __syncwarp();
         if (lane == 0) {
             c_arcs += ne - nb;
-            c_staged += mglob ? 0 : ll;
             c_vert += 1;
-            c_uniq += nS;
+            c_uniq += nc;
         }
-        // compact the set in place (write position never passes the read position)
-        int nc = 0;
-        for (int sb = 0; sb < (1 << log_s); sb += 32) {
-            const uint32_t h = S[sb + lane];
-            __syncwarp();
-            const bool has = h != kEmpty;
-            const unsigned m = __ballot_sync(kFull, has);
-            if (has) S[nc + __popc(m & ((1u << lane) - 1u))] = h;
-            nc += __popc(m);
-        }
+        if (nc == 0) continue;
+        stage_exact_levels(p.top, p.n, v, tv, lane, 32);
         __syncwarp();
+        // first prefilter step, 64 candidates at a time, then the distance
+        // checks of its survivors, 32 at a time; both compact S in place and in
+        // order.  A single chunk goes to the checks at once (i0 = 0: the masks
+        // and the check records of its candidates are then requested together)
+        int i0 = 0, ns = nc;
+        if (p.count_check)
+#pragma unroll 1
+            for (int j = lane; j < nc; j += 32) count_reads(p.loff_h, lv, ll, S[j], c_chk);
+        if (nc > 32) {
+            i0 = first_level(tv, imax, lane);
+            ns = 0;
+#pragma unroll 1
+            for (int cb = 0; cb < nc; cb += 64) {
+                const bool v0 = cb + lane < nc, v1 = cb + 32 + lane < nc;
+                const uint32_t h0 = v0 ? S[cb + lane] : 0u, h1 = v1 ? S[cb + 32 + lane] : 0u;
+                unsigned m0, m1;
+                prefilter_first(p, tv, (int)d, imax, i0, h0, v0, h1, v1, &m0, &m1);
+                if ((m0 >> lane) & 1u) S[ns + __popc(m0 & lt)] = h0;
+                ns += __popc(m0);
+                if ((m1 >> lane) & 1u) S[ns + __popc(m1 & lt)] = h1;
+                ns += __popc(m1);
+                __syncwarp();
+            }
+            if (lane == 0) c_pref += nc - ns;
+            if (ns == 0) continue;
+        }
+        // L(v) look-ups: the map staged in shared memory, or, for a receiver
+        // with few candidates against a long (indexed) row, v's row of the
+        // global probe index, which saves staging the whole row
+        const uint64_t hdv = (p.stage_ratio > 0 && ll >= kIndexMinLen &&
+                              (int64_t)bnd * p.stage_ratio < ll) ? p.hdesc[v] : 0ull;
+        const bool mglob = hdv != 0;
+        const int log_m = mglob ? (int)(hdv & 0xFFu) : max(5, ceil_log2_i64(2 * ll));
+        const uint32_t* Mv = mglob ? p.htab + (hdv >> 8) : X;
         // L(v)'s sorted row, copied behind the candidates (the set's slots
-        // past nc are free now) when it fits: the checks' binary searches in
+        // past ns are free now) when it fits: the checks' binary searches in
         // L(v) and their side-B scans of it then read shared memory
-        const uint32_t* lvp = p.lent + lb;
-        if (nc > 0 && (int64_t)nc + ll <= S_CAP) {
-            uint32_t* lvs = S + (S_CAP - ll);
-            for (int64_t j = lane; j < ll; j += 32) lvs[j] = p.lent[lb + j];
-            lvp = lvs;
+        const uint32_t* lvp = lv;
+        const bool copy = (int64_t)ns + ll <= S_CAP;
+        uint32_t* lvs = S + (S_CAP - ll);
+        if (copy) lvp = lvs;
+        if (!mglob) {
+#pragma unroll 1
+            for (int s = lane; s < (1 << log_m); s += 32) X[s] = kEmpty;
+            __syncwarp();
         }
-        // entries of L(v) with a top hub (the checks' side B starts past them)
-        const int lv_top =
-            nc > 0 ? (int)lower_bound_u32(lvp, ll, pack(base_of(p.vbase, v) + (uint32_t)kTopHubs, 0)) : 0;
-        // distance checks, 32 candidates at a time; survivors compacted in place
-        uint32_t* tv = tvs + wib * kTopRow;
-        if (nc > 0) stage_exact_levels(p.top, v, tv, lane, 32);
+        if (!mglob || copy) {
+#pragma unroll 1
+            for (int64_t j = lane; j < ll; j += 32) {
+                const uint32_t e = lv[j];
+                if (!mglob) map_insert(X, log_m, e);
+                if (copy) lvs[j] = e;
+            }
+        }
+        if (lane == 0) c_staged += mglob ? 0 : ll;
         __syncwarp();
-        int nacc = 0;
-        for (int cb = 0; cb < nc; cb += 32) {
-            const bool valid = cb + lane < nc;
+        // entries of L(v) with a top hub (the checks' side B starts past them)
+        const int lv_top = (int)lower_bound_u32(lvp, ll, pack(vb + (uint32_t)kTopHubs, 0));
+        int nacc = 0, ntail = 0;  // accepted; of them past the bitmap's hubs
+#pragma unroll 1
+        for (int cb = 0; cb < ns; cb += 32) {
+            const bool valid = cb + lane < ns;
             const uint32_t h = valid ? S[cb + lane] : 0u;
             __syncwarp();
             const unsigned okm = check_chunk(p, d, Mv, log_m, mglob, kWarpSideBMin, kWarpSideBShift, lvp, ll, lv_top,
-                                             h, valid, c_probed, tv, c_pref, c_chk);
-            if ((okm >> lane) & 1u) S[nacc + __popc(okm & ((1u << lane) - 1u))] = h;
+                                             h, valid, c_probed, tv, i0, c_pref);
+            const bool acc = (okm >> lane) & 1u;
+            if (acc) S[nacc + __popc(okm & lt)] = h;
             nacc += __popc(okm);
+            if (nset > 0) ntail += __popc(__ballot_sync(kFull, acc && h - vb >= W));
             __syncwarp();
         }
-        // the new row leaves sorted by hub rank: bitonic sort of S[0, nacc)
-        // (nacc <= cand_limit, a power of two at most half the set's slots)
-        if (nacc > 1) {
-            if (nacc <= 32) {
-                uint32_t x = lane < nacc ? S[lane] : kEmpty;
-#pragma unroll
-                for (int k = 2; k <= 32; k <<= 1) {
-#pragma unroll
-                    for (int j = k >> 1; j > 0; j >>= 1) {
-                        const uint32_t y = __shfl_xor_sync(kFull, x, j);
-                        const bool up = (lane & k) == 0, lower = (lane & j) == 0;
-                        x = (lower == up) ? min(x, y) : max(x, y);
-                    }
-                }
-                if (lane < nacc) S[lane] = x;
-            } else {
-                int P = 64;
-                while (P < nacc) P <<= 1;
-                for (int j = nacc + lane; j < P; j += 32) S[j] = kEmpty;
-                __syncwarp();
-                group_bitonic_sort(S, P, lane, 32, WarpSync());
-            }
-            __syncwarp();
-        }
+        if (!mglob)
+#pragma unroll 1
+            for (int s = lane; s < (1 << log_m); s += 32) X[s] = 0u;
         if (nacc > 0) {
             unsigned long long start = 0;
             if (lane == 0)
@@ -589,7 +789,27 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
                                  : atomicAdd(&p.ctr->cursor, (unsigned long long)nacc);
             start = __shfl_sync(kFull, start, 0);
             if (start + nacc <= p.fcap) {
-                for (int j = lane; j < nacc; j += 32) p.fhub_new[start + j] = S[j];
+                uint32_t* row = p.fhub_new + start;
+                // the new row leaves sorted by hub rank: the bitmap's hubs as
+                // they are, then the set's, moved to the front of S and sorted
+                const int n0 = nacc - ntail;
+#pragma unroll 1
+                for (int j = lane; j < n0; j += 32) row[j] = S[j];
+                if (ntail > 0) {
+                    int P = 32;
+#pragma unroll 1
+                    while (P < ntail) P <<= 1;  // <= S_CAP: at most cand_limit, half of it
+#pragma unroll 1
+                    for (int j0 = 0; j0 < P; j0 += 32) {
+                        const uint32_t h = j0 + lane < ntail ? S[n0 + j0 + lane] : kEmpty;
+                        __syncwarp();
+                        S[j0 + lane] = h;
+                        __syncwarp();
+                    }
+                    group_bitonic_sort(S, P, lane, 32, WarpSync());
+#pragma unroll 1
+                    for (int j = lane; j < ntail; j += 32) row[n0 + j] = S[j];
+                }
                 if (lane == 0) p.fse_new[v] = fpack(start, (uint32_t)nacc);
             } else if (lane == 0) {
                 p.ctr->fovf = 1;
@@ -620,20 +840,140 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
 }
 
 // Block-per-vertex scalars in shared memory (ints)
-enum { SH_UNIQ = 0, SH_OVF = 1, SH_ACC = 2, SH_NC = 3, SH_HI = 4, SH_TMP = 5, SH_START = 6 /* 2 ints */, SH_NEXT = 8,
-       SH_WORDS = 48 };
+enum { SH_UNIQ = 0, SH_OVF = 1, SH_ACC = 2 /* accepted, from the set */, SH_NC = 3, SH_HI = 4, SH_TMP = 5 /* 2 ints */,
+       SH_START = 8 /* 2 ints */, SH_NEXT = 10, SH_REST = 11, SH_MACC = 12 /* accepted, from the maps */,
+       SH_WCNT = 16 /* 2 x 8 warps */, SH_WORDS = 48 };
+
+// Accepted candidates of a chunk (okm): those of the maps are marked there
+// again (extraction cleared them), the set's go to this block's global scratch.
+__device__ __forceinline__ void keep_accepted(unsigned okm, uint32_t h, uint32_t vb, uint32_t W, uint8_t* B,
+                                              uint32_t* gacc, int* sh) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t hr = h - vb;
+    const bool ok = (okm >> lane) & 1u, inmap = hr < W;
+    if (ok && inmap) {
+        if (hr < (uint32_t)kByteHubs) {
+            B[hr] = 1;
+        } else {
+            const uint32_t q = hr - (uint32_t)kByteHubs;
+            atomicOr(reinterpret_cast<uint32_t*>(B + kByteHubs) + (q >> 5), 1u << (q & 31));
+        }
+    }
+    const unsigned mm = __ballot_sync(kFull, ok && inmap), ms = okm & ~mm;
+    int base = 0;
+    if (lane == 0) {
+        if (mm) atomicAdd(&sh[SH_MACC], __popc(mm));
+        if (ms) base = atomicAdd(&sh[SH_ACC], __popc(ms));
+    }
+    base = __shfl_sync(kFull, base, 0);
+    if (ok && !inmap) gacc[base + __popc(ms & ((1u << lane) - 1u))] = h;
+}
+
+// The bytes of four map words as 16 bits.
+__device__ __forceinline__ uint32_t byte_bits(uint32_t x) {
+    return (x & 1u) | ((x >> 7) & 2u) | ((x >> 14) & 4u) | ((x >> 21) & 8u);
+}
+__device__ __forceinline__ uint32_t byte_bits4(uint4 x) {
+    return byte_bits(x.x) | (byte_bits(x.y) << 4) | (byte_bits(x.z) << 8) | (byte_bits(x.w) << 12);
+}
+
+// Emits the marked hubs of the maps (W hubs from vb) to row in rank order and
+// clears them (row null: only clears).  Warp w takes the w-th slice of the
+// byte map and of the bitmap; all byte-map hubs precede the bitmap's.
+__device__ void emit_maps(uint8_t* B, uint32_t vb, uint32_t W, uint32_t* row, int* sh) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+    uint4* b4 = reinterpret_cast<uint4*>(B);
+    uint4* w4 = reinterpret_cast<uint4*>(B + kByteHubs);
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t Wb = min(W, (uint32_t)kByteHubs);
+    // units of 32 lanes x 16 bytes: 16 hubs per lane in the byte map, 128 in the bitmap
+    const int ub = (int)((Wb + 511) / 512), uw = (int)((W - Wb + 4095) / 4096);
+    const int b0 = ub * wid / nw, b1 = ub * (wid + 1) / nw, w0 = uw * wid / nw, w1 = uw * (wid + 1) / nw;
+    int cb = 0, cw = 0;
+#pragma unroll 1
+    for (int u = b0; u < b1; ++u) {
+        const uint4 x = b4[32 * u + lane];
+        cb += __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);  // one bit per marked byte
+    }
+#pragma unroll 1
+    for (int u = w0; u < w1; ++u) {
+        const uint4 x = w4[32 * u + lane];
+        cw += __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);
+    }
+    cb = warp_sum(cb);
+    cw = warp_sum(cw);
+    if (lane == 0) {
+        sh[SH_WCNT + wid] = cb;
+        sh[SH_WCNT + nw + wid] = cw;
+    }
+    __syncthreads();
+    const int c = lane < 2 * nw ? sh[SH_WCNT + lane] : 0;
+    const int before = warp_incl_scan(c, lane) - c;
+    int pos = __shfl_sync(kFull, before, wid);
+    if (cb > 0) {
+#pragma unroll 1
+        for (int u = b0; u < b1; ++u) {
+            const int x = 32 * u + lane;
+            uint32_t w = byte_bits4(b4[x]);
+            if (!__any_sync(kFull, w != 0u)) continue;
+            const int k = __popc(w);
+            const int incl = warp_incl_scan(k, lane);
+            int o = pos + incl - k;
+            const uint32_t hb = vb - 1u + 16u * (uint32_t)x;
+            if (w) b4[x] = zero;
+            if (row)
+#pragma unroll 1
+                for (; w; w &= w - 1u) row[o++] = hb + (uint32_t)__ffs(w);
+            pos += __shfl_sync(kFull, incl, 31);
+        }
+    }
+    pos = __shfl_sync(kFull, before, nw + wid);
+    if (cw > 0) {
+#pragma unroll 1
+        for (int u = w0; u < w1; ++u) {
+            const int x = 32 * u + lane;
+            const uint4 y = w4[x];
+            if (!__any_sync(kFull, (y.x | y.y | y.z | y.w) != 0u)) continue;
+            const int k = __popc(y.x) + __popc(y.y) + __popc(y.z) + __popc(y.w);
+            const int incl = warp_incl_scan(k, lane);
+            int o = pos + incl - k;
+            if (k) w4[x] = zero;
+            if (row && k) {
+                const uint32_t q[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint32_t hb = vb - 1u + (uint32_t)kByteHubs + 128u * (uint32_t)x + 32u * (uint32_t)j;
+#pragma unroll 1
+                    for (uint32_t w = q[j]; w; w &= w - 1u) row[o++] = hb + (uint32_t)__ffs(w);
+                }
+            }
+            pos += __shfl_sync(kFull, incl, 31);
+        }
+    }
+}
 
 // One block per vertex, any size.  The candidates are processed in passes
 // over hub ranges [lo, hi): each pass gathers the messages of its range into
-// the shared-memory set (shrinking hi when the set would overflow), checks
-// them and appends the survivors to this block's global scratch, copied to
-// the new frontier at the end.  L(v) is staged into the shared-memory map when it fits;
-// otherwise membership in L(v) is a binary search in its row.
+// the hub maps (the first pass) and the shared-memory set (shrinking hi when
+// the set would overflow) and checks them.
+//
+// What bounds it is latency: three blocks of 8 warps per SM wait on random
+// 32-byte sectors (masks, check records, probe tables) of arrays far larger
+// than L2, and one chunk of 32 candidates checked from end to end took 5,000
+// to 12,000 cycles although most of its candidates need one mask only.  So the
+// check is split: each warp takes units of the maps and of the set from a
+// shared counter, stages 64 candidates, tests one mask of each (two
+// independent sectors per lane), and runs check_chunk on full warps of
+// survivors; the warps' last survivors are pooled and spread over all warps.
+// L(v) is staged into the shared-memory map when it fits; otherwise it is
+// looked up in v's row of the global probe index.  Accepted hubs are marked in
+// the maps and leave them in rank order, so the new row needs no later sort.
 __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32_t* S, uint32_t* M, uint32_t* C,
                                 uint8_t* B, uint32_t* gacc, int* sh, int* wsum, int* sex, int64_t* sst, int* hist,
                                 uint32_t* tv, unsigned long long* cnt) {
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int lane = tid & 31, wid = tid >> 5, nw = nthr >> 5;
+    const unsigned lt = (1u << lane) - 1u;
     const int64_t lb = p.loff[v], ll = p.loff[v + 1] - lb;
     const int64_t nb = p.roff[v], ne = p.roff[v + 1];
     const uint32_t* lv = p.lent + lb;
@@ -653,35 +993,48 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
         log_mp = (int)(hd & 0xFFu);
     }
     if (useM) {
+#pragma unroll 1
         for (int s = tid; s < (1 << log_m); s += nthr) M[s] = kEmpty;
         __syncthreads();
+#pragma unroll 1
         for (int64_t j = tid; j < ll; j += nthr) map_insert(M, log_m, lv[j]);
     }
     if (tid == 0) {
         cnt[0] += ne - nb;
         cnt[3] += ll;
         cnt[6] += 1;
+        sh[SH_ACC] = 0;
+        sh[SH_MACC] = 0;
     }
-    stage_exact_levels(p.top, v, tv, tid, nthr);
-    int64_t total_acc = 0;
+    stage_exact_levels(p.top, p.n, v, tv, tid, nthr);
     const uint32_t vb = base_of(p.vbase, v);  // v's hubs are ranks [vb, v)
     uint32_t lo = vb;
     int64_t width = (int64_t)v - vb;
     uint32_t* hi_sm = reinterpret_cast<uint32_t*>(&sh[SH_HI]);
-    // hubs below vb + W (the most frequent messages) are deduplicated in the byte
-    // map, in the first pass, for vertices with many messages (for the others
-    // clearing and scanning the map costs more than the hashing it saves)
-    const uint32_t W = p.rbound[v] >= kByteMinBound ? min((uint32_t)kByteHubs, (uint32_t)v - vb) : 0u;
-    const int nbw = (int)((W + 3) / 4);  // byte-map words in use
-    for (int q = tid; q < nbw; q += nthr) reinterpret_cast<uint32_t*>(B)[q] = 0u;
-    while ((int64_t)lo < (int64_t)v) {
-        for (int s = tid; s < S_CAP; s += nthr) S[s] = kEmpty;
+    // hubs below vb + W (the most frequent messages) are deduplicated in the
+    // maps, in the first pass, for vertices with many messages (for the others
+    // scanning the maps costs more than the hashing it saves)
+    const uint32_t W =
+        p.rbound[v] >= kByteMinBound ? min((uint32_t)(kByteHubs + kBitHubs), (uint32_t)v - vb) : 0u;
+    const uint32_t Wb = min(W, (uint32_t)kByteHubs);
+    uint4* b4 = reinterpret_cast<uint4*>(B);
+    uint32_t* bits = reinterpret_cast<uint32_t*>(B + kByteHubs);
+    uint32_t* stage = S + wid * kWarpStage;  // (S is free once compacted)
+    uint32_t* surv = stage + kCandStage;
+    const int imax = min((int)d - 1, kTopLevels);
+#pragma unroll 1
+    while (lo < (uint32_t)v) {
+        if (lo > vb || (uint32_t)v - vb > W) {  // (no message reaches the set when the maps hold every hub of v)
+            uint4* s4 = reinterpret_cast<uint4*>(S);
+#pragma unroll 1
+            for (int s = tid; s < S_CAP / 4; s += nthr) s4[s] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+        }
         if (tid == 0) {
             sh[SH_UNIQ] = 0;
             sh[SH_OVF] = 0;
-            sh[SH_ACC] = 0;
             sh[SH_NC] = 0;
             sh[SH_NEXT] = 0;
+            sh[SH_REST] = 0;
             *hi_sm = (uint32_t)min((int64_t)v, (int64_t)lo + width);
         }
         __syncthreads();
@@ -689,117 +1042,150 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
                      (volatile int*)&sh[SH_OVF], wsum, sex, sst, C, hist, &sh[SH_TMP], cnt[1]);
         __syncthreads();
         const uint32_t hi = *(volatile uint32_t*)hi_sm;
-        if (lo - vb < W) {  // first pass: drop L(v)'s hubs from the byte map
+        const bool maps = lo == vb && W > 0;
+        if (maps) {  // first pass: drop L(v)'s hubs from the maps
+#pragma unroll 1
             for (int64_t j = tid; j < ll; j += nthr) {
                 const uint32_t w = hub_of(lv[j]) - vb;
-                if (w < W) B[w] = 0;
+                if (w < Wb) B[w] = 0;
+                else if (w < W) atomicAnd(&bits[(w - kByteHubs) >> 5], ~(1u << (w & 31)));
             }
         }
         // compact the set into C (any order)
-        for (int sb = 32 * wid; sb < S_CAP; sb += 32 * nw) {
-            const uint32_t h = S[sb + lane];
-            const bool has = h != kEmpty;
-            const unsigned m = __ballot_sync(kFull, has);
-            int base = 0;
-            if (lane == 0 && m) base = atomicAdd(&sh[SH_NC], __popc(m));
-            base = __shfl_sync(kFull, base, 0);
-            const int idx = base + __popc(m & ((1u << lane) - 1u));
-            if (has) {
-                if (idx < limit) C[idx] = h;
-                else p.ctr->guard = 1;  // invariant broken: report instead of writing out of bounds
+        if (*(volatile int*)&sh[SH_UNIQ] > 0) {
+#pragma unroll 1
+            for (int sb = 32 * wid; sb < S_CAP; sb += 32 * nw) {
+                const uint32_t h = S[sb + lane];
+                const bool has = h != kEmpty;
+                const unsigned m = __ballot_sync(kFull, has);
+                int base = 0;
+                if (lane == 0 && m) base = atomicAdd(&sh[SH_NC], __popc(m));
+                base = __shfl_sync(kFull, base, 0);
+                const int idx = base + __popc(m & lt);
+                if (has) {
+                    if (idx < limit) C[idx] = h;
+                    else p.ctr->guard = 1;  // invariant broken: report instead of writing out of bounds
+                }
             }
         }
         __syncthreads();  // every warp has read the set
-        // L(v)'s sorted row in the set's free tail (the byte-map staging below
-        // uses its head): the checks' binary searches in L(v) and their side-B
+        // L(v)'s sorted row in the set's free tail (its head stages the warps'
+        // candidates): the checks' binary searches in L(v) and their side-B
         // scans of it then read shared memory
         const uint32_t* lvp = lv;
-        if (ll + (int64_t)nw * kByteStage <= (int64_t)S_CAP) {
+        if (ll + (int64_t)nw * kWarpStage <= (int64_t)S_CAP) {
             uint32_t* lvs = S + (S_CAP - ll);
+#pragma unroll 1
             for (int64_t j = tid; j < ll; j += nthr) lvs[j] = lv[j];
             lvp = lvs;
         }
         __syncthreads();
         // entries of L(v) with a top hub (the checks' side B starts past them)
         const int lv_top = (int)lower_bound_u32(lvp, ll, pack(vb + (uint32_t)kTopHubs, 0));
+        const int i0 = first_level(tv, imax, lane);
         const int nc_set = min(*(volatile int*)&sh[SH_NC], limit);  // candidates from the set
-        if (tid == 0) cnt[2] += nc_set;
-        if (lo - vb < W) {
-            // the byte-map candidates: each warp extracts 32 words (up to 128
-            // hubs) at a time into its slice of S (free after the compaction;
-            // kByteStage words per warp), checks them in full chunks of 32 and
-            // carries the remainder; its final remainder (< 32) joins C
-            uint32_t* stage = S + wid * kByteStage;
-            int f = 0;  // candidates staged
-            for (int g = 32 * wid; g < nbw; g += 32 * nw) {
-                const uint32_t x = g + lane < nbw ? reinterpret_cast<const uint32_t*>(B)[g + lane] : 0u;
-                const uint32_t b4 = (x & 1u) | ((x >> 7) & 2u) | ((x >> 14) & 4u) | ((x >> 21) & 8u);
-                const int c = __popc(b4);
-                const int incl = warp_incl_scan(c, lane);
-                const int tot = __shfl_sync(kFull, incl, 31);
-                int o = f + incl - c;
-                for (int b = 0; b < 4; ++b)
-                    if ((b4 >> b) & 1u) stage[o++] = vb + 4u * (uint32_t)(g + lane) + (uint32_t)b;
-                if (lane == 0) cnt[2] += tot;
-                f += tot;
-                __syncwarp();
-                const int nchk = f & ~31;
-                for (int cb = 0; cb < nchk; cb += 32) {
-                    const uint32_t h = stage[cb + lane];
-                    const unsigned okm = check_chunk(p, d, Mp, log_mp, !useM, kBlockSideBMin, kBlockSideBShift, lvp,
-                                                     ll, lv_top, h, true, cnt[4], tv, cnt[7], cnt + 8);
-                    int base = 0;
-                    if (lane == 0 && okm) base = atomicAdd(&sh[SH_ACC], __popc(okm));
-                    base = __shfl_sync(kFull, base, 0);
-                    if ((okm >> lane) & 1u) gacc[total_acc + base + __popc(okm & ((1u << lane) - 1u))] = h;
+        // units of the maps (32 lanes x 16 bytes, 32 lanes x 32 bits, cleared
+        // as they are read) and of the set's candidates (32)
+        const int ub = maps ? (int)((Wb + 511) / 512) : 0, uw = maps ? (int)((W - Wb + 1023) / 1024) : 0;
+        const int units = ub + uw + (nc_set + 31) / 32;
+        bool more = true, last = false;
+        int nf = 0, ns = 0;        // staged candidates, survivors
+        uint32_t w = 0, hb = 0;    // this lane's candidates of the current unit: hub hb + b for every bit b of w
+#pragma unroll 1
+        while (!last) {
+#pragma unroll 1
+            while (nf < 64 && more) {
+                const unsigned m = __ballot_sync(kFull, w != 0u);
+                if (m) {
+                    if (w) {
+                        stage[nf + __popc(m & lt)] = hb + (uint32_t)(__ffs(w) - 1);
+                        w &= w - 1u;
+                    }
+                    nf += __popc(m);
+                    continue;
                 }
-                const int rem = f - nchk;
-                uint32_t carry = 0u;
-                if (lane < rem) carry = stage[nchk + lane];
-                __syncwarp();
-                if (lane < rem) stage[lane] = carry;
-                f = rem;
-                __syncwarp();
+                int u = 0;
+                if (lane == 0) u = atomicAdd(&sh[SH_NEXT], 1);
+                u = __shfl_sync(kFull, u, 0);
+                if (u >= units) {
+                    more = false;
+                } else if (u < ub) {
+                    const int x = 32 * u + lane;
+                    w = byte_bits4(b4[x]);
+                    if (w) b4[x] = make_uint4(0u, 0u, 0u, 0u);
+                    hb = vb + 16u * (uint32_t)x;
+                } else if (u < ub + uw) {
+                    const int x = 32 * (u - ub) + lane;
+                    w = bits[x];
+                    if (w) bits[x] = 0u;
+                    hb = vb + (uint32_t)kByteHubs + 32u * (uint32_t)x;
+                } else {
+                    const int x = 32 * (u - ub - uw) + lane;
+                    w = x < nc_set ? 1u : 0u;
+                    hb = x < nc_set ? C[x] : 0u;
+                    // without the map, set candidates may be hubs of v already
+                    if (!useM && w && map_has(Mp, log_mp, hb)) w = 0u;
+                }
             }
-            int base = 0;
-            if (lane == 0 && f) base = atomicAdd(&sh[SH_NC], f);
-            base = __shfl_sync(kFull, base, 0);
-            if (lane < f) C[base + lane] = stage[lane];  // C holds limit + 32 per warp
-            __syncthreads();
-        }
-        // distance checks of C (the set's candidates, then the byte map's
-        // remainders): each warp takes the next chunk of 32 from a shared
-        // counter (chunks differ in cost); the survivors are appended
-        // (unsorted) to this block's scratch
-        const int nc = *(volatile int*)&sh[SH_NC];
-        for (;;) {
-            int cb = 0;
-            if (lane == 0) cb = atomicAdd(&sh[SH_NEXT], 32);
-            cb = __shfl_sync(kFull, cb, 0);
-            if (cb >= nc) break;
-            bool valid = cb + lane < nc;
-            const uint32_t h = valid ? C[cb + lane] : 0u;
-            // without the map, set candidates may be hubs of v already (they
-            // were counted as unique candidates: take them back)
-            if (!useM) {
-                const bool known = valid && cb + lane < nc_set && map_find(Mp, log_mp, h) != kEmpty;
-                const unsigned km = __ballot_sync(kFull, known);
-                if (lane == 0) cnt[2] -= __popc(km);
-                if (known) valid = false;
+            if (nf > 0) {
+                __syncwarp();
+                // first prefilter step: the last 64 staged candidates (fewer at the end)
+                const int k = min(nf, 64), s0 = nf - k;
+                const bool v0 = lane < k, v1 = lane + 32 < k;
+                const uint32_t h0 = v0 ? stage[s0 + lane] : 0u, h1 = v1 ? stage[s0 + 32 + lane] : 0u;
+                nf = s0;
+                if (p.count_check) {
+                    if (v0) count_reads(p.loff_h, lvp, ll, h0, cnt + 8);
+                    if (v1) count_reads(p.loff_h, lvp, ll, h1, cnt + 8);
+                }
+                unsigned m0, m1;
+                prefilter_first(p, tv, (int)d, imax, i0, h0, v0, h1, v1, &m0, &m1);
+                if ((m0 >> lane) & 1u) surv[ns + __popc(m0 & lt)] = h0;
+                ns += __popc(m0);
+                if ((m1 >> lane) & 1u) surv[ns + __popc(m1 & lt)] = h1;
+                ns += __popc(m1);
+                if (lane == 0) {
+                    cnt[2] += k;
+                    cnt[7] += k - __popc(m0) - __popc(m1);
+                }
+                __syncwarp();
+            } else {
+                // no unit is left: the warps' last survivors (fewer than 32
+                // each) are pooled behind C's candidates and spread over the
+                // warps, so that one warp's scans are not what the others wait for
+                int base = 0;
+                if (lane == 0 && ns) base = atomicAdd(&sh[SH_REST], ns);
+                base = __shfl_sync(kFull, base, 0);
+                if (lane < ns) C[limit + base + lane] = surv[lane];
+                __syncthreads();
+                const int nrest = *(volatile int*)&sh[SH_REST];
+                const int per = max(4, (nrest + nw - 1) / nw);  // at most 31
+                ns = max(0, min(per, nrest - wid * per));
+                if (lane < ns) surv[lane] = C[limit + wid * per + lane];
+                __syncwarp();
+                last = true;
             }
-            const unsigned okm = check_chunk(p, d, Mp, log_mp, !useM, kBlockSideBMin, kBlockSideBShift, lvp, ll,
-                                             lv_top, h, valid, cnt[4], tv, cnt[7], cnt + 8);
-            int base = 0;
-            if (lane == 0 && okm) base = atomicAdd(&sh[SH_ACC], __popc(okm));
-            base = __shfl_sync(kFull, base, 0);
-            if ((okm >> lane) & 1u) gacc[total_acc + base + __popc(okm & ((1u << lane) - 1u))] = h;
+#pragma unroll 1
+            while (ns >= 32 || (last && ns > 0)) {
+                const int k = min(ns, 32);
+                ns -= k;
+                const bool valid = lane < k;
+                const uint32_t h = valid ? surv[ns + lane] : 0u;
+                const unsigned okm = check_chunk(p, d, Mp, log_mp, !useM, kBlockSideBMin, kBlockSideBShift, lvp, ll,
+                                                 lv_top, h, valid, cnt[4], tv, i0, cnt[7]);
+                keep_accepted(okm, h, vb, W, B, gacc, sh);
+            }
+            __syncwarp();
         }
-        __syncthreads();
-        total_acc += *(volatile int*)&sh[SH_ACC];
         __syncthreads();
         width = 2 * (int64_t)(hi - lo);
         lo = hi;
     }
+    // the new row: the maps' hubs in rank order, then the set's (all of them
+    // past the maps), sorted in shared memory (more than the set's slots hold:
+    // listed for the row sort)
+    const int macc = *(volatile int*)&sh[SH_MACC], sacc = *(volatile int*)&sh[SH_ACC];
+    const int64_t total_acc = (int64_t)macc + sacc;
     if (total_acc > 0) {
         if (tid == 0) {
             const unsigned long long start = p.ostart ? (unsigned long long)p.ostart[v]
@@ -808,11 +1194,28 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
         }
         __syncthreads();
         const unsigned long long start = *(volatile unsigned long long*)(sh + SH_START);
-        if (start + total_acc <= p.fcap) {
-            for (int64_t j = tid; j < total_acc; j += nthr) p.fhub_new[start + j] = gacc[j];
+        const bool fits = start + total_acc <= p.fcap;
+        uint32_t* row = p.fhub_new + start;
+        if (macc > 0) emit_maps(B, vb, W, fits ? row : nullptr, sh);
+        if (fits) {
+            const bool sorted = sacc <= S_CAP;
+            if (sacc > 1 && sorted) {
+                int P = 2;
+#pragma unroll 1
+                while (P < sacc) P <<= 1;
+#pragma unroll 1
+                for (int j = tid; j < P; j += nthr) S[j] = j < sacc ? gacc[j] : kEmpty;
+                __syncthreads();
+                group_bitonic_sort(S, P, tid, nthr, BlockSync());
+#pragma unroll 1
+                for (int j = tid; j < sacc; j += nthr) row[macc + j] = S[j];
+            } else {
+#pragma unroll 1
+                for (int j = tid; j < sacc; j += nthr) row[macc + j] = gacc[j];
+            }
             if (tid == 0) {
                 p.fse_new[v] = fpack(start, (uint32_t)total_acc);
-                if (p.unsorted && total_acc > 1) p.unsorted[atomicAdd(&p.ctr->nU, 1)] = v;  // sorted after the round
+                if (!sorted && p.unsorted) p.unsorted[atomicAdd(&p.ctr->nU, 1)] = v;  // sorted after the round
             }
         } else if (tid == 0) {
             p.ctr->fovf = 1;
@@ -825,20 +1228,25 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
 __global__ void __launch_bounds__(256, 3) k_gp_block(GpParams p) {
     extern __shared__ uint32_t sm[];
     int* sh = reinterpret_cast<int*>(sm);
-    int* wsum = sh + SH_WORDS;                                      // 33 ints (+ pad)
-    int* hist = wsum + 34;                                          // 256 ints
+    int* wsum = sh + SH_WORDS;                                      // 33 ints (+ 3 pad)
+    int* hist = wsum + 36;                                          // 256 ints
     uint32_t* tv = reinterpret_cast<uint32_t*>(hist + 256);         // v's exact-distance top-hub masks
     int* sex = reinterpret_cast<int*>(tv + kTopRow);                // blockDim + 1 ints
-    int64_t* sst = reinterpret_cast<int64_t*>(sex + ((blockDim.x + 2) & ~1u));  // blockDim int64
+    int64_t* sst = reinterpret_cast<int64_t*>(sex + ((blockDim.x + 4) & ~3u));  // blockDim int64
     uint32_t* S = reinterpret_cast<uint32_t*>(sst + blockDim.x);
     uint32_t* M = S + (1 << p.log_s);
     uint32_t* C = M + (1 << p.log_m);
-    uint8_t* B = reinterpret_cast<uint8_t*>(C + p.cand_limit + (int)blockDim.x);  // kByteHubs bytes
+    uint8_t* B = reinterpret_cast<uint8_t*>(C + p.cand_limit + (int)blockDim.x);  // kMapWords words
     uint32_t* gacc = p.gscratch + (int64_t)blockIdx.x * p.gscratch_words;
     unsigned long long cnt[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     if (p.ctr->done) return;
     const uint32_t d = p.ctr->d;
     const int n1 = *p.list_n;
+    // the hub maps are empty between vertices
+#pragma unroll 1
+    for (int q = threadIdx.x; q < kMapWords; q += blockDim.x) reinterpret_cast<uint32_t*>(B)[q] = 0u;
+    __syncthreads();
+#pragma unroll 1
     for (int i = blockIdx.x; i < n1; i += gridDim.x) {
         gp_block_vertex(p, d, p.list[i], S, M, C, B, gacc, sh, wsum, sex, sst, hist, tv, cnt);
         __syncthreads();
@@ -872,6 +1280,7 @@ __global__ void __launch_bounds__(256, 3) k_gp_block(GpParams p) {
 __global__ void k_pack_hrec(const int64_t* loff, const uint32_t* lent, const uint64_t* hdesc, const int32_t* vbase,
                             uint4* hrec, int64_t n, const RoundCounters* ctr) {
     if (ctr->done) return;
+#pragma unroll 1
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
         const int64_t a = loff[v], len = loff[v + 1] - a;
         const uint64_t row = hrec_row((uint64_t)a, (uint64_t)len);

@@ -86,7 +86,8 @@ struct GpParams {
     int64_t gscratch_words;    // words per block
     const uint64_t* hdesc;     // probe index of L: per row (table start << 8 | log2 slots), 0 = no table
     const uint32_t* htab;
-    const uint32_t* top;       // per vertex: top-hub masks by distance level (see kTopHubs)
+    int64_t n;                 // vertices
+    const uint32_t* top;       // top-hub masks by distance level, then vertex (see kTopHubs)
     // The candidates' side of the check: rows, probe index and top-hub masks
     // of the labels h contributes (the same arrays as above for undirected
     // graphs; for L_in(v) of a directed graph the L_out of h, and vice versa).
@@ -140,20 +141,33 @@ static_assert(kTopHubs % 128 == 0, "top-hub masks are read as uint4");
 constexpr int kTopWords = kTopHubs / 32;             // words per mask
 constexpr int kTopLevels = 7;                        // distance levels 1..7
 constexpr int kTopRow = kTopLevels * kTopWords;      // words per vertex
+// Layout: the masks of level 1 of all vertices, then level 2's, ...: a round
+// reads one or two levels of candidates that are mostly of high rank, so that
+// what it reads lies together (the 32-byte masks of 2^17 hubs in 4 MB; with
+// all levels of a vertex side by side they were spread over 29 MB).
 
 // Messages each lane loads before inserting them (gathers keep several loads
 // in flight per warp).
 constexpr int kGatherUnroll = 4;
-// Label entries each lane loads per step of a distance check.
-constexpr int kCheckUnroll = 2;
 
-// Block tier: hubs below this rank are deduplicated in a shared-memory byte
-// map (one byte per hub) instead of the hash set.
-constexpr int kByteHubs = 32768;
-// Receivers whose candidate bound reaches this use the byte map (for fewer
-// candidates clearing and scanning it costs more than the hashing it saves).
+// Block tier: the highest-ranked hubs (of the vertex's graph) are deduplicated
+// in shared-memory maps instead of the hash set: the first kByteHubs in a byte
+// map (plain stores: a row's hubs crowd into few words there, which would
+// serialise atomics), the next kBitHubs in a bitmap (shared-memory atomicOr).
+// On R-MAT 2^22 28% of round 3's messages and 32% of its candidates rank past
+// 32,768, 1.6% and 2% past 131,072: a 32 KB byte map of 32,768 hubs left them
+// to the set; 16 KB of bytes and 16 KB of bits cover 147,456.
+constexpr int kByteHubs = 16384;
+constexpr int kBitHubs = 131072;
+constexpr int kMapWords = kByteHubs / 4 + kBitHubs / 32;
+static_assert(kByteHubs % 512 == 0 && kBitHubs % 4096 == 0, "whole scan units");
+// Receivers whose candidate bound reaches this use the maps (for fewer
+// candidates scanning them costs more than the hashing it saves).
 constexpr uint32_t kByteMinBound = 2048;
-constexpr int kByteStage = 160;  // per-warp staging of byte-map candidates (< 32 carried + 128 new)
+// Block tier, per warp: staged candidates (fewer than 64, plus 32 of one
+// extraction) and survivors of the first prefilter step (fewer than 32, plus 64)
+constexpr int kCandStage = 96, kSurvStage = 96;
+constexpr int kWarpStage = kCandStage + kSurvStage;
 
 // Rows of L with at least this many entries get a hub-keyed probe table.
 constexpr int kIndexMinLen = 16;

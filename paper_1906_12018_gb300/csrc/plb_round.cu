@@ -221,8 +221,8 @@ __global__ void k_collect(unsigned long long* recv, const int64_t* roff, const i
         const unsigned long long below = (unsigned long long)(v - (int64_t)base_of(vbase, v));
         const unsigned long long bound = c < below ? c : below;
         if (obound) obound[v] = (int64_t)bound;
-        if (c) {
-            recv[v] = 0;
+        if (c) recv[v] = 0;
+        if (bound) {
             bsum += bound;
             rbound[v] = (uint32_t)bound;  // v < 2^24
             const int64_t ll = loff[v + 1] - loff[v];
@@ -771,7 +771,7 @@ __global__ void k_merge_old(const int64_t* loff, const uint32_t* lent, const int
 // New entries (dist d) of each active vertex: warp per vertex.
 __global__ void k_merge_new(const int64_t* loff, const uint32_t* lent, const int64_t* loff_new, uint32_t* lent_new,
                             const uint64_t* fse_new, const uint32_t* fhub_new, const int32_t* A,
-                            const int32_t* vbase, const RoundCounters* ctr, uint32_t* top) {
+                            const int32_t* vbase, const RoundCounters* ctr, uint32_t* top, int64_t n) {
     if (ctr->done) return;
     const uint32_t d = ctr->d;
     const int nA = ctr->nA;
@@ -805,8 +805,8 @@ __global__ void k_merge_new(const int64_t* loff, const uint32_t* lent, const int
             lent_new[pos] = pack(h, d);
             const uint32_t hr = h - vb;
             if (hr < (uint32_t)kTopHubs && d <= (uint32_t)kTopLevels) {
-                uint32_t* tv = top + (int64_t)v * kTopRow + (hr >> 5);
-                for (int t = (int)d; t <= kTopLevels; ++t) atomicOr(tv + (t - 1) * kTopWords, 1u << (hr & 31));
+                uint32_t* tv = top + (int64_t)v * kTopWords + (hr >> 5);
+                for (int t = (int)d; t <= kTopLevels; ++t) atomicOr(tv + (t - 1) * n * kTopWords, 1u << (hr & 31));
             }
         }
     }

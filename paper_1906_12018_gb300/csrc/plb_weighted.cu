@@ -356,7 +356,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     const int block_cand = pow2_at_least(std::max(bthr, o.block_cand_cap));
     const int b_log_s = ceil_log2_i64(std::max<int64_t>(
         std::max<int64_t>(2 * (int64_t)block_cand, block_cand + (int64_t)kGatherUnroll * bthr),
-        (int64_t)kByteStage * (bthr / 32)));
+        (int64_t)kWarpStage * (bthr / 32)));
     const int b_log_m = ceil_log2_i64(2 * (int64_t)std::max(o.block_label_cap, 64) + 2 * bthr);
     const size_t b_smem = gp_block_smem_bytes(bthr, b_log_s, b_log_m, block_cand);
     TierLimits lim;
@@ -398,6 +398,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     };
     auto gather = [&](uint64_t* fse_new) -> cudaError_t {
         GpParams p{};
+        p.n = n;
         p.roff = roff;
         p.rcol = vcol;
         p.loff = loff[cur];
@@ -537,7 +538,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
             k_merge_old<<<flat_grid_cap, kFlatThreads, 0, s>>>(loff[cur], lent[cur], loff[x], lent[x], fse_new, store,
                                                                n, ctr);
             k_merge_new<<<grid_for((int64_t)n * 32, kFlatThreads, flat_grid_cap), kFlatThreads, 0, s>>>(
-                loff[cur], lent[cur], loff[x], lent[x], fse_new, store, A, nullptr, ctr, top);
+                loff[cur], lent[cur], loff[x], lent[x], fse_new, store, A, nullptr, ctr, top, n);
             launches += 6 + scan_n;
             PLB_CK(cudaGetLastError());
             const int64_t Told = T;
