@@ -178,7 +178,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
             if (pool.failed) return PLB_ERR_OOM;
         }
         const int slots = index_slots(total);
-        k_index_build<<<grid_for((n + 255) / 256, 1, flat_grid_cap), kIndexWarps * 32,
+        k_index_build<<<grid_for((n + kIndexWarps - 1) / kIndexWarps, 1, flat_grid_cap), kIndexWarps * 32,
                         sizeof(uint32_t) * kIndexWarps * slots, s>>>(loff[which], lent[which], hoff, htab, hdesc, n,
                                                                      slots, ctr);
         k_index_total<<<1, 1, 0, s>>>(hoff, n, ctr);

@@ -208,7 +208,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
         k_index_size<<<gflat, kFlatThreads, 0, s>>>(S.loff[S.cur], n, tmp64, S.ctr);
         if (exclusive_scan_i64(tmp64, S.hoff, n, scan_scr, s) != cudaSuccess) return PLB_ERR_CUDA;
         const int slots = index_slots(total);
-        k_index_build<<<grid_for((n + 255) / 256, 1, flat_grid_cap), kIndexWarps * 32,
+        k_index_build<<<grid_for((n + kIndexWarps - 1) / kIndexWarps, 1, flat_grid_cap), kIndexWarps * 32,
                         sizeof(uint32_t) * kIndexWarps * slots, s>>>(S.loff[S.cur], S.lent[S.cur], S.hoff, S.htab,
                                                                      S.hdesc, n, slots, S.ctr);
         k_index_total<<<1, 1, 0, s>>>(S.hoff, n, S.ctr);

@@ -602,6 +602,7 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
     const uint32_t d = p.ctr->d;
     const int imax = min((int)d - 1, kTopLevels);
     const int nlist = *p.list_n;
+    if (nlist <= 0) return;
 #pragma unroll 1
     for (int s = lane; s < M_CAP; s += 32) X[s] = 0u;
 #pragma unroll 1
@@ -1242,6 +1243,7 @@ __global__ void __launch_bounds__(256, 3) k_gp_block(GpParams p) {
     if (p.ctr->done) return;
     const uint32_t d = p.ctr->d;
     const int n1 = *p.list_n;
+    if ((int)blockIdx.x >= n1) return;
     // the hub maps are empty between vertices
 #pragma unroll 1
     for (int q = threadIdx.x; q < kMapWords; q += blockDim.x) reinterpret_cast<uint32_t*>(B)[q] = 0u;

@@ -14,7 +14,7 @@
 
 namespace plb {
 
-constexpr int kFlatThreads = 256;
+constexpr int kFlatThreads = kTileThreads;
 constexpr int kGpWarpThreads = 256;
 
 // Device allocations of one build (stream-ordered, from the library pool),

@@ -161,6 +161,83 @@ __device__ __forceinline__ int64_t row_of(const int64_t* off, int64_t lo, int64_
     return lo;
 }
 
+// The same by a whole warp, 32 probes at a time (a binary search is a chain of
+// log2(rows) dependent loads; all lanes call and get the result).
+__device__ __forceinline__ int64_t warp_row_of(const int64_t* off, int64_t lo, int64_t hi, int64_t p) {
+    const int lane = threadIdx.x & 31;
+    while (lo < hi) {
+        const int64_t step = (hi - lo + 31) / 32;
+        const int64_t r = lo + (lane + 1) * step;
+        const int c = __popc(__ballot_sync(kFull, r <= hi && off[r] <= p));  // (off is non-decreasing)
+        lo += c * step;
+        hi = min(hi, lo + step - 1);
+    }
+    return lo;
+}
+
+// Flat passes over the items of rows (arcs, label entries): tiles of kTileItems
+// consecutive items per block of kTileThreads threads, so that rows of any
+// length are spread evenly.
+constexpr int kTileItems = 2048;
+constexpr int kTileThreads = 256;
+
+// Row of every item of the tile [p0, p1): srow[i] = row of item p0 + i, less
+// *r0 (the tile's first row; *r1 its last).  The first and last row are found
+// by two warps, each row's start is marked in srow and a running maximum gives
+// every item its row: one thread searching both ends cost 40 dependent loads
+// per tile (20 us), and a search per item 8 to 9 more (builds, before -> after,
+// with the two-launch scans: 4K vertices 1.76 -> 1.25 ms, 61K 3.4 -> 2.7 ms).
+// All threads call.
+struct TileScratch {
+    int64_t r[2];
+    int wmax[kTileThreads / 32];
+};
+__device__ __forceinline__ void tile_row_map(const int64_t* off, int64_t nrows, int64_t p0, int64_t p1, int* srow,
+                                             TileScratch* sh, int64_t* r0, int64_t* r1) {
+    constexpr int kPer = kTileItems / kTileThreads;
+    static_assert(kPer == 8, "eight items per thread");
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    __syncthreads();  // (srow and sh may still be read for the tile before)
+    if (wid < 2) {
+        const int64_t r = warp_row_of(off, 0, nrows - 1, wid == 0 ? p0 : p1 - 1);
+        if (lane == 0) sh->r[wid] = r;
+    }
+    int4* s4 = reinterpret_cast<int4*>(srow) + 2 * tid;
+    s4[0] = make_int4(0, 0, 0, 0);
+    s4[1] = make_int4(0, 0, 0, 0);
+    __syncthreads();
+    const int64_t a = sh->r[0], b = sh->r[1];
+    for (int64_t r = a + 1 + tid; r <= b; r += kTileThreads) {
+        const int64_t q = off[r] - p0;
+        if (q >= 0 && q < kTileItems) atomicMax(&srow[(int)q], (int)(r - a));  // (always, in a valid CSR)
+    }
+    __syncthreads();
+    int4 x = s4[0], y = s4[1];
+    x.y = max(x.y, x.x);
+    x.z = max(x.z, x.y);
+    x.w = max(x.w, x.z);
+    y.x = max(y.x, x.w);
+    y.y = max(y.y, y.x);
+    y.z = max(y.z, y.y);
+    y.w = max(y.w, y.z);
+    int m = y.w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(kFull, m, o);
+        if (lane >= o) m = max(m, t);
+    }
+    if (lane == 31) sh->wmax[wid] = m;
+    int before = __shfl_up_sync(kFull, m, 1);
+    if (lane == 0) before = 0;
+    __syncthreads();
+    for (int k = 0; k < wid; ++k) before = max(before, sh->wmax[k]);
+    s4[0] = make_int4(max(x.x, before), max(x.y, before), max(x.z, before), max(x.w, before));
+    s4[1] = make_int4(max(y.x, before), max(y.y, before), max(y.z, before), max(y.w, before));
+    __syncthreads();
+    *r0 = a;
+    *r1 = b;
+}
+
 // Bitonic sort of a[0..P) (P a power of two) by a group of nthreads threads.
 // Each step runs over the P/2 compare-exchange pairs (i, i + j), i the pair
 // index t with a zero bit inserted at bit log2(j): no idle half of the

@@ -7,16 +7,7 @@ namespace plb {
 
 namespace {
 
-constexpr int kTileItems = 2048;  // items per block tile in flat (load-balanced) kernels
-
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
-
-// First and last row of offsets off[0..nrows] that intersect items [p0, p1).
-__device__ __forceinline__ void tile_rows(const int64_t* off, int64_t nrows, int64_t p0, int64_t p1,
-                                          int64_t* r0, int64_t* r1) {
-    *r0 = row_of(off, 0, nrows - 1, p0);
-    *r1 = row_of(off, 0, nrows - 1, p1 - 1);
-}
 
 }  // namespace
 
@@ -36,16 +27,15 @@ __global__ void k_check_rowptr(const int64_t* row_ptr, int64_t n, int64_t nnz, i
 // symmetric) the reverse arc (c -> u) exists (binary search in row c).
 __global__ void k_check_cols(const int64_t* row_ptr, const int32_t* col, int64_t n, int64_t nnz, int symmetric,
                              int* err) {
-    __shared__ int64_t sh_r[2];
+    __shared__ __align__(16) int srow[kTileItems];
+    __shared__ TileScratch sh;
     const int64_t ntiles = (nnz + kTileItems - 1) / kTileItems;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
-        __syncthreads();
-        if (threadIdx.x == 0) tile_rows(row_ptr, n, p0, p1, &sh_r[0], &sh_r[1]);
-        __syncthreads();
-        const int64_t r0 = sh_r[0], r1 = sh_r[1];
+        int64_t r0, r1;
+        tile_row_map(row_ptr, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-            const int64_t u = row_of(row_ptr, r0, r1, p);
+            const int64_t u = r0 + srow[p - p0];
             const int32_t c = col[p];
             bool bad = c < 0 || (int64_t)c >= n || (int64_t)c == u;
             if (!bad && p > row_ptr[u] && col[p - 1] >= c) bad = true;
@@ -85,16 +75,15 @@ __global__ void k_in_degree(const int32_t* rcol, int64_t nnz, int64_t* indeg) {
 // the entries placed per row (zeroed by the caller; rows come out unsorted).
 __global__ void k_transpose(const int64_t* roff, const int32_t* rcol, int64_t n, int64_t nnz, const int64_t* roff_t,
                             unsigned long long* fill, int32_t* rcol_t) {
-    __shared__ int64_t sh_r[2];
+    __shared__ __align__(16) int srow[kTileItems];
+    __shared__ TileScratch sh;
     const int64_t ntiles = (nnz + kTileItems - 1) / kTileItems;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
-        __syncthreads();
-        if (threadIdx.x == 0) tile_rows(roff, n, p0, p1, &sh_r[0], &sh_r[1]);
-        __syncthreads();
-        const int64_t r0 = sh_r[0], r1 = sh_r[1];
+        int64_t r0, r1;
+        tile_row_map(roff, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-            const int64_t u = row_of(roff, r0, r1, p);
+            const int64_t u = r0 + srow[p - p0];
             const int32_t w = rcol[p];
             rcol_t[roff_t[w] + (int64_t)atomicAdd(&fill[w], 1ull)] = (int32_t)u;
         }
@@ -117,16 +106,15 @@ __global__ void k_rank_degree(const int64_t* row_ptr, const int32_t* order, int6
 // rcol[roff[r] + j] = rank of the j-th neighbour of order[r] (row order kept).
 __global__ void k_relabel(const int64_t* row_ptr, const int32_t* col, const int32_t* order, const int32_t* inv,
                           const int64_t* roff, int32_t* rcol, int64_t n, int64_t nnz) {
-    __shared__ int64_t sh_r[2];
+    __shared__ __align__(16) int srow[kTileItems];
+    __shared__ TileScratch sh;
     const int64_t ntiles = (nnz + kTileItems - 1) / kTileItems;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
-        __syncthreads();
-        if (threadIdx.x == 0) tile_rows(roff, n, p0, p1, &sh_r[0], &sh_r[1]);
-        __syncthreads();
-        const int64_t r0 = sh_r[0], r1 = sh_r[1];
+        int64_t r0, r1;
+        tile_row_map(roff, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-            const int64_t r = row_of(roff, r0, r1, p);
+            const int64_t r = r0 + srow[p - p0];
             const int32_t id = order[r];
             rcol[p] = inv[col[row_ptr[id] + (p - roff[r])]];
         }
@@ -177,7 +165,8 @@ __global__ void k_active_degree(const int64_t* roff, const int32_t* A, const Rou
 __global__ void k_mark(const int64_t* roff, const int32_t* rcol, const uint64_t* fse, const uint32_t* fhub,
                        const int32_t* A, const int64_t* aoff, const RoundCounters* ctr, unsigned long long* recv,
                        int64_t n) {
-    __shared__ int64_t sh_r[2];
+    __shared__ __align__(16) int srow[kTileItems];
+    __shared__ TileScratch sh;
     if (ctr->done) return;
     const int64_t nA = ctr->nA;
     if (nA == 0) return;
@@ -185,12 +174,10 @@ __global__ void k_mark(const int64_t* roff, const int32_t* rcol, const uint64_t*
     const int64_t ntiles = (total + kTileItems - 1) / kTileItems;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(total, p0 + kTileItems);
-        __syncthreads();
-        if (threadIdx.x == 0) tile_rows(aoff, nA, p0, p1, &sh_r[0], &sh_r[1]);
-        __syncthreads();
-        const int64_t r0 = sh_r[0], r1 = sh_r[1];
+        int64_t r0, r1;
+        tile_row_map(aoff, nA, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-            const int64_t i = row_of(aoff, r0, r1, p);
+            const int64_t i = r0 + srow[p - p0];
             const int32_t a = A[i];
             const uint64_t f = fse[a];
             const uint32_t minh = fhub[fstart(f)];
@@ -272,23 +259,22 @@ __global__ void k_after_collect(RoundCounters* ctr) {
 // atomic per row and warp).
 __global__ void k_round1_count(const int64_t* roff, const int32_t* rcol, int64_t n, int64_t nnz, int32_t s,
                                int32_t e, unsigned long long* cnt, const RoundCounters* ctr) {
-    __shared__ int64_t sh_r[2];
+    __shared__ __align__(16) int srow[kTileItems];
+    __shared__ TileScratch sh;
     if (ctr->done) return;
     const int lane = lane_id();
     const int64_t ntiles = (nnz + kTileItems - 1) / kTileItems;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
-        __syncthreads();
-        if (threadIdx.x == 0) tile_rows(roff, n, p0, p1, &sh_r[0], &sh_r[1]);
-        __syncthreads();
-        const int64_t r0 = sh_r[0], r1 = sh_r[1];
+        int64_t r0, r1;
+        tile_row_map(roff, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t q = p0; q < p1; q += blockDim.x) {  // uniform trip count: whole warps below
             const int64_t p = q + threadIdx.x;
             const bool ok = p < p1;
             int64_t v = -1;
             int c = 0;
             if (ok) {
-                v = row_of(roff, r0, r1, p);
+                v = r0 + srow[p - p0];
                 const int32_t a = rcol[p];
                 c = (a >= s && a < e && (int64_t)a < v) ? 1 : 0;
             }
@@ -307,7 +293,8 @@ __global__ void k_round1_count(const int64_t* roff, const int32_t* rcol, int64_t
 __global__ void k_round1(const int64_t* roff, const int32_t* rcol, int64_t n, int64_t nnz, int32_t s, int32_t e,
                          const int64_t* start, uint32_t* cur, uint64_t* fse_new, uint32_t* fhub_new,
                          unsigned long long fcap, RoundCounters* ctr) {
-    __shared__ int64_t sh_r[2];
+    __shared__ __align__(16) int srow[kTileItems];
+    __shared__ TileScratch sh;
     if (ctr->done) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctr->nA_saved = ctr->nA;
@@ -320,10 +307,8 @@ __global__ void k_round1(const int64_t* roff, const int32_t* rcol, int64_t n, in
     const int64_t ntiles = (nnz + kTileItems - 1) / kTileItems;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
-        __syncthreads();
-        if (threadIdx.x == 0) tile_rows(roff, n, p0, p1, &sh_r[0], &sh_r[1]);
-        __syncthreads();
-        const int64_t r0 = sh_r[0], r1 = sh_r[1];
+        int64_t r0, r1;
+        tile_row_map(roff, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t q = p0; q < p1; q += blockDim.x) {
             const int64_t p = q + threadIdx.x;
             const bool ok = p < p1;
@@ -331,7 +316,7 @@ __global__ void k_round1(const int64_t* roff, const int32_t* rcol, int64_t n, in
             int32_t a = 0;
             bool up = false;
             if (ok) {
-                v = row_of(roff, r0, r1, p);
+                v = r0 + srow[p - p0];
                 a = rcol[p];
                 up = a >= s && a < e && (int64_t)a < v;
             }
@@ -415,7 +400,9 @@ __device__ __forceinline__ void build_table(const uint32_t* lent, int64_t lb, in
     }
 }
 
-// Full rebuild, one warp per 32 rows: row x's table at hoff[x] (sizes from
+// Full rebuild, one warp per `per` rows (at most 32: fewer when the warps of the
+// grid outnumber the groups of 32, so that a small graph's rows are not built
+// one after the other on a few warps): row x's table at hoff[x] (sizes from
 // k_index_size and a scan); hdesc[x] = hoff[x] << 8 | log2 size, or 0.
 __global__ void __launch_bounds__(kIndexWarps * 32) k_index_build(const int64_t* loff, const uint32_t* lent,
                                                                   const int64_t* hoff, uint32_t* htab,
@@ -426,10 +413,11 @@ __global__ void __launch_bounds__(kIndexWarps * 32) k_index_build(const int64_t*
     const int lane = lane_id(), w = threadIdx.x >> 5;
     uint32_t* buf = ibuf + w * slots;
     const int64_t nwarps = (int64_t)gridDim.x * kIndexWarps;
-    for (int64_t base = ((int64_t)blockIdx.x * kIndexWarps + w) * 32; base < n; base += nwarps * 32) {
+    const int64_t per = min((int64_t)32, (n + nwarps - 1) / nwarps);
+    for (int64_t base = ((int64_t)blockIdx.x * kIndexWarps + w) * per; base < n; base += nwarps * per) {
         const int64_t x = base + lane;
         int64_t hb = 0, P = 0;
-        if (x < n) {
+        if (lane < per && x < n) {
             hb = hoff[x];
             P = hoff[x + 1] - hb;
             hdesc[x] = P > 0 ? ((uint64_t)hb << 8) | (uint64_t)(__ffsll((unsigned long long)P) - 1) : 0ull;
@@ -717,7 +705,8 @@ constexpr int kMergeRows = 512;
 
 __global__ void k_merge_old(const int64_t* loff, const uint32_t* lent, const int64_t* loff_new, uint32_t* lent_new,
                             const uint64_t* fse_new, const uint32_t* fhub_new, int64_t n, const RoundCounters* ctr) {
-    __shared__ int64_t sh_r[2];
+    __shared__ __align__(16) int srow[kTileItems];
+    __shared__ TileScratch sh;
     __shared__ int64_t s_off[kMergeRows + 1];
     __shared__ int64_t s_noff[kMergeRows];
     __shared__ uint64_t s_f[kMergeRows];
@@ -726,10 +715,8 @@ __global__ void k_merge_old(const int64_t* loff, const uint32_t* lent, const int
     const int64_t ntiles = (total + kTileItems - 1) / kTileItems;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(total, p0 + kTileItems);
-        __syncthreads();
-        if (threadIdx.x == 0) tile_rows(loff, n, p0, p1, &sh_r[0], &sh_r[1]);
-        __syncthreads();
-        const int64_t r0 = sh_r[0], r1 = sh_r[1];
+        int64_t r0, r1;
+        tile_row_map(loff, n, p0, p1, srow, &sh, &r0, &r1);
         const int64_t rows = r1 - r0 + 1;
         const int nr = rows <= kMergeRows ? (int)rows : kMergeRows + 1;
         const bool staged = nr <= kMergeRows;
@@ -744,17 +731,13 @@ __global__ void k_merge_old(const int64_t* loff, const uint32_t* lent, const int
         for (int64_t q = p0 + threadIdx.x; q < p1; q += blockDim.x) {
             int64_t ob, nb;
             uint64_t f;
+            const int lo = srow[q - p0];
             if (staged) {
-                int lo = 0, hi = nr - 1;  // last row of the tile whose offset is <= q
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (s_off[mid] <= q) lo = mid; else hi = mid - 1;
-                }
                 ob = s_off[lo];
                 nb = s_noff[lo];
                 f = s_f[lo];
             } else {
-                const int64_t v = row_of(loff, r0, r1, q);
+                const int64_t v = r0 + lo;
                 ob = loff[v];
                 nb = loff_new[v];
                 f = fse_new[v];
@@ -919,7 +902,8 @@ __global__ void k_final_len(const int64_t* loff, const int32_t* inv, int64_t n, 
 __global__ void k_finalize(const int64_t* loff, const uint32_t* lent, const int32_t* inv, const int64_t* out_off,
                            uint32_t* out_packed, uint32_t* out_hub, uint8_t* out_dist, int64_t n,
                            RoundCounters* ctr) {
-    __shared__ int64_t sh_r[2];
+    __shared__ __align__(16) int srow[kTileItems];
+    __shared__ TileScratch sh;
     __shared__ int64_t s_off[kMergeRows + 1];  // out_off of the tile's rows (as in k_merge_old)
     __shared__ int64_t s_src[kMergeRows];      // start of each row in rank space
     const int64_t total = out_off[n];
@@ -927,10 +911,8 @@ __global__ void k_finalize(const int64_t* loff, const uint32_t* lent, const int3
     uint32_t md = 0;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(total, p0 + kTileItems);
-        __syncthreads();
-        if (threadIdx.x == 0) tile_rows(out_off, n, p0, p1, &sh_r[0], &sh_r[1]);
-        __syncthreads();
-        const int64_t r0 = sh_r[0], r1 = sh_r[1];
+        int64_t r0, r1;
+        tile_row_map(out_off, n, p0, p1, srow, &sh, &r0, &r1);
         const int64_t rows = r1 - r0 + 1;
         const int nr = rows <= kMergeRows ? (int)rows : kMergeRows + 1;
         const bool staged = nr <= kMergeRows;
@@ -941,15 +923,11 @@ __global__ void k_finalize(const int64_t* loff, const uint32_t* lent, const int3
         __syncthreads();
         for (int64_t q = p0 + threadIdx.x; q < p1; q += blockDim.x) {
             int64_t src;
+            const int lo = srow[q - p0];
             if (staged) {
-                int lo = 0, hi = nr - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (s_off[mid] <= q) lo = mid; else hi = mid - 1;
-                }
                 src = s_src[lo] + (q - s_off[lo]);
             } else {
-                const int64_t id = row_of(out_off, r0, r1, q);
+                const int64_t id = r0 + lo;
                 src = loff[inv[id]] + (q - out_off[id]);
             }
             const uint32_t e = lent[src];

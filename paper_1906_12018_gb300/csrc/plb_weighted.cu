@@ -34,7 +34,7 @@ namespace plb {
 
 namespace {
 
-constexpr int kWFlatThreads = 256;
+constexpr int kWFlatThreads = kTileThreads;
 
 __device__ __forceinline__ int wlane() { return threadIdx.x & 31; }
 
@@ -57,31 +57,19 @@ __global__ void k_weight_range(const uint8_t* wt, int64_t nnz, int* mm) {
     }
 }
 
-// Flat kernels over the arcs: tiles of kWTile consecutive arcs, the tile's
-// first and last row found once, each arc's row by binary search between
-// them (rows of any length are spread evenly over the threads).
-constexpr int kWTile = 2048;
-
-__device__ __forceinline__ void tile_bounds(const int64_t* off, int64_t n, int64_t p0, int64_t p1, int64_t* sh) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        sh[0] = row_of(off, 0, n - 1, p0);
-        sh[1] = row_of(off, 0, n - 1, p1 - 1);
-    }
-    __syncthreads();
-}
-
 // Per arc (u -> c) of a validated symmetric CSR: the reverse arc (c -> u),
 // found by binary search in row c, has the same weight.
 __global__ void k_check_weights(const int64_t* row_ptr, const int32_t* col, const uint8_t* wt, int64_t n,
                                 int64_t nnz, int* err) {
-    __shared__ int64_t sh[2];
-    const int64_t ntiles = (nnz + kWTile - 1) / kWTile;
+    __shared__ __align__(16) int srow[kTileItems];
+    __shared__ TileScratch sh;
+    const int64_t ntiles = (nnz + kTileItems - 1) / kTileItems;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int64_t p0 = t * kWTile, p1 = min(nnz, p0 + kWTile);
-        tile_bounds(row_ptr, n, p0, p1, sh);
+        const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
+        int64_t r0, r1;
+        tile_row_map(row_ptr, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-            const int64_t u = row_of(row_ptr, sh[0], sh[1], p);
+            const int64_t u = r0 + srow[p - p0];
             const int32_t c = col[p];
             int64_t lo = row_ptr[c], hi = row_ptr[c + 1];
             while (lo < hi) {
@@ -97,13 +85,15 @@ __global__ void k_check_weights(const int64_t* row_ptr, const int32_t* col, cons
 // order[r] (k_relabel keeps the row order).
 __global__ void k_relabel_weights(const int64_t* row_ptr, const uint8_t* wt, const int32_t* order,
                                   const int64_t* roff, uint8_t* rwt, int64_t n, int64_t nnz) {
-    __shared__ int64_t sh[2];
-    const int64_t ntiles = (nnz + kWTile - 1) / kWTile;
+    __shared__ __align__(16) int srow[kTileItems];
+    __shared__ TileScratch sh;
+    const int64_t ntiles = (nnz + kTileItems - 1) / kTileItems;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int64_t p0 = t * kWTile, p1 = min(nnz, p0 + kWTile);
-        tile_bounds(roff, n, p0, p1, sh);
+        const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
+        int64_t r0, r1;
+        tile_row_map(roff, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-            const int64_t r = row_of(roff, sh[0], sh[1], p);
+            const int64_t r = r0 + srow[p - p0];
             rwt[p] = wt[row_ptr[order[r]] + (p - roff[r])];
         }
     }
@@ -120,19 +110,21 @@ __global__ void k_relabel_weights(const int64_t* row_ptr, const uint8_t* wt, con
 __global__ void k_w_pull(const int64_t* roff, const int32_t* rcol, const uint8_t* rwt, int64_t n, int64_t nnz,
                          uint32_t d, int S, int lgn, const uint64_t* fse_ring, const uint32_t* store, int32_t* vcol,
                          unsigned long long* recv) {
-    __shared__ int64_t sh[2];
+    __shared__ __align__(16) int srow[kTileItems];
+    __shared__ TileScratch sh;
     const int32_t empty = (int32_t)((int64_t)S << lgn);
-    const int64_t ntiles = (nnz + kWTile - 1) / kWTile;
+    const int64_t ntiles = (nnz + kTileItems - 1) / kTileItems;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int64_t p0 = t * kWTile, p1 = min(nnz, p0 + kWTile);
-        tile_bounds(roff, n, p0, p1, sh);
+        const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
+        int64_t r0, r1;
+        tile_row_map(roff, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t q = p0; q < p1; q += blockDim.x) {  // uniform trip count: whole warps below
             const int64_t p = q + threadIdx.x;
             const bool ok = p < p1;
             int64_t v = -1;
             unsigned c = 0;
             if (ok) {
-                v = row_of(roff, sh[0], sh[1], p);
+                v = r0 + srow[p - p0];
                 const int32_t a = rcol[p];
                 const int r = (int)d - (int)rwt[p];
                 const int32_t idx = r >= 0 ? (int32_t)(((int64_t)(r % S) << lgn) | a) : empty;
@@ -194,7 +186,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     const int sms = num_sms();
     const int flat_grid_cap = sms * 8;
     const int gflat = grid_for(n, kFlatThreads, flat_grid_cap);
-    const int gpull = grid_for((nnz + kWTile - 1) / kWTile, 1, flat_grid_cap);
+    const int gpull = grid_for((nnz + kTileItems - 1) / kTileItems, 1, flat_grid_cap);
     cudaEvent_t t_all0 = tm.on ? tm.mark() : nullptr;
     int64_t launches = 0;
 
@@ -249,7 +241,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
         pool.release(seen);
         if (herr[0]) return PLB_ERR_INVALID;
         if (nnz > 0) {  // arcs are symmetric and in range: compare the weights of both directions
-            k_check_weights<<<grid_for((nnz + kWTile - 1) / kWTile, 1, flat_grid_cap), kWFlatThreads, 0, s>>>(
+            k_check_weights<<<grid_for((nnz + kTileItems - 1) / kTileItems, 1, flat_grid_cap), kWFlatThreads, 0, s>>>(
                 row_ptr, col, wt, n, nnz, err);
             PLB_CK(cudaGetLastError());
             PLB_CK(cudaMemcpyAsync(herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -276,7 +268,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     if (nnz > 0) {
         k_relabel<<<grid_for((nnz + 2047) / 2048, 1, flat_grid_cap), kFlatThreads, 0, s>>>(row_ptr, col, order, inv,
                                                                                           roff, rcol, n, nnz);
-        k_relabel_weights<<<grid_for((nnz + kWTile - 1) / kWTile, 1, flat_grid_cap), kWFlatThreads, 0, s>>>(
+        k_relabel_weights<<<grid_for((nnz + kTileItems - 1) / kTileItems, 1, flat_grid_cap), kWFlatThreads, 0, s>>>(
             row_ptr, wt, order, roff, rwt, n, nnz);
     }
     PLB_CK(cudaGetLastError());
@@ -331,7 +323,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
         k_index_size<<<gflat, kFlatThreads, 0, s>>>(loff[cur], n, tmp64, ctr);
         if (exclusive_scan_i64(tmp64, hoff, n, scan_scr, s) != cudaSuccess) return PLB_ERR_CUDA;
         const int slots = index_slots(T);
-        k_index_build<<<grid_for((n + 255) / 256, 1, flat_grid_cap), kIndexWarps * 32,
+        k_index_build<<<grid_for((n + kIndexWarps - 1) / kIndexWarps, 1, flat_grid_cap), kIndexWarps * 32,
                         sizeof(uint32_t) * kIndexWarps * slots, s>>>(loff[cur], lent[cur], hoff, htab, hdesc, n,
                                                                      slots, ctr);
         k_index_total<<<1, 1, 0, s>>>(hoff, n, ctr);
