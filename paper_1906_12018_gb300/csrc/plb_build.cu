@@ -242,6 +242,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
     // block tier: per-block buffer of accepted hubs (at most v < n per vertex)
     const int64_t acc_words = std::max<int64_t>(std::min<int64_t>(n, max_part_n), 1);
     uint32_t* gacc = pool.alloc<uint32_t>((int64_t)grid_b * acc_words);
+    const SplitLists split = split_lists(pool, n, max_part_n, nnz, s);
     // per-vertex check records (row bounds and probe-table descriptor), packed before each gather
     uint4* hrec = pool.alloc<uint4>(std::max<int64_t>(n, 1));
     PLB_ALLOC_OK();
@@ -288,7 +289,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         cudaError_t e = exclusive_scan_i64(tmp64, aoff, n, scan_scr, s, skip);
         if (e != cudaSuccess) return e;
         k_mark<<<flat_grid_cap, kFlatThreads, 0, s>>>(roff, rcol, fse[c], fhub[c], A, aoff, ctr, recv, n);
-        k_collect<<<gflat, kFlatThreads, 0, s>>>(recv, roff, loff[c], n, fse[x], R, O1, rbound, tmp64, vbase, ctr, lim);
+        k_collect<<<gflat, kFlatThreads, 0, s>>>(recv, roff, loff[c], n, fse[x], R, O1, rbound, tmp64, vbase, split, ctr, lim);
         k_after_collect<<<1, 1, 0, s>>>(ctr);
         // the scan of the candidate bounds places each receiver's new frontier
         // row (aoff is free again after k_mark); used when the buffer holds
@@ -323,6 +324,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         GpParams w = p, b = p;
         w.list = R;  // warp tier
         w.list_n = &ctr->nR;
+        w.work = &ctr->wkR;
         w.log_s = w_log_s;
         w.log_m = w_log_m;
         w.cand_limit = warp_cand;
@@ -336,6 +338,8 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
             w.esc_n = &ctr->nO2;
             b.list = O1;
             b.list_n = &ctr->nO1;
+            b.work = &ctr->wkO1;
+            b.split = split;
             cudaError_t e = cudaEventRecord(ev_fork, s);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(side, ev_fork, 0);
             if (e != cudaSuccess) return e;
@@ -347,6 +351,8 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
             if (e != cudaSuccess) return e;
             b.list = O2;
             b.list_n = &ctr->nO2;
+            b.work = &ctr->wkO2;
+            b.split = SplitLists{};
             k_gp_block<<<grid_b, bthr, b_smem, s>>>(b);
             st.launches += 3;
             return cudaGetLastError();
@@ -357,6 +363,8 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         if (g1) *g1 = tm.mark();
         b.list = O1;
         b.list_n = &ctr->nO1;
+        b.work = &ctr->wkO1;
+        b.split = split;
         k_gp_block<<<grid_b, bthr, b_smem, s>>>(b);
         st.launches += 2;
         return cudaGetLastError();
@@ -477,7 +485,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         const int64_t acc = (int64_t)hctr->accepted;
         if (d < PLB_MAX_ROUNDS) {
             // per distance d (summed over the batches of Alg. 4)
-            st.receivers[d] += (int64_t)hctr->nR + hctr->nO1_base + hctr->nO2_base;
+            st.receivers[d] += (int64_t)hctr->nR + hctr->nO1_base + hctr->nG_base;
             st.accepted[d] += acc;
             st.unique_round[d] += (int64_t)hctr->uniq;
             st.prefiltered_round[d] += (int64_t)hctr->prefiltered;

@@ -260,6 +260,10 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
     uint32_t* gacc = pool.alloc<uint32_t>((int64_t)grid_b * std::max<int64_t>(n, 1));
     PLB_ALLOC_OK();
 
+    // split receivers (both sides' frontier steps run before either gather)
+    SplitLists split2[2];
+    for (int k = 0; k < 2; ++k) split2[k] = split_lists(pool, n, n, nnz, s);
+    PLB_ALLOC_OK();
     // ------------------------------------------------------------ rounds
     auto frontier = [&](Side& S) -> cudaError_t {
         const int c = S.cur, x = c ^ 1;
@@ -269,7 +273,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
         k_mark<<<flat_grid_cap, kFlatThreads, 0, s>>>(S.s_off, S.s_col, S.fse[c], S.fhub[c], S.A, S.aoff, S.ctr,
                                                       S.recv, n);
         k_collect<<<gflat, kFlatThreads, 0, s>>>(S.recv, S.g_off, S.loff[c], n, S.fse[x], S.R, S.O1, S.rbound, nullptr,
-                                                 nullptr, S.ctr, lim);
+                                                 nullptr, split2[&S - side], S.ctr, lim);
         k_after_collect<<<1, 1, 0, s>>>(S.ctr);
         launches += 4 + scan_n;
         return cudaGetLastError();
@@ -310,7 +314,10 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
         p.stage_ratio = o.warp_stage_ratio;
         p.count_check = o.profile != 0;
         p.unsorted = S.U;
+        p.work = &S.ctr->wkR;
         k_gp_warp<<<grid_w, kGpWarpThreads, w_smem, s>>>(p);
+        p.work = &S.ctr->wkO1;
+        p.split = split2[&S - side];
         p.list = S.O1;
         p.list_n = &S.ctr->nO1;
         p.esc = nullptr;
@@ -429,7 +436,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
             const RoundCounters& h = *S.hctr;
             const int64_t acc = (int64_t)h.accepted;
             if (d < PLB_MAX_ROUNDS) {
-                S.st.receivers[d] = (int64_t)h.nR + h.nO1_base + h.nO2_base;
+                S.st.receivers[d] = (int64_t)h.nR + h.nO1_base + h.nG_base;
                 S.st.accepted[d] = acc;
                 S.st.unique_round[d] = (int64_t)h.uniq;
                 S.st.prefiltered_round[d] = (int64_t)h.prefiltered;

@@ -605,9 +605,16 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
     if (nlist <= 0) return;
 #pragma unroll 1
     for (int s = lane; s < M_CAP; s += 32) X[s] = 0u;
+    // vertices are handed out one at a time (they differ in cost by orders of
+    // magnitude), the next one while this one is worked on
+    int next = 0;
+    if (lane == 0) next = atomicAdd(p.work, 1);
 #pragma unroll 1
-    for (int i = blockIdx.x * nwarps + wib; i < nlist; i += gridDim.x * nwarps) {
+    while (true) {
         __syncwarp();
+        const int i = __shfl_sync(kFull, next, 0);
+        if (i >= nlist) break;
+        if (lane == 0) next = atomicAdd(p.work, 1);
         const int32_t v = p.list[i];
         const uint32_t vb = base_of(p.vbase, v);
         const int64_t lb = p.loff[v], ll = p.loff[v + 1] - lb;
@@ -843,6 +850,7 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
 // Block-per-vertex scalars in shared memory (ints)
 enum { SH_UNIQ = 0, SH_OVF = 1, SH_ACC = 2 /* accepted, from the set */, SH_NC = 3, SH_HI = 4, SH_TMP = 5 /* 2 ints */,
        SH_START = 8 /* 2 ints */, SH_NEXT = 10, SH_REST = 11, SH_MACC = 12 /* accepted, from the maps */,
+       SH_ITEM = 13, SH_LAST = 14,
        SH_WCNT = 16 /* 2 x 8 warps */, SH_WORDS = 48 };
 
 // Accepted candidates of a chunk (okm): those of the maps are marked there
@@ -953,6 +961,47 @@ __device__ void emit_maps(uint8_t* B, uint32_t vb, uint32_t W, uint32_t* row, in
     }
 }
 
+// The marked hubs of the maps (W of them) OR-ed into a split receiver's global
+// bitmap; the maps are left empty.
+__device__ void flush_maps(uint8_t* B, uint32_t W, uint32_t* gbits) {
+    uint4* b4 = reinterpret_cast<uint4*>(B);
+    uint32_t* bits = reinterpret_cast<uint32_t*>(B + kByteHubs);
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    constexpr int kByteWords = kByteHubs / 32;
+#pragma unroll 1
+    for (int q = threadIdx.x; q < (int)((W + 31u) >> 5); q += blockDim.x) {
+        uint32_t w;
+        if (q < kByteWords) {
+            w = byte_bits4(b4[2 * q]) | (byte_bits4(b4[2 * q + 1]) << 16);
+            if (w) b4[2 * q] = b4[2 * q + 1] = zero;
+        } else {
+            w = bits[q - kByteWords];
+            if (w) bits[q - kByteWords] = 0u;
+        }
+        // (most of it is there already once a few parts have been merged)
+        if (w & ~__ldcg(gbits + q)) atomicOr(gbits + q, w);
+    }
+}
+
+// The maps of a split receiver from its global bitmap, which is left empty.
+__device__ void load_maps(uint8_t* B, uint32_t W, uint32_t* gbits) {
+    uint32_t* b1 = reinterpret_cast<uint32_t*>(B);
+    uint32_t* bits = reinterpret_cast<uint32_t*>(B + kByteHubs);
+    constexpr int kByteWords = kByteHubs / 32;
+#pragma unroll 1
+    for (int q = threadIdx.x; q < (int)((W + 31u) >> 5); q += blockDim.x) {
+        uint32_t w = __ldcg(gbits + q);
+        if (w == 0u) continue;
+        gbits[q] = 0u;
+        if (q < kByteWords) {
+#pragma unroll 1
+            for (int k = 0; k < 8; ++k, w >>= 4) b1[8 * q + k] = ((w & 15u) * 0x00204081u) & 0x01010101u;
+        } else {
+            bits[q - kByteWords] = w;
+        }
+    }
+}
+
 // One block per vertex, any size.  The candidates are processed in passes
 // over hub ranges [lo, hi): each pass gathers the messages of its range into
 // the hub maps (the first pass) and the shared-memory set (shrinking hi when
@@ -971,7 +1020,7 @@ __device__ void emit_maps(uint8_t* B, uint32_t vb, uint32_t W, uint32_t* row, in
 // the maps and leave them in rank order, so the new row needs no later sort.
 __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32_t* S, uint32_t* M, uint32_t* C,
                                 uint8_t* B, uint32_t* gacc, int* sh, int* wsum, int* sex, int64_t* sst, int* hist,
-                                uint32_t* tv, unsigned long long* cnt) {
+                                uint32_t* tv, unsigned long long* cnt, uint32_t* gbits) {
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int lane = tid & 31, wid = tid >> 5, nw = nthr >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -1015,8 +1064,8 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
     // hubs below vb + W (the most frequent messages) are deduplicated in the
     // maps, in the first pass, for vertices with many messages (for the others
     // scanning the maps costs more than the hashing it saves)
-    const uint32_t W =
-        p.rbound[v] >= kByteMinBound ? min((uint32_t)(kByteHubs + kBitHubs), (uint32_t)v - vb) : 0u;
+    const uint32_t W = gbits || p.rbound[v] >= kByteMinBound
+                           ? min((uint32_t)(kByteHubs + kBitHubs), (uint32_t)v - vb) : 0u;
     const uint32_t Wb = min(W, (uint32_t)kByteHubs);
     uint4* b4 = reinterpret_cast<uint4*>(B);
     uint32_t* bits = reinterpret_cast<uint32_t*>(B + kByteHubs);
@@ -1039,8 +1088,11 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
             *hi_sm = (uint32_t)min((int64_t)v, (int64_t)lo + width);
         }
         __syncthreads();
-        gather_block(p, nb, ne, lo, hi_sm, B, vb, W, S, log_s, useM ? M : nullptr, log_m, limit, &sh[SH_UNIQ],
-                     (volatile int*)&sh[SH_OVF], wsum, sex, sst, C, hist, &sh[SH_TMP], cnt[1]);
+        if (gbits)
+            load_maps(B, W, gbits);
+        else
+            gather_block(p, nb, ne, lo, hi_sm, B, vb, W, S, log_s, useM ? M : nullptr, log_m, limit, &sh[SH_UNIQ],
+                         (volatile int*)&sh[SH_OVF], wsum, sex, sst, C, hist, &sh[SH_TMP], cnt[1]);
         __syncthreads();
         const uint32_t hi = *(volatile uint32_t*)hi_sm;
         const bool maps = lo == vb && W > 0;
@@ -1242,15 +1294,57 @@ __global__ void __launch_bounds__(256, 3) k_gp_block(GpParams p) {
     unsigned long long cnt[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     if (p.ctr->done) return;
     const uint32_t d = p.ctr->d;
-    const int n1 = *p.list_n;
-    if ((int)blockIdx.x >= n1) return;
+    const int n1 = *p.list_n, np = p.split.max > 0 ? min(p.ctr->nP, p.split.max_parts) : 0;
+    if ((int)blockIdx.x >= np + n1) return;  // (as many blocks as entries are enough)
     // the hub maps are empty between vertices
 #pragma unroll 1
     for (int q = threadIdx.x; q < kMapWords; q += blockDim.x) reinterpret_cast<uint32_t*>(B)[q] = 0u;
+    // parts of split receivers first, then the list's vertices (in rank order:
+    // the largest first), handed out one at a time
+    int next = 0;
+    if (threadIdx.x == 0) sh[SH_ITEM] = atomicAdd(p.work, 1);
     __syncthreads();
 #pragma unroll 1
-    for (int i = blockIdx.x; i < n1; i += gridDim.x) {
-        gp_block_vertex(p, d, p.list[i], S, M, C, B, gacc, sh, wsum, sex, sst, hist, tv, cnt);
+    while (true) {
+        const int i = *(volatile int*)&sh[SH_ITEM];
+        if (i >= np + n1) break;
+        if (threadIdx.x == 0) next = atomicAdd(p.work, 1);
+        int32_t v = 0;
+        uint32_t* gbits = nullptr;
+        bool whole = true;
+        if (i < np) {
+            const int2 part = p.split.parts[i];
+            v = p.split.v[part.x];
+            gbits = p.split.bits + (int64_t)part.x * p.split.words;
+            const uint32_t vb = base_of(p.vbase, v), W = (uint32_t)v - vb;  // (all of v's hubs fit the maps)
+            const int64_t nb = p.roff[v] + (int64_t)part.y * kSplitPart;
+            const int64_t ne = min(p.roff[v + 1], nb + kSplitPart);
+            uint32_t* hi_sm = reinterpret_cast<uint32_t*>(&sh[SH_HI]);
+            if (threadIdx.x == 0) {
+                sh[SH_UNIQ] = 0;
+                sh[SH_OVF] = 0;
+                *hi_sm = (uint32_t)v;
+            }
+            __syncthreads();
+            gather_block(p, nb, ne, vb, hi_sm, B, vb, W, S, p.log_s, nullptr, 0, p.cand_limit, &sh[SH_UNIQ],
+                         (volatile int*)&sh[SH_OVF], wsum, sex, sst, C, hist, &sh[SH_TMP], cnt[1]);
+            __syncthreads();
+            flush_maps(B, W, gbits);
+            __threadfence();
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                const bool last = atomicAdd(&p.split.done[part.x], 1) == p.split.nparts[part.x] - 1;
+                if (last) p.split.done[part.x] = 0;
+                sh[SH_LAST] = last;
+            }
+            __syncthreads();
+            __threadfence();
+            whole = *(volatile int*)&sh[SH_LAST] != 0;
+        } else {
+            v = p.list[i - np];
+        }
+        if (whole) gp_block_vertex(p, d, v, S, M, C, B, gacc, sh, wsum, sex, sst, hist, tv, cnt, gbits);
+        if (threadIdx.x == 0) sh[SH_ITEM] = next;
         __syncthreads();
     }
     cnt[1] = warp_sum(cnt[1]);

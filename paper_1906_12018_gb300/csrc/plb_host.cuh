@@ -124,6 +124,28 @@ inline size_t gp_block_smem_bytes(int bthr, int log_s, int log_m, int cand_limit
                                kMapWords);
 }
 
+// Lists and bitmaps of the split receivers of a build over n vertices (the
+// largest graph of a union: max_part_n) and nnz arcs.  A receiver is split from
+// kSplitArcs arcs on, so at most nnz / kSplitArcs receivers are, and their
+// parts number at most nnz / kSplitPart + one each.
+inline SplitLists split_lists(DevPool& pool, int64_t n, int64_t max_part_n, int64_t nnz, cudaStream_t s) {
+    SplitLists l{};
+    const int64_t most = std::min<int64_t>(kMaxSplit, nnz / kSplitArcs);
+    if (most <= 0 || n <= 0) return l;
+    l.max = (int)most;
+    l.max_parts = (int)(nnz / kSplitPart + most);
+    l.words = (int)((std::min<int64_t>(max_part_n, kByteHubs + kBitHubs) + 31) / 32);
+    l.v = pool.alloc<int32_t>(most);
+    l.nparts = pool.alloc<int>(most);
+    l.done = pool.alloc<int>(most);
+    l.bits = pool.alloc<uint32_t>(most * l.words);
+    l.parts = pool.alloc<int2>(l.max_parts);
+    if (pool.failed || cudaMemsetAsync(l.done, 0, sizeof(int) * most, s) != cudaSuccess ||
+        cudaMemsetAsync(l.bits, 0, sizeof(uint32_t) * most * l.words, s) != cudaSuccess)
+        pool.failed = true;
+    return l;
+}
+
 // Records the failing CUDA call for plb_last_error (this thread).
 void set_last_error(cudaError_t e, int line);
 

@@ -35,8 +35,10 @@ struct RoundCounters {
     int nR, nO1, nO2;             // receivers: warp tier, block tier (nO2 unused)
     int nBig, nGiant;             // new frontier rows too long for a warp / for shared memory to sort
     int nU;                       // vertices whose new frontier row was written unsorted (block tier)
+    int wkR, wkO1, wkO2;          // next entry of each tier's list (taken by whoever is free)
+    int nG, nP;                   // split receivers and their parts (see SplitLists)
     int nA;                       // next active list (kept across the per-round reset)
-    int nO1_base, nO2_base;       // tier-list sizes made by k_collect (for reruns)
+    int nO1_base, nG_base;        // list sizes made by k_collect (for reruns and statistics)
     int fovf;                     // new-frontier buffer overflow
     unsigned int max_dist;        // finalize: largest stored distance
     int guard;                    // a kernel met a broken capacity invariant (internal error)
@@ -65,6 +67,24 @@ struct RoundStat {
     long long receivers, accepted, uniq, probed, msgs, pref, arcs, staged, tier0, tier1, chk_lv, chk_lh;
 };
 
+// Receivers with many arcs (hubs) are split: blocks gather parts of kSplitPart
+// arcs into shared-memory maps and OR these into the receiver's global bitmap;
+// the block that ends last goes on with the merged bitmap.  No block waits for
+// another.  (One block takes 4 to 5 us per 256 arcs of dependent loads: a hub
+// with 209,550 arcs kept a round from ending for up to 4 ms.)  Only for
+// receivers whose hubs all fit the maps.
+constexpr int kSplitArcs = 2048;   // arcs from which a receiver is split
+constexpr int kSplitPart = 1024;   // arcs per part
+constexpr int kMaxSplit = 512;     // split receivers per round (further ones are not split)
+struct SplitLists {
+    int32_t* v;        // [max] receivers
+    int* nparts;       // [max] parts of each
+    int* done;         // [max] parts gathered (zero between launches)
+    uint32_t* bits;    // [max x words] bitmaps (zero between launches)
+    int2* parts;       // (receiver's index, part)
+    int max, max_parts, words;
+};
+
 struct GpParams {
     const int64_t* roff;
     const int32_t* rcol;
@@ -77,6 +97,8 @@ struct GpParams {
     unsigned long long fcap;   // capacity of fhub_new
     const int32_t* list;       // vertices handled by this tier
     const int* list_n;
+    int* work;                 // counter that hands out the list's entries (after the parts)
+    SplitLists split;          // block tier: parts to gather before the list's vertices (split.max = 0: none)
     int32_t* esc;              // escalation list (next tier)
     int* esc_n;
     RoundCounters* ctr;        // also holds the round number d (ctr->d)

@@ -187,7 +187,8 @@ __global__ void k_mark(const int64_t* roff, const int32_t* rcol, const uint64_t*
     }
 }
 
-// Receivers (recv[v] > 0) are routed by the candidate bound min(v, recv[v])
+// Receivers (recv[v] > 0) with many arcs are split (SplitLists), the others
+// are routed by the candidate bound min(v, recv[v])
 // (v counted from the first rank of its graph in a disjoint union),
 // |L(v)| and degree: warp tier (R) or block tier (O1); the bound is kept in
 // rbound[v] (it sizes the warp tier's tables) and, when obound is given, in
@@ -196,7 +197,7 @@ __global__ void k_mark(const int64_t* roff, const int32_t* rcol, const uint64_t*
 // the bounds.
 __global__ void k_collect(unsigned long long* recv, const int64_t* roff, const int64_t* loff, int64_t n,
                           uint64_t* fse_new, int32_t* R, int32_t* O1, uint32_t* rbound, int64_t* obound,
-                          const int32_t* vbase, RoundCounters* ctr, TierLimits lim) {
+                          const int32_t* vbase, SplitLists split, RoundCounters* ctr, TierLimits lim) {
     if (ctr->done) return;
     unsigned long long bsum = 0;
     const int lane = lane_id();
@@ -215,6 +216,17 @@ __global__ void k_collect(unsigned long long* recv, const int64_t* roff, const i
             const int64_t ll = loff[v + 1] - loff[v];
             const int64_t deg = roff[v + 1] - roff[v];
             tier = ((int64_t)bound <= lim.warp_bound && ll <= lim.warp_label && deg <= lim.warp_deg) ? 0 : 1;
+            if (deg > kSplitArcs && below <= (unsigned long long)(kByteHubs + kBitHubs) && split.max > 0) {
+                const int np = (int)((deg + kSplitPart - 1) / kSplitPart);
+                const int g = atomicAdd(&ctr->nG, 1);
+                if (g < split.max) {
+                    tier = -1;
+                    split.v[g] = (int32_t)v;
+                    split.nparts[g] = np;
+                    const int at = atomicAdd(&ctr->nP, np);  // (in all at most max_parts: see split_lists)
+                    for (int t = 0; t < np; ++t) split.parts[at + t] = make_int2(g, t);
+                }
+            }
         }
         const unsigned am = __activemask();
         int32_t* lists[2] = {R, O1};
@@ -238,7 +250,8 @@ __global__ void k_collect(unsigned long long* recv, const int64_t* roff, const i
 __global__ void k_after_collect(RoundCounters* ctr) {
     if (ctr->done) return;
     ctr->nO1_base = ctr->nO1;
-    ctr->nO2_base = ctr->nO2;
+    ctr->nG = min(ctr->nG, kMaxSplit);
+    ctr->nG_base = ctr->nG;
     ctr->nA_saved = ctr->nA;
     ctr->nA = 0;
 }
@@ -362,7 +375,8 @@ __global__ void k_rerun_reset(RoundCounters* ctr, uint64_t* fse_new, int64_t n) 
         fse_new[v] = 0;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctr->nO1 = ctr->nO1_base;
-        ctr->nO2 = ctr->nO2_base;
+        ctr->nO2 = 0;
+        ctr->wkR = ctr->wkO1 = ctr->wkO2 = 0;
         ctr->cursor = 0;
         ctr->accepted = 0;
         ctr->fovf = 0;
@@ -839,7 +853,7 @@ __global__ void k_g_check(RoundCounters* ctr, RoundStat* stats) {
     }
     if (d < PLB_MAX_ROUNDS) {
         RoundStat& r = stats[d];
-        r.receivers = ctr->nR + ctr->nO1_base;
+        r.receivers = ctr->nR + ctr->nO1_base + ctr->nG_base;
         r.accepted = acc;
         r.uniq = (long long)ctr->uniq;
         r.probed = (long long)ctr->probed;
@@ -882,7 +896,8 @@ __global__ void k_g_finish(RoundCounters* ctr) {
     ctr->tier[0] = ctr->tier[1] = ctr->tier[2] = 0;
     ctr->bound_sum = ctr->prefiltered = 0;
     ctr->nR = ctr->nO1 = ctr->nO2 = ctr->nBig = ctr->nGiant = ctr->nU = 0;
-    ctr->nO1_base = ctr->nO2_base = ctr->fovf = 0;
+    ctr->wkR = ctr->wkO1 = ctr->wkO2 = ctr->nG = ctr->nP = 0;
+    ctr->nO1_base = ctr->nG_base = ctr->fovf = 0;
 }
 
 // Loop condition of the graph: continue while not done.

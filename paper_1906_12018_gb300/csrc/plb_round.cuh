@@ -26,7 +26,7 @@ __global__ void k_mark(const int64_t* roff, const int32_t* rcol, const uint64_t*
                        int64_t n);
 __global__ void k_collect(unsigned long long* recv, const int64_t* roff, const int64_t* loff, int64_t n,
                           uint64_t* fse_new, int32_t* R, int32_t* O1, uint32_t* rbound, int64_t* obound,
-                          const int32_t* vbase, RoundCounters* ctr, TierLimits lim);
+                          const int32_t* vbase, SplitLists split, RoundCounters* ctr, TierLimits lim);
 __global__ void k_after_collect(RoundCounters* ctr);
 __global__ void k_rerun_reset(RoundCounters* ctr, uint64_t* fse_new, int64_t n);
 __global__ void k_round1_count(const int64_t* roff, const int32_t* rcol, int64_t n, int64_t nnz, int32_t s,

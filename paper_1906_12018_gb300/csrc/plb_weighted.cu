@@ -153,7 +153,8 @@ __global__ void k_w_rerun(RoundCounters* ctr, uint64_t* fse_new, int64_t n, unsi
         fse_new[v] = 0;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctr->nO1 = ctr->nO1_base;
-        ctr->nO2 = ctr->nO2_base;
+        ctr->nO2 = 0;
+        ctr->wkR = ctr->wkO1 = ctr->wkO2 = 0;
         ctr->cursor = base;
         ctr->accepted = 0;
         ctr->fovf = 0;
@@ -373,6 +374,8 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     uint32_t* gacc = pool.alloc<uint32_t>((int64_t)grid_b * std::max<int64_t>(n, 1));
     PLB_ALLOC_OK();
 
+    const SplitLists split = split_lists(pool, n, n, nnz, s);
+    PLB_ALLOC_OK();
     auto read_ctr = [&]() -> cudaError_t {
         return cudaMemcpyAsync(hctr, ctr, sizeof(RoundCounters), cudaMemcpyDeviceToHost, s);
     };
@@ -424,7 +427,10 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
         p.stage_ratio = o.warp_stage_ratio;
         p.count_check = o.profile != 0;
         p.unsorted = U;
+        p.work = &ctr->wkR;
         k_gp_warp<<<grid_w, kGpWarpThreads, w_smem, s>>>(p);
+        p.work = &ctr->wkO1;
+        p.split = split;
         p.list = O1;
         p.list_n = &ctr->nO1;
         p.esc = nullptr;
@@ -448,7 +454,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
         if (nnz > 0)
             k_w_pull<<<gpull, kWFlatThreads, 0, s>>>(roff, rcol, rwt, n, nnz, (uint32_t)d, S, lgn, ring, store,
                                                      vcol, recv);
-        k_collect<<<gflat, kFlatThreads, 0, s>>>(recv, roff, loff[cur], n, fse_new, R, O1, rbound, nullptr, nullptr, ctr, lim);
+        k_collect<<<gflat, kFlatThreads, 0, s>>>(recv, roff, loff[cur], n, fse_new, R, O1, rbound, nullptr, nullptr, split, ctr, lim);
         k_after_collect<<<1, 1, 0, s>>>(ctr);
         launches += 4;
         PLB_CK(cudaGetLastError());
@@ -464,7 +470,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
         }
         if (tm.on) tm.span(T_FRONT, r0, tm.mark());
         cudaEvent_t g0 = tm.on ? tm.mark() : nullptr;
-        const bool any = hctr->nR + hctr->nO1_base > 0;
+        const bool any = hctr->nR + hctr->nO1_base + hctr->nG_base > 0;
         if (any) {
             for (int attempt = 0;; ++attempt) {
                 if (attempt > 0) {
@@ -485,7 +491,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
         if (tm.on) tm.span(T_GPW, g0, tm.mark());
         const int64_t acc = any ? (int64_t)hctr->accepted : 0;
         if (d < PLB_MAX_ROUNDS) {
-            st.receivers[d] = (int64_t)hctr->nR + hctr->nO1_base;
+            st.receivers[d] = (int64_t)hctr->nR + hctr->nO1_base + hctr->nG_base;
             st.accepted[d] = acc;
             st.unique_round[d] = any ? (int64_t)hctr->uniq : 0;
             st.prefiltered_round[d] = any ? (int64_t)hctr->prefiltered : 0;
