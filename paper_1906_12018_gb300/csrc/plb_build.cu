@@ -110,7 +110,9 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
     int64_t lcap[2] = {std::max<int64_t>(2 * n, 1024), std::max<int64_t>(2 * n, 1024)};
     int64_t* loff[2] = {pool.alloc<int64_t>(n + 1), pool.alloc<int64_t>(n + 1)};
     uint32_t* lent[2] = {pool.alloc<uint32_t>(lcap[0]), pool.alloc<uint32_t>(lcap[1])};
-    int64_t fcap[2] = {std::max<int64_t>(nnz / 2 + n, 1024), std::max<int64_t>(nnz / 2 + n, 1024)};
+    // (round 1 writes at most nnz / 2 hubs, padded rows)
+    int64_t fcap[2] = {std::max<int64_t>(nnz / 2 + kRowAlign * n, 1024),
+                       std::max<int64_t>(nnz / 2 + kRowAlign * n, 1024)};
     uint64_t* fse[2] = {pool.alloc<uint64_t>(n), pool.alloc<uint64_t>(n)};
     uint32_t* fhub[2] = {pool.alloc<uint32_t>(fcap[0]), pool.alloc<uint32_t>(fcap[1])};
     unsigned long long* recv = pool.alloc<unsigned long long>(n);
@@ -124,7 +126,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
     int64_t* aoff = pool.alloc<int64_t>(n + 1);
     PLB_ALLOC_OK();
     PLB_CK(cudaMemsetAsync(recv, 0, sizeof(unsigned long long) * std::max<int64_t>(n, 1), s));
-    k_init<<<gflat, kFlatThreads, 0, s>>>(roff, n, loff[0], lent[0], fse[0], fhub[0], A, ctr);
+    k_init<<<gflat, kFlatThreads, 0, s>>>(roff, n, loff[0], lent[0], fse[0], nullptr, A, ctr);
     PLB_CK(cudaGetLastError());
     st.launches += 1;
     int64_t T = n;  // labels so far
@@ -204,8 +206,8 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
     const int warp_cand = pow2_at_least(std::max(32, o.warp_cand_cap));
     const int warp_label = std::max(16, o.warp_label_cap);
     // set tables: load <= 1/2 at the candidate limit, plus the inserts a gather
-    // step can make before it sees the count (kGatherUnroll x 32 per warp)
-    const int w_log_s = ceil_log2_i64(std::max<int64_t>(2 * warp_cand, warp_cand + 32 * kGatherUnroll));
+    // step can make before it sees the count (block tier: kRowAlign per thread)
+    const int w_log_s = ceil_log2_i64(2 * (int64_t)warp_cand);
     const int w_log_m = ceil_log2_i64(2 * warp_label);
     const int warps_per_block = kGpWarpThreads / 32;
     const size_t w_smem = sizeof(uint32_t) * (4 * warps_per_block +
@@ -213,7 +215,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
     const int bthr = std::min(256, std::max(64, (o.block_threads / 32) * 32));  // k_gp_block: <= 256 threads
     const int block_cand = pow2_at_least(std::max(bthr, o.block_cand_cap));
     const int b_log_s = ceil_log2_i64(std::max<int64_t>(std::max<int64_t>(2 * (int64_t)block_cand,
-                                                                           block_cand + (int64_t)kGatherUnroll * bthr),
+                                                                           block_cand + (int64_t)kRowAlign * bthr),
                                                           (int64_t)kWarpStage * (bthr / 32)));
     const int b_log_m = ceil_log2_i64(2 * (int64_t)std::max(o.block_label_cap, 64) + 2 * bthr);
     const size_t b_smem = gp_block_smem_bytes(bthr, b_log_s, b_log_m, block_cand);
@@ -412,8 +414,8 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
             if (nnz > 0)
                 k_round1_count<<<g1, kFlatThreads, 0, s>>>(roff, rcol, n, nnz, (int32_t)batch_lo, (int32_t)batch_hi,
                                                           reinterpret_cast<unsigned long long*>(tmp64), ctr);
-            PLB_CK(exclusive_scan_i64(tmp64, tmp64, n, scan_scr, s));
-            k_round1<<<g1, kFlatThreads, 0, s>>>(roff, rcol, n, nnz, (int32_t)batch_lo, (int32_t)batch_hi, tmp64,
+            PLB_CK(exclusive_scan_i64(tmp64, aoff, n, scan_scr, s, nullptr, kRowAlign));
+            k_round1<<<g1, kFlatThreads, 0, s>>>(roff, rcol, n, nnz, (int32_t)batch_lo, (int32_t)batch_hi, tmp64, aoff,
                                                 cur1, fse[nxt], fhub[nxt], (unsigned long long)fcap[nxt], ctr);
             st.launches += 3 + scan_n;
             PLB_CK(cudaGetLastError());

@@ -165,7 +165,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
             S.lcap[b] = std::max<int64_t>(2 * n, 1024);
             S.loff[b] = pool.alloc<int64_t>(n + 1);
             S.lent[b] = pool.alloc<uint32_t>(S.lcap[b]);
-            S.fcap[b] = std::max<int64_t>(nnz + n, 1024);  // round 1 adds at most one label per arc
+            S.fcap[b] = std::max<int64_t>(nnz + kRowAlign * n, 1024);  // round 1 adds at most one label per arc
             S.fse[b] = pool.alloc<uint64_t>(n);
             S.fhub[b] = pool.alloc<uint32_t>(S.fcap[b]);
         }
@@ -183,7 +183,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
         S.aoff = pool.alloc<int64_t>(n + 1);
         PLB_ALLOC_OK();
         PLB_CK(cudaMemsetAsync(S.recv, 0, sizeof(unsigned long long) * std::max<int64_t>(n, 1), s));
-        k_init<<<gflat, kFlatThreads, 0, s>>>(S.s_off, n, S.loff[0], S.lent[0], S.fse[0], S.fhub[0], S.A, S.ctr);
+        k_init<<<gflat, kFlatThreads, 0, s>>>(S.s_off, n, S.loff[0], S.lent[0], S.fse[0], nullptr, S.A, S.ctr);
         k_top_init<<<flat_grid_cap, kFlatThreads, 0, s>>>(S.top, n);
         PLB_CK(cudaGetLastError());
         S.T = n;
@@ -224,7 +224,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
     // tier geometry (as in the undirected build)
     const int warp_cand = pow2_at_least(std::max(32, o.warp_cand_cap));
     const int warp_label = std::max(16, o.warp_label_cap);
-    const int w_log_s = ceil_log2_i64(std::max<int64_t>(2 * warp_cand, warp_cand + 32 * kGatherUnroll));
+    const int w_log_s = ceil_log2_i64(2 * (int64_t)warp_cand);
     const int w_log_m = ceil_log2_i64(2 * warp_label);
     const int warps_per_block = kGpWarpThreads / 32;
     const size_t w_smem = sizeof(uint32_t) * (4 * warps_per_block +
@@ -232,7 +232,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
     const int bthr = std::min(256, std::max(64, (o.block_threads / 32) * 32));
     const int block_cand = pow2_at_least(std::max(bthr, o.block_cand_cap));
     const int b_log_s = ceil_log2_i64(std::max<int64_t>(
-        std::max<int64_t>(2 * (int64_t)block_cand, block_cand + (int64_t)kGatherUnroll * bthr),
+        std::max<int64_t>(2 * (int64_t)block_cand, block_cand + (int64_t)kRowAlign * bthr),
         (int64_t)kWarpStage * (bthr / 32)));
     const int b_log_m = ceil_log2_i64(2 * (int64_t)std::max(o.block_label_cap, 64) + 2 * bthr);
     const size_t b_smem = gp_block_smem_bytes(bthr, b_log_s, b_log_m, block_cand);
@@ -369,8 +369,8 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
                 if (nnz > 0)
                     k_round1_count<<<g1, kFlatThreads, 0, s>>>(S.g_off, S.g_col, n, nnz, 0, (int32_t)n,
                                                               reinterpret_cast<unsigned long long*>(tmp64), S.ctr);
-                PLB_CK(exclusive_scan_i64(tmp64, tmp64, n, scan_scr, s));
-                k_round1<<<g1, kFlatThreads, 0, s>>>(S.g_off, S.g_col, n, nnz, 0, (int32_t)n, tmp64, cur1, S.fse[x],
+                PLB_CK(exclusive_scan_i64(tmp64, S.aoff, n, scan_scr, s, nullptr, kRowAlign));
+                k_round1<<<g1, kFlatThreads, 0, s>>>(S.g_off, S.g_col, n, nnz, 0, (int32_t)n, tmp64, S.aoff, cur1, S.fse[x],
                                                     S.fhub[x], (unsigned long long)S.fcap[x], S.ctr);
                 launches += 2 + scan_n;
                 PLB_CK(cudaGetLastError());

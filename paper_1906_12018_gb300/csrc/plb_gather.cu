@@ -426,48 +426,73 @@ __device__ void shrink_pass(uint32_t* S, int log_s, uint32_t* C, int limit, uint
     }
 }
 
+// A hub past the maps: into the set S, unless it is in L(v) (M) or the set is
+// full (*ovf_sm).  Returns 1 when it is new.
+__device__ __noinline__ int set_add(uint32_t* S, int log_s, const uint32_t* M, int log_m, int limit,
+                                    volatile int* cnt_sm, volatile int* ovf_sm, uint32_t h) {
+    if (M && map_has(M, log_m, h)) return 0;
+    if (*cnt_sm >= limit) {
+        *ovf_sm = 1;
+        return 0;
+    }
+    return set_insert(S, log_s, h) ? 1 : 0;
+}
+
 // Block-wide load-balanced gather of v's messages with hub in [lo, *hi_sm):
 // hubs below vb + W (vb: the first rank of v's graph) are marked in the maps B
 // (the first kByteHubs one byte each, plain stores: duplicates write the same
 // byte; the following ones one bit each; L(v)'s hubs are cleared afterwards),
-// the others go into the set S.  Neighbours are taken in tiles of blockDim; each thread finds its
-// neighbour's sub-range of dL_{d-1}(a) (binary searches in the sorted row), a
-// block-wide exclusive scan of the counts assigns every thread an equal,
-// contiguous share of the tile's messages.  When the set would exceed
-// `limit`, its range (hubs >= W) is shrunk (shrink_pass: S keeps the keys
-// below the new bound) and every warp resumes its share of the tile from the
-// step where it stopped, now dropping hubs at or above the new bound (a later
-// pass takes them): no message of the tile is read twice, except those of
-// the step that met the overflow.
-__device__ void gather_block(const GpParams& p, int64_t nb, int64_t ne, uint32_t lo, uint32_t* hi_sm, uint8_t* B,
-                             uint32_t vb, uint32_t W, uint32_t* S, int log_s, const uint32_t* M, int log_m, int limit, int* cnt_sm,
-                             volatile int* ovf_sm, int* wsum, int* sex, int64_t* sst, uint32_t* C, int* hist, int* tmp,
-                             unsigned long long& msgs) {
+// the others go into the set S.  Neighbours are taken in tiles of blockDim; each
+// thread finds the sectors (eight hubs) of its neighbour's row dL_{d-1}(a) that
+// overlap the range (the row is sorted), a block-wide exclusive scan of their
+// counts assigns every warp an equal, contiguous share, and every lane reads
+// one sector per step: the search for a lane's row, 20 instructions, then
+// serves eight messages instead of one (R-MAT 2^22 took 134 + 72 ms of warp
+// time in rounds 2 and 3 to gather its 52G messages one per lane).  When the
+// set would exceed `limit`, its range (hubs >= vb + W) is shrunk (shrink_pass: S
+// keeps the keys below the new bound) and every warp resumes its share of the
+// tile from the step where it stopped, now dropping hubs at or above the new
+// bound (a later pass takes them): no message of the tile is read twice, except
+// those of the step that met the overflow.
+__device__ __noinline__ void gather_block(const GpParams& p, int64_t nb, int64_t ne, uint32_t lo, uint32_t* hi_sm, uint8_t* B,
+                             uint32_t vb, uint32_t W, uint32_t* S, int log_s, const uint32_t* M, int log_m, int limit,
+                             int* cnt_sm, volatile int* ovf_sm, int* wsum, int* sex, int64_t* sst, uint32_t* C,
+                             int* hist, int* tmp, unsigned long long& msgs) {
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int nw = nthr >> 5, lane = tid & 31;
+    const uint32_t set_lo = max(lo, vb + W);  // S holds hubs from here on
+    if (lo > vb) W = 0;                       // the maps are the first pass's
     const uint32_t Wb = min(W, (uint32_t)kByteHubs);
     uint32_t* bits = reinterpret_cast<uint32_t*>(B + kByteHubs);
 #pragma unroll 1
     for (int64_t t0 = nb; t0 < ne; t0 += nthr) {
         const uint32_t hi = *(volatile uint32_t*)hi_sm;
         const int64_t j = t0 + tid;
-        int c = 0;
+        int c = 0;  // sectors
         int64_t st = 0;
         if (j < ne) {
             const int32_t a = p.rcol[j];
             const uint64_t f = p.fse[a];
-            const uint32_t n0 = fcount(f);
+            const int n0 = (int)fcount(f);
             if (n0) {
                 // the hubs of a frontier row of sender a are <= a (a itself
                 // only in round 0): for a < hi the whole row lies below hi
                 const uint32_t* row = p.fhub + fstart(f);
-                const int64_t a0 = lo > vb ? lower_bound_u32(row, n0, lo) : 0;
-                const int64_t a1 = sender_of(p, a) < hi ? (int64_t)n0 : lower_bound_u32(row, n0, hi);
-                st = (int64_t)fstart(f) + a0;
-                c = (int)(a1 - a0);
+                const int a0 = lo > vb ? (int)lower_bound_u32(row, n0, lo) / kRowAlign : 0;
+                int a1 = (n0 + kRowAlign - 1) / kRowAlign;
+                if (sender_of(p, a) >= hi) {  // sectors whose first hub is below hi
+                    int l = a0;
+#pragma unroll 1
+                    while (l < a1) {
+                        const int mid = (l + a1) >> 1;
+                        if (row[kRowAlign * mid] < hi) l = mid + 1; else a1 = mid;
+                    }
+                }
+                st = (int64_t)fstart(f) + (int64_t)kRowAlign * a0;
+                c = a1 - a0;
             }
         }
-        // message offsets of the tile's non-empty rows, compacted (rows cut
+        // sector offsets of the tile's non-empty rows, compacted (rows cut
         // to nothing by the hub range are common and would otherwise be
         // stepped over item by item)
         int total, nne;
@@ -480,13 +505,14 @@ __device__ void gather_block(const GpParams& p, int64_t nb, int64_t ne, uint32_t
         }
         if (tid == 0) sex[nne] = total;
         __syncthreads();
-        // each warp takes a contiguous range of the tile's messages and walks
+        // each warp takes a contiguous range of the tile's sectors and walks
         // it in windows of 32 rows: lane j holds the start of row k0 + j, and
-        // 32 consecutive messages at a time find their row by a warp-shuffle
-        // search, so that the lanes of a load read consecutive hubs of a row
+        // 32 consecutive sectors at a time find their row by a warp-shuffle
+        // search
         const int per_w = (((total + nw - 1) / nw) + 31) & ~31;
         const int wbeg = (tid >> 5) * per_w, wend = min(total, wbeg + per_w);
-        int pos = wbeg;  // this warp's messages before pos are done
+        int pos = wbeg;  // this warp's sectors before pos are done
+        unsigned n_msgs = 0;
 #pragma unroll 1
         while (true) {
             // hubs at or above hcut are left to a later pass (hcut = hi
@@ -504,51 +530,51 @@ __device__ void gather_block(const GpParams& p, int64_t nb, int64_t ne, uint32_t
                 for (int it0 = pos; it0 < wend && !stop; k0 += 32) {
                     const int kr = k0 + lane;
                     const int ex = kr < nne ? sex[kr] : total;
-                    const int64_t stv = kr < nne ? sst[kr] : 0;
-                    const int wcap = k0 + 32 < nne ? sex[k0 + 32] : total;
-                    const int wend_w = min(wend, wcap);
+                    // sector i of the tile, in this lane's row, is at row + 8 i
+                    const uint32_t* row = p.fhub + ((kr < nne ? sst[kr] : 0) - (int64_t)kRowAlign * ex);
+                    const int wend_w = min(wend, k0 + 32 < nne ? sex[k0 + 32] : total);
 #pragma unroll 1
-                    for (int ib = it0; ib < wend_w; ib += 32 * kGatherUnroll) {
-                        uint32_t hv[kGatherUnroll];
-                        // a step inside one row (long rows): every lane reads
-                        // that row, no per-lane owner search
-                        const int k1 = warp_owner(ex, ib);
-                        const int end1 = k1 < 31 ? __shfl_sync(kFull, ex, k1 + 1) : wcap;
-                        if (ib + 32 * kGatherUnroll <= min(end1, wend_w)) {
-                            const int64_t at = __shfl_sync(kFull, stv, k1) + (ib - __shfl_sync(kFull, ex, k1)) + lane;
-#pragma unroll
-                            for (int u = 0; u < kGatherUnroll; ++u) hv[u] = p.fhub[at + 32 * u];
+                    for (int ib = it0; ib < wend_w; ib += 32) {
+                        const int it = ib + lane;
+                        const int kk = warp_owner(ex, it);
+                        const uint32_t* rk =
+                            reinterpret_cast<const uint32_t*>(__shfl_sync(kFull, (unsigned long long)row, kk));
+                        uint32_t x[kRowAlign];
+                        if (it < wend_w) {
+                            load_sector(rk + (int64_t)kRowAlign * it, x);
                         } else {
 #pragma unroll
-                            for (int u = 0; u < kGatherUnroll; ++u) {
-                                const int it = ib + 32 * u + lane;
-                                const int kk = warp_owner(ex, it);
-                                const int exk = __shfl_sync(kFull, ex, kk);
-                                const int64_t stk = __shfl_sync(kFull, stv, kk);
-                                hv[u] = it < wend_w ? p.fhub[stk + (it - exk)] : kEmpty;
-                            }
+                            for (int q = 0; q < kRowAlign; ++q) x[q] = kEmpty;
                         }
-                        int nins = 0;
+                        unsigned past = 0, got = 0;  // hubs past the maps, messages of the range
 #pragma unroll
-                        for (int u = 0; u < kGatherUnroll; ++u) {
-                            const uint32_t h = hv[u];
-                            if (h - vb < Wb) {
-                                B[h - vb] = 1;
-                            } else if (h - vb < W) {
-                                const uint32_t q = h - vb - (uint32_t)kByteHubs;
-                                atomicOr(&bits[q >> 5], 1u << (q & 31));
-                            } else if (h - vb < hcut - vb && (!M || !map_has(M, log_m, h))) {
-                                if (*(volatile int*)cnt_sm >= limit) *ovf_sm = 1;
-                                else nins += set_insert(S, log_s, h) ? 1 : 0;
+                        for (int q = 0; q < kRowAlign; ++q) {
+                            const uint32_t hr = x[q] - vb;
+                            if (hr < Wb) {
+                                B[hr] = 1;
+                            } else if (hr < W) {
+                                const uint32_t z = hr - (uint32_t)kByteHubs;
+                                atomicOr(&bits[z >> 5], 1u << (z & 31));
+                            } else if (x[q] - set_lo < hcut - set_lo) {
+                                past |= 1u << q;
+                            }
+                            got += x[q] - lo < hi - lo ? 1u : 0u;
+                        }
+                        if (__any_sync(kFull, past != 0u)) {
+                            int nins = 0;
+#pragma unroll
+                            for (int q = 0; q < kRowAlign; ++q)
+                                if ((past >> q) & 1u)
+                                    nins += set_add(S, log_s, M, log_m, limit, cnt_sm, ovf_sm, x[q]);
+                            nins = warp_sum(nins);
+                            if (lane == 0 && nins) atomicAdd(cnt_sm, nins);
+                            if (__any_sync(kFull, *ovf_sm != 0)) {
+                                stop = true;  // resume from this step after the shrink
+                                pos = ib;
+                                break;
                             }
                         }
-                        nins = warp_sum(nins);
-                        if (lane == 0 && nins) atomicAdd(cnt_sm, nins);
-                        if (__any_sync(kFull, *ovf_sm != 0)) {
-                            stop = true;  // resume from this step after the shrink
-                            pos = ib;
-                            break;
-                        }
+                        n_msgs += got;
                     }
                     if (!stop) it0 = wend_w;
                 }
@@ -557,15 +583,14 @@ __device__ void gather_block(const GpParams& p, int64_t nb, int64_t ne, uint32_t
             __syncthreads();
             // concurrent inserts can pass the limit without raising the flag
             if (*ovf_sm || *(volatile int*)cnt_sm > limit) {
-                // S holds hubs >= vb + W
-                shrink_pass(S, log_s, C, limit, lo > vb + W ? lo : vb + W, hi_sm, cnt_sm, hist, tmp);
+                shrink_pass(S, log_s, C, limit, set_lo, hi_sm, cnt_sm, hist, tmp);
                 if (tid == 0) *ovf_sm = 0;
                 __syncthreads();
                 continue;  // every warp resumes at its pos with the smaller range
             }
             break;
         }
-        if (tid == 0) msgs += total;
+        msgs += n_msgs;
         __syncthreads();  // sex / sst are rewritten by the next tile
     }
 }
@@ -792,12 +817,14 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
             for (int s = lane; s < (1 << log_m); s += 32) X[s] = 0u;
         if (nacc > 0) {
             unsigned long long start = 0;
+            const int padded = (int)row_pad(nacc);
             if (lane == 0)
                 start = p.ostart ? (unsigned long long)p.ostart[v]
-                                 : atomicAdd(&p.ctr->cursor, (unsigned long long)nacc);
+                                 : atomicAdd(&p.ctr->cursor, (unsigned long long)padded);
             start = __shfl_sync(kFull, start, 0);
-            if (start + nacc <= p.fcap) {
+            if (start + padded <= p.fcap) {
                 uint32_t* row = p.fhub_new + start;
+                if (nacc + lane < padded) row[nacc + lane] = kEmpty;
                 // the new row leaves sorted by hub rank: the bitmap's hubs as
                 // they are, then the set's, moved to the front of S and sorted
                 const int n0 = nacc - ntail;
@@ -1241,14 +1268,16 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
     const int64_t total_acc = (int64_t)macc + sacc;
     if (total_acc > 0) {
         if (tid == 0) {
-            const unsigned long long start = p.ostart ? (unsigned long long)p.ostart[v]
-                                                      : atomicAdd(&p.ctr->cursor, (unsigned long long)total_acc);
+            const unsigned long long start =
+                p.ostart ? (unsigned long long)p.ostart[v]
+                         : atomicAdd(&p.ctr->cursor, (unsigned long long)row_pad(total_acc));
             *(unsigned long long*)(sh + SH_START) = start;
         }
         __syncthreads();
         const unsigned long long start = *(volatile unsigned long long*)(sh + SH_START);
-        const bool fits = start + total_acc <= p.fcap;
+        const bool fits = start + row_pad(total_acc) <= p.fcap;
         uint32_t* row = p.fhub_new + start;
+        if (fits && total_acc + tid < row_pad(total_acc)) row[total_acc + tid] = kEmpty;
         if (macc > 0) emit_maps(B, vb, W, fits ? row : nullptr, sh);
         if (fits) {
             const bool sorted = sacc <= S_CAP;

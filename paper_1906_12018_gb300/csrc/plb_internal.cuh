@@ -297,7 +297,7 @@ cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t s);
 // Device-wide exclusive scan of int64 values; out may alias in.
 // count(i) is evaluated for i in [0, n) and out[n] receives the total.
 cudaError_t exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* block_sums,
-                               cudaStream_t s, const int* skip = nullptr);
+                               cudaStream_t s, const int* skip = nullptr, int64_t align = 1);
 int64_t scan_scratch_elems(int64_t n);
 int scan_launch_count(int64_t n);
 

@@ -28,7 +28,7 @@ struct RoundCounters {
     unsigned long long accepted;  // new labels this round
     unsigned long long arcs, msgs, uniq, staged, probed;
     unsigned long long tier[3];
-    unsigned long long bound_sum; // sum over receivers of the candidate bound min(v, messages)
+    unsigned long long bound_sum; // sum over receivers of the candidate bound min(v, messages), as padded rows
     unsigned long long prefiltered; // candidates pruned by the top-hub witness prefilter
     unsigned long long chk_lv, chk_lh;  // checked candidates (h at v): sums of |L(v) entries with hub < h|
                                         // and of |L(h)| (counted when GpParams::count_check is set)
@@ -168,9 +168,10 @@ constexpr int kTopRow = kTopLevels * kTopWords;      // words per vertex
 // what it reads lies together (the 32-byte masks of 2^17 hubs in 4 MB; with
 // all levels of a vertex side by side they were spread over 29 MB).
 
-// Messages each lane loads before inserting them (gathers keep several loads
-// in flight per warp).
-constexpr int kGatherUnroll = 4;
+// Frontier rows start at multiples of kRowAlign hubs (32 bytes) and are filled
+// up to one with kEmpty: the block tier reads them a sector at a time.
+constexpr int kRowAlign = 8;
+__host__ __device__ __forceinline__ int64_t row_pad(int64_t c) { return (c + kRowAlign - 1) & ~(int64_t)(kRowAlign - 1); }
 
 // Block tier: the highest-ranked hubs (of the vertex's graph) are deduplicated
 // in shared-memory maps instead of the hash set: the first kByteHubs in a byte

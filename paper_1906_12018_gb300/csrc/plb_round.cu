@@ -122,13 +122,19 @@ __global__ void k_relabel(const int64_t* row_ptr, const int32_t* col, const int3
 }
 
 // L(v) = dL(v) = {(v, 0)}; active = vertices with at least one neighbour.
+// With fhub, the frontier rows of round 0 (padded: 8 n entries); else none (round
+// 1 reads the arcs instead: k_round1).
 __global__ void k_init(const int64_t* roff, int64_t n, int64_t* loff, uint32_t* lent, uint64_t* fse,
                        uint32_t* fhub, int32_t* A, RoundCounters* ctr) {
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
         loff[v] = v;
         lent[v] = pack((uint32_t)v, 0);
-        fhub[v] = (uint32_t)v;
-        fse[v] = fpack((uint64_t)v, 1);
+        if (fhub) {
+            uint4* row = reinterpret_cast<uint4*>(fhub + kRowAlign * v);
+            row[0] = make_uint4((uint32_t)v, kEmpty, kEmpty, kEmpty);
+            row[1] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+            fse[v] = fpack((uint64_t)(kRowAlign * v), 1);
+        }
         const bool act = roff[v + 1] > roff[v];
         const unsigned am = __activemask();
         const unsigned m = __ballot_sync(am, act);
@@ -208,10 +214,10 @@ __global__ void k_collect(unsigned long long* recv, const int64_t* roff, const i
         // v accepts hubs of its own graph that outrank it: at most v - base
         const unsigned long long below = (unsigned long long)(v - (int64_t)base_of(vbase, v));
         const unsigned long long bound = c < below ? c : below;
-        if (obound) obound[v] = (int64_t)bound;
+        if (obound) obound[v] = row_pad((int64_t)bound);
         if (c) recv[v] = 0;
         if (bound) {
-            bsum += bound;
+            bsum += (unsigned long long)row_pad((int64_t)bound);
             rbound[v] = (uint32_t)bound;  // v < 2^24
             const int64_t ll = loff[v + 1] - loff[v];
             const int64_t deg = roff[v + 1] - roff[v];
@@ -298,21 +304,21 @@ __global__ void k_round1_count(const int64_t* roff, const int32_t* rcol, int64_t
     }
 }
 
-// Write pass: row v of the new frontier at start[v] (the exclusive scan of
-// the counts: no shared cursor), start[n] entries in all; within a row the
+// Write pass: row v of the new frontier, cnt[v] hubs, at start[v] (the exclusive
+// scan of the padded counts: no shared cursor), start[n] entries in all; within a row the
 // entries are placed by the per-row cursor cur[v] (zero on entry; one atomic
 // per row and warp).  Then, per vertex, the frontier descriptor and the
 // counters.
 __global__ void k_round1(const int64_t* roff, const int32_t* rcol, int64_t n, int64_t nnz, int32_t s, int32_t e,
-                         const int64_t* start, uint32_t* cur, uint64_t* fse_new, uint32_t* fhub_new,
-                         unsigned long long fcap, RoundCounters* ctr) {
+                         const int64_t* cnt_row, const int64_t* start, uint32_t* cur, uint64_t* fse_new,
+                         uint32_t* fhub_new, unsigned long long fcap, RoundCounters* ctr) {
     __shared__ __align__(16) int srow[kTileItems];
     __shared__ TileScratch sh;
     if (ctr->done) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctr->nA_saved = ctr->nA;
         ctr->nA = 0;
-        if ((unsigned long long)start[n] > fcap) ctr->fovf = 1;  // cannot happen: the buffer holds every arc
+        if ((unsigned long long)start[n] > fcap) ctr->fovf = 1;  // cannot happen: the buffer holds every padded row
         else ctr->cursor = (unsigned long long)start[n];
     }
     if ((unsigned long long)start[n] > fcap) return;
@@ -348,9 +354,10 @@ __global__ void k_round1(const int64_t* roff, const int32_t* rcol, int64_t n, in
     unsigned long long c_acc = 0, c_arcs = 0, c_recv = 0;
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
         const int64_t st = start[v];
-        const int64_t c = start[v + 1] - st;
+        const int64_t c = cnt_row[v];
         fse_new[v] = c ? fpack((uint64_t)st, (uint32_t)c) : 0ull;
         if (c) {
+            for (int64_t j = st + c; j < start[v + 1]; ++j) fhub_new[j] = kEmpty;
             c_acc += (unsigned long long)c;
             c_arcs += (unsigned long long)(roff[v + 1] - roff[v]);
             c_recv += 1;

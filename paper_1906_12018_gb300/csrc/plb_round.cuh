@@ -32,8 +32,8 @@ __global__ void k_rerun_reset(RoundCounters* ctr, uint64_t* fse_new, int64_t n);
 __global__ void k_round1_count(const int64_t* roff, const int32_t* rcol, int64_t n, int64_t nnz, int32_t s,
                                int32_t e, unsigned long long* cnt, const RoundCounters* ctr);
 __global__ void k_round1(const int64_t* roff, const int32_t* rcol, int64_t n, int64_t nnz, int32_t s, int32_t e,
-                         const int64_t* start, uint32_t* cur, uint64_t* fse_new, uint32_t* fhub_new,
-                         unsigned long long fcap, RoundCounters* ctr);
+                         const int64_t* cnt_row, const int64_t* start, uint32_t* cur, uint64_t* fse_new,
+                         uint32_t* fhub_new, unsigned long long fcap, RoundCounters* ctr);
 __global__ void k_gp_warp(GpParams p);
 __global__ void k_gp_block(GpParams p);
 __global__ void k_index_size(const int64_t* loff, int64_t n, int64_t* hsz, const RoundCounters* ctr);

@@ -44,8 +44,9 @@ __device__ int64_t block_excl_scan(int64_t x, int64_t* sh_warp, int64_t* total) 
     return r;
 }
 
+// (pad: the values are rounded up to multiples of pad + 1, a power of two)
 __global__ void __launch_bounds__(kThreads) k_scan_sums(const int64_t* in, int64_t n, int64_t* tile_sums,
-                                                        const int* skip) {
+                                                        int64_t pad, const int* skip) {
     __shared__ int64_t sh_warp[kThreads / 32];
     if (skip && *skip) return;
     const int64_t base = (int64_t)blockIdx.x * kTile;
@@ -53,7 +54,7 @@ __global__ void __launch_bounds__(kThreads) k_scan_sums(const int64_t* in, int64
 #pragma unroll
     for (int k = 0; k < kPerThread; ++k) {
         const int64_t i = base + k * kThreads + threadIdx.x;
-        if (i < n) sum += in[i];
+        if (i < n) sum += (in[i] + pad) & ~pad;
     }
     sum = warp_sum(sum);
     if ((threadIdx.x & 31) == 0) sh_warp[threadIdx.x >> 5] = sum;
@@ -65,7 +66,7 @@ __global__ void __launch_bounds__(kThreads) k_scan_sums(const int64_t* in, int64
 }
 
 __global__ void __launch_bounds__(kThreads) k_scan_write(const int64_t* in, int64_t* out, int64_t n,
-                                                         const int64_t* tile_sums, const int* skip) {
+                                                         const int64_t* tile_sums, int64_t pad, const int* skip) {
     __shared__ int64_t sh_warp[kThreads / 32 + 1];
     if (skip && *skip) return;
     const int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kPerThread;
@@ -74,7 +75,7 @@ __global__ void __launch_bounds__(kThreads) k_scan_write(const int64_t* in, int6
 #pragma unroll
     for (int k = 0; k < kPerThread; ++k) {
         const int64_t i = base + k;
-        v[k] = i < n ? in[i] : 0;
+        v[k] = i < n ? (in[i] + pad) & ~pad : 0;
         sum += v[k];
     }
     for (int64_t t = threadIdx.x; t < blockIdx.x; t += kThreads) before += tile_sums[t];
@@ -91,7 +92,7 @@ __global__ void __launch_bounds__(kThreads) k_scan_write(const int64_t* in, int6
 }
 
 // single-tile scan writing out[n] = total
-__global__ void __launch_bounds__(kThreads) k_scan_single(const int64_t* in, int64_t* out, int64_t n,
+__global__ void __launch_bounds__(kThreads) k_scan_single(const int64_t* in, int64_t* out, int64_t n, int64_t pad,
                                                           const int* skip) {
     __shared__ int64_t sh_warp[kThreads / 32 + 1];
     if (skip && *skip) return;
@@ -101,7 +102,7 @@ __global__ void __launch_bounds__(kThreads) k_scan_single(const int64_t* in, int
 #pragma unroll
     for (int k = 0; k < kPerThread; ++k) {
         const int64_t i = base + k;
-        v[k] = i < n ? in[i] : 0;
+        v[k] = i < n ? (in[i] + pad) & ~pad : 0;
         sum += v[k];
     }
     int64_t total;
@@ -124,16 +125,18 @@ int scan_launch_count(int64_t n) { return n <= kTile ? 1 : 2; }
 
 // out[0..n] = exclusive scan of in[0..n), out[n] = sum (out may be in).  With
 // skip, every kernel returns at once while *skip is non-zero (graph-driven
-// rounds after the loop has finished).
+// rounds after the loop has finished).  With align (a power of two) every value
+// is rounded up to a multiple of it first.
 cudaError_t exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* scratch, cudaStream_t s,
-                               const int* skip) {
+                               const int* skip, int64_t align) {
+    const int64_t pad = align - 1;
     if (n <= kTile) {
-        k_scan_single<<<1, kThreads, 0, s>>>(in, out, n, skip);
+        k_scan_single<<<1, kThreads, 0, s>>>(in, out, n, pad, skip);
         return cudaGetLastError();
     }
     const int64_t tiles = (n + kTile - 1) / kTile;
-    k_scan_sums<<<(unsigned)tiles, kThreads, 0, s>>>(in, n, scratch, skip);
-    k_scan_write<<<(unsigned)tiles, kThreads, 0, s>>>(in, out, n, scratch, skip);
+    k_scan_sums<<<(unsigned)tiles, kThreads, 0, s>>>(in, n, scratch, pad, skip);
+    k_scan_write<<<(unsigned)tiles, kThreads, 0, s>>>(in, out, n, scratch, pad, skip);
     return cudaGetLastError();
 }
 

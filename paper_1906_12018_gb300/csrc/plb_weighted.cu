@@ -281,7 +281,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     uint32_t* lent[2] = {pool.alloc<uint32_t>(lcap[0]), pool.alloc<uint32_t>(lcap[1])};
     // frontier ring (S slots of 2^lgn descriptors, then the empty one) and store
     uint64_t* ring = pool.alloc<uint64_t>(ring_n + 1);
-    int64_t scap = std::max<int64_t>(n + nnz + 1024, 4096);
+    int64_t scap = std::max<int64_t>(kRowAlign * n + nnz + 1024, 4096);
     uint32_t* store = pool.alloc<uint32_t>(scap);
     uint32_t* top = pool.alloc<uint32_t>(n * kTopRow);
     int64_t* hoff = pool.alloc<int64_t>(n + 1);
@@ -297,14 +297,14 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     PLB_ALLOC_OK();
     PLB_CK(cudaMemsetAsync(ring, 0, sizeof(uint64_t) * ((size_t)ring_n + 1), s));
     PLB_CK(cudaMemsetAsync(recv, 0, sizeof(unsigned long long) * (size_t)n, s));
-    // round 0: L(v) = dL_0(v) = {(v, 0)}; its frontier rows are store[0, n)
+    // round 0: L(v) = dL_0(v) = {(v, 0)}; its frontier rows are store[0, 8 n)
     k_init<<<gflat, kFlatThreads, 0, s>>>(roff, n, loff[0], lent[0], ring, store, A, ctr);
     k_top_init<<<flat_grid_cap, kFlatThreads, 0, s>>>(top, n);
     PLB_CK(cudaGetLastError());
     launches += 2;
     int cur = 0;
     int64_t T = n;       // labels so far
-    int64_t base = n;    // store entries used (next round's rows start here)
+    int64_t base = kRowAlign * n;  // store entries used (next round's rows start here)
     plb_build_stats st{};
     st.n = n;
     st.nnz = nnz;
@@ -340,7 +340,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     // tier geometry (as in the undirected build)
     const int warp_cand = pow2_at_least(std::max(32, o.warp_cand_cap));
     const int warp_label = std::max(16, o.warp_label_cap);
-    const int w_log_s = ceil_log2_i64(std::max<int64_t>(2 * warp_cand, warp_cand + 32 * kGatherUnroll));
+    const int w_log_s = ceil_log2_i64(2 * (int64_t)warp_cand);
     const int w_log_m = ceil_log2_i64(2 * warp_label);
     const int warps_per_block = kGpWarpThreads / 32;
     const size_t w_smem = sizeof(uint32_t) * (4 * warps_per_block +
@@ -348,7 +348,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     const int bthr = std::min(256, std::max(64, (o.block_threads / 32) * 32));
     const int block_cand = pow2_at_least(std::max(bthr, o.block_cand_cap));
     const int b_log_s = ceil_log2_i64(std::max<int64_t>(
-        std::max<int64_t>(2 * (int64_t)block_cand, block_cand + (int64_t)kGatherUnroll * bthr),
+        std::max<int64_t>(2 * (int64_t)block_cand, block_cand + (int64_t)kRowAlign * bthr),
         (int64_t)kWarpStage * (bthr / 32)));
     const int b_log_m = ceil_log2_i64(2 * (int64_t)std::max(o.block_label_cap, 64) + 2 * bthr);
     const size_t b_smem = gp_block_smem_bytes(bthr, b_log_s, b_log_m, block_cand);

@@ -2,6 +2,7 @@
 oracle (bit-exact)."""
 import numpy as np
 import pytest
+import torch
 
 import oracle as O
 from paper_1906_12018_gb300 import graphs as G
@@ -47,3 +48,53 @@ def test_hubs_around_the_map_boundaries(n, deg, lead, opts):
     assert_labels_equal(lab, O.pll(g.off, g.col, order), f"lead {lead}")
     if lead > 4096 and deg == 400:  # (with few ranks the candidate bounds stay within the warp tier)
         assert lab.stats()["tier_vertices"][1] > 0
+
+
+def hub_edges(leaves, arcs, seed):
+    """Hubs 0..len(arcs)-1 with the given numbers of random leaves, and a sparse
+    random graph on the leaves."""
+    rng = np.random.default_rng(seed)
+    k = len(arcs)
+    src = [np.full(c, i) for i, c in enumerate(arcs)] + [k + rng.integers(0, leaves, leaves)]
+    dst = [k + rng.choice(leaves, c, replace=False) for c in arcs] + [k + rng.integers(0, leaves, leaves)]
+    return k + leaves, np.concatenate(src), np.concatenate(dst)
+
+
+# arcs per hub: at and next to the least number that is split (2,048) and whole
+# and ragged numbers of parts (1,024); the leaves' graph adds none to the hubs
+HUB_ARCS = [2047, 2048, 2049, 3072, 3073, 5000, 9000]
+
+
+@pytest.mark.parametrize("opts", [{}, {"use_graph": 1}, {"batch_hubs": 5000}], ids=["host", "graph", "rank batches"])
+def test_split_receivers(opts):
+    n, src, dst = hub_edges(9500, HUB_ARCS, 1)
+    g = G.clean_csr(n, src.astype(np.int32), dst.astype(np.int32))
+    rng = np.random.default_rng(2)
+    mixed = rng.permutation(n).astype(np.int32)  # hubs anywhere in the order
+    for order in (G.degree_order(g), mixed if not opts else None):
+        if order is None:
+            continue
+        rp, col, o = to_device(g, order)
+        assert_labels_equal(plb.build(rp, col, o, **opts), O.pll(g.off, g.col, order))
+
+
+def test_split_receivers_weighted():
+    n, src, dst = hub_edges(9500, HUB_ARCS, 3)
+    g = G.clean_csr(n, src.astype(np.int32), dst.astype(np.int32))
+    order = G.degree_order(g)
+    wt = G.edge_weights(g, 1, 5, 4)
+    rp, col, o = to_device(g, order)
+    lab = plb.build_weighted(rp, col, torch.from_numpy(wt).cuda(), o)
+    assert_labels_equal(lab, O.pll_weighted(g.off, g.col, wt, order))
+
+
+def test_split_receivers_directed():
+    n, src, dst = hub_edges(9500, HUB_ARCS, 5)
+    flip = np.random.default_rng(6).random(src.size) < 0.4
+    g = G.directed_csr(n, np.where(flip, dst, src), np.where(flip, src, dst))
+    order = G.directed_degree_order(g)
+    ref_in, ref_out = O.pll_directed(g.off, g.col, g.off_in, g.col_in, order)
+    lin, lout = plb.build_directed(torch.from_numpy(g.off).cuda(), torch.from_numpy(g.col).cuda(),
+                                   torch.from_numpy(order).cuda())
+    assert_labels_equal(lin, ref_in, "in")
+    assert_labels_equal(lout, ref_out, "out")
