@@ -301,32 +301,13 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         st.launches += 4 + 2 * scan_n;
         return cudaGetLastError();
     };
-    // Host-driven rounds run the two tiers concurrently: the block tier on a
-    // side stream over k_collect's block list while the warp tier runs on the
-    // build's stream and escalates into a second list, taken by one more
-    // block-tier launch after both (the tails of the two kernels overlap).
-    // Captured rounds (graph mode) run them one after the other.
-    cudaStream_t side = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    PLB_CK(cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking));
-    PLB_CK(cudaEventCreateWithFlags(&ev_fork, cudaEventDisableTiming));
-    PLB_CK(cudaEventCreateWithFlags(&ev_join, cudaEventDisableTiming));
-    struct SideGuard {
-        cudaStream_t st;
-        cudaEvent_t a, b;
-        ~SideGuard() {
-            cudaEventDestroy(a);
-            cudaEventDestroy(b);
-            cudaStreamDestroy(st);
-        }
-    } side_guard{side, ev_fork, ev_join};
+    SideStream side_stream;
+    PLB_CK(side_stream.create());
     auto launch_gp = [&](GpParams p, cudaEvent_t* g1) -> cudaError_t {
         k_pack_hrec<<<gflat, kFlatThreads, 0, s>>>(p.loff, p.lent, hdesc, vbase, hrec, n, ctr);
         st.launches += 1;
         GpParams w = p, b = p;
         w.list = R;  // warp tier
-        w.list_n = &ctr->nR;
-        w.work = &ctr->wkR;
         w.log_s = w_log_s;
         w.log_m = w_log_m;
         w.cand_limit = warp_cand;
@@ -336,29 +317,13 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         b.log_m = b_log_m;
         b.cand_limit = block_cand;
         if (skip == nullptr) {
-            w.esc = O2;
-            w.esc_n = &ctr->nO2;
-            b.list = O1;
-            b.list_n = &ctr->nO1;
-            b.work = &ctr->wkO1;
-            b.split = split;
-            cudaError_t e = cudaEventRecord(ev_fork, s);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(side, ev_fork, 0);
-            if (e != cudaSuccess) return e;
-            k_gp_block<<<grid_b, bthr, b_smem, side>>>(b);
-            k_gp_warp<<<grid_w, kGpWarpThreads, w_smem, s>>>(w);
-            if (g1) *g1 = tm.mark();
-            e = cudaEventRecord(ev_join, side);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev_join, 0);
-            if (e != cudaSuccess) return e;
-            b.list = O2;
-            b.list_n = &ctr->nO2;
-            b.work = &ctr->wkO2;
-            b.split = SplitLists{};
-            k_gp_block<<<grid_b, bthr, b_smem, s>>>(b);
             st.launches += 3;
-            return cudaGetLastError();
+            return launch_tiers(w, b, split, O1, O2, ctr, grid_w, w_smem, grid_b, bthr, b_smem, s, side_stream,
+                                g1 ? &tm : nullptr, g1);
         }
+        // captured rounds (graph mode): one after the other
+        w.list_n = &ctr->nR;
+        w.work = &ctr->wkR;
         w.esc = O1;
         w.esc_n = &ctr->nO1;
         k_gp_warp<<<grid_w, kGpWarpThreads, w_smem, s>>>(w);

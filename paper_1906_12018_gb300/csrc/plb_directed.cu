@@ -261,6 +261,11 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
     PLB_ALLOC_OK();
 
     // split receivers (both sides' frontier steps run before either gather)
+    uint4* hrec = pool.alloc<uint4>(std::max<int64_t>(n, 1));  // check records of the candidates' side
+    int32_t* O2 = pool.alloc<int32_t>(n);                      // warp-tier escalations
+    PLB_ALLOC_OK();
+    SideStream side_stream;
+    PLB_CK(side_stream.create());
     SplitLists split2[2];
     for (int k = 0; k < 2; ++k) split2[k] = split_lists(pool, n, n, nnz, s);
     PLB_ALLOC_OK();
@@ -306,28 +311,21 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
         p.rbound = S.rbound;
         p.list = S.R;
         p.list_n = &S.ctr->nR;
-        p.esc = S.O1;
-        p.esc_n = &S.ctr->nO1;
+        p.hrec_h = hrec;
         p.log_s = w_log_s;
         p.log_m = w_log_m;
         p.cand_limit = warp_cand;
         p.stage_ratio = o.warp_stage_ratio;
         p.count_check = o.profile != 0;
         p.unsorted = S.U;
-        p.work = &S.ctr->wkR;
-        k_gp_warp<<<grid_w, kGpWarpThreads, w_smem, s>>>(p);
-        p.work = &S.ctr->wkO1;
-        p.split = split2[&S - side];
-        p.list = S.O1;
-        p.list_n = &S.ctr->nO1;
-        p.esc = nullptr;
-        p.esc_n = nullptr;
-        p.log_s = b_log_s;
-        p.log_m = b_log_m;
-        p.cand_limit = block_cand;
-        k_gp_block<<<grid_b, bthr, b_smem, s>>>(p);
-        launches += 2;
-        return cudaGetLastError();
+        k_pack_hrec<<<gflat, kFlatThreads, 0, s>>>(p.loff_h, p.lent_h, p.hdesc_h, nullptr, hrec, n, S.ctr);
+        GpParams b = p;
+        b.log_s = b_log_s;
+        b.log_m = b_log_m;
+        b.cand_limit = block_cand;
+        launches += 4;
+        return launch_tiers(p, b, split2[&S - side], S.O1, O2, S.ctr, grid_w, w_smem, grid_b, bthr, b_smem, s,
+                            side_stream, nullptr);
     };
     auto merge = [&](Side& S) -> cudaError_t {
         const int c = S.cur, x = c ^ 1;

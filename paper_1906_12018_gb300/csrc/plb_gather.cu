@@ -172,7 +172,7 @@ __device__ __forceinline__ unsigned check_chunk(const GpParams& p, uint32_t d, c
     // load, one memory sector) is requested before the rest of the top-hub
     // prefilter reads h's masks, so the loads overlap
     uint4 rec = make_uint4(0u, 0u, 0u, 0u);
-    if (valid && p.hrec_h) rec = p.hrec_h[h];
+    if (valid) rec = p.hrec_h[h];
     const int imax = min((int)d - 1, kTopLevels);
     if (i0 == 0 || (p.sender_bits == 0 && imax > 1)) {
         uint32_t hit = 0;
@@ -187,21 +187,11 @@ __device__ __forceinline__ unsigned check_chunk(const GpParams& p, uint32_t d, c
     // past the top hubs when the prefilter settles them (see above)
     const bool skip_top = d <= (uint32_t)kTopLevels + 1u;
     if (valid) {
-        int64_t hb, he;
-        uint64_t hd;
-        int top_h = 0;  // entries of L(h) with hub < kTopHubs
-        if (p.hrec_h) {
-            const uint64_t row = ((uint64_t)rec.y << 32) | rec.x;
-            hb = (int64_t)(row >> 24);
-            he = hb + (int64_t)(row & 0xFFFFFFu);
-            hd = (((uint64_t)rec.w << 32) | rec.z) & kHrecDescMask;
-            top_h = (int)(rec.w >> kHrecTopShift);
-        } else {
-            hb = p.loff_h[h];
-            he = p.loff_h[h + 1];
-            hd = p.hdesc_h[h];
-        }
-        const int la = (int)(he - hb) - 1;
+        const uint64_t row = ((uint64_t)rec.y << 32) | rec.x;
+        const int64_t hb = (int64_t)(row >> 24);
+        const int la = (int)(row & 0xFFFFFFu) - 1;
+        const uint64_t hd = (((uint64_t)rec.w << 32) | rec.z) & kHrecDescMask;
+        const int top_h = (int)(rec.w >> kHrecTopShift);  // entries of L(h) with a top hub
         const int sa = skip_top ? min(top_h, la) : 0;  // side A starts past L(h)'s top hubs
         ent = p.lent_h + hb + sa;
         items = la - sa;
@@ -1089,10 +1079,8 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
     int64_t width = (int64_t)v - vb;
     uint32_t* hi_sm = reinterpret_cast<uint32_t*>(&sh[SH_HI]);
     // hubs below vb + W (the most frequent messages) are deduplicated in the
-    // maps, in the first pass, for vertices with many messages (for the others
-    // scanning the maps costs more than the hashing it saves)
-    const uint32_t W = gbits || p.rbound[v] >= kByteMinBound
-                           ? min((uint32_t)(kByteHubs + kBitHubs), (uint32_t)v - vb) : 0u;
+    // maps, in the first pass
+    const uint32_t W = min((uint32_t)(kByteHubs + kBitHubs), (uint32_t)v - vb);
     const uint32_t Wb = min(W, (uint32_t)kByteHubs);
     uint4* b4 = reinterpret_cast<uint4*>(B);
     uint32_t* bits = reinterpret_cast<uint32_t*>(B + kByteHubs);
@@ -1122,7 +1110,7 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
                          (volatile int*)&sh[SH_OVF], wsum, sex, sst, C, hist, &sh[SH_TMP], cnt[1]);
         __syncthreads();
         const uint32_t hi = *(volatile uint32_t*)hi_sm;
-        const bool maps = lo == vb && W > 0;
+        const bool maps = lo == vb;
         if (maps) {  // first pass: drop L(v)'s hubs from the maps
 #pragma unroll 1
             for (int64_t j = tid; j < ll; j += nthr) {

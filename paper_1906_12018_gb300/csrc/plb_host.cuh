@@ -146,6 +146,59 @@ inline SplitLists split_lists(DevPool& pool, int64_t n, int64_t max_part_n, int6
     return l;
 }
 
+// The block tier's stream beside the build's own, with its fork and join events.
+struct SideStream {
+    cudaStream_t st = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
+    cudaError_t create() {
+        cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
+        return e;
+    }
+    ~SideStream() {
+        if (fork) cudaEventDestroy(fork);
+        if (join) cudaEventDestroy(join);
+        if (st) cudaStreamDestroy(st);
+    }
+};
+
+// One gather + prune of host-driven rounds.  The two tiers run side by side:
+// the block tier on the side stream over k_collect's block list O1 (and the
+// split receivers), the warp tier on the build's stream, escalating into O2,
+// which one more block-tier launch takes after both (the tails of the two
+// kernels overlap).  w, b: the tiers' parameters without lists; tm and mark:
+// where to record the end of the warp tier (profiled builds), or null.
+inline cudaError_t launch_tiers(GpParams w, GpParams b, const SplitLists& split, int32_t* O1, int32_t* O2,
+                                RoundCounters* ctr, int grid_w, size_t w_smem, int grid_b, int bthr, size_t b_smem,
+                                cudaStream_t s, SideStream& side, Timer* tm, cudaEvent_t* mark = nullptr) {
+    w.list_n = &ctr->nR;
+    w.work = &ctr->wkR;
+    w.esc = O2;
+    w.esc_n = &ctr->nO2;
+    b.esc = nullptr;  // the block tier never escalates
+    b.esc_n = nullptr;
+    b.list = O1;
+    b.list_n = &ctr->nO1;
+    b.work = &ctr->wkO1;
+    b.split = split;
+    cudaError_t e = cudaEventRecord(side.fork, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(side.st, side.fork, 0);
+    if (e != cudaSuccess) return e;
+    k_gp_block<<<grid_b, bthr, b_smem, side.st>>>(b);
+    k_gp_warp<<<grid_w, kGpWarpThreads, w_smem, s>>>(w);
+    if (tm) *mark = tm->mark();
+    e = cudaEventRecord(side.join, side.st);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, side.join, 0);
+    if (e != cudaSuccess) return e;
+    b.list = O2;
+    b.list_n = &ctr->nO2;
+    b.work = &ctr->wkO2;
+    b.split = SplitLists{};
+    k_gp_block<<<grid_b, bthr, b_smem, s>>>(b);
+    return cudaGetLastError();
+}
+
 // Records the failing CUDA call for plb_last_error (this thread).
 void set_last_error(cudaError_t e, int line);
 

@@ -118,8 +118,8 @@ struct GpParams {
     const uint64_t* hdesc_h;
     const uint32_t* htab_h;
     const uint32_t* top_h;
-    const uint4* hrec_h;       // per vertex of the candidates' side, or null: {row start << 24 | row length
-                               // (64 bits), probe-table descriptor (64 bits)}, one 16-byte load per check
+    const uint4* hrec_h;       // per vertex of the candidates' side: {row start << 24 | row length (64
+                               // bits), probe-table descriptor (64 bits)}, one 16-byte load per check
     const uint32_t* rbound;    // per receiver: candidate bound min(v, messages)
     const int64_t* ostart;     // per receiver: start of its new frontier row (the scan of the bounds),
                                // or null (rows reserved with an atomic cursor)
@@ -179,14 +179,14 @@ __host__ __device__ __forceinline__ int64_t row_pad(int64_t c) { return (c + kRo
 // serialise atomics), the next kBitHubs in a bitmap (shared-memory atomicOr).
 // On R-MAT 2^22 28% of round 3's messages and 32% of its candidates rank past
 // 32,768, 1.6% and 2% past 131,072: a 32 KB byte map of 32,768 hubs left them
-// to the set; 16 KB of bytes and 16 KB of bits cover 147,456.
+// to the set; 16 KB of bytes and 16 KB of bits cover 147,456.  Every receiver
+// of the block tier uses them (only those with 2,048 candidates or more, the
+// others hashing: R-MAT 2^22 741 instead of 722 ms, directed R-MAT 2^20 125
+// instead of 119 ms).
 constexpr int kByteHubs = 16384;
 constexpr int kBitHubs = 131072;
 constexpr int kMapWords = kByteHubs / 4 + kBitHubs / 32;
 static_assert(kByteHubs % 512 == 0 && kBitHubs % 4096 == 0, "whole scan units");
-// Receivers whose candidate bound reaches this use the maps (for fewer
-// candidates scanning them costs more than the hashing it saves).
-constexpr uint32_t kByteMinBound = 2048;
 // Block tier, per warp: staged candidates (fewer than 64, plus 32 of one
 // extraction) and survivors of the first prefilter step (fewer than 32, plus 64)
 constexpr int kCandStage = 96, kSurvStage = 96;

@@ -375,6 +375,10 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     PLB_ALLOC_OK();
 
     const SplitLists split = split_lists(pool, n, n, nnz, s);
+    uint4* hrec = pool.alloc<uint4>(std::max<int64_t>(n, 1));  // check records
+    int32_t* O2 = pool.alloc<int32_t>(n);                      // warp-tier escalations
+    SideStream side_stream;
+    PLB_CK(side_stream.create());
     PLB_ALLOC_OK();
     auto read_ctr = [&]() -> cudaError_t {
         return cudaMemcpyAsync(hctr, ctr, sizeof(RoundCounters), cudaMemcpyDeviceToHost, s);
@@ -419,28 +423,20 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
         p.sender_bits = lgn;
         p.list = R;
         p.list_n = &ctr->nR;
-        p.esc = O1;
-        p.esc_n = &ctr->nO1;
         p.log_s = w_log_s;
         p.log_m = w_log_m;
         p.cand_limit = warp_cand;
         p.stage_ratio = o.warp_stage_ratio;
         p.count_check = o.profile != 0;
         p.unsorted = U;
-        p.work = &ctr->wkR;
-        k_gp_warp<<<grid_w, kGpWarpThreads, w_smem, s>>>(p);
-        p.work = &ctr->wkO1;
-        p.split = split;
-        p.list = O1;
-        p.list_n = &ctr->nO1;
-        p.esc = nullptr;
-        p.esc_n = nullptr;
-        p.log_s = b_log_s;
-        p.log_m = b_log_m;
-        p.cand_limit = block_cand;
-        k_gp_block<<<grid_b, bthr, b_smem, s>>>(p);
-        launches += 2;
-        return cudaGetLastError();
+        p.hrec_h = hrec;
+        k_pack_hrec<<<gflat, kFlatThreads, 0, s>>>(p.loff, p.lent, hdesc, nullptr, hrec, n, ctr);
+        GpParams b = p;
+        b.log_s = b_log_s;
+        b.log_m = b_log_m;
+        b.cand_limit = block_cand;
+        launches += 4;
+        return launch_tiers(p, b, split, O1, O2, ctr, grid_w, w_smem, grid_b, bthr, b_smem, s, side_stream, nullptr);
     };
 
     // ------------------------------------------------------------ rounds
