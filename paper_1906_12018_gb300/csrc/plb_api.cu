@@ -3,12 +3,13 @@
 #include <atomic>
 #include <vector>
 
-#include "plb_internal.cuh"
+#include "plb_kernels.cuh"
 
 namespace plb {
 
 int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order, int64_t n, int64_t nnz,
-               const plb_options& o, cudaStream_t s, plb_labels** out, int64_t max_part_n, const int32_t* vbase);
+               const plb_options& o, cudaStream_t s, plb_labels** out, int64_t max_part_n, const int32_t* vbase,
+               const int2* col_base, int64_t col_quads);
 int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order, int64_t n, int64_t nnz,
                         const plb_options& o, cudaStream_t s, plb_labels** out_in, plb_labels** out_out);
 int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_t* wt, const int32_t* order,
@@ -28,6 +29,7 @@ struct GraphDesc {
     const int32_t* col;
     const int32_t* order;
     int64_t vbase, ebase, n, nnz;
+    int2 cols;  // place of its top-hub columns (TopColumns::by_base)
 };
 
 __device__ __forceinline__ int find_part(const int64_t* base, int k, int64_t x) {
@@ -42,7 +44,7 @@ __device__ __forceinline__ int find_part(const int64_t* base, int k, int64_t x) 
 // Disjoint union: vertex u of part g becomes vbase[g] + u; the union order
 // lists part 0's order, then part 1's, ... (each part keeps its own order).
 __global__ void k_union_rows(const GraphDesc* gd, const int64_t* vb, int k, int64_t N, int64_t E, int64_t* U_off,
-                             int32_t* U_ord, int32_t* U_base) {
+                             int32_t* U_ord, int32_t* U_base, int2* U_cols) {
     for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < N; u += (int64_t)gridDim.x * blockDim.x) {
         const int g = find_part(vb, k, u);
         const GraphDesc d = gd[g];
@@ -50,6 +52,7 @@ __global__ void k_union_rows(const GraphDesc* gd, const int64_t* vb, int k, int6
         U_off[u] = d.ebase + d.row_ptr[lu];
         U_ord[u] = d.order[lu] + (int32_t)d.vbase;
         U_base[u] = (int32_t)d.vbase;  // ranks and ids of a part fill the same range
+        if (lu == 0) U_cols[u] = d.cols;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) U_off[N] = E;
 }
@@ -163,7 +166,8 @@ int plb_build(const plb_csr* g, const int32_t* vertex_order, const plb_options* 
     cudaStream_t s = (cudaStream_t)stream;
     (void)cudaGetLastError();
     if (g->n == 0) return empty_labels(out, s);
-    return plb::build_core(g->row_ptr, g->col, vertex_order, g->n, g->nnz, o, s, out, g->n, nullptr);
+    return plb::build_core(g->row_ptr, g->col, vertex_order, g->n, g->nnz, o, s, out, g->n, nullptr, nullptr,
+                           plb::column_quads(g->n));
 }
 
 int plb_build_directed(const plb_csr* g, const int32_t* vertex_order, const plb_options* opt, plb_stream stream,
@@ -206,11 +210,13 @@ static int build_union(const plb_csr* gs, const int32_t* const* orders, int64_t 
                        cudaStream_t s, plb_labels** outs) {
     std::vector<plb::GraphDesc> hd((size_t)k);
     std::vector<int64_t> vb((size_t)k + 1), eb((size_t)k + 1);
-    int64_t N = 0, E = 0;
+    int64_t N = 0, E = 0, quads = 0;
     for (int64_t i = 0; i < k; ++i) {
         vb[i] = N;
         eb[i] = E;
-        hd[i] = {gs[i].row_ptr, gs[i].col, orders[i], N, E, gs[i].n, gs[i].nnz};
+        hd[i] = {gs[i].row_ptr, gs[i].col, orders[i], N, E, gs[i].n, gs[i].nnz,
+                 make_int2((int)quads, plb::column_quads(gs[i].n))};
+        quads += plb::column_quads(gs[i].n);
         N += gs[i].n;
         E += gs[i].nnz;
     }
@@ -220,9 +226,10 @@ static int build_union(const plb_csr* gs, const int32_t* const* orders, int64_t 
     plb::GraphDesc* dgd = nullptr;
     int64_t *dvb = nullptr, *deb = nullptr, *U_off = nullptr, *eoff = nullptr;
     int32_t *U_col = nullptr, *U_ord = nullptr, *U_base = nullptr;
+    int2* U_cols = nullptr;
     auto cleanup = [&]() {
         for (void* p : {(void*)dgd, (void*)dvb, (void*)deb, (void*)U_off, (void*)eoff, (void*)U_col, (void*)U_ord,
-                        (void*)U_base})
+                        (void*)U_base, (void*)U_cols})
             if (p) cudaFreeAsync(p, s);
     };
     if (plb::dev_alloc((void**)&dgd, sizeof(plb::GraphDesc) * k, s) != cudaSuccess ||
@@ -232,7 +239,8 @@ static int build_union(const plb_csr* gs, const int32_t* const* orders, int64_t 
         plb::dev_alloc((void**)&U_off, sizeof(int64_t) * (N + 1), s) != cudaSuccess ||
         plb::dev_alloc((void**)&U_col, sizeof(int32_t) * std::max<int64_t>(E, 1), s) != cudaSuccess ||
         plb::dev_alloc((void**)&U_ord, sizeof(int32_t) * std::max<int64_t>(N, 1), s) != cudaSuccess ||
-        plb::dev_alloc((void**)&U_base, sizeof(int32_t) * std::max<int64_t>(N, 1), s) != cudaSuccess) {
+        plb::dev_alloc((void**)&U_base, sizeof(int32_t) * std::max<int64_t>(N, 1), s) != cudaSuccess ||
+        plb::dev_alloc((void**)&U_cols, sizeof(int2) * std::max<int64_t>(N, 1), s) != cudaSuccess) {
         (void)cudaGetLastError();
         cleanup();
         return PLB_ERR_OOM;
@@ -244,7 +252,7 @@ static int build_union(const plb_csr* gs, const int32_t* const* orders, int64_t 
         return PLB_ERR_CUDA;
     }
     if (N > 0) plb::k_union_rows<<<plb::grid_of(N), 256, 0, s>>>(dgd, dvb, (int)k, N, E, U_off, U_ord,
-                                                                      U_base);
+                                                                      U_base, U_cols);
     if (E > 0) plb::k_union_cols<<<plb::grid_of(E), 256, 0, s>>>(dgd, deb, (int)k, E, U_col);
     if (cudaGetLastError() != cudaSuccess) {
         cleanup();
@@ -253,7 +261,7 @@ static int build_union(const plb_csr* gs, const int32_t* const* orders, int64_t 
     plb_labels* U = nullptr;
     int64_t max_part = 1;  // a vertex accepts hubs of its own graph only
     for (int64_t i = 0; i < k; ++i) max_part = std::max<int64_t>(max_part, gs[i].n);
-    int st = N > 0 ? plb::build_core(U_off, U_col, U_ord, N, E, o, s, &U, max_part, U_base) : empty_labels(&U, s);
+    int st = N > 0 ? plb::build_core(U_off, U_col, U_ord, N, E, o, s, &U, max_part, U_base, U_cols, quads) : empty_labels(&U, s);
     if (st != PLB_OK) {
         cleanup();
         return st;

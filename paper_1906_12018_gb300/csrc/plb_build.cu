@@ -21,9 +21,12 @@ void set_last_error(cudaError_t e, int line) {
 // *out holds the labels (rows by original id).  max_part_n: the most vertices
 // of one graph when the CSR is a disjoint union (else n); a vertex's label
 // holds at most that many hubs, which sizes the block tier's accepted rows.
-// vbase: the first rank of each vertex's graph in that union (else null).
+// vbase: the first rank of each vertex's graph in that union (else null);
+// col_base, col_quads: the places of the graphs' top-hub columns and the size
+// of all (else null and column_quads(n)).
 int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order, int64_t n, int64_t nnz,
-               const plb_options& o, cudaStream_t s, plb_labels** out, int64_t max_part_n, const int32_t* vbase) {
+               const plb_options& o, cudaStream_t s, plb_labels** out, int64_t max_part_n, const int32_t* vbase,
+               const int2* col_base, int64_t col_quads) {
 #define PLB_CK(x)                                            \
     do {                                                     \
         const cudaError_t plb_e_ = (x);                      \
@@ -134,6 +137,8 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
     // top-hub distance rows (witness prefilter), updated by each merge
     uint32_t* top = pool.alloc<uint32_t>(n * kTopRow);
     PLB_ALLOC_OK();
+    const TopColumns cols = top_columns(pool, col_quads, col_base, s);
+    PLB_ALLOC_OK();
     k_top_init<<<flat_grid_cap, kFlatThreads, 0, s>>>(top, n);
     st.launches += 1;
     // probe index of L: a hub-keyed table per row of >= kIndexMinLen entries in
@@ -241,14 +246,17 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
     PLB_CK(cudaFuncSetAttribute(k_sort_rows_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)(16384 * sizeof(uint32_t))));
     PLB_CK(cudaFuncSetAttribute(k_sort_rows_radix, cudaFuncAttributeMaxDynamicSharedMemorySize, kSortRadixSmemBytes));
-    // block tier: per-block buffer of accepted hubs (at most v < n per vertex)
-    const int64_t acc_words = std::max<int64_t>(std::min<int64_t>(n, max_part_n), 1);
+    // block tier: per-block buffer of accepted hubs past the maps
+    const int64_t acc_words = accepted_words(std::min<int64_t>(n, max_part_n));
     uint32_t* gacc = pool.alloc<uint32_t>((int64_t)grid_b * acc_words);
     const SplitLists split = split_lists(pool, n, max_part_n, nnz, s);
     // per-vertex check records (row bounds and probe-table descriptor), packed before each gather
     uint4* hrec = pool.alloc<uint4>(std::max<int64_t>(n, 1));
     PLB_ALLOC_OK();
 
+    // hubs of the current batch (Alg. 4): ranks [batch_lo, batch_hi); one batch
+    // of all vertices is Alg. 3
+    const int64_t batch = o.batch_hubs > 0 ? std::min<int64_t>(o.batch_hubs, n) : n;
     // ------------------------------------------------------------ rounds
     // launch sequences of one round (buffers of parity c -> x = c ^ 1)
     // placed: the new-frontier buffer holds the bound sum, so the rows go where
@@ -275,6 +283,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         p.htab_h = htab;
         p.top = top;
         p.top_h = top;
+        p.cols_h = cols;
         p.hrec_h = hrec;
         p.gscratch = gacc;
         p.gscratch_words = acc_words;
@@ -349,16 +358,14 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
                                                            ctr);
         k_merge_new<<<grid_for((int64_t)n * 32, kFlatThreads, flat_grid_cap), kFlatThreads, 0, s>>>(
             loff[c], lent[c], loff[x], lent[x], fse[x], fhub[x], A, vbase, ctr, top, n);
-        st.launches += 6 + scan_n;
+        k_top_columns<<<grid_for((n + 31) / 32, 1, flat_grid_cap), 256, 0, s>>>(top, n, vbase, cols, batch < n, ctr);
+        st.launches += 7 + scan_n;
         return cudaGetLastError();
     };
 
     int status = PLB_OK;
     int d = 0;          // last completed round (of the current batch)
     bool finished = false;
-    // hubs of the current batch (Alg. 4): ranks [batch_lo, batch_hi); one batch
-    // of all vertices is Alg. 3
-    const int64_t batch = o.batch_hubs > 0 ? std::min<int64_t>(o.batch_hubs, n) : n;
     int64_t batch_lo = 0, batch_hi = n;
     std::vector<std::pair<int, cudaEvent_t>> round_ev;  // (round, start event)
     std::vector<char> host_stat(PLB_MAX_ROUNDS, 0);     // rounds whose statistics the host recorded

@@ -33,6 +33,7 @@ struct Side {
     uint32_t* fhub[2] = {nullptr, nullptr};
     int64_t fcap[2] = {0, 0};
     uint32_t* top = nullptr;
+    TopColumns cols{};
     int64_t* hoff = nullptr;
     uint64_t* hdesc = nullptr;
     uint32_t* htab = nullptr;
@@ -170,6 +171,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
             S.fhub[b] = pool.alloc<uint32_t>(S.fcap[b]);
         }
         S.top = pool.alloc<uint32_t>(n * kTopRow);
+        S.cols = top_columns(pool, column_quads(n), nullptr, s);
         S.hoff = pool.alloc<int64_t>(n + 1);
         S.hdesc = pool.alloc<uint64_t>(n);
         S.hcap = std::max<int64_t>(4 * n, 1024);
@@ -257,7 +259,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
     const int sort_blocks = 8;
     const int64_t sort_words = pow2_at_least(std::max<int64_t>(n, 1));
     uint32_t* sortscr = pool.alloc<uint32_t>(sort_words * sort_blocks);
-    uint32_t* gacc = pool.alloc<uint32_t>((int64_t)grid_b * std::max<int64_t>(n, 1));
+    uint32_t* gacc = pool.alloc<uint32_t>((int64_t)grid_b * accepted_words(n));
     PLB_ALLOC_OK();
 
     // split receivers (both sides' frontier steps run before either gather)
@@ -306,8 +308,9 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
         p.hdesc_h = H.hdesc;
         p.htab_h = H.htab;
         p.top_h = H.top;
+        p.cols_h = H.cols;
         p.gscratch = gacc;
-        p.gscratch_words = std::max<int64_t>(n, 1);
+        p.gscratch_words = accepted_words(n);
         p.rbound = S.rbound;
         p.list = S.R;
         p.list_n = &S.ctr->nR;
@@ -341,7 +344,8 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
                                                            S.fhub[x], n, S.ctr);
         k_merge_new<<<grid_for((int64_t)n * 32, kFlatThreads, flat_grid_cap), kFlatThreads, 0, s>>>(
             S.loff[c], S.lent[c], S.loff[x], S.lent[x], S.fse[x], S.fhub[x], S.A, nullptr, S.ctr, S.top, n);
-        launches += 6 + scan_n;
+        k_top_columns<<<grid_for((n + 31) / 32, 1, flat_grid_cap), 256, 0, s>>>(S.top, n, nullptr, S.cols, 0, S.ctr);
+        launches += 7 + scan_n;
         return cudaGetLastError();
     };
     auto read_ctr = [&](Side& S) -> cudaError_t {

@@ -867,7 +867,7 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
 // Block-per-vertex scalars in shared memory (ints)
 enum { SH_UNIQ = 0, SH_OVF = 1, SH_ACC = 2 /* accepted, from the set */, SH_NC = 3, SH_HI = 4, SH_TMP = 5 /* 2 ints */,
        SH_START = 8 /* 2 ints */, SH_NEXT = 10, SH_REST = 11, SH_MACC = 12 /* accepted, from the maps */,
-       SH_ITEM = 13, SH_LAST = 14,
+       SH_ITEM = 13, SH_LAST = 14, SH_NE = 15 /* rows of the first prefilter step */,
        SH_WCNT = 16 /* 2 x 8 warps */, SH_WORDS = 48 };
 
 // Accepted candidates of a chunk (okm): those of the maps are marked there
@@ -895,10 +895,9 @@ __device__ __forceinline__ void keep_accepted(unsigned okm, uint32_t h, uint32_t
     if (ok && !inmap) gacc[base + __popc(ms & ((1u << lane) - 1u))] = h;
 }
 
-// The bytes of four map words as 16 bits.
-__device__ __forceinline__ uint32_t byte_bits(uint32_t x) {
-    return (x & 1u) | ((x >> 7) & 2u) | ((x >> 14) & 4u) | ((x >> 21) & 8u);
-}
+// The bytes (0 or 1) of four map words as 16 bits (the product's bits 28..31
+// are bytes 0..3; its other bits never meet, so nothing carries).
+__device__ __forceinline__ uint32_t byte_bits(uint32_t x) { return (x * 0x10204080u) >> 28; }
 __device__ __forceinline__ uint32_t byte_bits4(uint4 x) {
     return byte_bits(x.x) | (byte_bits(x.y) << 4) | (byte_bits(x.z) << 8) | (byte_bits(x.w) << 12);
 }
@@ -1029,9 +1028,11 @@ __device__ void load_maps(uint8_t* B, uint32_t W, uint32_t* gbits) {
 // than L2, and one chunk of 32 candidates checked from end to end took 5,000
 // to 12,000 cycles although most of its candidates need one mask only.  So the
 // check is split: each warp takes units of the maps and of the set from a
-// shared counter, stages 64 candidates, tests one mask of each (two
-// independent sectors per lane), and runs check_chunk on full warps of
-// survivors; the warps' last survivors are pooled and spread over all warps.
+// shared counter, prunes them by the top-hub columns (64 candidates per lane:
+// testing one 32-byte mask per candidate, and listing candidates for it, took
+// 108 and 143 ms of warp time in rounds 2 and 3 of R-MAT 2^22), and runs
+// check_chunk on full warps of survivors; the warps' last survivors are pooled
+// and spread over all warps.
 // L(v) is staged into the shared-memory map when it fits; otherwise it is
 // looked up in v's row of the global probe index.  Accepted hubs are marked in
 // the maps and leave them in rank order, so the new row needs no later sort.
@@ -1084,8 +1085,9 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
     const uint32_t Wb = min(W, (uint32_t)kByteHubs);
     uint4* b4 = reinterpret_cast<uint4*>(B);
     uint32_t* bits = reinterpret_cast<uint32_t*>(B + kByteHubs);
-    uint32_t* stage = S + wid * kWarpStage;  // (S is free once compacted)
-    uint32_t* surv = stage + kCandStage;
+    uint32_t* surv = S + wid * kWarpStage;  // (S is free once compacted)
+    uint32_t cwords;
+    const uint32_t* cols = columns_of(p.cols_h, vb, &cwords);
     const int imax = min((int)d - 1, kTopLevels);
 #pragma unroll 1
     while (lo < (uint32_t)v) {
@@ -1147,29 +1149,55 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
             for (int64_t j = tid; j < ll; j += nthr) lvs[j] = lv[j];
             lvp = lvs;
         }
+        // the rows of the first prefilter step (column offsets, in hist; filled
+        // up to a multiple of four): v's top hubs at distance i0, or at every
+        // distance in weighted rounds
+        const int i0 = first_level(tv, imax, lane);
+        if (wid == nw - 1) {
+            int ne = 0;
+#pragma unroll 1
+            for (int i = p.sender_bits ? 1 : i0; i <= (p.sender_bits ? imax : i0); ++i) {
+                uint32_t m = lane < kTopWords ? tv[(i - 1) * kTopWords + lane] : 0u;
+                const int c = __popc(m);
+                const int incl = warp_incl_scan(c, lane);
+                int o = ne + incl - c;
+                const int row0 = (min((int)d - i, kTopLevels) - 1) * kTopHubs + 32 * lane - 1;
+#pragma unroll 1
+                for (; m; m &= m - 1u) hist[o++] = (row0 + __ffs(m)) * (int)cwords;
+                ne += __shfl_sync(kFull, incl, 31);
+            }
+            __syncwarp();
+            if (ne > 0 && lane < ((4 - ne) & 3)) hist[ne + lane] = hist[0];
+            if (lane == 0) sh[SH_NE] = ne;
+        }
         __syncthreads();
+        const int n_rows = *(volatile int*)&sh[SH_NE];
         // entries of L(v) with a top hub (the checks' side B starts past them)
         const int lv_top = (int)lower_bound_u32(lvp, ll, pack(vb + (uint32_t)kTopHubs, 0));
-        const int i0 = first_level(tv, imax, lane);
         const int nc_set = min(*(volatile int*)&sh[SH_NC], limit);  // candidates from the set
-        // units of the maps (32 lanes x 16 bytes, 32 lanes x 32 bits, cleared
-        // as they are read) and of the set's candidates (32)
-        const int ub = maps ? (int)((Wb + 511) / 512) : 0, uw = maps ? (int)((W - Wb + 1023) / 1024) : 0;
-        const int units = ub + uw + (nc_set + 31) / 32;
+        // units: 2,048 hubs of the maps (64 per lane, cleared as they are read),
+        // pruned by the receiver's rows of the top-hub columns, or 32 of the
+        // set's candidates, pruned by their own masks.  The warps take them from
+        // a shared counter and check full warps of survivors
+        const int um = maps ? (int)((W + 2047) / 2048) : 0;
+        const int units = um + (nc_set + 31) / 32;
         bool more = true, last = false;
-        int nf = 0, ns = 0;        // staged candidates, survivors
-        uint32_t w = 0, hb = 0;    // this lane's candidates of the current unit: hub hb + b for every bit b of w
+        int ns = 0;                           // survivors
+        uint32_t c0 = 0, c1 = 0, hb = 0;      // this lane's of the current unit: hub hb + b for every bit b of c1 c0
 #pragma unroll 1
         while (!last) {
 #pragma unroll 1
-            while (nf < 64 && more) {
-                const unsigned m = __ballot_sync(kFull, w != 0u);
+            while (ns < 32 && more) {
+                const bool has = (c0 | c1) != 0u;
+                const unsigned m = __ballot_sync(kFull, has);
                 if (m) {
-                    if (w) {
-                        stage[nf + __popc(m & lt)] = hb + (uint32_t)(__ffs(w) - 1);
-                        w &= w - 1u;
+                    if (has) {
+                        const uint32_t b = c0 ? (uint32_t)__ffs(c0) - 1u : (uint32_t)__ffs(c1) + 31u;
+                        if (c0) c0 &= c0 - 1u;
+                        else c1 &= c1 - 1u;
+                        surv[ns + __popc(m & lt)] = hb + b;
                     }
-                    nf += __popc(m);
+                    ns += __popc(m);
                     continue;
                 }
                 int u = 0;
@@ -1177,47 +1205,62 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
                 u = __shfl_sync(kFull, u, 0);
                 if (u >= units) {
                     more = false;
-                } else if (u < ub) {
-                    const int x = 32 * u + lane;
-                    w = byte_bits4(b4[x]);
-                    if (w) b4[x] = make_uint4(0u, 0u, 0u, 0u);
-                    hb = vb + 16u * (uint32_t)x;
-                } else if (u < ub + uw) {
-                    const int x = 32 * (u - ub) + lane;
-                    w = bits[x];
-                    if (w) bits[x] = 0u;
-                    hb = vb + (uint32_t)kByteHubs + 32u * (uint32_t)x;
+                } else if (u < um) {
+                    const int x = 64 * u + 2 * lane;  // first of the lane's two words, as bits
+                    if (x < kByteHubs / 32) {
+                        uint4* q = b4 + 2 * x;
+                        const uint4 y0 = q[0], y1 = q[1], y2 = q[2], y3 = q[3];
+                        c0 = byte_bits4(y0) | (byte_bits4(y1) << 16);
+                        c1 = byte_bits4(y2) | (byte_bits4(y3) << 16);
+                        if (c0 | c1) q[0] = q[1] = q[2] = q[3] = make_uint4(0u, 0u, 0u, 0u);
+                    } else {
+                        uint2* q = reinterpret_cast<uint2*>(bits + (x - kByteHubs / 32));
+                        const uint2 y = *q;
+                        c0 = y.x;
+                        c1 = y.y;
+                        if (c0 | c1) *q = make_uint2(0u, 0u);
+                    }
+                    hb = vb + 32u * (uint32_t)x;
+                    if (!__any_sync(kFull, (c0 | c1) != 0u)) continue;
+                    const int found = __popc(c0) + __popc(c1);
+                    if (p.count_check)
+#pragma unroll 1
+                        for (int b = 0; b < 64; ++b)
+                            if (((b < 32 ? c0 : c1) >> (b & 31)) & 1u)
+                                count_reads(p.loff_h, lvp, ll, hb + (uint32_t)b, cnt + 8);
+                    // (x < the row's words: hubs of v's graph within the maps,
+                    // rounded up to 128; rows are 16-byte aligned)
+                    const uint32_t* cx = cols + min((uint32_t)x, cwords - 2u);
+#pragma unroll 1
+                    for (int k = 0; k < n_rows; k += 4) {
+                        const int4 o = *reinterpret_cast<const int4*>(hist + k);
+                        const uint2 t0 = *reinterpret_cast<const uint2*>(cx + o.x);
+                        const uint2 t1 = *reinterpret_cast<const uint2*>(cx + o.y);
+                        const uint2 t2 = *reinterpret_cast<const uint2*>(cx + o.z);
+                        const uint2 t3 = *reinterpret_cast<const uint2*>(cx + o.w);
+                        c0 &= ~(t0.x | t1.x | t2.x | t3.x);
+                        c1 &= ~(t0.y | t1.y | t2.y | t3.y);
+                        if (!__any_sync(kFull, (c0 | c1) != 0u)) break;
+                    }
+                    cnt[2] += found;
+                    cnt[7] += found - __popc(c0) - __popc(c1);
                 } else {
-                    const int x = 32 * (u - ub - uw) + lane;
-                    w = x < nc_set ? 1u : 0u;
-                    hb = x < nc_set ? C[x] : 0u;
+                    const int x = 32 * (u - um) + lane;
+                    bool valid = x < nc_set;
+                    hb = valid ? C[x] : 0u;
                     // without the map, set candidates may be hubs of v already
-                    if (!useM && w && map_has(Mp, log_mp, hb)) w = 0u;
+                    if (!useM && valid && map_has(Mp, log_mp, hb)) valid = false;
+                    if (p.count_check && valid) count_reads(p.loff_h, lvp, ll, hb, cnt + 8);
+                    unsigned m0, m1;
+                    prefilter_first(p, tv, (int)d, imax, i0, hb, valid, 0u, false, &m0, &m1);
+                    c0 = (m0 >> lane) & 1u;
+                    c1 = 0;
+                    cnt[2] += valid ? 1 : 0;
+                    cnt[7] += valid && !c0 ? 1 : 0;
                 }
             }
-            if (nf > 0) {
-                __syncwarp();
-                // first prefilter step: the last 64 staged candidates (fewer at the end)
-                const int k = min(nf, 64), s0 = nf - k;
-                const bool v0 = lane < k, v1 = lane + 32 < k;
-                const uint32_t h0 = v0 ? stage[s0 + lane] : 0u, h1 = v1 ? stage[s0 + 32 + lane] : 0u;
-                nf = s0;
-                if (p.count_check) {
-                    if (v0) count_reads(p.loff_h, lvp, ll, h0, cnt + 8);
-                    if (v1) count_reads(p.loff_h, lvp, ll, h1, cnt + 8);
-                }
-                unsigned m0, m1;
-                prefilter_first(p, tv, (int)d, imax, i0, h0, v0, h1, v1, &m0, &m1);
-                if ((m0 >> lane) & 1u) surv[ns + __popc(m0 & lt)] = h0;
-                ns += __popc(m0);
-                if ((m1 >> lane) & 1u) surv[ns + __popc(m1 & lt)] = h1;
-                ns += __popc(m1);
-                if (lane == 0) {
-                    cnt[2] += k;
-                    cnt[7] += k - __popc(m0) - __popc(m1);
-                }
-                __syncwarp();
-            } else {
+            __syncwarp();
+            if (ns < 32) {
                 // no unit is left: the warps' last survivors (fewer than 32
                 // each) are pooled behind C's candidates and spread over the
                 // warps, so that one warp's scans are not what the others wait for
@@ -1365,7 +1408,9 @@ __global__ void __launch_bounds__(256, 3) k_gp_block(GpParams p) {
         __syncthreads();
     }
     cnt[1] = warp_sum(cnt[1]);
+    cnt[2] = warp_sum(cnt[2]);
     cnt[4] = warp_sum(cnt[4]);
+    cnt[7] = warp_sum(cnt[7]);
     if (p.count_check) {
         cnt[8] = warp_sum(cnt[8]);
         cnt[9] = warp_sum(cnt[9]);
@@ -1374,7 +1419,7 @@ __global__ void __launch_bounds__(256, 3) k_gp_block(GpParams p) {
             atomicAdd(&p.ctr->chk_lh, cnt[9]);
         }
     }
-    if ((threadIdx.x & 31) == 0) {  // lane 0 of each warp holds its warp's unique and prefiltered counts
+    if ((threadIdx.x & 31) == 0) {
         atomicAdd(&p.ctr->msgs, cnt[1]);
         atomicAdd(&p.ctr->probed, cnt[4]);
         atomicAdd(&p.ctr->prefiltered, cnt[7]);

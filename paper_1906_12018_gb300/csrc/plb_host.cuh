@@ -199,6 +199,24 @@ inline cudaError_t launch_tiers(GpParams w, GpParams b, const SplitLists& split,
     return cudaGetLastError();
 }
 
+// Block tier, per block: accepted hubs past the maps (those within them stay
+// marked there).
+inline int64_t accepted_words(int64_t max_part_n) {
+    return std::max<int64_t>(max_part_n - (kByteHubs + kBitHubs), 1);
+}
+
+// The top-hub columns of a graph of n vertices, empty (quads: the words per row,
+// in units of 4, of all graphs of a union; by_base: their places).
+inline TopColumns top_columns(DevPool& pool, int64_t quads, const int2* by_base, cudaStream_t s) {
+    TopColumns c{};
+    c.by_base = by_base;
+    c.one = make_int2(0, (int)quads);
+    c.bits = pool.alloc<uint32_t>(quads * 4 * kTopRows);
+    if (!pool.failed && cudaMemsetAsync(c.bits, 0, sizeof(uint32_t) * quads * 4 * kTopRows, s) != cudaSuccess)
+        pool.failed = true;
+    return c;
+}
+
 // Records the failing CUDA call for plb_last_error (this thread).
 void set_last_error(cudaError_t e, int line);
 

@@ -85,6 +85,16 @@ struct SplitLists {
     int max, max_parts, words;
 };
 
+// The top-hub masks by hub instead of by vertex: per graph, level t and top hub
+// w a row of bits over the graph's first vertices (those the block tier's maps
+// hold), bit x: w in L(x) at distance <= t.  A receiver prunes the candidates
+// in its maps 64 per lane and row: OR of the rows of its own top hubs.
+struct TopColumns {
+    uint32_t* bits;       // rows (t, w) of 4 one.y words each, from 4 x kTopRows x one.x words on
+    const int2* by_base;  // disjoint union: {x, y} of each graph, at the index of its first rank; else null
+    int2 one;             // one graph: {0, y}
+};
+
 struct GpParams {
     const int64_t* roff;
     const int32_t* rcol;
@@ -129,6 +139,7 @@ struct GpParams {
                                // count ctr->nU), or null (every new row is sorted after the round)
     int sender_bits;           // rcol holds frontier descriptor indices whose low sender_bits bits are
                                // the sending vertex (weighted rounds), or 0: the vertex itself
+    TopColumns cols_h;         // the candidates' side's top-hub masks by hub
     const int32_t* vbase;      // per vertex: first rank of its graph in a disjoint union, or null (one graph:
                                // 0).  The top hubs and the byte map are those of the vertex's own graph
     int count_check;           // 1: count the label entries each check would read by the paper's cost
@@ -163,6 +174,7 @@ static_assert(kTopHubs % 128 == 0, "top-hub masks are read as uint4");
 constexpr int kTopWords = kTopHubs / 32;             // words per mask
 constexpr int kTopLevels = 7;                        // distance levels 1..7
 constexpr int kTopRow = kTopLevels * kTopWords;      // words per vertex
+constexpr int kTopRows = kTopLevels * kTopHubs;      // rows of TopColumns
 // Layout: the masks of level 1 of all vertices, then level 2's, ...: a round
 // reads one or two levels of candidates that are mostly of high rank, so that
 // what it reads lies together (the 32-byte masks of 2^17 hubs in 4 MB; with
@@ -186,11 +198,10 @@ __host__ __device__ __forceinline__ int64_t row_pad(int64_t c) { return (c + kRo
 constexpr int kByteHubs = 16384;
 constexpr int kBitHubs = 131072;
 constexpr int kMapWords = kByteHubs / 4 + kBitHubs / 32;
-static_assert(kByteHubs % 512 == 0 && kBitHubs % 4096 == 0, "whole scan units");
-// Block tier, per warp: staged candidates (fewer than 64, plus 32 of one
-// extraction) and survivors of the first prefilter step (fewer than 32, plus 64)
-constexpr int kCandStage = 96, kSurvStage = 96;
-constexpr int kWarpStage = kCandStage + kSurvStage;
+static_assert(kByteHubs % 512 == 0 && kBitHubs % 4096 == 0 && kByteHubs % 2048 == 0, "whole scan units");
+// Block tier, per warp: survivors of the first prefilter step (fewer than 32,
+// plus 32 of one extraction).
+constexpr int kWarpStage = 64;
 
 // Rows of L with at least this many entries get a hub-keyed probe table.
 constexpr int kIndexMinLen = 16;
@@ -207,6 +218,17 @@ constexpr int kIndexSmemSlotsMax = 2048;
 __host__ __device__ __forceinline__ uint64_t hrec_row(uint64_t start, uint64_t len) { return (start << 24) | len; }
 constexpr int kHrecTopShift = 16;  // within the record's last word
 constexpr uint64_t kHrecDescMask = (uint64_t(1) << 48) - 1;
+// A graph's rows and words per row (in units of 4) of the top-hub columns.
+__device__ __forceinline__ uint32_t* columns_of(const TopColumns& c, uint32_t vb, uint32_t* words) {
+    const int2 t = c.by_base ? c.by_base[vb] : c.one;
+    *words = 4u * (uint32_t)t.y;
+    return c.bits + (int64_t)t.x * (4 * kTopRows);
+}
+// Words per row, in units of 4, for a graph of n vertices.
+__host__ __device__ __forceinline__ int column_quads(int64_t n) {
+    const int64_t m = n < kByteHubs + kBitHubs ? n : kByteHubs + kBitHubs;
+    return (int)((m + 127) / 128);
+}
 __global__ void k_pack_hrec(const int64_t* loff, const uint32_t* lent, const uint64_t* hdesc, const int32_t* vbase,
                             uint4* hrec, int64_t n, const RoundCounters* ctr);
 

@@ -816,6 +816,50 @@ __global__ void k_merge_new(const int64_t* loff, const uint32_t* lent, const int
     }
 }
 
+// After the merge of round d: level d of the masks, which is final now, by hub
+// (TopColumns; with more != 0, as in rank batches, whose rounds start again at
+// distance 1, the levels above it too).  A block takes 32 vertices; those that
+// start a run of 128 of their graph are transposed, one warp per mask word.
+__global__ void __launch_bounds__(256) k_top_columns(const uint32_t* top, int64_t n, const int32_t* vbase,
+                                                     TopColumns cols, int more, const RoundCounters* ctr) {
+    static_assert(kTopWords == 8, "one warp per mask word");
+    if (ctr->done) return;
+    const int d = (int)ctr->d;
+    if (d > kTopLevels) return;
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    const int64_t chunks = (n + 31) / 32;
+    for (int64_t g = blockIdx.x; g < chunks; g += gridDim.x) {
+        const int64_t v = 32 * g + lane;
+        const uint32_t vb = v < n ? base_of(vbase, v) : 0u;
+        const uint32_t rel = (uint32_t)v - vb;
+        unsigned starts = __ballot_sync(kFull, v < n && (rel & 127u) == 0u && rel < (uint32_t)(kByteHubs + kBitHubs));
+        while (starts) {
+            const int k = __ffs(starts) - 1;
+            starts &= starts - 1u;
+            const uint32_t b = __shfl_sync(kFull, vb, k), r0 = __shfl_sync(kFull, rel, k);
+            uint32_t words;
+            uint32_t* rows = columns_of(cols, b, &words);
+            for (int t = d; t <= (more ? kTopLevels : d); ++t) {
+                uint32_t out[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int64_t x = (int64_t)b + r0 + 32 * q + lane;
+                    uint32_t m = 0;
+                    if (x < n && base_of(vbase, x) == b) m = top[((t - 1) * n + x) * kTopWords + w];
+                    out[q] = 0;
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) {
+                        const uint32_t bits = __ballot_sync(kFull, (m >> i) & 1u);
+                        if (lane == i) out[q] = bits;
+                    }
+                }
+                uint32_t* row = rows + (int64_t)((t - 1) * kTopHubs + 32 * w + lane) * words + (r0 >> 5);
+                *reinterpret_cast<uint4*>(row) = make_uint4(out[0], out[1], out[2], out[3]);
+            }
+        }
+    }
+}
+
 // Masks start empty (distance-0 self labels are not part of any level).
 __global__ void k_top_init(uint32_t* top, int64_t n) {
     const int64_t words = n * kTopRow;

@@ -284,6 +284,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     int64_t scap = std::max<int64_t>(kRowAlign * n + nnz + 1024, 4096);
     uint32_t* store = pool.alloc<uint32_t>(scap);
     uint32_t* top = pool.alloc<uint32_t>(n * kTopRow);
+    const TopColumns cols = top_columns(pool, column_quads(n), nullptr, s);
     int64_t* hoff = pool.alloc<int64_t>(n + 1);
     uint64_t* hdesc = pool.alloc<uint64_t>(n);
     int64_t hcap = std::max<int64_t>(4 * n, 1024);
@@ -371,7 +372,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     const int sort_blocks = 8;
     const int64_t sort_words = pow2_at_least(std::max<int64_t>(n, 1));
     uint32_t* sortscr = pool.alloc<uint32_t>(sort_words * sort_blocks);
-    uint32_t* gacc = pool.alloc<uint32_t>((int64_t)grid_b * std::max<int64_t>(n, 1));
+    uint32_t* gacc = pool.alloc<uint32_t>((int64_t)grid_b * accepted_words(n));
     PLB_ALLOC_OK();
 
     const SplitLists split = split_lists(pool, n, n, nnz, s);
@@ -416,8 +417,9 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
         p.hdesc_h = hdesc;
         p.htab_h = htab;
         p.top_h = top;
+        p.cols_h = cols;
         p.gscratch = gacc;
-        p.gscratch_words = std::max<int64_t>(n, 1);
+        p.gscratch_words = accepted_words(n);
         p.rbound = rbound;
         p.ostart = nullptr;
         p.sender_bits = lgn;
@@ -533,7 +535,8 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
                                                                n, ctr);
             k_merge_new<<<grid_for((int64_t)n * 32, kFlatThreads, flat_grid_cap), kFlatThreads, 0, s>>>(
                 loff[cur], lent[cur], loff[x], lent[x], fse_new, store, A, nullptr, ctr, top, n);
-            launches += 6 + scan_n;
+            k_top_columns<<<grid_for((n + 31) / 32, 1, flat_grid_cap), 256, 0, s>>>(top, n, nullptr, cols, 0, ctr);
+            launches += 7 + scan_n;
             PLB_CK(cudaGetLastError());
             const int64_t Told = T;
             T = Tn;
