@@ -354,12 +354,10 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
                                                                             sortscr, sort_words, ctr);
         cudaError_t e = exclusive_scan_i64(tmp64, loff[x], n, scan_scr, s, skip);
         if (e != cudaSuccess) return e;
-        k_merge_old<<<flat_grid_cap, kFlatThreads, 0, s>>>(loff[c], lent[c], loff[x], lent[x], fse[x], fhub[x], n,
-                                                           ctr);
-        k_merge_new<<<grid_for((int64_t)n * 32, kFlatThreads, flat_grid_cap), kFlatThreads, 0, s>>>(
-            loff[c], lent[c], loff[x], lent[x], fse[x], fhub[x], A, vbase, ctr, top, n);
+        k_merge_rows<<<grid_for((n + 7) / 8, 1, flat_grid_cap), 256, 0, s>>>(
+            loff[c], lent[c], loff[x], lent[x], fse[x], fhub[x], n, vbase, ctr, top);
         k_top_columns<<<grid_for((n + 31) / 32, 1, flat_grid_cap), 256, 0, s>>>(top, n, vbase, cols, batch < n, ctr);
-        st.launches += 7 + scan_n;
+        st.launches += 6 + scan_n;
         return cudaGetLastError();
     };
 
@@ -778,7 +776,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
     L->bytes = (int64_t)(sizeof(int64_t) * (n + 1) + 9 * (size_t)T + 4 * (size_t)n);
     k_final_len<<<gflat, kFlatThreads, 0, s>>>(loff[cur], inv, n, tmp64);
     if (exclusive_scan_i64(tmp64, L->off, n, scan_scr, s) != cudaSuccess) return fail(PLB_ERR_CUDA);
-    k_finalize<<<grid_for((T + 2047) / 2048, 1, flat_grid_cap), kFlatThreads, 0, s>>>(
+    k_finalize<<<grid_for((n + 7) / 8, 1, flat_grid_cap), kFlatThreads, 0, s>>>(
         loff[cur], lent[cur], inv, L->off, L->packed, L->hub, L->dist, n, ctr);
     if (cudaMemcpyAsync(L->order, order, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
         return fail(PLB_ERR_CUDA);

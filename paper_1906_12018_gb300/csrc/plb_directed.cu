@@ -340,12 +340,10 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
                                                                             S.ctr);
         cudaError_t e = exclusive_scan_i64(tmp64, S.loff[x], n, scan_scr, s);
         if (e != cudaSuccess) return e;
-        k_merge_old<<<flat_grid_cap, kFlatThreads, 0, s>>>(S.loff[c], S.lent[c], S.loff[x], S.lent[x], S.fse[x],
-                                                           S.fhub[x], n, S.ctr);
-        k_merge_new<<<grid_for((int64_t)n * 32, kFlatThreads, flat_grid_cap), kFlatThreads, 0, s>>>(
-            S.loff[c], S.lent[c], S.loff[x], S.lent[x], S.fse[x], S.fhub[x], S.A, nullptr, S.ctr, S.top, n);
+        k_merge_rows<<<grid_for((n + 7) / 8, 1, flat_grid_cap), 256, 0, s>>>(
+            S.loff[c], S.lent[c], S.loff[x], S.lent[x], S.fse[x], S.fhub[x], n, nullptr, S.ctr, S.top);
         k_top_columns<<<grid_for((n + 31) / 32, 1, flat_grid_cap), 256, 0, s>>>(S.top, n, nullptr, S.cols, 0, S.ctr);
-        launches += 7 + scan_n;
+        launches += 6 + scan_n;
         return cudaGetLastError();
     };
     auto read_ctr = [&](Side& S) -> cudaError_t {
@@ -536,7 +534,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
         L->bytes = (int64_t)(sizeof(int64_t) * (n + 1) + 9 * (size_t)T + 4 * (size_t)n);
         k_final_len<<<gflat, kFlatThreads, 0, s>>>(S.loff[S.cur], inv, n, tmp64);
         if (exclusive_scan_i64(tmp64, L->off, n, scan_scr, s) != cudaSuccess) return fail(PLB_ERR_CUDA);
-        k_finalize<<<grid_for((T + 2047) / 2048, 1, flat_grid_cap), kFlatThreads, 0, s>>>(
+        k_finalize<<<grid_for((n + 7) / 8, 1, flat_grid_cap), kFlatThreads, 0, s>>>(
             S.loff[S.cur], S.lent[S.cur], inv, L->off, L->packed, L->hub, L->dist, n, S.ctr);
         if (cudaMemcpyAsync(L->order, order, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
             read_ctr(S) != cudaSuccess)

@@ -15,7 +15,7 @@
 //   k_sort_rows_*  rows of the new frontier that were written unsorted (round
 //                  1; the block tier's) sorted by hub rank (the warp tier
 //                  writes its rows sorted);
-//   k_merge_*      L(v) <- L(v) U dL_d(v), keeping rows sorted by hub rank;
+//   k_merge_rows   L(v) <- L(v) U dL_d(v), keeping rows sorted by hub rank;
 //                  then the probe index of L is rebuilt (k_index_*).
 #pragma once
 

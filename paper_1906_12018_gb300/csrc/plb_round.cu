@@ -409,14 +409,23 @@ __global__ void k_index_size(const int64_t* loff, int64_t n, int64_t* hsz, const
 // written out whole, empty slots included), else cleared and filled in place.
 __device__ __forceinline__ void build_table(const uint32_t* lent, int64_t lb, int64_t ll, uint32_t* htab,
                                             int64_t hb, int lg, uint32_t* buf, int slots, int lane) {
-    const int P = 1 << lg;
-    uint32_t* tab = P <= slots ? buf : htab + hb;
-    for (int sl = lane; sl < P; sl += 32) tab[sl] = kEmpty;
+    const int P4 = 1 << (lg - 2);  // in 16-byte words (tables have at least 32 slots and start at multiples of 32)
+    uint32_t* tab = 4 * P4 <= slots ? buf : htab + hb;
+    for (int sl = lane; sl < P4; sl += 32)
+        reinterpret_cast<uint4*>(tab)[sl] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
     __syncwarp();
-    for (int64_t j = lane; j < ll; j += 32) map_insert(tab, lg, lent[lb + j]);
+    for (int64_t j = lane; j < ll; j += 128) {  // four entries in flight per lane
+        uint32_t x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = j + 32 * u < ll ? lent[lb + j + 32 * u] : kEmpty;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (x[u] != kEmpty) map_insert(tab, lg, x[u]);
+    }
     __syncwarp();
-    if (P <= slots) {
-        for (int sl = lane; sl < P; sl += 32) htab[hb + sl] = buf[sl];
+    if (4 * P4 <= slots) {
+        uint4* out = reinterpret_cast<uint4*>(htab + hb);
+        for (int sl = lane; sl < P4; sl += 32) out[sl] = reinterpret_cast<const uint4*>(buf)[sl];
         __syncwarp();
     }
 }
@@ -717,102 +726,135 @@ __global__ void __launch_bounds__(kRadixThreads) k_sort_rows_radix(const uint64_
     }
 }
 
-// Old entries move to their place in the merged row: flat over old entries.
-// A tile of entries that spans at most kMergeRows rows stages those rows'
-// old and new offsets and new-frontier descriptors in shared memory (each
-// entry's row is a binary search there); a tile over more rows reads them
-// from global memory.
-constexpr int kMergeRows = 512;
+// Copies len words from src to dst with nthr threads (this one is t): eight
+// loads in flight per thread.
+__device__ __forceinline__ void copy_words(const uint32_t* src, uint32_t* dst, int64_t len, int t, int nthr) {
+    constexpr int kUn = 8;
+    int64_t i = t;
+    for (; i + (int64_t)(kUn - 1) * nthr < len; i += (int64_t)kUn * nthr) {
+        uint32_t x[kUn];
+#pragma unroll
+        for (int u = 0; u < kUn; ++u) x[u] = src[i + (int64_t)u * nthr];
+#pragma unroll
+        for (int u = 0; u < kUn; ++u) dst[i + (int64_t)u * nthr] = x[u];
+    }
+    for (; i < len; i += nthr) dst[i] = src[i];
+}
 
-__global__ void k_merge_old(const int64_t* loff, const uint32_t* lent, const int64_t* loff_new, uint32_t* lent_new,
-                            const uint64_t* fse_new, const uint32_t* fhub_new, int64_t n, const RoundCounters* ctr) {
-    __shared__ __align__(16) int srow[kTileItems];
-    __shared__ TileScratch sh;
-    __shared__ int64_t s_off[kMergeRows + 1];
-    __shared__ int64_t s_noff[kMergeRows];
-    __shared__ uint64_t s_f[kMergeRows];
-    if (ctr->done) return;
-    const int64_t total = loff[n];
-    const int64_t ntiles = (total + kTileItems - 1) / kTileItems;
-    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int64_t p0 = t * kTileItems, p1 = min(total, p0 + kTileItems);
-        int64_t r0, r1;
-        tile_row_map(loff, n, p0, p1, srow, &sh, &r0, &r1);
-        const int64_t rows = r1 - r0 + 1;
-        const int nr = rows <= kMergeRows ? (int)rows : kMergeRows + 1;
-        const bool staged = nr <= kMergeRows;
-        if (staged) {
-            for (int i = threadIdx.x; i <= nr; i += blockDim.x) s_off[i] = loff[r0 + i];
-            for (int i = threadIdx.x; i < nr; i += blockDim.x) {
-                s_noff[i] = loff_new[r0 + i];
-                s_f[i] = fse_new[r0 + i];
-            }
-        }
-        __syncthreads();
-        for (int64_t q = p0 + threadIdx.x; q < p1; q += blockDim.x) {
-            int64_t ob, nb;
-            uint64_t f;
-            const int lo = srow[q - p0];
-            if (staged) {
-                ob = s_off[lo];
-                nb = s_noff[lo];
-                f = s_f[lo];
-            } else {
-                const int64_t v = r0 + lo;
-                ob = loff[v];
-                nb = loff_new[v];
-                f = fse_new[v];
-            }
-            const uint32_t e = lent[q];
-            int64_t pos = nb + (q - ob);
-            const uint32_t c = fcount(f);
-            if (c) pos += lower_bound_u32(fhub_new + fstart(f), c, hub_of(e));
-            lent_new[pos] = e;
-        }
+// One row's merge by nthr threads (this one is t): the old entries (sorted) and
+// the c new hubs (sorted, distance d) to their places.
+__device__ __forceinline__ void merge_row(const uint32_t* old, int64_t ol, const uint32_t* fr, int64_t c, uint32_t* dst,
+                                          uint32_t d, int t, int nthr) {
+    for (int64_t i = t; i < ol; i += nthr) {
+        const uint32_t e = old[i];
+        dst[i + lower_bound_u32(fr, c, hub_of(e))] = e;
+    }
+    for (int64_t j = t; j < c; j += nthr) {
+        const uint32_t e = pack(fr[j], d);
+        dst[j + lower_bound_u32(old, ol, pack(fr[j], 0))] = e;
     }
 }
 
-// New entries (dist d) of each active vertex: warp per vertex.
-__global__ void k_merge_new(const int64_t* loff, const uint32_t* lent, const int64_t* loff_new, uint32_t* lent_new,
-                            const uint64_t* fse_new, const uint32_t* fhub_new, const int32_t* A,
-                            const int32_t* vbase, const RoundCounters* ctr, uint32_t* top, int64_t n) {
+// L(v) <- L(v) U dL_d(v) into the other label buffer, rows sorted by hub, and the
+// new top hubs into the masks.  A warp takes 32 rows: runs of rows without new
+// entries are one copy each, the others are merged row by row; what is longer
+// than kLongRow is left to the whole block.  Bound by memory; before, a pass
+// flat over the old entries (the row of every entry looked up, 2.1 TB/s when
+// nothing was new) and one over the new ones with an atomic per top hub and
+// distance level (builds with both, k_finalize by rows and wider index builds:
+// Chung-Lu 2^20 26.2 -> 24.7 ms, weighted 61.9 -> 58.2 ms).
+constexpr int64_t kLongRow = 8192;
+constexpr int kMergeWarps = 8;
+
+// Rows per warp: 32, fewer when the grid has more warps than groups of 32 rows (a
+// small graph's rows would otherwise wait for one another on a few warps).
+__device__ __forceinline__ int rows_per_warp(int64_t n) {
+    const int64_t warps = (int64_t)gridDim.x * kMergeWarps;
+    return (int)min((int64_t)32, (n + warps - 1) / warps);
+}
+
+__global__ void __launch_bounds__(kMergeWarps * 32) k_merge_rows(const int64_t* loff, const uint32_t* lent,
+                                                                 const int64_t* loff_new, uint32_t* lent_new,
+                                                                 const uint64_t* fse_new, const uint32_t* fhub_new,
+                                                                 int64_t n, const int32_t* vbase,
+                                                                 const RoundCounters* ctr, uint32_t* top) {
+    __shared__ int64_t s_row[kMergeWarps * 32];  // long rows and runs: first row, rows << 40
+    __shared__ int s_n;
     if (ctr->done) return;
     const uint32_t d = ctr->d;
-    const int nA = ctr->nA;
-    const int lane = lane_id();
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < nA; i += nw) {
-        const int32_t v = A[i];
-        const uint64_t f = fse_new[v];
-        const uint32_t c = fcount(f);
-        const uint32_t* fr = fhub_new + fstart(f);
-        const int64_t ob = loff[v], ol = loff[v + 1] - ob;
-        // an old row of at most 32 entries sits in the lanes' registers: the
-        // old hubs below h are counted with shuffles instead of a binary
-        // search in global memory (c and ol are the same in every lane)
-        const bool reg = ol <= 32;
-        const uint32_t vb = base_of(vbase, v);
-        const uint32_t oe = reg && lane < ol ? lent[ob + lane] : 0xFFFFFFFFu;
-        for (uint32_t j0 = 0; j0 < c; j0 += 32) {
-            const uint32_t j = j0 + lane;
-            const uint32_t h = j < c ? fr[j] : 0u;
-            int64_t below;
-            if (reg) {
-                int cnt = 0;
-                for (int k = 0; k < (int)ol; ++k) cnt += __shfl_sync(kFull, oe, k) < pack(h, 0) ? 1 : 0;
-                below = cnt;
-            } else {
-                below = j < c ? lower_bound_u32(lent + ob, ol, pack(h, 0)) : 0;
-            }
-            if (j >= c) continue;
-            const int64_t pos = loff_new[v] + j + below;
-            lent_new[pos] = pack(h, d);
-            const uint32_t hr = h - vb;
-            if (hr < (uint32_t)kTopHubs && d <= (uint32_t)kTopLevels) {
-                uint32_t* tv = top + (int64_t)v * kTopWords + (hr >> 5);
-                for (int t = (int)d; t <= kTopLevels; ++t) atomicOr(tv + (t - 1) * n * kTopWords, 1u << (hr & 31));
-            }
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    const int per = rows_per_warp(n);
+    const int64_t groups = (n + kMergeWarps * per - 1) / (kMergeWarps * per);
+    for (int64_t g = blockIdx.x; g < groups; g += gridDim.x) {
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();
+        const int64_t v0 = (g * kMergeWarps + w) * per, v = lane < per ? v0 + lane : n;
+        int64_t ob = 0, oe = 0, nb = 0;
+        uint64_t f = 0;
+        if (v < n) {
+            ob = loff[v];
+            oe = loff[v + 1];
+            nb = loff_new[v];
+            f = fse_new[v];
         }
+        const unsigned live = __ballot_sync(kFull, v < n);
+        const unsigned act = __ballot_sync(kFull, fcount(f) > 0);
+        for (int k = 0; k < 32 && (live >> k) != 0u;) {
+            const bool merge = (act >> k) & 1u;
+            int e = k + 1;  // one row, or a run of rows without new entries
+            if (!merge) {
+                const unsigned stop = (act | ~live) & ~((2u << k) - 1u);
+                e = stop ? __ffs(stop) - 1 : 32;
+            }
+            const int64_t b = __shfl_sync(kFull, ob, k), len = __shfl_sync(kFull, oe, e - 1) - b;
+            const int64_t to = __shfl_sync(kFull, nb, k);
+            const uint64_t fk = __shfl_sync(kFull, f, k);
+            const int64_t c = fcount(fk);
+            if (max(len, c) > kLongRow) {
+                if (lane == 0) s_row[atomicAdd(&s_n, 1)] = (v0 + k) | ((int64_t)(e - k) << 40);
+            } else if (!merge) {
+                copy_words(lent + b, lent_new + to, len, lane, 32);
+            } else {
+                merge_row(lent + b, len, fhub_new + fstart(fk), c, lent_new + to, d, lane, 32);
+            }
+            if (merge && d <= (uint32_t)kTopLevels) {
+                // the row's new top hubs (they come first): lane i < kTopWords
+                // gathers word i, then ORs it into the levels from d on (only
+                // this warp writes v's masks)
+                const uint32_t* fr = fhub_new + fstart(fk);
+                const uint32_t vb = base_of(vbase, v0 + k);
+                uint32_t word = 0;
+                for (int64_t j0 = 0; j0 < c; j0 += 32) {
+                    const uint32_t hr = j0 + lane < c ? fr[j0 + lane] - vb : 0xFFFFFFFFu;
+                    unsigned todo = __ballot_sync(kFull, hr < (uint32_t)kTopHubs);
+                    const bool more = todo == kFull;
+                    while (todo) {
+                        const uint32_t q = __shfl_sync(kFull, hr, __ffs(todo) - 1) >> 5;
+                        const bool mine = (hr >> 5) == q;
+                        const uint32_t x = __reduce_or_sync(kFull, mine ? 1u << (hr & 31) : 0u);
+                        if (lane == (int)q) word |= x;
+                        todo &= ~__ballot_sync(kFull, mine);
+                    }
+                    if (!more) break;
+                }
+                if (word) {
+                    uint32_t* tv = top + (v0 + k) * kTopWords + lane;
+                    for (int t = (int)d; t <= kTopLevels; ++t) tv[(int64_t)(t - 1) * n * kTopWords] |= word;
+                }
+            }
+            k = e;
+        }
+        __syncthreads();
+        const int nl = s_n;
+        for (int i = 0; i < nl; ++i) {
+            const int64_t row = s_row[i] & ((int64_t(1) << 40) - 1), rows = s_row[i] >> 40;
+            const int64_t b = loff[row], len = loff[row + rows] - b, to = loff_new[row];
+            const uint64_t fk = fse_new[row];
+            const int64_t c = fcount(fk);
+            if (c == 0) copy_words(lent + b, lent_new + to, len, threadIdx.x, blockDim.x);
+            else merge_row(lent + b, len, fhub_new + fstart(fk), c, lent_new + to, d, threadIdx.x, blockDim.x);
+        }
+        __syncthreads();
     }
 }
 
@@ -964,51 +1006,69 @@ __global__ void k_final_len(const int64_t* loff, const int32_t* inv, int64_t n, 
     }
 }
 
-// Rows by original id: packed copy + separate hub / dist arrays.
-__global__ void k_finalize(const int64_t* loff, const uint32_t* lent, const int32_t* inv, const int64_t* out_off,
-                           uint32_t* out_packed, uint32_t* out_hub, uint8_t* out_dist, int64_t n,
-                           RoundCounters* ctr) {
-    __shared__ __align__(16) int srow[kTileItems];
-    __shared__ TileScratch sh;
-    __shared__ int64_t s_off[kMergeRows + 1];  // out_off of the tile's rows (as in k_merge_old)
-    __shared__ int64_t s_src[kMergeRows];      // start of each row in rank space
-    const int64_t total = out_off[n];
-    const int64_t ntiles = (total + kTileItems - 1) / kTileItems;
+// Words [t, len) in steps of nthr of one row: packed copy, hub and distance.
+__device__ __forceinline__ uint32_t final_row(const uint32_t* src, uint32_t* packed, uint32_t* hub, uint8_t* dist,
+                                              int64_t len, int t, int nthr) {
+    constexpr int kUn = 4;
     uint32_t md = 0;
-    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int64_t p0 = t * kTileItems, p1 = min(total, p0 + kTileItems);
-        int64_t r0, r1;
-        tile_row_map(out_off, n, p0, p1, srow, &sh, &r0, &r1);
-        const int64_t rows = r1 - r0 + 1;
-        const int nr = rows <= kMergeRows ? (int)rows : kMergeRows + 1;
-        const bool staged = nr <= kMergeRows;
-        if (staged) {
-            for (int i = threadIdx.x; i <= nr; i += blockDim.x) s_off[i] = out_off[r0 + i];
-            for (int i = threadIdx.x; i < nr; i += blockDim.x) s_src[i] = loff[inv[r0 + i]];
-        }
-        __syncthreads();
-        for (int64_t q = p0 + threadIdx.x; q < p1; q += blockDim.x) {
-            int64_t src;
-            const int lo = srow[q - p0];
-            if (staged) {
-                src = s_src[lo] + (q - s_off[lo]);
-            } else {
-                const int64_t id = r0 + lo;
-                src = loff[inv[id]] + (q - out_off[id]);
-            }
-            const uint32_t e = lent[src];
-            out_packed[q] = e;
-            out_hub[q] = hub_of(e);
-            out_dist[q] = (uint8_t)dist_of(e);
-            md = max(md, dist_of(e));
+    for (int64_t i = t; i < len; i += (int64_t)kUn * nthr) {
+        uint32_t x[kUn];
+#pragma unroll
+        for (int u = 0; u < kUn; ++u) x[u] = i + (int64_t)u * nthr < len ? src[i + (int64_t)u * nthr] : 0u;
+#pragma unroll
+        for (int u = 0; u < kUn; ++u) {
+            const int64_t q = i + (int64_t)u * nthr;
+            if (q >= len) break;
+            packed[q] = x[u];
+            hub[q] = hub_of(x[u]);
+            dist[q] = (uint8_t)dist_of(x[u]);
+            md = max(md, dist_of(x[u]));
         }
     }
-    md = max(md, __shfl_xor_sync(kFull, md, 16));
-    md = max(md, __shfl_xor_sync(kFull, md, 8));
-    md = max(md, __shfl_xor_sync(kFull, md, 4));
-    md = max(md, __shfl_xor_sync(kFull, md, 2));
-    md = max(md, __shfl_xor_sync(kFull, md, 1));
-    if ((threadIdx.x & 31) == 0 && md) atomicMax(&ctr->max_dist, md);
+    return md;
+}
+
+// Rows by original id: packed copy + separate hub / dist arrays, one warp per
+// row (long rows: the whole block; see k_merge_rows).
+__global__ void __launch_bounds__(kMergeWarps * 32) k_finalize(const int64_t* loff, const uint32_t* lent,
+                                                               const int32_t* inv, const int64_t* out_off,
+                                                               uint32_t* out_packed, uint32_t* out_hub,
+                                                               uint8_t* out_dist, int64_t n, RoundCounters* ctr) {
+    __shared__ int64_t s_id[kMergeWarps * 32];
+    __shared__ int s_n;
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    const int per = rows_per_warp(n);
+    const int64_t groups = (n + kMergeWarps * per - 1) / (kMergeWarps * per);
+    uint32_t md = 0;
+    for (int64_t g = blockIdx.x; g < groups; g += gridDim.x) {
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();
+        const int64_t id0 = (g * kMergeWarps + w) * per, id = lane < per ? id0 + lane : n;
+        int64_t src = 0, dst = 0, len = 0;
+        if (id < n) {
+            src = loff[inv[id]];
+            dst = out_off[id];
+            len = out_off[id + 1] - dst;
+        }
+        const int rows = (int)max((int64_t)0, min((int64_t)per, n - id0));
+        for (int k = 0; k < rows; ++k) {
+            const int64_t s = __shfl_sync(kFull, src, k), t = __shfl_sync(kFull, dst, k), l = __shfl_sync(kFull, len, k);
+            if (l > kLongRow) {
+                if (lane == 0) s_id[atomicAdd(&s_n, 1)] = id0 + k;
+            } else {
+                md = max(md, final_row(lent + s, out_packed + t, out_hub + t, out_dist + t, l, lane, 32));
+            }
+        }
+        __syncthreads();
+        const int nl = s_n;
+        for (int i = 0; i < nl; ++i) {
+            const int64_t s = loff[inv[s_id[i]]], t = out_off[s_id[i]], l = out_off[s_id[i] + 1] - t;
+            md = max(md, final_row(lent + s, out_packed + t, out_hub + t, out_dist + t, l, threadIdx.x, blockDim.x));
+        }
+        __syncthreads();
+    }
+    md = __reduce_max_sync(kFull, md);
+    if (lane == 0 && md) atomicMax(&ctr->max_dist, md);
 }
 
 }  // namespace plb

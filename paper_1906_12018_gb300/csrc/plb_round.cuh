@@ -60,11 +60,9 @@ __global__ void k_sort_rows_radix(const uint64_t* fse_new, uint32_t* fhub_new, c
                                   const RoundCounters* ctr);
 __global__ void k_sort_rows_block(const uint64_t* fse_new, uint32_t* fhub_new, const int32_t* big, const int* nbig,
                                   uint32_t* scratch, int64_t scratch_words, const RoundCounters* ctr);
-__global__ void k_merge_old(const int64_t* loff, const uint32_t* lent, const int64_t* loff_new, uint32_t* lent_new,
-                            const uint64_t* fse_new, const uint32_t* fhub_new, int64_t n, const RoundCounters* ctr);
-__global__ void k_merge_new(const int64_t* loff, const uint32_t* lent, const int64_t* loff_new, uint32_t* lent_new,
-                            const uint64_t* fse_new, const uint32_t* fhub_new, const int32_t* A,
-                            const int32_t* vbase, const RoundCounters* ctr, uint32_t* top, int64_t n);
+__global__ void k_merge_rows(const int64_t* loff, const uint32_t* lent, const int64_t* loff_new, uint32_t* lent_new,
+                             const uint64_t* fse_new, const uint32_t* fhub_new, int64_t n, const int32_t* vbase,
+                             const RoundCounters* ctr, uint32_t* top);
 __global__ void k_top_columns(const uint32_t* top, int64_t n, const int32_t* vbase, TopColumns cols, int more,
                               const RoundCounters* ctr);
 __global__ void k_top_init(uint32_t* top, int64_t n);

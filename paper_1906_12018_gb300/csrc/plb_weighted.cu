@@ -531,12 +531,10 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
                                                                                 &ctr->nGiant, sortscr, sort_words,
                                                                                 ctr);
             PLB_CK(exclusive_scan_i64(tmp64, loff[x], n, scan_scr, s));
-            k_merge_old<<<flat_grid_cap, kFlatThreads, 0, s>>>(loff[cur], lent[cur], loff[x], lent[x], fse_new, store,
-                                                               n, ctr);
-            k_merge_new<<<grid_for((int64_t)n * 32, kFlatThreads, flat_grid_cap), kFlatThreads, 0, s>>>(
-                loff[cur], lent[cur], loff[x], lent[x], fse_new, store, A, nullptr, ctr, top, n);
+            k_merge_rows<<<grid_for((n + 7) / 8, 1, flat_grid_cap), 256, 0, s>>>(
+                loff[cur], lent[cur], loff[x], lent[x], fse_new, store, n, nullptr, ctr, top);
             k_top_columns<<<grid_for((n + 31) / 32, 1, flat_grid_cap), 256, 0, s>>>(top, n, nullptr, cols, 0, ctr);
-            launches += 7 + scan_n;
+            launches += 6 + scan_n;
             PLB_CK(cudaGetLastError());
             const int64_t Told = T;
             T = Tn;
@@ -587,7 +585,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     L->bytes = (int64_t)(sizeof(int64_t) * (n + 1) + 9 * (size_t)T + 4 * (size_t)n);
     k_final_len<<<gflat, kFlatThreads, 0, s>>>(loff[cur], inv, n, tmp64);
     if (exclusive_scan_i64(tmp64, L->off, n, scan_scr, s) != cudaSuccess) return fail(PLB_ERR_CUDA);
-    k_finalize<<<grid_for((T + 2047) / 2048, 1, flat_grid_cap), kFlatThreads, 0, s>>>(
+    k_finalize<<<grid_for((n + 7) / 8, 1, flat_grid_cap), kFlatThreads, 0, s>>>(
         loff[cur], lent[cur], inv, L->off, L->packed, L->hub, L->dist, n, ctr);
     if (cudaMemcpyAsync(L->order, order, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
         read_ctr() != cudaSuccess)
