@@ -1,12 +1,8 @@
 // Batched 2-hop distance queries (Sec. 2.1):
 //   Dis(s, t) = min over hubs h in L(s) and L(t) of d(s,h) + d(h,t).
-// One warp per pair.  The 32 highest-ranked hubs of both rows, compared in
-// registers, give an upper bound `best` that is usually the answer or next to
-// it.  A smaller sum has an entry of at most (best - 1) / 2 on one of its
-// sides: both rows are streamed once, entries that near are collected, and only
-// full warps of these are looked up in the other row by binary search (on
-// R-MAT 2^22, 750 entries per row, 27 of them at distance 1, about 60 of 750
-// searches remain).
+// One warp per pair: lanes stride over the shorter of the two hub-sorted rows
+// and binary-search each hub in the longer row; a warp min-reduction gives
+// the answer.
 #include <algorithm>
 
 #include "plb_internal.cuh"
@@ -27,117 +23,64 @@ struct SetTable {
     SetDesc s[kMaxSets];
 };
 
-// Smallest sum (at most 510, or kEmpty) of the entry x of one row (kEmpty: none)
-// with its hub's entry in the other row ent[0, len).
-__device__ __forceinline__ uint32_t look_up(uint32_t x, const uint32_t* ent, int len) {
-    if (x == kEmpty) return kEmpty;
-    const uint32_t key = pack(hub_of(x), 0);
-    int lo = 0, hi = len;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (ent[mid] < key) lo = mid + 1; else hi = mid;
-    }
-    if (lo >= len) return kEmpty;
-    const uint32_t y = ent[lo];
-    return hub_of(y) == hub_of(x) ? dist_of(x) + dist_of(y) : kEmpty;
-}
-
-// The entries of row a[0, al) whose distance is at most (*best - 1) / 2, looked up
-// in row b[0, bl), 32 at a time (buf: 64 words of the warp's shared memory).
-__device__ __forceinline__ void near_entries(const uint32_t* a, int al, const uint32_t* b, int bl, uint32_t* buf,
-                                             uint32_t* best) {
-    constexpr int kUn = 4;
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    int nf = 0;
-    for (int j0 = 0; j0 < al; j0 += 32 * kUn) {
-        uint32_t x[kUn];
-#pragma unroll
-        for (int u = 0; u < kUn; ++u) x[u] = j0 + 32 * u + lane < al ? a[j0 + 32 * u + lane] : kEmpty;
-#pragma unroll
-        for (int u = 0; u < kUn; ++u) {
-            // (best = kEmpty, no common hub yet: every entry; else best >= 1:
-            // a sum of 0 ends the pair before this)
-            const uint32_t reach = (*best - 1u) >> 1;
-            const bool take = x[u] != kEmpty && dist_of(x[u]) <= reach;
-            const unsigned m = __ballot_sync(kFull, take);
-            if (take) buf[nf + __popc(m & lt)] = x[u];
-            nf += __popc(m);
-            __syncwarp();
-            if (nf >= 32) {
-                nf -= 32;
-                *best = min(*best, __reduce_min_sync(kFull, look_up(buf[nf + lane], b, bl)));
-                __syncwarp();
-            }
-        }
-    }
-    if (nf > 0) *best = min(*best, __reduce_min_sync(kFull, look_up(lane < nf ? buf[lane] : kEmpty, b, bl)));
-    __syncwarp();
-}
-
 // Rows: s in the set (off_s, ent_s), t in (off_t, ent_t); the same set for
 // undirected labels, L_out and L_in for directed ones (d(s -> t)).
 __device__ __forceinline__ int32_t answer_pair2(const int64_t* off_s, const uint32_t* ent_s, const int64_t* off_t,
-                                                const uint32_t* ent_t, int64_t n, int32_t s, int32_t t, uint32_t* buf) {
+                                                const uint32_t* ent_t, int64_t n, int32_t s, int32_t t, int lane) {
     if (s < 0 || t < 0 || (int64_t)s >= n || (int64_t)t >= n) return PLB_BAD_PAIR;
-    const int lane = threadIdx.x & 31;
-    const int64_t ab = off_s[s], ae = off_s[s + 1], bb = off_t[t], be = off_t[t + 1];
-    const uint32_t* a = ent_s + ab;
-    const uint32_t* b = ent_t + bb;
-    int al = (int)(ae - ab), bl = (int)(be - bb);  // (a row has at most n < 2^24 entries)
+    const uint32_t* ent = ent_s;
+    const uint32_t* ent2 = ent_t;
+    int64_t ab = off_s[s], al = off_s[s + 1] - ab;
+    int64_t bb = off_t[t], bl = off_t[t + 1] - bb;
     if (al > bl) {
-        const uint32_t* e = a;
-        a = b;
-        b = e;
-        const int x = al;
+        const uint32_t* e = ent;
+        ent = ent2;
+        ent2 = e;
+        int64_t x = ab;
+        ab = bb;
+        bb = x;
+        x = al;
         al = bl;
         bl = x;
     }
-    // the first 32 hubs of both rows: lane i's hub of a among b's lanes
-    const uint32_t x = lane < al ? a[lane] : kEmpty, y = lane < bl ? b[lane] : kEmpty;
-    int k = 0;  // largest lane with y <= x's hub at any distance
+    uint32_t best = 0xFFFFFFFFu;
+    for (int64_t j = lane; j < al; j += 32) {
+        const uint32_t x = ent[ab + j];
+        const uint32_t key = pack(hub_of(x), 0);
+        const int64_t pos = lower_bound_u32(ent2 + bb, bl, key);
+        if (pos < bl) {
+            const uint32_t y = ent2[bb + pos];
+            if (hub_of(y) == hub_of(x)) best = min(best, dist_of(x) + dist_of(y));
+        }
+    }
 #pragma unroll
-    for (int step = 16; step >= 1; step >>= 1) {
-        const uint32_t z = __shfl_sync(kFull, y, k + step);
-        if (z <= (x | 0xFFu)) k += step;
-    }
-    const uint32_t z = __shfl_sync(kFull, y, k);
-    uint32_t best = x != kEmpty && z != kEmpty && hub_of(z) == hub_of(x) ? dist_of(x) + dist_of(z) : kEmpty;
-    best = __reduce_min_sync(kFull, best);
-    if (best > 1 && (best != kEmpty || al > 32 || bl > 32)) {  // (two rows of up to 32 entries without a common hub: done)
-        near_entries(a, al, b, bl, buf, &best);
-        if (best > 1 && best != kEmpty) near_entries(b, bl, a, al, buf, &best);
-    }
-    return best == kEmpty ? PLB_UNREACHABLE : (int32_t)best;
+    for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(kFull, best, o));
+    return best == 0xFFFFFFFFu ? PLB_UNREACHABLE : (int32_t)best;
 }
 
 __device__ __forceinline__ int32_t answer_pair(const int64_t* off, const uint32_t* ent, int64_t n, int32_t s,
-                                               int32_t t, uint32_t* buf) {
-    return answer_pair2(off, ent, off, ent, n, s, t, buf);
+                                               int32_t t, int lane) {
+    return answer_pair2(off, ent, off, ent, n, s, t, lane);
 }
 
 __global__ void __launch_bounds__(kQThreads) k_query2(const int64_t* off_s, const uint32_t* ent_s,
                                                       const int64_t* off_t, const uint32_t* ent_t, int64_t n,
                                                       const int32_t* pairs, int64_t q, int32_t* out) {
-    __shared__ uint32_t bufs[kQThreads / 32][64];
-    uint32_t* buf = bufs[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < q; i += nw) {
-        const int32_t r = answer_pair2(off_s, ent_s, off_t, ent_t, n, pairs[2 * i], pairs[2 * i + 1], buf);
+        const int32_t r = answer_pair2(off_s, ent_s, off_t, ent_t, n, pairs[2 * i], pairs[2 * i + 1], lane);
         if (lane == 0) out[i] = r;
     }
 }
 
 __global__ void __launch_bounds__(kQThreads) k_query(const int64_t* off, const uint32_t* ent, int64_t n,
                                                      const int32_t* pairs, int64_t q, int32_t* out) {
-    __shared__ uint32_t bufs[kQThreads / 32][64];
-    uint32_t* buf = bufs[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < q; i += nw) {
         const int32_t s = pairs[2 * i], t = pairs[2 * i + 1];
-        const int32_t r = answer_pair(off, ent, n, s, t, buf);
+        const int32_t r = answer_pair(off, ent, n, s, t, lane);
         if (lane == 0) out[i] = r;
     }
 }
@@ -145,8 +88,6 @@ __global__ void __launch_bounds__(kQThreads) k_query(const int64_t* off, const u
 __global__ void __launch_bounds__(kQThreads) k_query_multi(SetTable tab, int set_lo, int set_hi, int64_t m,
                                                            const int32_t* set_idx, const int32_t* pairs, int64_t q,
                                                            int32_t* out) {
-    __shared__ uint32_t bufs[kQThreads / 32][64];
-    uint32_t* buf = bufs[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < q; i += nw) {
@@ -157,7 +98,7 @@ __global__ void __launch_bounds__(kQThreads) k_query_multi(SetTable tab, int set
         }
         if (k < set_lo || k >= set_hi) continue;
         const SetDesc& d = tab.s[k - set_lo];
-        const int32_t r = answer_pair(d.off, d.packed, d.n, pairs[2 * i], pairs[2 * i + 1], buf);
+        const int32_t r = answer_pair(d.off, d.packed, d.n, pairs[2 * i], pairs[2 * i + 1], lane);
         if (lane == 0) out[i] = r;
     }
 }
