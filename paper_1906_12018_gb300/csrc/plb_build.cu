@@ -51,7 +51,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
     cudaEvent_t t_all0 = tm.on ? tm.mark() : nullptr;
 
     RoundCounters* ctr = pool.alloc<RoundCounters>(1);
-    int* err = pool.alloc<int>(4);
+    int* err = pool.alloc<int>(6);  // [4..5]: the balance of k_check_cols
     PLB_ALLOC_OK();
     RoundCounters* hctr = nullptr;
     PLB_CK(cudaMallocHost(&hctr, sizeof(RoundCounters)));
@@ -60,7 +60,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         ~HostFree() { cudaFreeHost(p); }
     } hf{hctr};
     PLB_CK(cudaMemsetAsync(ctr, 0, sizeof(RoundCounters), s));
-    PLB_CK(cudaMemsetAsync(err, 0, 4 * sizeof(int), s));
+    PLB_CK(cudaMemsetAsync(err, 0, 6 * sizeof(int), s));
 
     cudaEvent_t t0 = tm.on ? tm.mark() : nullptr;
     // ---------------------------------------------------------- validation
@@ -77,14 +77,16 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         PLB_CK(cudaMemsetAsync(seen, 0, sizeof(int) * std::max<int64_t>(n, 1), s));
         if (nnz > 0) {
             k_check_cols<<<grid_for((nnz + 2047) / 2048, 1, flat_grid_cap), kFlatThreads, 0, s>>>(row_ptr, col, n,
-                                                                                               nnz, 1, err);
+                                                                                               nnz, 1, err,
+                                                                                               reinterpret_cast<unsigned long long*>(err + 4));
+            k_check_balance<<<1, 1, 0, s>>>(reinterpret_cast<unsigned long long*>(err + 4), err);
             PLB_CK(cudaGetLastError());
         }
         k_check_order<<<grid_for(n, kFlatThreads, flat_grid_cap), kFlatThreads, 0, s>>>(order, n, seen, err);
         PLB_CK(cudaGetLastError());
         PLB_CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
         PLB_CK(cudaStreamSynchronize(s));
-        st.launches += 2;
+        st.launches += 3;
         pool.release(seen);
         if (herr) return PLB_ERR_INVALID;
     }

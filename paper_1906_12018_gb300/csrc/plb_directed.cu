@@ -81,7 +81,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
     int64_t launches = 0;
 
     Side side[2];  // 0: L_in, 1: L_out
-    int* err = pool.alloc<int>(4);
+    int* err = pool.alloc<int>(6);  // [4..5]: the balance of k_check_cols
     for (int k = 0; k < 2; ++k) side[k].ctr = pool.alloc<RoundCounters>(1);
     PLB_ALLOC_OK();
     RoundCounters* hbuf = nullptr;
@@ -94,7 +94,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
         side[k].hctr = hbuf + k;
         PLB_CK(cudaMemsetAsync(side[k].ctr, 0, sizeof(RoundCounters), s));
     }
-    PLB_CK(cudaMemsetAsync(err, 0, 4 * sizeof(int), s));
+    PLB_CK(cudaMemsetAsync(err, 0, 6 * sizeof(int), s));
 
     cudaEvent_t t0 = tm.on ? tm.mark() : nullptr;
     // ---------------------------------------------------------- validation
@@ -109,7 +109,8 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
         if (herr) return PLB_ERR_INVALID;
         if (nnz > 0)
             k_check_cols<<<grid_for((nnz + 2047) / 2048, 1, flat_grid_cap), kFlatThreads, 0, s>>>(row_ptr, col, n,
-                                                                                               nnz, 0, err);
+                                                                                               nnz, 0, err,
+                                                                                               reinterpret_cast<unsigned long long*>(err + 4));
         k_check_order<<<grid_for(n, kFlatThreads, flat_grid_cap), kFlatThreads, 0, s>>>(order, n, seen, err);
         PLB_CK(cudaGetLastError());
         PLB_CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));

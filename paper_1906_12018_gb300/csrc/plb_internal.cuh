@@ -238,6 +238,12 @@ __device__ __forceinline__ void tile_row_map(const int64_t* off, int64_t nrows, 
     *r1 = b;
 }
 
+// Which of an edge's two arcs the input checks look up (see k_check_cols).
+__device__ __forceinline__ bool looked_up(const int64_t* row_ptr, int64_t u, int64_t c) {
+    const int64_t du = row_ptr[u + 1] - row_ptr[u], dc = row_ptr[c + 1] - row_ptr[c];
+    return dc < du || (dc == du && c < u);
+}
+
 // Bitonic sort of a[0..P) (P a power of two) by a group of nthreads threads.
 // Each step runs over the P/2 compare-exchange pairs (i, i + j), i the pair
 // index t with a zero bit inserted at bit log2(j): no idle half of the

@@ -24,12 +24,18 @@ __global__ void k_check_rowptr(const int64_t* row_ptr, int64_t n, int64_t nnz, i
 }
 
 // Per arc (u -> c): 0 <= c < n, c != u, rows strictly ascending, and (when
-// symmetric) the reverse arc (c -> u) exists (binary search in row c).
+// symmetric) the reverse arc (c -> u) exists.  Of an edge's two arcs only the
+// one into the row that is not longer (ties: into the smaller id) is looked up,
+// by binary search there: `balance` counts these arcs up and the others down.
+// Each arc that was looked up has its reverse among the others, and different
+// arcs different ones, so with equal counts (balance 0) every arc has one.
+// (Looking up every arc took 13.5 ms on R-MAT 2^22, mostly in hubs' rows.)
 __global__ void k_check_cols(const int64_t* row_ptr, const int32_t* col, int64_t n, int64_t nnz, int symmetric,
-                             int* err) {
+                             int* err, unsigned long long* balance) {
     __shared__ __align__(16) int srow[kTileItems];
     __shared__ TileScratch sh;
     const int64_t ntiles = (nnz + kTileItems - 1) / kTileItems;
+    int64_t bal = 0;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
         int64_t r0, r1;
@@ -40,17 +46,31 @@ __global__ void k_check_cols(const int64_t* row_ptr, const int32_t* col, int64_t
             bool bad = c < 0 || (int64_t)c >= n || (int64_t)c == u;
             if (!bad && p > row_ptr[u] && col[p - 1] >= c) bad = true;
             if (!bad && symmetric) {
-                const int64_t b = row_ptr[c], e = row_ptr[c + 1];
-                int64_t lo = b, hi = e;
-                while (lo < hi) {
-                    const int64_t mid = (lo + hi) >> 1;
-                    if ((int64_t)col[mid] < u) lo = mid + 1; else hi = mid;
+                if (looked_up(row_ptr, u, c)) {
+                    const int64_t e = row_ptr[c + 1];
+                    int64_t lo = row_ptr[c], hi = e;
+                    while (lo < hi) {
+                        const int64_t mid = (lo + hi) >> 1;
+                        if ((int64_t)col[mid] < u) lo = mid + 1; else hi = mid;
+                    }
+                    if (lo >= e || (int64_t)col[lo] != u) bad = true;
+                    ++bal;
+                } else {
+                    --bal;
                 }
-                if (lo >= e || (int64_t)col[lo] != u) bad = true;
             }
             if (bad) atomicOr(err, 2);
         }
     }
+    if (symmetric) {
+        bal = warp_sum(bal);
+        if ((threadIdx.x & 31) == 0 && bal != 0) atomicAdd(balance, (unsigned long long)bal);
+    }
+}
+
+// After k_check_cols (and in order with it): unequal counts are an error.
+__global__ void k_check_balance(const unsigned long long* balance, int* err) {
+    if (*balance != 0ull) atomicOr(err, 2);
 }
 
 __global__ void k_check_order(const int32_t* order, int64_t n, int* seen, int* err) {
@@ -430,21 +450,32 @@ __device__ __forceinline__ void build_table(const uint32_t* lent, int64_t lb, in
     }
 }
 
-// Full rebuild, one warp per `per` rows (at most 32: fewer when the warps of the
-// grid outnumber the groups of 32, so that a small graph's rows are not built
-// one after the other on a few warps): row x's table at hoff[x] (sizes from
-// k_index_size and a scan); hdesc[x] = hoff[x] << 8 | log2 size, or 0.
+// Full rebuild: row x's table at hoff[x] (sizes from k_index_size and a scan);
+// hdesc[x] = hoff[x] << 8 | log2 size, or 0.  One warp per `per` rows (at most
+// 32: fewer when the warps of the grid outnumber the groups of 32, so that a
+// small graph's rows are not built one after the other on a few warps), each
+// table in the warp's shared-memory buffer; tables that outgrow it are built
+// by the whole block in the eight warps' buffers together, and only those
+// that outgrow these too in place (atomics in global memory: with every
+// table beyond a warp's buffer built so, R-MAT 2^22's last rebuild, 1.7G labels
+// in rows of 720 on average, took 32.7 ms).
 __global__ void __launch_bounds__(kIndexWarps * 32) k_index_build(const int64_t* loff, const uint32_t* lent,
                                                                   const int64_t* hoff, uint32_t* htab,
                                                                   uint64_t* hdesc, int64_t n, int slots,
                                                                   const RoundCounters* ctr) {
     extern __shared__ uint32_t ibuf[];
+    __shared__ int64_t s_row[kIndexWarps * 32];
+    __shared__ int s_n;
     if (ctr->done) return;
     const int lane = lane_id(), w = threadIdx.x >> 5;
     uint32_t* buf = ibuf + w * slots;
     const int64_t nwarps = (int64_t)gridDim.x * kIndexWarps;
     const int64_t per = min((int64_t)32, (n + nwarps - 1) / nwarps);
-    for (int64_t base = ((int64_t)blockIdx.x * kIndexWarps + w) * per; base < n; base += nwarps * per) {
+    const int64_t groups = (n + kIndexWarps * per - 1) / (kIndexWarps * per);
+    for (int64_t g = blockIdx.x; g < groups; g += gridDim.x) {
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();
+        const int64_t base = (g * kIndexWarps + w) * per;
         const int64_t x = base + lane;
         int64_t hb = 0, P = 0;
         if (lane < per && x < n) {
@@ -452,15 +483,32 @@ __global__ void __launch_bounds__(kIndexWarps * 32) k_index_build(const int64_t*
             P = hoff[x + 1] - hb;
             hdesc[x] = P > 0 ? ((uint64_t)hb << 8) | (uint64_t)(__ffsll((unsigned long long)P) - 1) : 0ull;
         }
-        unsigned m = __ballot_sync(kFull, P > 0);
+        const bool wide = P > slots && P <= (int64_t)slots * kIndexWarps;
+        if (wide) s_row[atomicAdd(&s_n, 1)] = x;
+        unsigned m = __ballot_sync(kFull, P > 0 && !wide);
         while (m) {
             const int k = __ffs(m) - 1;
             m &= m - 1;
             const int64_t xk = base + k;
             const int64_t hbk = __shfl_sync(kFull, hb, k);
-            const int Pk = (int)__shfl_sync(kFull, P, k);
+            const int64_t Pk = __shfl_sync(kFull, P, k);
             const int64_t lb = loff[xk], ll = loff[xk + 1] - lb;
-            build_table(lent, lb, ll, htab, hbk, __ffs(Pk) - 1, buf, slots, lane);
+            build_table(lent, lb, ll, htab, hbk, __ffsll((unsigned long long)Pk) - 1, buf, slots, lane);
+        }
+        __syncthreads();
+        const int nw = s_n;
+        for (int i = 0; i < nw; ++i) {
+            const int64_t xk = s_row[i], hbk = hoff[xk], lb = loff[xk], ll = loff[xk + 1] - lb;
+            const int P4 = (int)((hoff[xk + 1] - hbk) >> 2);
+            const int lg = __ffs(P4) + 1;
+            uint4* b4 = reinterpret_cast<uint4*>(ibuf);
+            for (int sl = threadIdx.x; sl < P4; sl += blockDim.x) b4[sl] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+            __syncthreads();
+            for (int64_t j = threadIdx.x; j < ll; j += blockDim.x) map_insert(ibuf, lg, lent[lb + j]);
+            __syncthreads();
+            uint4* out = reinterpret_cast<uint4*>(htab + hbk);
+            for (int sl = threadIdx.x; sl < P4; sl += blockDim.x) out[sl] = b4[sl];
+            __syncthreads();
         }
     }
 }

@@ -57,8 +57,8 @@ __global__ void k_weight_range(const uint8_t* wt, int64_t nnz, int* mm) {
     }
 }
 
-// Per arc (u -> c) of a validated symmetric CSR: the reverse arc (c -> u),
-// found by binary search in row c, has the same weight.
+// Per edge of a validated symmetric CSR: the reverse of its arc that
+// k_check_cols looks up, found by binary search, has the same weight.
 __global__ void k_check_weights(const int64_t* row_ptr, const int32_t* col, const uint8_t* wt, int64_t n,
                                 int64_t nnz, int* err) {
     __shared__ __align__(16) int srow[kTileItems];
@@ -71,6 +71,7 @@ __global__ void k_check_weights(const int64_t* row_ptr, const int32_t* col, cons
         for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
             const int64_t u = r0 + srow[p - p0];
             const int32_t c = col[p];
+            if (!looked_up(row_ptr, u, c)) continue;
             int64_t lo = row_ptr[c], hi = row_ptr[c + 1];
             while (lo < hi) {
                 const int64_t mid = (lo + hi) >> 1;
@@ -191,7 +192,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     cudaEvent_t t_all0 = tm.on ? tm.mark() : nullptr;
     int64_t launches = 0;
 
-    int* err = pool.alloc<int>(4);
+    int* err = pool.alloc<int>(6);  // [4..5]: the balance of k_check_cols
     RoundCounters* ctr = pool.alloc<RoundCounters>(1);
     PLB_ALLOC_OK();
     RoundCounters* hctr = nullptr;
@@ -202,7 +203,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     } hf{hctr};
     int* herr = reinterpret_cast<int*>(hctr + 1);
     PLB_CK(cudaMemsetAsync(ctr, 0, sizeof(RoundCounters), s));
-    PLB_CK(cudaMemsetAsync(err, 0, 4 * sizeof(int), s));
+    PLB_CK(cudaMemsetAsync(err, 0, 6 * sizeof(int), s));
 
     cudaEvent_t t0 = tm.on ? tm.mark() : nullptr;
     // ------------------------------------------------- weights and validation
@@ -231,9 +232,12 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
         PLB_CK(cudaMemcpyAsync(herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
         PLB_CK(cudaStreamSynchronize(s));
         if (herr[0]) return PLB_ERR_INVALID;
-        if (nnz > 0)
+        if (nnz > 0) {
             k_check_cols<<<grid_for((nnz + 2047) / 2048, 1, flat_grid_cap), kFlatThreads, 0, s>>>(row_ptr, col, n,
-                                                                                               nnz, 1, err);
+                                                                                               nnz, 1, err,
+                                                                                               reinterpret_cast<unsigned long long*>(err + 4));
+            k_check_balance<<<1, 1, 0, s>>>(reinterpret_cast<unsigned long long*>(err + 4), err);
+        }
         k_check_order<<<grid_for(n, kFlatThreads, flat_grid_cap), kFlatThreads, 0, s>>>(order, n, seen, err);
         PLB_CK(cudaGetLastError());
         PLB_CK(cudaMemcpyAsync(herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
