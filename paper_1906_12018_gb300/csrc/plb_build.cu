@@ -17,6 +17,16 @@ void set_last_error(cudaError_t e, int line) {
              cudaGetErrorName(e));
 }
 
+// Graph mode saves launches and host reads, 60 us a round, once capture and
+// instantiation (700 us) are paid: a path of 250 vertices (249 rounds) takes 34.7
+// ms host-driven and 20.1 in a graph, but power-law graphs finish in 5 to 8
+// rounds, most of their labels in round 2, where a graph stops to grow its
+// buffers (batches of 8 x 61K vertices: 10.1 ms host-driven, 11.1 in a graph; of
+// 200 graphs, 2.6M vertices: 46.5 and 50.1).  So a build of kGraphSmall vertices
+// or more is host-driven until it has had kGraphAfter rounds.
+constexpr int64_t kGraphSmall = 4096;
+constexpr int kGraphAfter = 8;
+
 // Core build on a validated-or-trusted CSR.  Returns a status; on success
 // *out holds the labels (rows by original id).  max_part_n: the most vertices
 // of one graph when the CSR is a disjoint union (else n); a vertex's label
@@ -327,25 +337,10 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         b.log_s = b_log_s;
         b.log_m = b_log_m;
         b.cand_limit = block_cand;
-        if (skip == nullptr) {
-            st.launches += 3;
-            return launch_tiers(w, b, split, O1, O2, ctr, grid_w, w_smem, grid_b, bthr, b_smem, s, side_stream,
-                                g1 ? &tm : nullptr, g1);
-        }
-        // captured rounds (graph mode): one after the other
-        w.list_n = &ctr->nR;
-        w.work = &ctr->wkR;
-        w.esc = O1;
-        w.esc_n = &ctr->nO1;
-        k_gp_warp<<<grid_w, kGpWarpThreads, w_smem, s>>>(w);
-        if (g1) *g1 = tm.mark();
-        b.list = O1;
-        b.list_n = &ctr->nO1;
-        b.work = &ctr->wkO1;
-        b.split = split;
-        k_gp_block<<<grid_b, bthr, b_smem, s>>>(b);
-        st.launches += 2;
-        return cudaGetLastError();
+        // (in captured rounds the side stream becomes a branch of the graph)
+        st.launches += 3;
+        return launch_tiers(w, b, split, O1, O2, ctr, grid_w, w_smem, grid_b, bthr, b_smem, s, side_stream,
+                            g1 ? &tm : nullptr, g1);
     };
     auto launch_merge = [&](int c, int x) -> cudaError_t {
         k_next_active<<<gflat, kFlatThreads, 0, s>>>(loff[c], fse[x], n, tmp64, A, ctr);
@@ -540,7 +535,10 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
             PLB_CK(cudaMemsetAsync(ctr, 0, offsetof(RoundCounters, nA), s));
             PLB_CK(cudaMemsetAsync(&ctr->nO1_base, 0, sizeof(int) * 3, s));
         }
-        {  // round 1 is always host-driven (one kernel)
+        // round 1 is always host-driven (one kernel); above kGraphSmall vertices
+        // the first kGraphAfter rounds are
+        const int before = o.use_graph && batch == n && n >= kGraphSmall ? kGraphAfter : 1;
+        for (int k = 0; k < before && !finished; ++k) {
             const int e = host_round(false);
             if (e != PLB_OK) return e;
         }
@@ -548,7 +546,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
             RoundStat* dstat = pool.alloc<RoundStat>(PLB_MAX_ROUNDS);
             PLB_ALLOC_OK();
             PLB_CK(cudaMemsetAsync(dstat, 0, sizeof(RoundStat) * PLB_MAX_ROUNDS, s));
-            int64_t lc = std::max<int64_t>(std::max<int64_t>(32 * n, T + 1024), 1 << 20);
+            int64_t lc = std::max<int64_t>(d > 1 ? T + T / 2 + 1024 : std::max<int64_t>(32 * n, T + 1024), 1 << 20);
             auto grow = [&](uint32_t*& buf, int64_t& cap, int64_t want, int64_t keep) -> bool {
                 if (cap >= want) return true;
                 uint32_t* nb = pool.alloc<uint32_t>(want);
