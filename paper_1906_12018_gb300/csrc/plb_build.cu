@@ -24,6 +24,7 @@ void set_last_error(cudaError_t e, int line) {
 // buffers (batches of 8 x 61K vertices: 10.1 ms host-driven, 11.1 in a graph; of
 // 200 graphs, 2.6M vertices: 46.5 and 50.1).  So a build of kGraphSmall vertices
 // or more is host-driven until it has had kGraphAfter rounds.
+constexpr int64_t kSmallIndex = 1 << 20;  // labels up to which the table pool is sized without a host read
 constexpr int64_t kGraphSmall = 4096;
 constexpr int kGraphAfter = 8;
 
@@ -179,7 +180,9 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         k_index_size<<<gflat, kFlatThreads, 0, s>>>(loff[which], n, tmp64, ctr);
         if (exclusive_scan_i64(tmp64, hoff, n, scan_scr, s) != cudaSuccess) return PLB_ERR_CUDA;
         int64_t need = 6 * total + 1024, want = 8 * total + 1024;
-        if (!roomy) {
+        if (total <= kSmallIndex) {  // (from the bound too: a host read costs more than the memory)
+            need = 4 * total + 1024;
+        } else if (!roomy) {
             int64_t packed = 0;
             int done = 0;
             if (cudaMemcpyAsync(&packed, hoff + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
@@ -190,7 +193,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
             need = packed + 1024;
             want = packed + packed / 2 + 1024;
         }
-        if (hcap < need || (!roomy && hcap > 2 * want)) {
+        if (hcap < need || (!roomy && hcap > 2 * want && total > kSmallIndex)) {
             pool.release(htab);
             hcap = want;
             htab = pool.alloc<uint32_t>(hcap);
@@ -200,8 +203,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         k_index_build<<<grid_for((n + kIndexWarps - 1) / kIndexWarps, 1, flat_grid_cap), kIndexWarps * 32,
                         sizeof(uint32_t) * kIndexWarps * slots, s>>>(loff[which], lent[which], hoff, htab, hdesc, n,
                                                                      slots, ctr);
-        k_index_total<<<1, 1, 0, s>>>(hoff, n, ctr);
-        st.launches += 3 + scan_n;
+        st.launches += 2 + scan_n;
         return cudaGetLastError() == cudaSuccess ? PLB_OK : PLB_ERR_CUDA;
     };
     // after a merge into parity c (labels and this round's frontier): update the
@@ -307,19 +309,18 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         return p;
     };
     const int* skip = nullptr;  // graph mode: &ctr->done (scans of finished rounds do nothing)
-    auto launch_frontier = [&](int c, int x) -> cudaError_t {
-        k_active_degree<<<gflat, kFlatThreads, 0, s>>>(roff, A, ctr, tmp64, n);
+    auto launch_frontier = [&](int c, int x, uint32_t round) -> cudaError_t {
+        k_active_degree<<<gflat, kFlatThreads, 0, s>>>(roff, A, ctr, tmp64, n, round);
         cudaError_t e = exclusive_scan_i64(tmp64, aoff, n, scan_scr, s, skip);
         if (e != cudaSuccess) return e;
         k_mark<<<flat_grid_cap, kFlatThreads, 0, s>>>(roff, rcol, fse[c], fhub[c], A, aoff, ctr, recv, n);
         k_collect<<<gflat, kFlatThreads, 0, s>>>(recv, roff, loff[c], n, fse[x], R, O1, rbound, tmp64, vbase, split, ctr, lim);
-        k_after_collect<<<1, 1, 0, s>>>(ctr);
         // the scan of the candidate bounds places each receiver's new frontier
         // row (aoff is free again after k_mark); used when the buffer holds
         // the bound sum, so that no shared cursor is contended
         e = exclusive_scan_i64(tmp64, aoff, n, scan_scr, s, skip);
         if (e != cudaSuccess) return e;
-        st.launches += 4 + 2 * scan_n;
+        st.launches += 3 + 2 * scan_n;
         return cudaGetLastError();
     };
     SideStream side_stream;
@@ -342,19 +343,23 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         return launch_tiers(w, b, split, O1, O2, ctr, grid_w, w_smem, grid_b, bthr, b_smem, s, side_stream,
                             g1 ? &tm : nullptr, g1);
     };
-    auto launch_merge = [&](int c, int x) -> cudaError_t {
+    // sort: whether rows may have been written unsorted (round 1, or rows the
+    // block tier listed; captured rounds: always launched)
+    auto launch_merge = [&](int c, int x, bool sort) -> cudaError_t {
         k_next_active<<<gflat, kFlatThreads, 0, s>>>(loff[c], fse[x], n, tmp64, A, ctr);
-        // sort the new frontier rows (appended unsorted by the gather/prune kernels)
-        k_sort_rows_warp<<<sms * 8, 256, 0, s>>>(fse[x], fhub[x], A, U, 1, ctr, big, giant);
-        k_sort_rows_radix<<<sms, 1024, kSortRadixSmemBytes, s>>>(fse[x], fhub[x], big, &ctr->nBig, ctr);
-        k_sort_rows_block<<<sort_blocks, 1024, 16384 * sizeof(uint32_t), s>>>(fse[x], fhub[x], giant, &ctr->nGiant,
-                                                                            sortscr, sort_words, ctr);
+        if (sort) {
+            k_sort_rows_warp<<<sms * 8, 256, 0, s>>>(fse[x], fhub[x], A, U, 1, ctr, big, giant);
+            k_sort_rows_radix<<<sms, 1024, kSortRadixSmemBytes, s>>>(fse[x], fhub[x], big, &ctr->nBig, ctr);
+            k_sort_rows_block<<<sort_blocks, 1024, 16384 * sizeof(uint32_t), s>>>(fse[x], fhub[x], giant, &ctr->nGiant,
+                                                                                sortscr, sort_words, ctr);
+            st.launches += 3;
+        }
         cudaError_t e = exclusive_scan_i64(tmp64, loff[x], n, scan_scr, s, skip);
         if (e != cudaSuccess) return e;
         k_merge_rows<<<grid_for((n + 7) / 8, 1, flat_grid_cap), 256, 0, s>>>(
             loff[c], lent[c], loff[x], lent[x], fse[x], fhub[x], n, vbase, ctr, top);
         k_top_columns<<<grid_for((n + 31) / 32, 1, flat_grid_cap), 256, 0, s>>>(top, n, vbase, cols, batch < n, ctr);
-        st.launches += 6 + scan_n;
+        st.launches += 3 + scan_n;
         return cudaGetLastError();
     };
 
@@ -395,10 +400,8 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
             }
         } else {
             if (!frontier_done) {
-                k_set_round<<<1, 1, 0, s>>>(ctr, (uint32_t)d);
-                st.launches += 1;
                 // frontier: mark receivers from the active list, collect them
-                PLB_CK(launch_frontier(cur, nxt));
+                PLB_CK(launch_frontier(cur, nxt, (uint32_t)d));
             }
             // size the new frontier buffer from the candidate bound (no re-run)
             PLB_CK(cudaMemcpyAsync(hctr, ctr, sizeof(RoundCounters), cudaMemcpyDeviceToHost, s));
@@ -489,7 +492,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
             lent[nxt] = pool.alloc<uint32_t>(lcap[nxt]);
             PLB_ALLOC_OK();
         }
-        PLB_CK(launch_merge(cur, nxt));
+        PLB_CK(launch_merge(cur, nxt, d == 1 || hctr->nU > 0));
         T = Tn;
         cur = nxt;
         if (d == 1 || acc > T - acc) {
@@ -504,7 +507,6 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         if (tm.on) tm.span(T_MERGE, m0, tm.mark());
         // round-start reset of the per-round counters (nA carries over)
         PLB_CK(cudaMemsetAsync(ctr, 0, offsetof(RoundCounters, nA), s));
-        PLB_CK(cudaMemsetAsync(&ctr->nO1_base, 0, sizeof(int) * 3, s));
         // grow the frontier buffer ahead of a large round
         if (acc > fcap[cur ^ 1] / 2) {
             const int nx2 = cur ^ 1;
@@ -533,7 +535,6 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
             d = 0;
             finished = false;
             PLB_CK(cudaMemsetAsync(ctr, 0, offsetof(RoundCounters, nA), s));
-            PLB_CK(cudaMemsetAsync(&ctr->nO1_base, 0, sizeof(int) * 3, s));
         }
         // round 1 is always host-driven (one kernel); above kGraphSmall vertices
         // the first kGraphAfter rounds are
@@ -615,14 +616,14 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
                 for (int r = 0; r < 2 && ce == cudaSuccess; ++r) {
                     const int c = cur ^ r, x = c ^ 1;
                     k_g_begin<<<1, 1, 0, s>>>(ctr);
-                    ce = launch_frontier(c, x);
+                    ce = launch_frontier(c, x, 0u);
                     if (ce == cudaSuccess) {
                         k_g_bound<<<1, 1, 0, s>>>(ctr, x);
                         ce = launch_gp(gp_params(c, x, fcap[x], true), nullptr);  // k_g_bound checked the bound
                     }
                     if (ce == cudaSuccess) {
                         k_g_check<<<1, 1, 0, s>>>(ctr, dstat);
-                        ce = launch_merge(c, x);
+                        ce = launch_merge(c, x, true);
                     }
                     if (ce == cudaSuccess) ce = update_index(x, T);
                     if (ce == cudaSuccess) {
@@ -685,7 +686,6 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
                     d = dd - 1;
                     hctr->nA = hctr->nA_saved;
                     PLB_CK(cudaMemsetAsync(ctr, 0, offsetof(RoundCounters, nA), s));
-                    PLB_CK(cudaMemsetAsync(&ctr->nO1_base, 0, sizeof(int) * 3, s));
                     PLB_CK(cudaMemcpyAsync(&ctr->nA, &hctr->nA, sizeof(int), cudaMemcpyHostToDevice, s));
                     const int e = host_round(false);
                     if (e != PLB_OK) return e;
@@ -697,7 +697,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
                 const int64_t Tn = T + (int64_t)hctr->accepted;
                 lc = std::max<int64_t>(Tn + Tn / 2, lc + lc / 2);
                 if (!grow(lent[nxt], lcap[nxt], lc, 0)) return PLB_ERR_OOM;
-                PLB_CK(launch_merge(cur, nxt));
+                PLB_CK(launch_merge(cur, nxt, true));
                 T = Tn;
                 cur = nxt;
                 d = dd;
@@ -706,7 +706,6 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
                     if (e != PLB_OK) return e;
                 }
                 PLB_CK(cudaMemsetAsync(ctr, 0, offsetof(RoundCounters, nA), s));
-                PLB_CK(cudaMemsetAsync(&ctr->nO1_base, 0, sizeof(int) * 3, s));
             }
             // per-round statistics written on the device
             std::vector<RoundStat> hstat(PLB_MAX_ROUNDS);

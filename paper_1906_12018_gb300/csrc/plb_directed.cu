@@ -214,8 +214,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
         k_index_build<<<grid_for((n + kIndexWarps - 1) / kIndexWarps, 1, flat_grid_cap), kIndexWarps * 32,
                         sizeof(uint32_t) * kIndexWarps * slots, s>>>(S.loff[S.cur], S.lent[S.cur], S.hoff, S.htab,
                                                                      S.hdesc, n, slots, S.ctr);
-        k_index_total<<<1, 1, 0, s>>>(S.hoff, n, S.ctr);
-        launches += 3 + scan_n;
+        launches += 2 + scan_n;
         return cudaGetLastError() == cudaSuccess ? PLB_OK : PLB_ERR_CUDA;
     };
     for (int k = 0; k < 2; ++k) {
@@ -273,17 +272,17 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
     for (int k = 0; k < 2; ++k) split2[k] = split_lists(pool, n, n, nnz, s);
     PLB_ALLOC_OK();
     // ------------------------------------------------------------ rounds
+    int d = 0;
     auto frontier = [&](Side& S) -> cudaError_t {
         const int c = S.cur, x = c ^ 1;
-        k_active_degree<<<gflat, kFlatThreads, 0, s>>>(S.s_off, S.A, S.ctr, tmp64, n);
+        k_active_degree<<<gflat, kFlatThreads, 0, s>>>(S.s_off, S.A, S.ctr, tmp64, n, (uint32_t)d);
         cudaError_t e = exclusive_scan_i64(tmp64, S.aoff, n, scan_scr, s);
         if (e != cudaSuccess) return e;
         k_mark<<<flat_grid_cap, kFlatThreads, 0, s>>>(S.s_off, S.s_col, S.fse[c], S.fhub[c], S.A, S.aoff, S.ctr,
                                                       S.recv, n);
         k_collect<<<gflat, kFlatThreads, 0, s>>>(S.recv, S.g_off, S.loff[c], n, S.fse[x], S.R, S.O1, S.rbound, nullptr,
                                                  nullptr, split2[&S - side], S.ctr, lim);
-        k_after_collect<<<1, 1, 0, s>>>(S.ctr);
-        launches += 4 + scan_n;
+        launches += 3 + scan_n;
         return cudaGetLastError();
     };
     // gather + prune of side S; the candidates' side of the check is side H
@@ -334,17 +333,20 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
     auto merge = [&](Side& S) -> cudaError_t {
         const int c = S.cur, x = c ^ 1;
         k_next_active<<<gflat, kFlatThreads, 0, s>>>(S.loff[c], S.fse[x], n, tmp64, S.A, S.ctr);
-        k_sort_rows_warp<<<sms * 8, 256, 0, s>>>(S.fse[x], S.fhub[x], S.A, S.U, 1, S.ctr, big, giant);
-        k_sort_rows_radix<<<sms, 1024, kSortRadixSmemBytes, s>>>(S.fse[x], S.fhub[x], big, &S.ctr->nBig, S.ctr);
-        k_sort_rows_block<<<sort_blocks, 1024, 16384 * sizeof(uint32_t), s>>>(S.fse[x], S.fhub[x], giant,
-                                                                            &S.ctr->nGiant, sortscr, sort_words,
-                                                                            S.ctr);
+        if (d == 1 || S.hctr->nU > 0) {  // rows written unsorted
+            k_sort_rows_warp<<<sms * 8, 256, 0, s>>>(S.fse[x], S.fhub[x], S.A, S.U, 1, S.ctr, big, giant);
+            k_sort_rows_radix<<<sms, 1024, kSortRadixSmemBytes, s>>>(S.fse[x], S.fhub[x], big, &S.ctr->nBig, S.ctr);
+            k_sort_rows_block<<<sort_blocks, 1024, 16384 * sizeof(uint32_t), s>>>(S.fse[x], S.fhub[x], giant,
+                                                                                &S.ctr->nGiant, sortscr, sort_words,
+                                                                                S.ctr);
+            launches += 3;
+        }
         cudaError_t e = exclusive_scan_i64(tmp64, S.loff[x], n, scan_scr, s);
         if (e != cudaSuccess) return e;
         k_merge_rows<<<grid_for((n + 7) / 8, 1, flat_grid_cap), 256, 0, s>>>(
             S.loff[c], S.lent[c], S.loff[x], S.lent[x], S.fse[x], S.fhub[x], n, nullptr, S.ctr, S.top);
         k_top_columns<<<grid_for((n + 31) / 32, 1, flat_grid_cap), 256, 0, s>>>(S.top, n, nullptr, S.cols, 0, S.ctr);
-        launches += 6 + scan_n;
+        launches += 3 + scan_n;
         return cudaGetLastError();
     };
     auto read_ctr = [&](Side& S) -> cudaError_t {
@@ -352,7 +354,6 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
     };
 
     int status = PLB_OK;
-    int d = 0;
     while (!(side[0].done && side[1].done)) {
         ++d;
         cudaEvent_t r0 = tm.on ? tm.mark() : nullptr;
@@ -361,9 +362,9 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
             Side& S = side[k];
             if (S.done) continue;
             const int x = S.cur ^ 1;
-            k_set_round<<<1, 1, 0, s>>>(S.ctr, (uint32_t)d);
-            launches += 1;
             if (d == 1) {
+                k_set_round<<<1, 1, 0, s>>>(S.ctr, 1u);
+                launches += 1;
                 const int g1 = grid_for((nnz + 2047) / 2048, 1, flat_grid_cap);
                 PLB_CK(cudaMemsetAsync(tmp64, 0, sizeof(int64_t) * (n + 1), s));
                 PLB_CK(cudaMemsetAsync(cur1, 0, sizeof(uint32_t) * std::max<int64_t>(n, 1), s));
@@ -486,7 +487,6 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
                 PLB_CK(cudaGetLastError());
             }
             PLB_CK(cudaMemsetAsync(S.ctr, 0, offsetof(RoundCounters, nA), s));
-            PLB_CK(cudaMemsetAsync(&S.ctr->nO1_base, 0, sizeof(int) * 3, s));
             if ((int64_t)S.hctr->accepted > S.fcap[S.cur ^ 1] / 2) {  // grow the next frontier buffer ahead
                 const int nx2 = S.cur ^ 1;
                 pool.release(S.fhub[nx2]);

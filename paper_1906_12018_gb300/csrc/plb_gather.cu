@@ -1436,8 +1436,14 @@ __global__ void __launch_bounds__(256, 3) k_gp_block(GpParams p) {
 // Check records of all rows, from the label offsets and the probe index as
 // they stand for the coming gather (a finished round returns at once).
 __global__ void k_pack_hrec(const int64_t* loff, const uint32_t* lent, const uint64_t* hdesc, const int32_t* vbase,
-                            uint4* hrec, int64_t n, const RoundCounters* ctr) {
+                            uint4* hrec, int64_t n, RoundCounters* ctr) {
     if (ctr->done) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {  // after k_collect: its list sizes; the next active list starts empty
+        ctr->nO1_base = ctr->nO1;
+        ctr->nG_base = ctr->nG = min(ctr->nG, kMaxSplit);
+        if (ctr->nA > 0) ctr->nA_saved = ctr->nA;  // (0: the gather runs again)
+        ctr->nA = 0;
+    }
 #pragma unroll 1
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
         const int64_t a = loff[v], len = loff[v + 1] - a;

@@ -37,9 +37,9 @@ struct RoundCounters {
     int nU;                       // vertices whose new frontier row was written unsorted (block tier)
     int wkR, wkO1, wkO2;          // next entry of each tier's list (taken by whoever is free)
     int nG, nP;                   // split receivers and their parts (see SplitLists)
-    int nA;                       // next active list (kept across the per-round reset)
     int nO1_base, nG_base;        // list sizes made by k_collect (for reruns and statistics)
     int fovf;                     // new-frontier buffer overflow
+    int nA;                       // next active list (kept across the per-round reset, which ends here)
     unsigned int max_dist;        // finalize: largest stored distance
     int guard;                    // a kernel met a broken capacity invariant (internal error)
     // loop control (kept across rounds)
@@ -230,7 +230,7 @@ __host__ __device__ __forceinline__ int column_quads(int64_t n) {
     return (int)((m + 127) / 128);
 }
 __global__ void k_pack_hrec(const int64_t* loff, const uint32_t* lent, const uint64_t* hdesc, const int32_t* vbase,
-                            uint4* hrec, int64_t n, const RoundCounters* ctr);
+                            uint4* hrec, int64_t n, RoundCounters* ctr);
 
 // Routing limits of k_collect (see the tier geometry in build_core).
 struct TierLimits {

@@ -170,10 +170,12 @@ __global__ void k_init(const int64_t* roff, int64_t n, int64_t* loff, uint32_t* 
 }
 
 // ------------------------------------------------------------ frontier
-// adeg[i] = degree of active vertex A[i] (0 beyond nA), for the flat mark.
-__global__ void k_active_degree(const int64_t* roff, const int32_t* A, const RoundCounters* ctr, int64_t* adeg,
-                                int64_t n) {
+// adeg[i] = degree of active vertex A[i] (0 beyond nA), for the flat mark.  Host-
+// driven rounds start here: d > 0 is the round number (graph mode: k_g_begin).
+__global__ void k_active_degree(const int64_t* roff, const int32_t* A, RoundCounters* ctr, int64_t* adeg, int64_t n,
+                                uint32_t d) {
     if (ctr->done) return;
+    if (d > 0 && blockIdx.x == 0 && threadIdx.x == 0) ctr->d = d;
     const int nA = ctr->nA;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         int64_t x = 0;
@@ -271,15 +273,6 @@ __global__ void k_collect(unsigned long long* recv, const int64_t* roff, const i
     }
     bsum = warp_sum(bsum);
     if (lane == 0 && bsum) atomicAdd(&ctr->bound_sum, bsum);
-}
-
-__global__ void k_after_collect(RoundCounters* ctr) {
-    if (ctr->done) return;
-    ctr->nO1_base = ctr->nO1;
-    ctr->nG = min(ctr->nG, kMaxSplit);
-    ctr->nG_base = ctr->nG;
-    ctr->nA_saved = ctr->nA;
-    ctr->nA = 0;
 }
 
 // Round 1 (Alg. 3 with d = 1) of the hubs [s, e) (all hubs, or one batch of
@@ -462,11 +455,15 @@ __device__ __forceinline__ void build_table(const uint32_t* lent, int64_t lb, in
 __global__ void __launch_bounds__(kIndexWarps * 32) k_index_build(const int64_t* loff, const uint32_t* lent,
                                                                   const int64_t* hoff, uint32_t* htab,
                                                                   uint64_t* hdesc, int64_t n, int slots,
-                                                                  const RoundCounters* ctr) {
+                                                                  RoundCounters* ctr) {
     extern __shared__ uint32_t ibuf[];
     __shared__ int64_t s_row[kIndexWarps * 32];
     __shared__ int s_n;
     if (ctr->done) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {  // the next free slot of the table pool
+        ctr->hnext = hoff[n];
+        ctr->hovf = 0;
+    }
     const int lane = lane_id(), w = threadIdx.x >> 5;
     uint32_t* buf = ibuf + w * slots;
     const int64_t nwarps = (int64_t)gridDim.x * kIndexWarps;
@@ -511,13 +508,6 @@ __global__ void __launch_bounds__(kIndexWarps * 32) k_index_build(const int64_t*
             __syncthreads();
         }
     }
-}
-
-// After a full rebuild: the next free slot of the table pool.
-__global__ void k_index_total(const int64_t* hoff, int64_t n, RoundCounters* ctr) {
-    if (ctr->done) return;
-    ctr->hnext = hoff[n];
-    ctr->hovf = 0;
 }
 
 // Incremental update after a merge, one warp per row that changed (the new

@@ -20,15 +20,14 @@ __global__ void k_relabel(const int64_t* row_ptr, const int32_t* col, const int3
                           const int64_t* roff, int32_t* rcol, int64_t n, int64_t nnz);
 __global__ void k_init(const int64_t* roff, int64_t n, int64_t* loff, uint32_t* lent, uint64_t* fse,
                        uint32_t* fhub, int32_t* A, RoundCounters* ctr);
-__global__ void k_active_degree(const int64_t* roff, const int32_t* A, const RoundCounters* ctr, int64_t* adeg,
-                                int64_t n);
+__global__ void k_active_degree(const int64_t* roff, const int32_t* A, RoundCounters* ctr, int64_t* adeg, int64_t n,
+                                uint32_t d);
 __global__ void k_mark(const int64_t* roff, const int32_t* rcol, const uint64_t* fse, const uint32_t* fhub,
                        const int32_t* A, const int64_t* aoff, const RoundCounters* ctr, unsigned long long* recv,
                        int64_t n);
 __global__ void k_collect(unsigned long long* recv, const int64_t* roff, const int64_t* loff, int64_t n,
                           uint64_t* fse_new, int32_t* R, int32_t* O1, uint32_t* rbound, int64_t* obound,
                           const int32_t* vbase, SplitLists split, RoundCounters* ctr, TierLimits lim);
-__global__ void k_after_collect(RoundCounters* ctr);
 __global__ void k_rerun_reset(RoundCounters* ctr, uint64_t* fse_new, int64_t n);
 __global__ void k_round1_count(const int64_t* roff, const int32_t* rcol, int64_t n, int64_t nnz, int32_t s,
                                int32_t e, unsigned long long* cnt, const RoundCounters* ctr);
@@ -39,8 +38,7 @@ __global__ void k_gp_warp(GpParams p);
 __global__ void k_gp_block(GpParams p);
 __global__ void k_index_size(const int64_t* loff, int64_t n, int64_t* hsz, const RoundCounters* ctr);
 __global__ void k_index_build(const int64_t* loff, const uint32_t* lent, const int64_t* hoff, uint32_t* htab,
-                              uint64_t* hdesc, int64_t n, int slots, const RoundCounters* ctr);
-__global__ void k_index_total(const int64_t* hoff, int64_t n, RoundCounters* ctr);
+                              uint64_t* hdesc, int64_t n, int slots, RoundCounters* ctr);
 __global__ void k_index_update(const int64_t* loff, const uint32_t* lent, const uint64_t* fse_new,
                                const uint32_t* fhub_new, const int32_t* A, uint32_t* htab, uint64_t* hdesc,
                                long long hcap, int slots, RoundCounters* ctr);

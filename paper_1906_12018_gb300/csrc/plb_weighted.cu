@@ -332,8 +332,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
         k_index_build<<<grid_for((n + kIndexWarps - 1) / kIndexWarps, 1, flat_grid_cap), kIndexWarps * 32,
                         sizeof(uint32_t) * kIndexWarps * slots, s>>>(loff[cur], lent[cur], hoff, htab, hdesc, n,
                                                                      slots, ctr);
-        k_index_total<<<1, 1, 0, s>>>(hoff, n, ctr);
-        launches += 3 + scan_n;
+        launches += 2 + scan_n;
         return cudaGetLastError() == cudaSuccess ? PLB_OK : PLB_ERR_CUDA;
     };
     {
@@ -457,8 +456,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
             k_w_pull<<<gpull, kWFlatThreads, 0, s>>>(roff, rcol, rwt, n, nnz, (uint32_t)d, S, lgn, ring, store,
                                                      vcol, recv);
         k_collect<<<gflat, kFlatThreads, 0, s>>>(recv, roff, loff[cur], n, fse_new, R, O1, rbound, nullptr, nullptr, split, ctr, lim);
-        k_after_collect<<<1, 1, 0, s>>>(ctr);
-        launches += 4;
+        launches += 3;
         PLB_CK(cudaGetLastError());
         PLB_CK(read_ctr());
         PLB_CK(cudaStreamSynchronize(s));
@@ -472,7 +470,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
         }
         if (tm.on) tm.span(T_FRONT, r0, tm.mark());
         cudaEvent_t g0 = tm.on ? tm.mark() : nullptr;
-        const bool any = hctr->nR + hctr->nO1_base + hctr->nG_base > 0;
+        const bool any = hctr->nR + hctr->nO1 + hctr->nG > 0;
         if (any) {
             for (int attempt = 0;; ++attempt) {
                 if (attempt > 0) {
@@ -528,17 +526,20 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
                 PLB_ALLOC_OK();
             }
             k_next_active<<<gflat, kFlatThreads, 0, s>>>(loff[cur], fse_new, n, tmp64, A, ctr);
-            k_sort_rows_warp<<<sms * 8, 256, 0, s>>>(fse_new, store, A, U, 0, ctr, big, giant);
-            k_sort_rows_block<<<sms * 2, 1024, 16384 * sizeof(uint32_t), s>>>(fse_new, store, big, &ctr->nBig,
-                                                                            nullptr, 0, ctr);
-            k_sort_rows_block<<<sort_blocks, 1024, 16384 * sizeof(uint32_t), s>>>(fse_new, store, giant,
-                                                                                &ctr->nGiant, sortscr, sort_words,
-                                                                                ctr);
+            if (hctr->nU > 0) {  // rows written unsorted
+                k_sort_rows_warp<<<sms * 8, 256, 0, s>>>(fse_new, store, A, U, 0, ctr, big, giant);
+                k_sort_rows_block<<<sms * 2, 1024, 16384 * sizeof(uint32_t), s>>>(fse_new, store, big, &ctr->nBig,
+                                                                                nullptr, 0, ctr);
+                k_sort_rows_block<<<sort_blocks, 1024, 16384 * sizeof(uint32_t), s>>>(fse_new, store, giant,
+                                                                                    &ctr->nGiant, sortscr, sort_words,
+                                                                                    ctr);
+                launches += 3;
+            }
             PLB_CK(exclusive_scan_i64(tmp64, loff[x], n, scan_scr, s));
             k_merge_rows<<<grid_for((n + 7) / 8, 1, flat_grid_cap), 256, 0, s>>>(
                 loff[cur], lent[cur], loff[x], lent[x], fse_new, store, n, nullptr, ctr, top);
             k_top_columns<<<grid_for((n + 31) / 32, 1, flat_grid_cap), 256, 0, s>>>(top, n, nullptr, cols, 0, ctr);
-            launches += 6 + scan_n;
+            launches += 3 + scan_n;
             PLB_CK(cudaGetLastError());
             const int64_t Told = T;
             T = Tn;
@@ -557,7 +558,6 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
             if (tm.on) tm.span(T_MERGE, m0, tm.mark());
         }
         PLB_CK(cudaMemsetAsync(ctr, 0, offsetof(RoundCounters, nA), s));
-        PLB_CK(cudaMemsetAsync(&ctr->nO1_base, 0, sizeof(int) * 3, s));
     }
     if (status != PLB_OK) return status;
 
