@@ -312,7 +312,9 @@ __device__ __forceinline__ bool gather_range(const GpParams& p, int64_t nb, int6
             const uint32_t hn = it < total ? rk[it] : kEmpty;
             const uint32_t hr = h - vb;
             if (hr < W) {
-                atomicOr(&X[hr >> 5], 1u << (hr & 31));
+                // (a set bit is not set again: in dense graphs the lanes of a
+                // step share few words, and atomics on one word take turns)
+                if (!((X[hr >> 5] >> (hr & 31)) & 1u)) atomicOr(&X[hr >> 5], 1u << (hr & 31));
                 hmax = max(hmax, hr + 1u);
             }
             const bool big = h != kEmpty && hr >= W;
