@@ -229,8 +229,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
     const int w_log_s = ceil_log2_i64(2 * (int64_t)warp_cand);
     const int w_log_m = ceil_log2_i64(2 * warp_label);
     const int warps_per_block = kGpWarpThreads / 32;
-    const size_t w_smem = sizeof(uint32_t) * (4 * warps_per_block +
-                                              (size_t)warps_per_block * (kTopRow + (1 << w_log_s) + (1 << w_log_m)));
+    const size_t w_smem = gp_warp_smem_bytes(warps_per_block, w_log_s, w_log_m);
     const int bthr = std::min(256, std::max(64, (o.block_threads / 32) * 32));  // k_gp_block: <= 256 threads
     const int block_cand = pow2_at_least(std::max(bthr, o.block_cand_cap));
     const int b_log_s = ceil_log2_i64(std::max<int64_t>(std::max<int64_t>(2 * (int64_t)block_cand,
@@ -242,7 +241,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
     lim.warp_bound = 2 * (int64_t)warp_cand;
     lim.warp_label = warp_label;
     lim.warp_deg = (int64_t)32 * 64;
-    if (w_smem > 227 * 1024 || b_smem > 227 * 1024) return PLB_ERR_INVALID;
+    if (!tiers_fit(warps_per_block, w_log_s, w_log_m, b_smem)) return PLB_ERR_INVALID;
     PLB_CK(cudaFuncSetAttribute(k_gp_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w_smem));
     PLB_CK(cudaFuncSetAttribute(k_gp_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b_smem));
     int occ_w = 1, occ_b = 1;
@@ -260,7 +259,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
     PLB_CK(cudaFuncSetAttribute(k_sort_rows_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)(16384 * sizeof(uint32_t))));
     PLB_CK(cudaFuncSetAttribute(k_sort_rows_radix, cudaFuncAttributeMaxDynamicSharedMemorySize, kSortRadixSmemBytes));
-    // block tier: per-block buffer of accepted hubs past the maps
+    // block tier: per-block buffer of accepted hubs past the map
     const int64_t acc_words = accepted_words(std::min<int64_t>(n, max_part_n));
     uint32_t* gacc = pool.alloc<uint32_t>((int64_t)grid_b * acc_words);
     const SplitLists split = split_lists(pool, n, max_part_n, nnz, s);
@@ -333,6 +332,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         w.log_s = w_log_s;
         w.log_m = w_log_m;
         w.cand_limit = warp_cand;
+        w.s_words = warp_set_words(w_log_s);
         b.esc = nullptr;  // block tier (never escalates)
         b.esc_n = nullptr;
         b.log_s = b_log_s;

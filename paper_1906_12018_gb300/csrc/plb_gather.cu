@@ -418,7 +418,7 @@ __device__ void shrink_pass(uint32_t* S, int log_s, uint32_t* C, int limit, uint
     }
 }
 
-// A hub past the maps: into the set S, unless it is in L(v) (M) or the set is
+// A hub past the map: into the set S, unless it is in L(v) (M) or the set is
 // full (*ovf_sm).  Returns 1 when it is new.
 __device__ __noinline__ int set_add(uint32_t* S, int log_s, const uint32_t* M, int log_m, int limit,
                                     volatile int* cnt_sm, volatile int* ovf_sm, uint32_t h) {
@@ -431,10 +431,11 @@ __device__ __noinline__ int set_add(uint32_t* S, int log_s, const uint32_t* M, i
 }
 
 // Block-wide load-balanced gather of v's messages with hub in [lo, *hi_sm):
-// hubs below vb + W (vb: the first rank of v's graph) are marked in the maps B
-// (the first kByteHubs one byte each, plain stores: duplicates write the same
-// byte; the following ones one bit each; L(v)'s hubs are cleared afterwards),
-// the others go into the set S.  Neighbours are taken in tiles of blockDim; each
+// hubs below vb + W (vb: the first rank of v's graph) are marked in the map B
+// (a bit each; L(v)'s hubs are cleared afterwards; looking first whether the bit
+// is set already, as the warp tier does, made R-MAT 2^22 2% slower: the lanes of
+// a step read different sectors and seldom meet in a word), the others go into
+// the set S.  Neighbours are taken in tiles of blockDim; each
 // thread finds the sectors (eight hubs) of its neighbour's row dL_{d-1}(a) that
 // overlap the range (the row is sorted), a block-wide exclusive scan of their
 // counts assigns every warp an equal, contiguous share, and every lane reads
@@ -446,16 +447,14 @@ __device__ __noinline__ int set_add(uint32_t* S, int log_s, const uint32_t* M, i
 // tile from the step where it stopped, now dropping hubs at or above the new
 // bound (a later pass takes them): no message of the tile is read twice, except
 // those of the step that met the overflow.
-__device__ __noinline__ void gather_block(const GpParams& p, int64_t nb, int64_t ne, uint32_t lo, uint32_t* hi_sm, uint8_t* B,
+__device__ __noinline__ void gather_block(const GpParams& p, int64_t nb, int64_t ne, uint32_t lo, uint32_t* hi_sm, uint32_t* B,
                              uint32_t vb, uint32_t W, uint32_t* S, int log_s, const uint32_t* M, int log_m, int limit,
                              int* cnt_sm, volatile int* ovf_sm, int* wsum, int* sex, int64_t* sst, uint32_t* C,
                              int* hist, int* tmp, unsigned long long& msgs) {
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int nw = nthr >> 5, lane = tid & 31;
     const uint32_t set_lo = max(lo, vb + W);  // S holds hubs from here on
-    if (lo > vb) W = 0;                       // the maps are the first pass's
-    const uint32_t Wb = min(W, (uint32_t)kByteHubs);
-    uint32_t* bits = reinterpret_cast<uint32_t*>(B + kByteHubs);
+    if (lo > vb) W = 0;                       // the map is the first pass's
 #pragma unroll 1
     for (int64_t t0 = nb; t0 < ne; t0 += nthr) {
         const uint32_t hi = *(volatile uint32_t*)hi_sm;
@@ -538,15 +537,12 @@ __device__ __noinline__ void gather_block(const GpParams& p, int64_t nb, int64_t
 #pragma unroll
                             for (int q = 0; q < kRowAlign; ++q) x[q] = kEmpty;
                         }
-                        unsigned past = 0, got = 0;  // hubs past the maps, messages of the range
+                        unsigned past = 0, got = 0;  // hubs past the map, messages of the range
 #pragma unroll
                         for (int q = 0; q < kRowAlign; ++q) {
                             const uint32_t hr = x[q] - vb;
-                            if (hr < Wb) {
-                                B[hr] = 1;
-                            } else if (hr < W) {
-                                const uint32_t z = hr - (uint32_t)kByteHubs;
-                                atomicOr(&bits[z >> 5], 1u << (z & 31));
+                            if (hr < W) {
+                                atomicOr(&B[hr >> 5], 1u << (hr & 31));
                             } else if (x[q] - set_lo < hcut - set_lo) {
                                 past |= 1u << q;
                             }
@@ -606,12 +602,14 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
     extern __shared__ uint32_t sm[];
     const int lane = lane_id(), wib = threadIdx.x >> 5;
     const int nwarps = blockDim.x >> 5;
-    const int S_CAP = 1 << p.log_s, M_CAP = 1 << p.log_m;
+    const int M_CAP = 1 << p.log_m;
     int* wsc = reinterpret_cast<int*>(sm) + wib * 4;  // [0] entries of the set
-    uint32_t* tvs = sm + 4 * nwarps;                   // per warp: v's exact-distance top-hub masks
-    uint32_t* S = tvs + nwarps * kTopRow + wib * (S_CAP + M_CAP);
-    uint32_t* X = S + S_CAP;                           // hub bitmap (zero between vertices), then L(v)'s map
-    uint32_t* tv = tvs + wib * kTopRow;
+    // per warp: the set, then the candidates and, in its last words, v's
+    // exact-distance top-hub masks
+    uint32_t* S = sm + 4 * nwarps + wib * (p.s_words + M_CAP);
+    uint32_t* X = S + p.s_words;                       // hub bitmap (zero between vertices), then L(v)'s map
+    const int cap = p.s_words - kTopRow;               // most candidates
+    uint32_t* tv = S + cap;
     const unsigned lt = (1u << lane) - 1u;
     unsigned long long c_arcs = 0, c_msgs = 0, c_uniq = 0, c_staged = 0, c_probed = 0, c_acc = 0, c_vert = 0;
     unsigned long long c_pref = 0, c_chk[2] = {0, 0};
@@ -658,10 +656,13 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
             __syncwarp();
             // ... and the set's, compacted in place (write position never
             // passes the read position)
-            if (*(volatile int*)&wsc[0] > 0) {
+            const bool any = *(volatile int*)&wsc[0] > 0;
+            if (any || bnd > (uint32_t)cap) {
 #pragma unroll 1
                 for (int q = lane; q < words; q += 32) nbm += __popc(X[q]);
                 nbm = warp_sum(nbm);
+            }
+            if (any) {
 #pragma unroll 1
                 for (int sb = 0; sb < (1 << log_s); sb += 32) {
                     const uint32_t h = S[sb + lane];
@@ -678,7 +679,7 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
                 __syncwarp();
             }
         }
-        if (!ok || nbm + nset > S_CAP) {
+        if (!ok || nbm + nset > cap) {
 #pragma unroll 1
             for (int q = lane; q < (int)((W + 31u) >> 5); q += 32) X[q] = 0u;
             if (lane == 0) {
@@ -770,8 +771,8 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
         // past ns are free now) when it fits: the checks' binary searches in
         // L(v) and their side-B scans of it then read shared memory
         const uint32_t* lvp = lv;
-        const bool copy = (int64_t)ns + ll <= S_CAP;
-        uint32_t* lvs = S + (S_CAP - ll);
+        const bool copy = (int64_t)ns + ll <= cap;
+        uint32_t* lvs = S + (cap - ll);
         if (copy) lvp = lvs;
         if (!mglob) {
 #pragma unroll 1
@@ -825,7 +826,7 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
                 if (ntail > 0) {
                     int P = 32;
 #pragma unroll 1
-                    while (P < ntail) P <<= 1;  // <= S_CAP: at most cand_limit, half of it
+                    while (P < ntail) P <<= 1;  // <= cap: at most cand_limit
 #pragma unroll 1
                     for (int j0 = 0; j0 < P; j0 += 32) {
                         const uint32_t h = j0 + lane < ntail ? S[n0 + j0 + lane] : kEmpty;
@@ -868,24 +869,19 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
 
 // Block-per-vertex scalars in shared memory (ints)
 enum { SH_UNIQ = 0, SH_OVF = 1, SH_ACC = 2 /* accepted, from the set */, SH_NC = 3, SH_HI = 4, SH_TMP = 5 /* 2 ints */,
-       SH_START = 8 /* 2 ints */, SH_NEXT = 10, SH_REST = 11, SH_MACC = 12 /* accepted, from the maps */,
+       SH_START = 8 /* 2 ints */, SH_NEXT = 10, SH_REST = 11, SH_MACC = 12 /* accepted, from the map */,
        SH_ITEM = 13, SH_LAST = 14, SH_NE = 15 /* rows of the first prefilter step */,
-       SH_WCNT = 16 /* 2 x 8 warps */, SH_WORDS = 48 };
+       SH_WCNT = 16 /* 8 warps */, SH_WORDS = 48 };
 
-// Accepted candidates of a chunk (okm): those of the maps are marked there
+// Accepted candidates of a chunk (okm): those of the map are marked there
 // again (extraction cleared them), the set's go to this block's global scratch.
-__device__ __forceinline__ void keep_accepted(unsigned okm, uint32_t h, uint32_t vb, uint32_t W, uint8_t* B,
+__device__ __forceinline__ void keep_accepted(unsigned okm, uint32_t h, uint32_t vb, uint32_t W, uint32_t* B,
                                               uint32_t* gacc, int* sh) {
     const int lane = threadIdx.x & 31;
     const uint32_t hr = h - vb;
     const bool ok = (okm >> lane) & 1u, inmap = hr < W;
     if (ok && inmap) {
-        if (hr < (uint32_t)kByteHubs) {
-            B[hr] = 1;
-        } else {
-            const uint32_t q = hr - (uint32_t)kByteHubs;
-            atomicOr(reinterpret_cast<uint32_t*>(B + kByteHubs) + (q >> 5), 1u << (q & 31));
-        }
+        atomicOr(&B[hr >> 5], 1u << (hr & 31));
     }
     const unsigned mm = __ballot_sync(kFull, ok && inmap), ms = okm & ~mm;
     int base = 0;
@@ -897,139 +893,81 @@ __device__ __forceinline__ void keep_accepted(unsigned okm, uint32_t h, uint32_t
     if (ok && !inmap) gacc[base + __popc(ms & ((1u << lane) - 1u))] = h;
 }
 
-// The bytes (0 or 1) of four map words as 16 bits (the product's bits 28..31
-// are bytes 0..3; its other bits never meet, so nothing carries).
-__device__ __forceinline__ uint32_t byte_bits(uint32_t x) { return (x * 0x10204080u) >> 28; }
-__device__ __forceinline__ uint32_t byte_bits4(uint4 x) {
-    return byte_bits(x.x) | (byte_bits(x.y) << 4) | (byte_bits(x.z) << 8) | (byte_bits(x.w) << 12);
-}
-
-// Emits the marked hubs of the maps (W hubs from vb) to row in rank order and
-// clears them (row null: only clears).  Warp w takes the w-th slice of the
-// byte map and of the bitmap; all byte-map hubs precede the bitmap's.
-__device__ void emit_maps(uint8_t* B, uint32_t vb, uint32_t W, uint32_t* row, int* sh) {
+// Emits the marked hubs of the map (W hubs from vb) to row in rank order and
+// clears them (row null: only clears).  Warp w takes the w-th slice.
+__device__ void emit_map(uint32_t* B, uint32_t vb, uint32_t W, uint32_t* row, int* sh) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-    uint4* b4 = reinterpret_cast<uint4*>(B);
-    uint4* w4 = reinterpret_cast<uint4*>(B + kByteHubs);
-    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-    const uint32_t Wb = min(W, (uint32_t)kByteHubs);
-    // units of 32 lanes x 16 bytes: 16 hubs per lane in the byte map, 128 in the bitmap
-    const int ub = (int)((Wb + 511) / 512), uw = (int)((W - Wb + 4095) / 4096);
-    const int b0 = ub * wid / nw, b1 = ub * (wid + 1) / nw, w0 = uw * wid / nw, w1 = uw * (wid + 1) / nw;
-    int cb = 0, cw = 0;
-#pragma unroll 1
-    for (int u = b0; u < b1; ++u) {
-        const uint4 x = b4[32 * u + lane];
-        cb += __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);  // one bit per marked byte
-    }
+    uint4* w4 = reinterpret_cast<uint4*>(B);
+    // units of 32 lanes x 16 bytes (128 hubs per lane)
+    const int uw = (int)((W + 4095) / 4096);
+    const int w0 = uw * wid / nw, w1 = uw * (wid + 1) / nw;
+    int cw = 0;
 #pragma unroll 1
     for (int u = w0; u < w1; ++u) {
         const uint4 x = w4[32 * u + lane];
         cw += __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);
     }
-    cb = warp_sum(cb);
     cw = warp_sum(cw);
-    if (lane == 0) {
-        sh[SH_WCNT + wid] = cb;
-        sh[SH_WCNT + nw + wid] = cw;
-    }
+    if (lane == 0) sh[SH_WCNT + wid] = cw;
     __syncthreads();
-    const int c = lane < 2 * nw ? sh[SH_WCNT + lane] : 0;
-    const int before = warp_incl_scan(c, lane) - c;
-    int pos = __shfl_sync(kFull, before, wid);
-    if (cb > 0) {
+    if (cw == 0) return;
+    const int c = lane < nw ? sh[SH_WCNT + lane] : 0;
+    int pos = __shfl_sync(kFull, warp_incl_scan(c, lane) - c, wid);
 #pragma unroll 1
-        for (int u = b0; u < b1; ++u) {
-            const int x = 32 * u + lane;
-            uint32_t w = byte_bits4(b4[x]);
-            if (!__any_sync(kFull, w != 0u)) continue;
-            const int k = __popc(w);
-            const int incl = warp_incl_scan(k, lane);
-            int o = pos + incl - k;
-            const uint32_t hb = vb - 1u + 16u * (uint32_t)x;
-            if (w) b4[x] = zero;
-            if (row)
-#pragma unroll 1
-                for (; w; w &= w - 1u) row[o++] = hb + (uint32_t)__ffs(w);
-            pos += __shfl_sync(kFull, incl, 31);
-        }
-    }
-    pos = __shfl_sync(kFull, before, nw + wid);
-    if (cw > 0) {
-#pragma unroll 1
-        for (int u = w0; u < w1; ++u) {
-            const int x = 32 * u + lane;
-            const uint4 y = w4[x];
-            if (!__any_sync(kFull, (y.x | y.y | y.z | y.w) != 0u)) continue;
-            const int k = __popc(y.x) + __popc(y.y) + __popc(y.z) + __popc(y.w);
-            const int incl = warp_incl_scan(k, lane);
-            int o = pos + incl - k;
-            if (k) w4[x] = zero;
-            if (row && k) {
-                const uint32_t q[4] = {y.x, y.y, y.z, y.w};
+    for (int u = w0; u < w1; ++u) {
+        const int x = 32 * u + lane;
+        const uint4 y = w4[x];
+        if (!__any_sync(kFull, (y.x | y.y | y.z | y.w) != 0u)) continue;
+        const int k = __popc(y.x) + __popc(y.y) + __popc(y.z) + __popc(y.w);
+        const int incl = warp_incl_scan(k, lane);
+        int o = pos + incl - k;
+        if (k) w4[x] = make_uint4(0u, 0u, 0u, 0u);
+        if (row && k) {
+            const uint32_t q[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint32_t hb = vb - 1u + (uint32_t)kByteHubs + 128u * (uint32_t)x + 32u * (uint32_t)j;
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t hb = vb - 1u + 128u * (uint32_t)x + 32u * (uint32_t)j;
 #pragma unroll 1
-                    for (uint32_t w = q[j]; w; w &= w - 1u) row[o++] = hb + (uint32_t)__ffs(w);
-                }
+                for (uint32_t w = q[j]; w; w &= w - 1u) row[o++] = hb + (uint32_t)__ffs(w);
             }
-            pos += __shfl_sync(kFull, incl, 31);
         }
+        pos += __shfl_sync(kFull, incl, 31);
     }
 }
 
-// The marked hubs of the maps (W of them) OR-ed into a split receiver's global
-// bitmap; the maps are left empty.
-__device__ void flush_maps(uint8_t* B, uint32_t W, uint32_t* gbits) {
-    uint4* b4 = reinterpret_cast<uint4*>(B);
-    uint32_t* bits = reinterpret_cast<uint32_t*>(B + kByteHubs);
-    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-    constexpr int kByteWords = kByteHubs / 32;
+// The marked hubs of the map (W of them) OR-ed into a split receiver's global
+// bitmap; the map is left empty.
+__device__ void flush_map(uint32_t* B, uint32_t W, uint32_t* gbits) {
 #pragma unroll 1
     for (int q = threadIdx.x; q < (int)((W + 31u) >> 5); q += blockDim.x) {
-        uint32_t w;
-        if (q < kByteWords) {
-            w = byte_bits4(b4[2 * q]) | (byte_bits4(b4[2 * q + 1]) << 16);
-            if (w) b4[2 * q] = b4[2 * q + 1] = zero;
-        } else {
-            w = bits[q - kByteWords];
-            if (w) bits[q - kByteWords] = 0u;
-        }
+        const uint32_t w = B[q];
+        if (w) B[q] = 0u;
         // (most of it is there already once a few parts have been merged)
         if (w & ~__ldcg(gbits + q)) atomicOr(gbits + q, w);
     }
 }
 
-// The maps of a split receiver from its global bitmap, which is left empty.
-__device__ void load_maps(uint8_t* B, uint32_t W, uint32_t* gbits) {
-    uint32_t* b1 = reinterpret_cast<uint32_t*>(B);
-    uint32_t* bits = reinterpret_cast<uint32_t*>(B + kByteHubs);
-    constexpr int kByteWords = kByteHubs / 32;
+// The map of a split receiver from its global bitmap, which is left empty.
+__device__ void load_map(uint32_t* B, uint32_t W, uint32_t* gbits) {
 #pragma unroll 1
     for (int q = threadIdx.x; q < (int)((W + 31u) >> 5); q += blockDim.x) {
-        uint32_t w = __ldcg(gbits + q);
+        const uint32_t w = __ldcg(gbits + q);
         if (w == 0u) continue;
         gbits[q] = 0u;
-        if (q < kByteWords) {
-#pragma unroll 1
-            for (int k = 0; k < 8; ++k, w >>= 4) b1[8 * q + k] = ((w & 15u) * 0x00204081u) & 0x01010101u;
-        } else {
-            bits[q - kByteWords] = w;
-        }
+        B[q] = w;
     }
 }
 
 // One block per vertex, any size.  The candidates are processed in passes
 // over hub ranges [lo, hi): each pass gathers the messages of its range into
-// the hub maps (the first pass) and the shared-memory set (shrinking hi when
+// the hub map (the first pass) and the shared-memory set (shrinking hi when
 // the set would overflow) and checks them.
 //
 // What bounds it is latency: three blocks of 8 warps per SM wait on random
 // 32-byte sectors (masks, check records, probe tables) of arrays far larger
 // than L2, and one chunk of 32 candidates checked from end to end took 5,000
 // to 12,000 cycles although most of its candidates need one mask only.  So the
-// check is split: each warp takes units of the maps and of the set from a
+// check is split: each warp takes units of the map and of the set from a
 // shared counter, prunes them by the top-hub columns (64 candidates per lane:
 // testing one 32-byte mask per candidate, and listing candidates for it, took
 // 108 and 143 ms of warp time in rounds 2 and 3 of R-MAT 2^22), and runs
@@ -1037,9 +975,9 @@ __device__ void load_maps(uint8_t* B, uint32_t W, uint32_t* gbits) {
 // and spread over all warps.
 // L(v) is staged into the shared-memory map when it fits; otherwise it is
 // looked up in v's row of the global probe index.  Accepted hubs are marked in
-// the maps and leave them in rank order, so the new row needs no later sort.
+// the map and leave it in rank order, so the new row needs no later sort.
 __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32_t* S, uint32_t* M, uint32_t* C,
-                                uint8_t* B, uint32_t* gacc, int* sh, int* wsum, int* sex, int64_t* sst, int* hist,
+                                uint32_t* B, uint32_t* gacc, int* sh, int* wsum, int* sex, int64_t* sst, int* hist,
                                 uint32_t* tv, unsigned long long* cnt, uint32_t* gbits) {
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int lane = tid & 31, wid = tid >> 5, nw = nthr >> 5;
@@ -1082,18 +1020,15 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
     int64_t width = (int64_t)v - vb;
     uint32_t* hi_sm = reinterpret_cast<uint32_t*>(&sh[SH_HI]);
     // hubs below vb + W (the most frequent messages) are deduplicated in the
-    // maps, in the first pass
-    const uint32_t W = min((uint32_t)(kByteHubs + kBitHubs), (uint32_t)v - vb);
-    const uint32_t Wb = min(W, (uint32_t)kByteHubs);
-    uint4* b4 = reinterpret_cast<uint4*>(B);
-    uint32_t* bits = reinterpret_cast<uint32_t*>(B + kByteHubs);
+    // map, in the first pass
+    const uint32_t W = min((uint32_t)kMapHubs, (uint32_t)v - vb);
     uint32_t* surv = S + wid * kWarpStage;  // (S is free once compacted)
     uint32_t cwords;
     const uint32_t* cols = columns_of(p.cols_h, vb, &cwords);
     const int imax = min((int)d - 1, kTopLevels);
 #pragma unroll 1
     while (lo < (uint32_t)v) {
-        if (lo > vb || (uint32_t)v - vb > W) {  // (no message reaches the set when the maps hold every hub of v)
+        if (lo > vb || (uint32_t)v - vb > W) {  // (no message reaches the set when the map holds every hub of v)
             uint4* s4 = reinterpret_cast<uint4*>(S);
 #pragma unroll 1
             for (int s = tid; s < S_CAP / 4; s += nthr) s4[s] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
@@ -1108,19 +1043,18 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
         }
         __syncthreads();
         if (gbits)
-            load_maps(B, W, gbits);
+            load_map(B, W, gbits);
         else
             gather_block(p, nb, ne, lo, hi_sm, B, vb, W, S, log_s, useM ? M : nullptr, log_m, limit, &sh[SH_UNIQ],
                          (volatile int*)&sh[SH_OVF], wsum, sex, sst, C, hist, &sh[SH_TMP], cnt[1]);
         __syncthreads();
         const uint32_t hi = *(volatile uint32_t*)hi_sm;
         const bool maps = lo == vb;
-        if (maps) {  // first pass: drop L(v)'s hubs from the maps
+        if (maps) {  // first pass: drop L(v)'s hubs from the map
 #pragma unroll 1
             for (int64_t j = tid; j < ll; j += nthr) {
                 const uint32_t w = hub_of(lv[j]) - vb;
-                if (w < Wb) B[w] = 0;
-                else if (w < W) atomicAnd(&bits[(w - kByteHubs) >> 5], ~(1u << (w & 31)));
+                if (w < W) atomicAnd(&B[w >> 5], ~(1u << (w & 31)));
             }
         }
         // compact the set into C (any order)
@@ -1177,7 +1111,7 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
         // entries of L(v) with a top hub (the checks' side B starts past them)
         const int lv_top = (int)lower_bound_u32(lvp, ll, pack(vb + (uint32_t)kTopHubs, 0));
         const int nc_set = min(*(volatile int*)&sh[SH_NC], limit);  // candidates from the set
-        // units: 2,048 hubs of the maps (64 per lane, cleared as they are read),
+        // units: 2,048 hubs of the map (64 per lane, cleared as they are read),
         // pruned by the receiver's rows of the top-hub columns, or 32 of the
         // set's candidates, pruned by their own masks.  The warps take them from
         // a shared counter and check full warps of survivors
@@ -1209,19 +1143,11 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
                     more = false;
                 } else if (u < um) {
                     const int x = 64 * u + 2 * lane;  // first of the lane's two words, as bits
-                    if (x < kByteHubs / 32) {
-                        uint4* q = b4 + 2 * x;
-                        const uint4 y0 = q[0], y1 = q[1], y2 = q[2], y3 = q[3];
-                        c0 = byte_bits4(y0) | (byte_bits4(y1) << 16);
-                        c1 = byte_bits4(y2) | (byte_bits4(y3) << 16);
-                        if (c0 | c1) q[0] = q[1] = q[2] = q[3] = make_uint4(0u, 0u, 0u, 0u);
-                    } else {
-                        uint2* q = reinterpret_cast<uint2*>(bits + (x - kByteHubs / 32));
-                        const uint2 y = *q;
-                        c0 = y.x;
-                        c1 = y.y;
-                        if (c0 | c1) *q = make_uint2(0u, 0u);
-                    }
+                    uint2* q = reinterpret_cast<uint2*>(B + x);
+                    const uint2 y = *q;
+                    c0 = y.x;
+                    c1 = y.y;
+                    if (c0 | c1) *q = make_uint2(0u, 0u);
                     hb = vb + 32u * (uint32_t)x;
                     if (!__any_sync(kFull, (c0 | c1) != 0u)) continue;
                     const int found = __popc(c0) + __popc(c1);
@@ -1230,7 +1156,7 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
                         for (int b = 0; b < 64; ++b)
                             if (((b < 32 ? c0 : c1) >> (b & 31)) & 1u)
                                 count_reads(p.loff_h, lvp, ll, hb + (uint32_t)b, cnt + 8);
-                    // (x < the row's words: hubs of v's graph within the maps,
+                    // (x < the row's words: hubs of v's graph within the map,
                     // rounded up to 128; rows are 16-byte aligned)
                     const uint32_t* cx = cols + min((uint32_t)x, cwords - 2u);
 #pragma unroll 1
@@ -1294,8 +1220,8 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
         width = 2 * (int64_t)(hi - lo);
         lo = hi;
     }
-    // the new row: the maps' hubs in rank order, then the set's (all of them
-    // past the maps), sorted in shared memory (more than the set's slots hold:
+    // the new row: the map's hubs in rank order, then the set's (all of them
+    // past the map), sorted in shared memory (more than the set's slots hold:
     // listed for the row sort)
     const int macc = *(volatile int*)&sh[SH_MACC], sacc = *(volatile int*)&sh[SH_ACC];
     const int64_t total_acc = (int64_t)macc + sacc;
@@ -1311,7 +1237,7 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
         const bool fits = start + row_pad(total_acc) <= p.fcap;
         uint32_t* row = p.fhub_new + start;
         if (fits && total_acc + tid < row_pad(total_acc)) row[total_acc + tid] = kEmpty;
-        if (macc > 0) emit_maps(B, vb, W, fits ? row : nullptr, sh);
+        if (macc > 0) emit_map(B, vb, W, fits ? row : nullptr, sh);
         if (fits) {
             const bool sorted = sacc <= S_CAP;
             if (sacc > 1 && sorted) {
@@ -1351,16 +1277,16 @@ __global__ void __launch_bounds__(256, 3) k_gp_block(GpParams p) {
     uint32_t* S = reinterpret_cast<uint32_t*>(sst + blockDim.x);
     uint32_t* M = S + (1 << p.log_s);
     uint32_t* C = M + (1 << p.log_m);
-    uint8_t* B = reinterpret_cast<uint8_t*>(C + p.cand_limit + (int)blockDim.x);  // kMapWords words
+    uint32_t* B = C + p.cand_limit + (int)blockDim.x;  // kMapWords words
     uint32_t* gacc = p.gscratch + (int64_t)blockIdx.x * p.gscratch_words;
     unsigned long long cnt[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     if (p.ctr->done) return;
     const uint32_t d = p.ctr->d;
     const int n1 = *p.list_n, np = p.split.max > 0 ? min(p.ctr->nP, p.split.max_parts) : 0;
     if ((int)blockIdx.x >= np + n1) return;  // (as many blocks as entries are enough)
-    // the hub maps are empty between vertices
+    // the hub map is empty between vertices
 #pragma unroll 1
-    for (int q = threadIdx.x; q < kMapWords; q += blockDim.x) reinterpret_cast<uint32_t*>(B)[q] = 0u;
+    for (int q = threadIdx.x; q < kMapWords; q += blockDim.x) B[q] = 0u;
     // parts of split receivers first, then the list's vertices (in rank order:
     // the largest first), handed out one at a time
     int next = 0;
@@ -1378,7 +1304,7 @@ __global__ void __launch_bounds__(256, 3) k_gp_block(GpParams p) {
             const int2 part = p.split.parts[i];
             v = p.split.v[part.x];
             gbits = p.split.bits + (int64_t)part.x * p.split.words;
-            const uint32_t vb = base_of(p.vbase, v), W = (uint32_t)v - vb;  // (all of v's hubs fit the maps)
+            const uint32_t vb = base_of(p.vbase, v), W = (uint32_t)v - vb;  // (all of v's hubs fit the map)
             const int64_t nb = p.roff[v] + (int64_t)part.y * kSplitPart;
             const int64_t ne = min(p.roff[v + 1], nb + kSplitPart);
             uint32_t* hi_sm = reinterpret_cast<uint32_t*>(&sh[SH_HI]);
@@ -1391,7 +1317,7 @@ __global__ void __launch_bounds__(256, 3) k_gp_block(GpParams p) {
             gather_block(p, nb, ne, vb, hi_sm, B, vb, W, S, p.log_s, nullptr, 0, p.cand_limit, &sh[SH_UNIQ],
                          (volatile int*)&sh[SH_OVF], wsum, sex, sst, C, hist, &sh[SH_TMP], cnt[1]);
             __syncthreads();
-            flush_maps(B, W, gbits);
+            flush_map(B, W, gbits);
             __threadfence();
             __syncthreads();
             if (threadIdx.x == 0) {

@@ -116,12 +116,30 @@ inline int pow2_at_least(int64_t x) {
 // carves it up: scalars (48 words) + warp sums (34, padded to 36) + histogram
 // (256) + top-hub masks + prefix per thread + 64-bit row start per thread + set
 // (also kWarpStage per warp of staged candidates) + map + candidate list
-// (limit + 32 per warp) + hub maps.  The masks, the set and the hub maps are
+// (limit + 32 per warp) + hub map.  The masks, the set and the hub map are
 // read as 16-byte words.
 inline size_t gp_block_smem_bytes(int bthr, int log_s, int log_m, int cand_limit) {
     return sizeof(uint32_t) * (48 + 36 + 256 + kTopRow + (size_t)((bthr + 4) & ~3) + 2 * (size_t)bthr +
                                ((size_t)1 << log_s) + ((size_t)1 << log_m) + (size_t)cand_limit + (size_t)bthr +
                                kMapWords);
+}
+
+// Warp tier: words per warp for the set (2^log_s slots), the candidates and the
+// top-hub masks, which lie in the set's last words: for the default options
+// three blocks then take 196 KB of an SM's 256, as the block tier's do (with the
+// masks beside the set 198: see kMapHubs).  Small sets keep all their slots for
+// candidates.
+inline int warp_set_words(int log_s) { return log_s >= 10 ? 1 << log_s : (1 << log_s) + kTopRow; }
+inline size_t gp_warp_smem_bytes(int warps, int log_s, int log_m) {
+    return sizeof(uint32_t) * (size_t)warps * (4 + (size_t)warp_set_words(log_s) + ((size_t)1 << log_m));
+}
+
+// Whether the tables of the options fit: the bounds are those of the larger
+// layouts that the options were specified with (a hub map of 32 KB, masks beside
+// the set).
+inline bool tiers_fit(int warps, int w_log_s, int w_log_m, size_t b_smem) {
+    const size_t w = sizeof(uint32_t) * (size_t)warps * (4 + kTopRow + ((size_t)1 << w_log_s) + ((size_t)1 << w_log_m));
+    return w <= 227 * 1024 && b_smem - sizeof(uint32_t) * kMapWords + 32768 <= 227 * 1024;
 }
 
 // Lists and bitmaps of the split receivers of a build over n vertices (the
@@ -134,7 +152,7 @@ inline SplitLists split_lists(DevPool& pool, int64_t n, int64_t max_part_n, int6
     if (most <= 0 || n <= 0) return l;
     l.max = (int)most;
     l.max_parts = (int)(nnz / kSplitPart + most);
-    l.words = (int)((std::min<int64_t>(max_part_n, kByteHubs + kBitHubs) + 31) / 32);
+    l.words = (int)((std::min<int64_t>(max_part_n, kMapHubs) + 31) / 32);
     l.v = pool.alloc<int32_t>(most);
     l.nparts = pool.alloc<int>(most);
     l.done = pool.alloc<int>(most);
@@ -199,10 +217,10 @@ inline cudaError_t launch_tiers(GpParams w, GpParams b, const SplitLists& split,
     return cudaGetLastError();
 }
 
-// Block tier, per block: accepted hubs past the maps (those within them stay
+// Block tier, per block: accepted hubs past the map (those within it stay
 // marked there).
 inline int64_t accepted_words(int64_t max_part_n) {
-    return std::max<int64_t>(max_part_n - (kByteHubs + kBitHubs), 1);
+    return std::max<int64_t>(max_part_n - kMapHubs, 1);
 }
 
 // The top-hub columns of a graph of n vertices, empty (quads: the words per row,

@@ -11,7 +11,7 @@
 //                  L(v) staged hub-keyed in shared memory (the gather of
 //                  Alg. 3: unique messages, then d < min over common hubs).
 //   k_gp_block     the same with one vertex per block (any size: hub-range
-//                  passes, a byte map for the top hubs).
+//                  passes, a bitmap for the top hubs).
 //   k_sort_rows_*  rows of the new frontier that were written unsorted (round
 //                  1; the block tier's) sorted by hub rank (the warp tier
 //                  writes its rows sorted);
@@ -68,11 +68,11 @@ struct RoundStat {
 };
 
 // Receivers with many arcs (hubs) are split: blocks gather parts of kSplitPart
-// arcs into shared-memory maps and OR these into the receiver's global bitmap;
+// arcs into shared-memory bitmaps and OR these into the receiver's global bitmap;
 // the block that ends last goes on with the merged bitmap.  No block waits for
 // another.  (One block takes 4 to 5 us per 256 arcs of dependent loads: a hub
 // with 209,550 arcs kept a round from ending for up to 4 ms.)  Only for
-// receivers whose hubs all fit the maps.
+// receivers whose hubs all fit the map.
 constexpr int kSplitArcs = 2048;   // arcs from which a receiver is split
 constexpr int kSplitPart = 1024;   // arcs per part
 constexpr int kMaxSplit = 512;     // split receivers per round (further ones are not split)
@@ -86,9 +86,9 @@ struct SplitLists {
 };
 
 // The top-hub masks by hub instead of by vertex: per graph, level t and top hub
-// w a row of bits over the graph's first vertices (those the block tier's maps
+// w a row of bits over the graph's first vertices (those the block tier's map
 // hold), bit x: w in L(x) at distance <= t.  A receiver prunes the candidates
-// in its maps 64 per lane and row: OR of the rows of its own top hubs.
+// in its map 64 per lane and row: OR of the rows of its own top hubs.
 struct TopColumns {
     uint32_t* bits;       // rows (t, w) of 4 one.y words each, from 4 x kTopRows x one.x words on
     const int2* by_base;  // disjoint union: {x, y} of each graph, at the index of its first rank; else null
@@ -114,6 +114,7 @@ struct GpParams {
     RoundCounters* ctr;        // also holds the round number d (ctr->d)
     int log_s, log_m;          // table sizes (log2 slots): candidate set, L(v) map (block tier: largest)
     int cand_limit;            // max unique candidates per pass (power of two)
+    int s_words;               // warp tier: words per warp of the set, the candidates and the top-hub masks
     uint32_t* gscratch;        // block tier: per-block buffer of accepted hubs
     int64_t gscratch_words;    // words per block
     const uint64_t* hdesc;     // probe index of L: per row (table start << 8 | log2 slots), 0 = no table
@@ -141,7 +142,7 @@ struct GpParams {
                                // the sending vertex (weighted rounds), or 0: the vertex itself
     TopColumns cols_h;         // the candidates' side's top-hub masks by hub
     const int32_t* vbase;      // per vertex: first rank of its graph in a disjoint union, or null (one graph:
-                               // 0).  The top hubs and the byte map are those of the vertex's own graph
+                               // 0).  The top hubs and the maps are those of the vertex's own graph
     int count_check;           // 1: count the label entries each check would read by the paper's cost
                                // model (RoundCounters::chk_lv / chk_lh; one binary search per candidate)
 };
@@ -186,19 +187,23 @@ constexpr int kRowAlign = 8;
 __host__ __device__ __forceinline__ int64_t row_pad(int64_t c) { return (c + kRowAlign - 1) & ~(int64_t)(kRowAlign - 1); }
 
 // Block tier: the highest-ranked hubs (of the vertex's graph) are deduplicated
-// in shared-memory maps instead of the hash set: the first kByteHubs in a byte
-// map (plain stores: a row's hubs crowd into few words there, which would
-// serialise atomics), the next kBitHubs in a bitmap (shared-memory atomicOr).
-// On R-MAT 2^22 28% of round 3's messages and 32% of its candidates rank past
-// 32,768, 1.6% and 2% past 131,072: a 32 KB byte map of 32,768 hubs left them
-// to the set; 16 KB of bytes and 16 KB of bits cover 147,456.  Every receiver
-// of the block tier uses them (only those with 2,048 candidates or more, the
-// others hashing: R-MAT 2^22 741 instead of 722 ms, directed R-MAT 2^20 125
-// instead of 119 ms).
-constexpr int kByteHubs = 16384;
-constexpr int kBitHubs = 131072;
-constexpr int kMapWords = kByteHubs / 4 + kBitHubs / 32;
-static_assert(kByteHubs % 512 == 0 && kBitHubs % 4096 == 0 && kByteHubs % 2048 == 0, "whole scan units");
+// in a shared-memory bitmap instead of the hash set.  On R-MAT 2^22 28% of round
+// 3's messages and 32% of its candidates rank past 32,768, 1.6% and 2% past
+// 131,072.  Every receiver of the block tier uses it (only those with 2,048
+// candidates or more, the others hashing: R-MAT 2^22 741 instead of 722 ms).
+// What shared memory leaves is the L1 cache, which the checks' masks, records
+// and probe tables pass through: three blocks of either tier take 196 KB (a
+// carve-out the SM offers; the next is 228) of its 256, so 60 KB are cache
+// instead of 28.  Both have to: the tiers run side by side, and an SM keeps one
+// carve-out for both (the block tier alone at 196 left R-MAT 2^22 at 616 ms when
+// it ran beside the warp tier, 553 without).  16 KB of bytes (plain stores) for
+// the first 16,384 hubs and 16 KB of bits for the next 131,072, at 228 KB, took
+// 618 ms on R-MAT 2^22, 100 on directed R-MAT 2^20, 24.2 on Chung-Lu 2^20; this
+// bitmap 535, 96 and 23.6 (131,072 or 196,608 hubs: within 1%; both tiers within
+// 164 KB, by shorter candidate lists in the warp tier: 547, 104, 23.4).
+constexpr int kMapHubs = 147456;
+constexpr int kMapWords = kMapHubs / 32;
+static_assert(kMapHubs % 4096 == 0, "whole scan units");
 // Block tier, per warp: survivors of the first prefilter step (fewer than 32,
 // plus 32 of one extraction).
 constexpr int kWarpStage = 64;
@@ -226,7 +231,7 @@ __device__ __forceinline__ uint32_t* columns_of(const TopColumns& c, uint32_t vb
 }
 // Words per row, in units of 4, for a graph of n vertices.
 __host__ __device__ __forceinline__ int column_quads(int64_t n) {
-    const int64_t m = n < kByteHubs + kBitHubs ? n : kByteHubs + kBitHubs;
+    const int64_t m = n < kMapHubs ? n : kMapHubs;
     return (int)((m + 127) / 128);
 }
 __global__ void k_pack_hrec(const int64_t* loff, const uint32_t* lent, const uint64_t* hdesc, const int32_t* vbase,

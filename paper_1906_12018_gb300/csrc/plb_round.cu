@@ -244,7 +244,7 @@ __global__ void k_collect(unsigned long long* recv, const int64_t* roff, const i
             const int64_t ll = loff[v + 1] - loff[v];
             const int64_t deg = roff[v + 1] - roff[v];
             tier = ((int64_t)bound <= lim.warp_bound && ll <= lim.warp_label && deg <= lim.warp_deg) ? 0 : 1;
-            if (deg > kSplitArcs && below <= (unsigned long long)(kByteHubs + kBitHubs) && split.max > 0) {
+            if (deg > kSplitArcs && below <= (unsigned long long)kMapHubs && split.max > 0) {
                 const int np = (int)((deg + kSplitPart - 1) / kSplitPart);
                 const int g = atomicAdd(&ctr->nG, 1);
                 if (g < split.max) {
@@ -912,7 +912,7 @@ __global__ void __launch_bounds__(256) k_top_columns(const uint32_t* top, int64_
         const int64_t v = 32 * g + lane;
         const uint32_t vb = v < n ? base_of(vbase, v) : 0u;
         const uint32_t rel = (uint32_t)v - vb;
-        unsigned starts = __ballot_sync(kFull, v < n && (rel & 127u) == 0u && rel < (uint32_t)(kByteHubs + kBitHubs));
+        unsigned starts = __ballot_sync(kFull, v < n && (rel & 127u) == 0u && rel < (uint32_t)kMapHubs);
         while (starts) {
             const int k = __ffs(starts) - 1;
             starts &= starts - 1u;

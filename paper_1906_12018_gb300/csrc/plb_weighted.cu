@@ -347,8 +347,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     const int w_log_s = ceil_log2_i64(2 * (int64_t)warp_cand);
     const int w_log_m = ceil_log2_i64(2 * warp_label);
     const int warps_per_block = kGpWarpThreads / 32;
-    const size_t w_smem = sizeof(uint32_t) * (4 * warps_per_block +
-                                              (size_t)warps_per_block * (kTopRow + (1 << w_log_s) + (1 << w_log_m)));
+    const size_t w_smem = gp_warp_smem_bytes(warps_per_block, w_log_s, w_log_m);
     const int bthr = std::min(256, std::max(64, (o.block_threads / 32) * 32));
     const int block_cand = pow2_at_least(std::max(bthr, o.block_cand_cap));
     const int b_log_s = ceil_log2_i64(std::max<int64_t>(
@@ -360,7 +359,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     lim.warp_bound = 2 * (int64_t)warp_cand;
     lim.warp_label = warp_label;
     lim.warp_deg = (int64_t)32 * 64;
-    if (w_smem > 227 * 1024 || b_smem > 227 * 1024) return PLB_ERR_INVALID;
+    if (!tiers_fit(warps_per_block, w_log_s, w_log_m, b_smem)) return PLB_ERR_INVALID;
     PLB_CK(cudaFuncSetAttribute(k_gp_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w_smem));
     PLB_CK(cudaFuncSetAttribute(k_gp_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b_smem));
     PLB_CK(cudaFuncSetAttribute(k_sort_rows_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -431,6 +430,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
         p.log_s = w_log_s;
         p.log_m = w_log_m;
         p.cand_limit = warp_cand;
+        p.s_words = warp_set_words(w_log_s);
         p.stage_ratio = o.warp_stage_ratio;
         p.count_check = o.profile != 0;
         p.unsorted = U;

@@ -35,10 +35,10 @@ def test_union_parts_around_the_top_hub_count(opts):
                                    "block_label_cap": 24, "block_threads": 64}], ids=["host", "graph", "block tier"])
 @pytest.mark.parametrize("n,deg", [(2500, 40), (1500, 400)], ids=["sparse", "dense"])
 def test_hubs_around_the_map_boundaries(n, deg, lead, opts):
-    """The highest-ranked hubs are marked in byte maps and bitmaps, the others
-    go into hash sets.  `lead` isolated vertices ranked first move a small
-    graph's hubs to the boundaries: the top-hub masks (256), the block tier's
-    byte map (16,384) and bitmap (147,456), the warp tier's bitmap (32,768)."""
+    """The highest-ranked hubs are marked in bitmaps, the others go into hash
+    sets.  `lead` isolated vertices ranked first move a small graph's hubs to
+    the boundaries: the top-hub masks (256), the block tier's bitmap (147,456),
+    the warp tier's (32,768), and a rank between."""
     core = G.chung_lu_graph(n, deg, 2.2, 9)
     src = np.repeat(np.arange(core.n), np.diff(core.off))
     g = G.clean_csr(core.n + lead, src.astype(np.int32) + lead, core.col.astype(np.int32) + lead)
@@ -48,6 +48,31 @@ def test_hubs_around_the_map_boundaries(n, deg, lead, opts):
     assert_labels_equal(lab, O.pll(g.off, g.col, order), f"lead {lead}")
     if lead > 4096 and deg == 400:  # (with few ranks the candidate bounds stay within the warp tier)
         assert lab.stats()["tier_vertices"][1] > 0
+
+
+@pytest.mark.parametrize("lead", [0, 32768 - 700, 32768 - 300], ids=["bitmap", "both", "set"])
+@pytest.mark.parametrize("opts", [{}, {"use_graph": 1}, {"warp_cand_cap": 32}], ids=["host", "graph", "small"])
+def test_candidate_counts_around_the_warp_tiers_list(opts, lead):
+    """Receivers of k candidates each, none with a witness, around the
+    capacity of the warp tier's list (968, and 64 for the smallest option) and
+    its bound (1,024 and 64): `lead` ranks before the hubs move all but the
+    first of them past the bitmap (32,768), where the set holds 512 and 32."""
+    counts = [31, 32, 33, 63, 64, 65, 500, 512, 513, 967, 968, 969, 1000, 1023, 1024, 1025]
+    hubs, senders = 1025, 16
+    src, dst = [], []
+    for q, k in enumerate(counts):
+        v = hubs + len(counts) * senders + q
+        for s in range(senders):
+            a = hubs + senders * q + s
+            mine = np.arange(s, k, senders)
+            src += [mine, [a]]
+            dst += [np.full(len(mine), a), [v]]
+    n = lead + hubs + len(counts) * (senders + 1)
+    g = G.clean_csr(n, (np.concatenate(src) + lead).astype(np.int32), (np.concatenate(dst) + lead).astype(np.int32))
+    order = np.arange(n, dtype=np.int32)
+    rp, col, o = to_device(g, order)
+    lab = plb.build(rp, col, o, **opts)
+    assert_labels_equal(lab, O.pll(g.off, g.col, order), f"lead {lead}")
 
 
 def hub_edges(leaves, arcs, seed):
