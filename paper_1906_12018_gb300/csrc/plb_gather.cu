@@ -648,10 +648,17 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
         const int words = (int)((top + 31u) >> 5);
         int nbm = 0, nset = 0;
         if (ok) {
+            // (four loads in flight, here and where the map is staged: one at a
+            // time, each waited for, weighted Chung-Lu 2^20 took 56.0 ms instead
+            // of 54.1, the batch of 200 graphs 49.1 instead of 47.7)
 #pragma unroll 1
-            for (int64_t j = lane; j < ll; j += 32) {
-                const uint32_t w = hub_of(lv[j]) - vb;
-                if (w < top) atomicAnd(&X[w >> 5], ~(1u << (w & 31)));
+            for (int j = lane; j < (int)ll; j += 128) {
+                uint32_t w[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) w[q] = j + 32 * q < (int)ll ? hub_of(lv[j + 32 * q]) - vb : kEmpty;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (w[q] < top) atomicAnd(&X[w[q] >> 5], ~(1u << (w[q] & 31)));
             }
             __syncwarp();
             // ... and the set's, compacted in place (write position never
@@ -781,10 +788,16 @@ __global__ void __launch_bounds__(256, 3) k_gp_warp(GpParams p) {
         }
         if (!mglob || copy) {
 #pragma unroll 1
-            for (int64_t j = lane; j < ll; j += 32) {
-                const uint32_t e = lv[j];
-                if (!mglob) map_insert(X, log_m, e);
-                if (copy) lvs[j] = e;
+            for (int j = lane; j < (int)ll; j += 128) {
+                uint32_t e[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) e[q] = j + 32 * q < (int)ll ? lv[j + 32 * q] : kEmpty;
+#pragma unroll 1
+                for (int q = 0; q < 4; ++q, e[0] = e[1], e[1] = e[2], e[2] = e[3]) {
+                    if (j + 32 * q >= (int)ll) break;
+                    if (!mglob) map_insert(X, log_m, e[0]);
+                    if (copy) lvs[j + 32 * q] = e[0];
+                }
             }
         }
         if (lane == 0) c_staged += mglob ? 0 : ll;
