@@ -142,6 +142,25 @@ inline bool tiers_fit(int warps, int w_log_s, int w_log_m, size_t b_smem) {
     return w <= 227 * 1024 && b_smem - sizeof(uint32_t) * kMapWords + 32768 <= 227 * 1024;
 }
 
+// Tier of a receiver.  The bound counts messages; the candidates, which have to
+// fit the warp tier's list (968 for the default 512), are fewer, by 2 to 5 times
+// on power-law graphs, and a receiver with more goes on to the block tier.  With
+// the bound at 2 x warp_cand the block tier took receivers that a warp finishes
+// sooner than a block starts; with long rows L(v) a warp does less well (staging
+// them, and no pruning by columns).  2 | 3 | 4 | 8 x warp_cand | the rule below, ms:
+// Chung-Lu 2^20 23.4 | 22.2 | 21.9 | 22.0 | 21.8; batch of 200 graphs 47.7 |
+// 46.2 | 45.5 | 45.6 | 45.6; directed R-MAT 2^20 95.8 | 93.4 | 94.4 | 98.7 | 93.4;
+// R-MAT 2^22 535.6 | 536 | 538 | 545 | 537; 1.5 x: 25.1, 49.3, 100.6, 547.
+inline TierLimits tier_limits(int warp_cand, int warp_label) {
+    TierLimits lim;
+    lim.warp_bound = 5 * (int64_t)warp_cand / 2;
+    lim.short_bound = 4 * (int64_t)warp_cand;
+    lim.short_label = 128;
+    lim.warp_label = warp_label;
+    lim.warp_deg = (int64_t)32 * 64;
+    return lim;
+}
+
 // Lists and bitmaps of the split receivers of a build over n vertices (the
 // largest graph of a union: max_part_n) and nnz arcs.  A receiver is split from
 // kSplitArcs arcs on, so at most nnz / kSplitArcs receivers are, and their

@@ -240,6 +240,8 @@ __global__ void k_pack_hrec(const int64_t* loff, const uint32_t* lent, const uin
 // Routing limits of k_collect (see the tier geometry in build_core).
 struct TierLimits {
     int64_t warp_bound;   // candidate bound up to which the warp tier is tried
+    int64_t short_bound;  // the same with |L(v)| <= short_label
+    int64_t short_label;
     int64_t warp_label;   // largest |L(v)| of the warp tier
     int64_t warp_deg;     // largest degree of the warp tier
 };

@@ -243,7 +243,8 @@ __global__ void k_collect(unsigned long long* recv, const int64_t* roff, const i
             rbound[v] = (uint32_t)bound;  // v < 2^24
             const int64_t ll = loff[v + 1] - loff[v];
             const int64_t deg = roff[v + 1] - roff[v];
-            tier = ((int64_t)bound <= lim.warp_bound && ll <= lim.warp_label && deg <= lim.warp_deg) ? 0 : 1;
+            tier = ((int64_t)bound <= (ll <= lim.short_label ? lim.short_bound : lim.warp_bound) &&
+                    ll <= lim.warp_label && deg <= lim.warp_deg) ? 0 : 1;
             if (deg > kSplitArcs && below <= (unsigned long long)kMapHubs && split.max > 0) {
                 const int np = (int)((deg + kSplitPart - 1) / kSplitPart);
                 const int g = atomicAdd(&ctr->nG, 1);

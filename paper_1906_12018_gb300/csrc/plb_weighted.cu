@@ -355,10 +355,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
         (int64_t)kWarpStage * (bthr / 32)));
     const int b_log_m = ceil_log2_i64(2 * (int64_t)std::max(o.block_label_cap, 64) + 2 * bthr);
     const size_t b_smem = gp_block_smem_bytes(bthr, b_log_s, b_log_m, block_cand);
-    TierLimits lim;
-    lim.warp_bound = 2 * (int64_t)warp_cand;
-    lim.warp_label = warp_label;
-    lim.warp_deg = (int64_t)32 * 64;
+    const TierLimits lim = tier_limits(warp_cand, warp_label);
     if (!tiers_fit(warps_per_block, w_log_s, w_log_m, b_smem)) return PLB_ERR_INVALID;
     PLB_CK(cudaFuncSetAttribute(k_gp_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w_smem));
     PLB_CK(cudaFuncSetAttribute(k_gp_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b_smem));

@@ -55,10 +55,10 @@ def test_hubs_around_the_map_boundaries(n, deg, lead, opts):
 def test_candidate_counts_around_the_warp_tiers_list(opts, lead):
     """Receivers of k candidates each, none with a witness, around the
     capacity of the warp tier's list (968, and 64 for the smallest option) and
-    its bound (1,024 and 64): `lead` ranks before the hubs move all but the
+    the bounds up to which it is tried: `lead` ranks before the hubs move all but the
     first of them past the bitmap (32,768), where the set holds 512 and 32."""
-    counts = [31, 32, 33, 63, 64, 65, 500, 512, 513, 967, 968, 969, 1000, 1023, 1024, 1025]
-    hubs, senders = 1025, 16
+    counts = [31, 32, 33, 63, 64, 65, 80, 81, 128, 129, 512, 513, 967, 968, 969, 1024, 1025, 1280, 1281, 2048, 2049]
+    hubs, senders = 2049, 16
     src, dst = [], []
     for q, k in enumerate(counts):
         v = hubs + len(counts) * senders + q
