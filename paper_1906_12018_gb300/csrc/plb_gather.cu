@@ -11,10 +11,12 @@
 // different places of these kernels, and code that outgrows the instruction
 // caches costs more than the loop control (see witness4).
 //
-// Measured, with hub maps, the two-step prefilter, the lane/group/warp checks
-// and the bucketed tables (before -> after, builds): R-MAT 2^22, 64M edges
-// 1,213 -> 834 ms; Chung-Lu 2^20 39.1 -> 34.8 ms; directed R-MAT 2^20 185.9 ->
-// 140.9 ms.
+// Measured (builds, hash sets and one check of all candidates -> hub maps, the
+// two-step prefilter, the lane/group/warp checks and the bucketed tables -> with
+// frontier sectors, split hubs, top-hub columns, the cache's share of shared
+// memory and the warp tier's wider bound besides): R-MAT 2^22, 64M edges 1,213 ->
+// 834 -> 534 ms; Chung-Lu 2^20 39.1 -> 34.8 -> 21.7 ms; directed R-MAT 2^20
+// 185.9 -> 140.9 -> 91 ms.
 #include "plb_kernels.cuh"
 #include "plb_round.cuh"
 
@@ -592,8 +594,8 @@ __device__ __noinline__ void gather_block(const GpParams& p, int64_t nb, int64_t
 //     map M, in the bitmap's place (or, with few candidates against a long row,
 //     look L(v) up in v's row of the global probe index), and check them;
 //  4. append the accepted hubs to the new frontier: in order, the set's sorted.
-// A vertex with more than cand_limit candidates in the set goes to the block
-// tier.
+// A vertex with more than cand_limit candidates in the set, or more in all than
+// the list holds, goes to the block tier.
 // What bounds it is instruction issue (each of 24 independent warps per SM
 // issues every 12 cycles) and the instructions' way to the SM: the bitmap
 // replaced a hash set with a look-up in M per message, its compaction and a

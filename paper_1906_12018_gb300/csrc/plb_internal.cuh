@@ -192,7 +192,7 @@ struct TileScratch {
     int64_t r[2];
     int wmax[kTileThreads / 32];
 };
-__device__ __forceinline__ void tile_row_map(const int64_t* off, int64_t nrows, int64_t p0, int64_t p1, int* srow,
+__device__ __forceinline__ void tile_rows(const int64_t* off, int64_t nrows, int64_t p0, int64_t p1, int* srow,
                                              TileScratch* sh, int64_t* r0, int64_t* r1) {
     constexpr int kPer = kTileItems / kTileThreads;
     static_assert(kPer == 8, "eight items per thread");

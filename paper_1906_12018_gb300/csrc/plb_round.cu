@@ -39,7 +39,7 @@ __global__ void k_check_cols(const int64_t* row_ptr, const int32_t* col, int64_t
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
         int64_t r0, r1;
-        tile_row_map(row_ptr, n, p0, p1, srow, &sh, &r0, &r1);
+        tile_rows(row_ptr, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
             const int64_t u = r0 + srow[p - p0];
             const int32_t c = col[p];
@@ -101,7 +101,7 @@ __global__ void k_transpose(const int64_t* roff, const int32_t* rcol, int64_t n,
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
         int64_t r0, r1;
-        tile_row_map(roff, n, p0, p1, srow, &sh, &r0, &r1);
+        tile_rows(roff, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
             const int64_t u = r0 + srow[p - p0];
             const int32_t w = rcol[p];
@@ -132,7 +132,7 @@ __global__ void k_relabel(const int64_t* row_ptr, const int32_t* col, const int3
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
         int64_t r0, r1;
-        tile_row_map(roff, n, p0, p1, srow, &sh, &r0, &r1);
+        tile_rows(roff, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
             const int64_t r = r0 + srow[p - p0];
             const int32_t id = order[r];
@@ -203,7 +203,7 @@ __global__ void k_mark(const int64_t* roff, const int32_t* rcol, const uint64_t*
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(total, p0 + kTileItems);
         int64_t r0, r1;
-        tile_row_map(aoff, nA, p0, p1, srow, &sh, &r0, &r1);
+        tile_rows(aoff, nA, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
             const int64_t i = r0 + srow[p - p0];
             const int32_t a = A[i];
@@ -300,7 +300,7 @@ __global__ void k_round1_count(const int64_t* roff, const int32_t* rcol, int64_t
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
         int64_t r0, r1;
-        tile_row_map(roff, n, p0, p1, srow, &sh, &r0, &r1);
+        tile_rows(roff, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t q = p0; q < p1; q += blockDim.x) {  // uniform trip count: whole warps below
             const int64_t p = q + threadIdx.x;
             const bool ok = p < p1;
@@ -341,7 +341,7 @@ __global__ void k_round1(const int64_t* roff, const int32_t* rcol, int64_t n, in
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
         int64_t r0, r1;
-        tile_row_map(roff, n, p0, p1, srow, &sh, &r0, &r1);
+        tile_rows(roff, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t q = p0; q < p1; q += blockDim.x) {
             const int64_t p = q + threadIdx.x;
             const bool ok = p < p1;
@@ -452,7 +452,7 @@ __device__ __forceinline__ void build_table(const uint32_t* lent, int64_t lb, in
 // by the whole block in the eight warps' buffers together, and only those
 // that outgrow these too in place (atomics in global memory: with every
 // table beyond a warp's buffer built so, R-MAT 2^22's last rebuild, 1.7G labels
-// in rows of 720 on average, took 32.7 ms).
+// in rows of 720 on average, took 32.7 ms; the build 644 instead of 618).
 __global__ void __launch_bounds__(kIndexWarps * 32) k_index_build(const int64_t* loff, const uint32_t* lent,
                                                                   const int64_t* hoff, uint32_t* htab,
                                                                   uint64_t* hdesc, int64_t n, int slots,
@@ -576,8 +576,8 @@ __global__ void k_next_active(const int64_t* loff, const uint64_t* fse_new, int6
 }
 
 // ------------------------------------------------- sort new frontier rows
-// The gather/prune kernels append each vertex's accepted hubs unsorted; one
-// warp per active vertex sorts its row: up to 32 entries in registers (a
+// Round 1 appends each vertex's accepted hubs unsorted (and the block tier those
+// rows it has no room to sort); one warp per such vertex sorts its row: up to 32 entries in registers (a
 // bitonic network over the lanes), up to kWarpSortMax in shared memory;
 // longer rows are listed for k_sort_rows_block.
 constexpr int kWarpSortMax = 1024;

@@ -67,7 +67,7 @@ __global__ void k_check_weights(const int64_t* row_ptr, const int32_t* col, cons
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
         int64_t r0, r1;
-        tile_row_map(row_ptr, n, p0, p1, srow, &sh, &r0, &r1);
+        tile_rows(row_ptr, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
             const int64_t u = r0 + srow[p - p0];
             const int32_t c = col[p];
@@ -92,7 +92,7 @@ __global__ void k_relabel_weights(const int64_t* row_ptr, const uint8_t* wt, con
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
         int64_t r0, r1;
-        tile_row_map(roff, n, p0, p1, srow, &sh, &r0, &r1);
+        tile_rows(roff, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
             const int64_t r = r0 + srow[p - p0];
             rwt[p] = wt[row_ptr[order[r]] + (p - roff[r])];
@@ -118,7 +118,7 @@ __global__ void k_w_pull(const int64_t* roff, const int32_t* rcol, const uint8_t
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t p0 = t * kTileItems, p1 = min(nnz, p0 + kTileItems);
         int64_t r0, r1;
-        tile_row_map(roff, n, p0, p1, srow, &sh, &r0, &r1);
+        tile_rows(roff, n, p0, p1, srow, &sh, &r0, &r1);
         for (int64_t q = p0; q < p1; q += blockDim.x) {  // uniform trip count: whole warps below
             const int64_t p = q + threadIdx.x;
             const bool ok = p < p1;
