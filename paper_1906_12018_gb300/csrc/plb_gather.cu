@@ -271,6 +271,23 @@ __device__ __noinline__ void count_reads(const int64_t* loff_h, const uint32_t* 
     chk[1] += (unsigned long long)(loff_h[h + 1] - loff_h[h]);
 }
 
+// The same for the candidates hb + b, b the bits of c, with one search for all of
+// them (one each: 1,330 instead of 650 ms for a profiled build of R-MAT 2^22).
+__device__ __noinline__ void count_reads64(const int64_t* loff, const uint32_t* lv, int64_t lvlen, uint32_t hb,
+                                           unsigned long long c, unsigned long long* cnt) {
+    if (c == 0) return;
+    int64_t at = lower_bound_u32(lv, lvlen, pack(hb, 0));
+    cnt[0] += (unsigned long long)at * (unsigned)__popcll(c);
+#pragma unroll 1
+    for (; at < lvlen && hub_of(lv[at]) - hb < 64u; ++at)
+        cnt[0] += (unsigned)__popcll(c >> (hub_of(lv[at]) - hb) >> 1);  // candidates past this hub
+#pragma unroll 1
+    for (; c; c &= c - 1) {
+        const int64_t* l = loff + hb + (__ffsll((long long)c) - 1);
+        cnt[1] += (unsigned long long)(l[1] - l[0]);
+    }
+}
+
 // Warp tier: gather of v's messages (hubs below v of the neighbours' frontier
 // rows; the rows are sorted, so each row's share is found by binary search).
 // Hubs below vb + W are marked in the bitmap X, the others go into the set S
@@ -1167,10 +1184,7 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
                     if (!__any_sync(kFull, (c0 | c1) != 0u)) continue;
                     const int found = __popc(c0) + __popc(c1);
                     if (p.count_check)
-#pragma unroll 1
-                        for (int b = 0; b < 64; ++b)
-                            if (((b < 32 ? c0 : c1) >> (b & 31)) & 1u)
-                                count_reads(p.loff_h, lvp, ll, hb + (uint32_t)b, cnt + 8);
+                        count_reads64(p.loff_h, lvp, ll, hb, (unsigned long long)c1 << 32 | c0, cnt + 8);
                     // (x < the row's words: hubs of v's graph within the map,
                     // rounded up to 128; rows are 16-byte aligned)
                     const uint32_t* cx = cols + min((uint32_t)x, cwords - 2u);
