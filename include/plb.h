@@ -76,11 +76,13 @@ typedef struct {
 typedef struct {
     int32_t validate;          /* 1: check CSR and order on the device first (default 1) */
     int32_t warp_label_cap;    /* largest |L(v)| handled one-vertex-per-warp (default 512) */
-    int32_t warp_cand_cap;     /* largest unique-candidate count per warp-vertex (default 512) */
+    int32_t warp_cand_cap;     /* one-vertex-per-warp: unique candidates past the first hubs of the
+                                  graph; all its candidates: about twice as many (default 512) */
     int32_t block_label_cap;   /* largest |L(v)| the block tier stages in shared memory (default 512) */
     int32_t block_cand_cap;    /* unique candidates per hub-range pass of the block tier (default 2048) */
     int32_t block_threads;     /* threads of the block tier, 64..256, rounded down to a multiple of 32 (default 256) */
-    int32_t use_graph;         /* 1: run the rounds after round 1 as a captured CUDA graph with
+    int32_t use_graph;         /* 1: run the rounds after round 1 (with 4,096 vertices or more:
+                                  after round 8) as a captured CUDA graph with
                                   a device-side while condition (no per-round host sync);
                                   buffers get fixed capacities; a round that may not fit
                                   stops the graph, finishes host-driven after the buffers
@@ -254,8 +256,8 @@ int plb_memory_stats(int64_t* out, int reset);
 
 /* Degree order (Sec. 6.1: vertices ordered by degree): order_out (device,
  * int32[n]) receives rank -> id, degree descending, ties by smaller id.
- * Only row_ptr is read.  Allocates device scratch (8 bytes per vertex,
- * rounded up to a power of two).  Asynchronous on the stream. */
+ * Only row_ptr is read.  Allocates device scratch (about 17 bytes per vertex).
+ * Asynchronous on the stream. */
 int plb_degree_order(const plb_csr* g, int32_t* order_out, plb_stream stream);
 
 /* Allocation-free degree order (no counterpart in the paper; a service of

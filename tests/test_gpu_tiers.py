@@ -75,6 +75,23 @@ def test_candidate_counts_around_the_warp_tiers_list(opts, lead):
     assert_labels_equal(lab, O.pll(g.off, g.col, order), f"lead {lead}")
 
 
+@pytest.mark.parametrize("lead", [0, 40, 147456 - 1000], ids=["map", "offset", "map and set"])
+def test_profiled_counts_agree_between_the_tiers(lead):
+    """A profiled build counts the label entries below and of every checked
+    candidate: the warp tier one candidate at a time, the block tier 64 hubs of
+    its bitmap at a time."""
+    core = G.chung_lu_graph(1800, 60, 2.2, 11)
+    src = np.repeat(np.arange(core.n), np.diff(core.off))
+    g = G.clean_csr(core.n + lead, src.astype(np.int32) + lead, core.col.astype(np.int32) + lead)
+    order = np.concatenate([np.arange(lead, dtype=np.int32), G.degree_order(core) + np.int32(lead)])
+    rp, col, o = to_device(g, order)
+    warp = plb.build(rp, col, o, profile=1, warp_cand_cap=2048, warp_label_cap=512).stats()
+    block = plb.build(rp, col, o, profile=1, warp_cand_cap=32, warp_label_cap=16).stats()
+    assert block["tier_vertices"][1] > warp["tier_vertices"][1]
+    for key in ("check_lv_entries", "check_lh_entries"):
+        assert warp[key] == block[key] > 0, key
+
+
 def hub_edges(leaves, arcs, seed):
     """Hubs 0..len(arcs)-1 with the given numbers of random leaves, and a sparse
     random graph on the leaves."""
