@@ -899,7 +899,10 @@ __global__ void __launch_bounds__(kMergeWarps * 32) k_merge_rows(const int64_t* 
 
 // After the merge of round d: level d of the masks, which is final now, by hub
 // (TopColumns; with more != 0, as in rank batches, whose rounds start again at
-// distance 1, the levels above it too).  A block takes 32 vertices; those that
+// distance 1, the levels above it too).
+// A round of distance d reads every level below d (at most kTopLevels), so a round
+// that accepts nothing needs its level as well: it equals the one before, but the
+// columns start empty.  A block takes 32 vertices; those that
 // start a run of 128 of their graph are transposed, one warp per mask word.
 // What bounds it is instruction issue: with a vote per bit (32 votes and selects
 // per word) it took 380 us a round for a union of 200 graphs, 2.3 of 50 ms; a

@@ -535,8 +535,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
             PLB_CK(exclusive_scan_i64(tmp64, loff[x], n, scan_scr, s));
             k_merge_rows<<<grid_for((n + 7) / 8, 1, flat_grid_cap), 256, 0, s>>>(
                 loff[cur], lent[cur], loff[x], lent[x], fse_new, store, n, nullptr, ctr, top);
-            k_top_columns<<<grid_for((n + 31) / 32, 1, flat_grid_cap), 256, 0, s>>>(top, n, nullptr, cols, 0, ctr);
-            launches += 3 + scan_n;
+            launches += 2 + scan_n;
             PLB_CK(cudaGetLastError());
             const int64_t Told = T;
             T = Tn;
@@ -553,6 +552,13 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
             }
             base = (int64_t)hctr->cursor;  // this round's rows end here
             if (tm.on) tm.span(T_MERGE, m0, tm.mark());
+        }
+        // level d of the top-hub columns, also when no label has distance d: it
+        // then equals the level below, and later rounds look for witnesses in it
+        if (d <= kTopLevels) {
+            k_top_columns<<<grid_for((n + 31) / 32, 1, flat_grid_cap), 256, 0, s>>>(top, n, nullptr, cols, 0, ctr);
+            launches += 1;
+            PLB_CK(cudaGetLastError());
         }
         PLB_CK(cudaMemsetAsync(ctr, 0, offsetof(RoundCounters, nA), s));
     }
