@@ -451,8 +451,17 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
             S.st.check_lh_entries += (int64_t)h.chk_lh;
             for (int q = 0; q < 3; ++q) S.st.tier_vertices[q] += (int64_t)h.tier[q];
             S.rounds = d;
-            if (acc == 0) S.done = true;
-            else if (d > PLB_MAX_DIST) status = PLB_ERR_DIST_OVERFLOW;
+            if (acc == 0) {
+                S.done = true;
+                // the other side's rounds go on to look for witnesses at the levels
+                // from d on, which this side no longer merges: all are final now
+                k_top_columns<<<grid_for((n + 31) / 32, 1, flat_grid_cap), 256, 0, s>>>(S.top, n, nullptr, S.cols, 1,
+                                                                                      S.ctr);
+                launches += 1;
+                PLB_CK(cudaGetLastError());
+            } else if (d > PLB_MAX_DIST) {
+                status = PLB_ERR_DIST_OVERFLOW;
+            }
         }
         if (status != PLB_OK) break;
         // merges after both gathers (snapshot of round d - 1 for both checks)

@@ -898,8 +898,8 @@ __global__ void __launch_bounds__(kMergeWarps * 32) k_merge_rows(const int64_t* 
 }
 
 // After the merge of round d: level d of the masks, which is final now, by hub
-// (TopColumns; with more != 0, as in rank batches, whose rounds start again at
-// distance 1, the levels above it too).
+// (TopColumns; with more != 0 the levels above it too: in rank batches, whose
+// rounds start again at distance 1, and for a directed side that has finished).
 // A round of distance d reads every level below d (at most kTopLevels), so a round
 // that accepts nothing needs its level as well: it equals the one before, but the
 // columns start empty.  A block takes 32 vertices; those that

@@ -1,7 +1,7 @@
 """Distances at which nothing is accepted: weighted rounds without a label at
-their distance.  The labels known at such a distance are those of the distance
-below it, and a witness among them still refutes a candidate (bit-exact against
-the oracle)."""
+their distance, and directed builds whose two sides need different numbers of
+rounds.  The labels known at such a distance are those of the distance below it,
+and a witness among them still refutes a candidate (bit-exact against the oracle)."""
 import numpy as np
 import pytest
 import torch
@@ -59,3 +59,40 @@ def test_weighted_random_graphs_with_empty_distances(weights, seed):
     g, wt = weighted_csr(n, list(zip(s.tolist(), t.tolist(), rng.choice(weights, len(s)).tolist())))
     for order in (G.degree_order(g), rng.permutation(n).astype(np.int32)):
         check_weighted(g, wt, order, **FORCED)
+
+
+def check_directed(g, order, **opts):
+    ref_in, ref_out = O.pll_directed(g.off, g.col, g.off_in, g.col_in, order)
+    lin, lout = plb.build_directed(torch.from_numpy(g.off).cuda(), torch.from_numpy(g.col).cuda(),
+                                   torch.from_numpy(order).cuda(), **opts)
+    assert_labels_equal(lin, ref_in, "in")
+    assert_labels_equal(lout, ref_out, "out")
+    return lin, lout
+
+
+@pytest.mark.parametrize("leaves,opts", RECEIVERS)
+@pytest.mark.parametrize("flip", [False, True], ids=["in ends first", "out ends first"])
+def test_directed_witness_on_a_side_that_has_finished(leaves, opts, flip):
+    """v -> 0 -> 1 and v -> a -> b -> 1: candidate 1 at distance 3 of v has the
+    witness 0 (1 + 1); nothing is reached over two arcs on the other side, which
+    accepts nothing after round 1."""
+    a, b, v = leaves + 2, leaves + 3, leaves + 4
+    arcs = [(v, 0), (0, 1), (v, a), (a, b), (b, 1)] + [(v, i) for i in range(2, a)]
+    src, dst = (np.array(x, dtype=np.int32) for x in zip(*arcs))
+    if flip:
+        src, dst = dst, src
+    lin, lout = check_directed(G.directed_csr(v + 1, src, dst), np.arange(v + 1, dtype=np.int32), **opts)
+    rounds = (lin.stats()["rounds"], lout.stats()["rounds"])
+    assert rounds[flip] < rounds[not flip]
+    assert (lin if flip else lout).stats()["tier_vertices"][1] > 0
+
+
+@pytest.mark.parametrize("seed", range(8))
+def test_directed_random_graphs(seed):
+    rng = np.random.default_rng(seed)
+    for _ in range(25):
+        n = int(rng.integers(70, 140))
+        m = int(n * rng.uniform(1.5, 4))
+        g = G.directed_csr(n, rng.integers(0, n, m), rng.integers(0, n, m))
+        check_directed(g, G.directed_degree_order(g), **FORCED)
+        check_directed(g, rng.permutation(n).astype(np.int32), **FORCED)
