@@ -3,7 +3,7 @@
 #include <atomic>
 #include <vector>
 
-#include "plb_kernels.cuh"
+#include "plb_host.cuh"
 
 namespace plb {
 
@@ -167,7 +167,7 @@ int plb_build(const plb_csr* g, const int32_t* vertex_order, const plb_options* 
     (void)cudaGetLastError();
     if (g->n == 0) return empty_labels(out, s);
     return plb::build_core(g->row_ptr, g->col, vertex_order, g->n, g->nnz, o, s, out, g->n, nullptr, nullptr,
-                           plb::column_quads(g->n));
+                           plb::column_quads(g->n, plb::warp_only_vertices(o)));
 }
 
 int plb_build_directed(const plb_csr* g, const int32_t* vertex_order, const plb_options* opt, plb_stream stream,
@@ -211,12 +211,13 @@ static int build_union(const plb_csr* gs, const int32_t* const* orders, int64_t 
     std::vector<plb::GraphDesc> hd((size_t)k);
     std::vector<int64_t> vb((size_t)k + 1), eb((size_t)k + 1);
     int64_t N = 0, E = 0, quads = 0;
+    const int64_t warp_only = plb::warp_only_vertices(o);
     for (int64_t i = 0; i < k; ++i) {
         vb[i] = N;
         eb[i] = E;
         hd[i] = {gs[i].row_ptr, gs[i].col, orders[i], N, E, gs[i].n, gs[i].nnz,
-                 make_int2((int)quads, plb::column_quads(gs[i].n))};
-        quads += plb::column_quads(gs[i].n);
+                 make_int2((int)quads, plb::column_quads(gs[i].n, warp_only))};
+        quads += hd[i].cols.y;
         N += gs[i].n;
         E += gs[i].nnz;
     }

@@ -34,7 +34,7 @@ constexpr int kGraphAfter = 8;
 // holds at most that many hubs, which sizes the block tier's accepted rows.
 // vbase: the first rank of each vertex's graph in that union (else null);
 // col_base, col_quads: the places of the graphs' top-hub columns and the size
-// of all (else null and column_quads(n)).
+// of all (else null and those of n).
 int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order, int64_t n, int64_t nnz,
                const plb_options& o, cudaStream_t s, plb_labels** out, int64_t max_part_n, const int32_t* vbase,
                const int2* col_base, int64_t col_quads) {

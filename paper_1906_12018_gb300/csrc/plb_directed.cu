@@ -172,7 +172,7 @@ int build_directed_core(const int64_t* row_ptr, const int32_t* col, const int32_
             S.fhub[b] = pool.alloc<uint32_t>(S.fcap[b]);
         }
         S.top = pool.alloc<uint32_t>(n * kTopRow);
-        S.cols = top_columns(pool, column_quads(n), nullptr, s);
+        S.cols = top_columns(pool, column_quads(n, warp_only_vertices(o)), nullptr, s);
         S.hoff = pool.alloc<int64_t>(n + 1);
         S.hdesc = pool.alloc<uint64_t>(n);
         S.hcap = std::max<int64_t>(4 * n, 1024);

@@ -1119,12 +1119,13 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
         }
         // the rows of the first prefilter step (column offsets, in hist; filled
         // up to a multiple of four): v's top hubs at distance i0, or at every
-        // distance in weighted rounds
+        // distance in weighted rounds; none for a graph without columns, whose
+        // candidates take the whole prefilter in check_chunk
         const int i0 = first_level(tv, imax, lane);
         if (wid == nw - 1) {
             int ne = 0;
 #pragma unroll 1
-            for (int i = p.sender_bits ? 1 : i0; i <= (p.sender_bits ? imax : i0); ++i) {
+            for (int i = p.sender_bits ? 1 : i0; cwords && i <= (p.sender_bits ? imax : i0); ++i) {
                 uint32_t m = lane < kTopWords ? tv[(i - 1) * kTopWords + lane] : 0u;
                 const int c = __popc(m);
                 const int incl = warp_incl_scan(c, lane);
@@ -1186,7 +1187,8 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
                     if (p.count_check)
                         count_reads64(p.loff_h, lvp, ll, hb, (unsigned long long)c1 << 32 | c0, cnt + 8);
                     // (x < the row's words: hubs of v's graph within the map,
-                    // rounded up to 128; rows are 16-byte aligned)
+                    // rounded up to 128; rows are 16-byte aligned; a graph
+                    // without columns has no rows to read)
                     const uint32_t* cx = cols + min((uint32_t)x, cwords - 2u);
 #pragma unroll 1
                     for (int k = 0; k < n_rows; k += 4) {
@@ -1240,7 +1242,7 @@ __device__ void gp_block_vertex(const GpParams& p, uint32_t d, int32_t v, uint32
                 const bool valid = lane < k;
                 const uint32_t h = valid ? surv[ns + lane] : 0u;
                 const unsigned okm = check_chunk(p, d, Mp, log_mp, !useM, kBlockSideBMin, kBlockSideBShift, lvp, ll,
-                                                 lv_top, h, valid, cnt[4], tv, i0, cnt[7]);
+                                                 lv_top, h, valid, cnt[4], tv, cwords ? i0 : 0, cnt[7]);
                 keep_accepted(okm, h, vb, W, B, gacc, sh);
             }
             __syncwarp();

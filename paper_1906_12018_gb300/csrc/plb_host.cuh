@@ -161,6 +161,16 @@ inline TierLimits tier_limits(int warp_cand, int warp_label) {
     return lim;
 }
 
+// The most vertices of a graph whose receivers all stay in the warp tier: arcs,
+// label row, candidate bound and candidates are each at most the vertex count,
+// and the tier's limits on them are no smaller than these (tier_limits; the set
+// holds warp_cand entries, the candidate list as many).  Only a CSR with repeated
+// arcs, which the input check refuses, can take such a receiver to the block tier.
+inline int64_t warp_only_vertices(const plb_options& o) {
+    const int warp_cand = pow2_at_least(std::max(32, o.warp_cand_cap)), warp_label = std::max(16, o.warp_label_cap);
+    return std::min<int64_t>({warp_cand, warp_label, tier_limits(warp_cand, warp_label).warp_deg});
+}
+
 // Lists and bitmaps of the split receivers of a build over n vertices (the
 // largest graph of a union: max_part_n) and nnz arcs.  A receiver is split from
 // kSplitArcs arcs on, so at most nnz / kSplitArcs receivers are, and their
@@ -242,8 +252,8 @@ inline int64_t accepted_words(int64_t max_part_n) {
     return std::max<int64_t>(max_part_n - kMapHubs, 1);
 }
 
-// The top-hub columns of a graph of n vertices, empty (quads: the words per row,
-// in units of 4, of all graphs of a union; by_base: their places).
+// The top-hub columns of a graph, empty (quads: the words per row, in units of 4,
+// of all graphs of a union, see column_quads; by_base: their places).
 inline TopColumns top_columns(DevPool& pool, int64_t quads, const int2* by_base, cudaStream_t s) {
     TopColumns c{};
     c.by_base = by_base;

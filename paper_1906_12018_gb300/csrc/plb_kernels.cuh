@@ -229,8 +229,12 @@ __device__ __forceinline__ uint32_t* columns_of(const TopColumns& c, uint32_t vb
     *words = 4u * (uint32_t)t.y;
     return c.bits + (int64_t)t.x * (4 * kTopRows);
 }
-// Words per row, in units of 4, for a graph of n vertices.
-__host__ __device__ __forceinline__ int column_quads(int64_t n) {
+// Words per row, in units of 4, for a graph of n vertices: none for one of up to
+// warp_only vertices (see warp_only_vertices), whose candidates are pruned by
+// their own masks.  (A quad of columns takes 28,672 bytes: a union of a million
+// graphs of 16 vertices had 28.7 GB of them, never read.)
+inline int column_quads(int64_t n, int64_t warp_only) {
+    if (n <= warp_only) return 0;
     const int64_t m = n < kMapHubs ? n : kMapHubs;
     return (int)((m + 127) / 128);
 }

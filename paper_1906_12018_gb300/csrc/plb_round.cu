@@ -926,6 +926,7 @@ __global__ void __launch_bounds__(256) k_top_columns(const uint32_t* top, int64_
             const uint32_t b = __shfl_sync(kFull, vb, k), r0 = __shfl_sync(kFull, rel, k);
             uint32_t words;
             uint32_t* rows = columns_of(cols, b, &words);
+            if (words == 0u) continue;  // (a graph without columns)
             for (int t = d; t <= (more ? kTopLevels : d); ++t) {
                 uint32_t out[4];
 #pragma unroll

@@ -288,7 +288,7 @@ int build_weighted_core(const int64_t* row_ptr, const int32_t* col, const uint8_
     int64_t scap = std::max<int64_t>(kRowAlign * n + nnz + 1024, 4096);
     uint32_t* store = pool.alloc<uint32_t>(scap);
     uint32_t* top = pool.alloc<uint32_t>(n * kTopRow);
-    const TopColumns cols = top_columns(pool, column_quads(n), nullptr, s);
+    const TopColumns cols = top_columns(pool, column_quads(n, warp_only_vertices(o)), nullptr, s);
     int64_t* hoff = pool.alloc<int64_t>(n + 1);
     uint64_t* hdesc = pool.alloc<uint64_t>(n);
     int64_t hcap = std::max<int64_t>(4 * n, 1024);
