@@ -180,7 +180,7 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
         k_index_size<<<gflat, kFlatThreads, 0, s>>>(loff[which], n, tmp64, ctr);
         if (exclusive_scan_i64(tmp64, hoff, n, scan_scr, s) != cudaSuccess) return PLB_ERR_CUDA;
         int64_t need = 6 * total + 1024, want = 8 * total + 1024;
-        if (total <= kSmallIndex) {  // (from the bound too: a host read costs more than the memory)
+        if (!roomy && total <= kSmallIndex) {  // (from the bound too: a host read costs more than the memory)
             need = 4 * total + 1024;
         } else if (!roomy) {
             int64_t packed = 0;
