@@ -126,9 +126,9 @@ int build_core(const int64_t* row_ptr, const int32_t* col, const int32_t* order,
     int64_t lcap[2] = {std::max<int64_t>(2 * n, 1024), std::max<int64_t>(2 * n, 1024)};
     int64_t* loff[2] = {pool.alloc<int64_t>(n + 1), pool.alloc<int64_t>(n + 1)};
     uint32_t* lent[2] = {pool.alloc<uint32_t>(lcap[0]), pool.alloc<uint32_t>(lcap[1])};
-    // (round 1 writes at most nnz / 2 hubs, padded rows)
-    int64_t fcap[2] = {std::max<int64_t>(nnz / 2 + kRowAlign * n, 1024),
-                       std::max<int64_t>(nnz / 2 + kRowAlign * n, 1024)};
+    // (round 1 writes at most nnz / 2 hubs; a row's padding is at most kRowAlign - 1)
+    const int64_t fcap0 = std::max<int64_t>(nnz / 2 + n, 1024) + (kRowAlign - 1) * n;
+    int64_t fcap[2] = {fcap0, fcap0};
     uint64_t* fse[2] = {pool.alloc<uint64_t>(n), pool.alloc<uint64_t>(n)};
     uint32_t* fhub[2] = {pool.alloc<uint32_t>(fcap[0]), pool.alloc<uint32_t>(fcap[1])};
     unsigned long long* recv = pool.alloc<unsigned long long>(n);

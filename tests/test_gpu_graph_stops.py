@@ -18,3 +18,16 @@ def test_probe_index_with_room_for_a_segments_updates():
     lab = gpu_build(g, order, use_graph=1)
     assert_labels_equal(lab, O.pll(g.off, g.col, order))
     assert lab.stats()["rounds"] > 8 and lab.stats()["reruns"] == 0
+
+
+def test_small_frontiers_with_padded_rows():
+    """The frontier buffers of a small graph hold 1,024 hubs however short their
+    rows are (rows are padded to eight hubs).  The rounds of this graph bring
+    fewer: its only stop is not one for their sake."""
+    w = 10
+    g = G.from_edges(w * w, [(w * i + j, w * i + j + 1) for i in range(w) for j in range(w - 1)] +
+                     [(w * i + j, w * i + j + w) for i in range(w - 1) for j in range(w)])
+    order = G.degree_order(g)
+    lab = gpu_build(g, order, use_graph=1)
+    assert_labels_equal(lab, O.pll(g.off, g.col, order))
+    assert lab.stats()["reruns"] <= 1
