@@ -194,9 +194,13 @@ inline SplitLists split_lists(DevPool& pool, int64_t n, int64_t max_part_n, int6
 }
 
 // The block tier's stream beside the build's own, with its fork and join events.
+// Declared after the build's DevPool: a build that fails between fork and join
+// waits here for the side stream's kernels, since the pool takes their buffers
+// back in the order of the build's own stream, which has not joined them.
 struct SideStream {
     cudaStream_t st = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
+    bool open = false;  // launched into, and not joined
     cudaError_t create() {
         cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
@@ -204,6 +208,7 @@ struct SideStream {
         return e;
     }
     ~SideStream() {
+        if (open) cudaStreamSynchronize(st);
         if (fork) cudaEventDestroy(fork);
         if (join) cudaEventDestroy(join);
         if (st) cudaStreamDestroy(st);
@@ -232,12 +237,14 @@ inline cudaError_t launch_tiers(GpParams w, GpParams b, const SplitLists& split,
     cudaError_t e = cudaEventRecord(side.fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(side.st, side.fork, 0);
     if (e != cudaSuccess) return e;
+    side.open = true;
     k_gp_block<<<grid_b, bthr, b_smem, side.st>>>(b);
     k_gp_warp<<<grid_w, kGpWarpThreads, w_smem, s>>>(w);
     if (tm) *mark = tm->mark();
     e = cudaEventRecord(side.join, side.st);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, side.join, 0);
     if (e != cudaSuccess) return e;
+    side.open = false;
     b.list = O2;
     b.list_n = &ctr->nO2;
     b.work = &ctr->wkO2;
