@@ -102,8 +102,8 @@ __device__ __forceinline__ int32_t answer_pair2(const int64_t* off_s, const uint
                                                                              : look_up_all<kShortRow>(a, al, b, bl);
         return m == kEmpty ? PLB_UNREACHABLE : (int32_t)m;
     }
-    // the first 32 hubs of both rows: lane i's hub of a among b's lanes
-    const uint32_t x = lane < al ? a[lane] : kEmpty, y = lane < bl ? b[lane] : kEmpty;
+    // the first 32 hubs of both rows (each longer): lane i's hub of a among b's lanes
+    const uint32_t x = a[lane], y = b[lane];
     int k = 0;  // largest lane with y <= x's hub at any distance
 #pragma unroll
     for (int step = 16; step >= 1; step >>= 1) {
@@ -111,11 +111,8 @@ __device__ __forceinline__ int32_t answer_pair2(const int64_t* off_s, const uint
         if (z <= (x | 0xFFu)) k += step;
     }
     const uint32_t z = __shfl_sync(kFull, y, k);
-    uint32_t best = x != kEmpty && z != kEmpty && hub_of(z) == hub_of(x) ? dist_of(x) + dist_of(z) : kEmpty;
-    best = __reduce_min_sync(kFull, best);
-    // two rows of up to 32 entries have been compared whole; a sum of 0 or 1 is
-    // the distance
-    if (best > 1 && (al > 32 || bl > 32)) {
+    uint32_t best = __reduce_min_sync(kFull, hub_of(z) == hub_of(x) ? dist_of(x) + dist_of(z) : kEmpty);
+    if (best > 1) {  // (a sum of 0 or 1 is the distance)
         // near entries of a, then of b, looked up in the other row, 32 at a
         // time from the end of buf (its first na are a's)
         const unsigned lt = (1u << lane) - 1u;
