@@ -150,7 +150,12 @@ inline bool tiers_fit(int warps, int w_log_s, int w_log_m, size_t b_smem) {
 // them, and no pruning by columns).  2 | 3 | 4 | 8 x warp_cand | the rule below, ms:
 // Chung-Lu 2^20 23.4 | 22.2 | 21.9 | 22.0 | 21.8; batch of 200 graphs 47.7 |
 // 46.2 | 45.5 | 45.6 | 45.6; directed R-MAT 2^20 95.8 | 93.4 | 94.4 | 98.7 | 93.4;
-// R-MAT 2^22 535.6 | 536 | 538 | 545 | 537; 1.5 x: 25.1, 49.3, 100.6, 547.
+// R-MAT 2^22 535.6 | 536 | 538 | 545 | 537; 1.5 x: 25.1, 49.3, 100.6, 547.  Rows up
+// to which the larger bound holds, none | 64 | 128 | 256 | any: Chung-Lu 22.8 |
+// 22.1 | 22.1 | 22.1 | 22.2; batch 45.5 | 44.5 | 44.5 | 44.5 | 44.6; directed 91.6 |
+// 90.7 | 90.9 | 91.8 | 92.1; R-MAT 2^22 532 | 534 | 535 | 535 | 535.  What a wider
+// bound costs: receivers whose candidates do not fit after all are gathered
+// twice, the second time beside nothing else (see launch_tiers).
 inline TierLimits tier_limits(int warp_cand, int warp_label) {
     TierLimits lim;
     lim.warp_bound = 5 * (int64_t)warp_cand / 2;
@@ -215,7 +220,8 @@ struct SideStream {
     }
 };
 
-// One gather + prune of host-driven rounds.  The two tiers run side by side:
+// One gather + prune of a round.  The two tiers run side by side (in a captured
+// round the side stream becomes a branch of the graph):
 // the block tier on the side stream over k_collect's block list O1 (and the
 // split receivers), the warp tier on the build's stream, escalating into O2,
 // which one more block-tier launch takes after both (the tails of the two

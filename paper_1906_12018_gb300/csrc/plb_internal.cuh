@@ -151,17 +151,8 @@ __device__ __forceinline__ int64_t lower_bound_u32(const uint32_t* a, int64_t le
     return lo;
 }
 
-// Row r of offsets off[] containing item p (largest r with off[r] <= p) in [lo, hi].
-__device__ __forceinline__ int64_t row_of(const int64_t* off, int64_t lo, int64_t hi, int64_t p) {
-#pragma unroll 1
-    while (lo < hi) {
-        const int64_t mid = (lo + hi + 1) >> 1;
-        if (off[mid] <= p) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-// The same by a whole warp, 32 probes at a time (a binary search is a chain of
+// Row r of offsets off[] containing item p (largest r with off[r] <= p) in [lo,
+// hi], by a whole warp, 32 probes at a time (a binary search is a chain of
 // log2(rows) dependent loads; all lanes call and get the result).
 __device__ __forceinline__ int64_t warp_row_of(const int64_t* off, int64_t lo, int64_t hi, int64_t p) {
     const int lane = threadIdx.x & 31;

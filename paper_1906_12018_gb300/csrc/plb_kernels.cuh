@@ -32,7 +32,7 @@ struct RoundCounters {
     unsigned long long prefiltered; // candidates pruned by the top-hub witness prefilter
     unsigned long long chk_lv, chk_lh;  // checked candidates (h at v): sums of |L(v) entries with hub < h|
                                         // and of |L(h)| (counted when GpParams::count_check is set)
-    int nR, nO1, nO2;             // receivers: warp tier, block tier (nO2 unused)
+    int nR, nO1, nO2;             // receivers: warp tier, block tier, escalated by the warp tier
     int nBig, nGiant;             // new frontier rows too long for a warp / for shared memory to sort
     int nU;                       // vertices whose new frontier row was written unsorted (block tier)
     int wkR, wkO1, wkO2;          // next entry of each tier's list (taken by whoever is free)
@@ -144,7 +144,8 @@ struct GpParams {
     const int32_t* vbase;      // per vertex: first rank of its graph in a disjoint union, or null (one graph:
                                // 0).  The top hubs and the maps are those of the vertex's own graph
     int count_check;           // 1: count the label entries each check would read by the paper's cost
-                               // model (RoundCounters::chk_lv / chk_lh; one binary search per candidate)
+                               // model (RoundCounters::chk_lv / chk_lh; a search per candidate, or per 64
+                               // hubs of the block tier's bitmap)
 };
 
 // First rank of v's graph (see GpParams::vbase).

@@ -286,8 +286,7 @@ __global__ void k_collect(unsigned long long* recv, const int64_t* roff, const i
 // active list restarts.  Counted like the general round:
 // one message, one unique candidate and one accepted label per such neighbour.
 // Both passes run flat over tiles of arcs (a hub's row is spread over many
-// warps instead of one), each arc's row found by binary search in the tile's
-// row range.
+// warps instead of one; tile_rows gives each arc its row).
 // Count pass: cnt[v] = |N(v) n [s, min(e, v))| (cnt zero on entry; one
 // atomic per row and warp).
 __global__ void k_round1_count(const int64_t* roff, const int32_t* rcol, int64_t n, int64_t nnz, int32_t s,
