@@ -1,6 +1,6 @@
 // Degree order (Sec. 6.1: vertices ordered by degree, the heuristic of the
 // original PLL): rank -> id with degree descending and ties by smaller id.
-// Up to kSortTile vertices, and without scratch of its own (the allocation-free
+// Up to kBitonicMax vertices, and without scratch of its own (the allocation-free
 // entry point), a bitonic network over unique keys (0x7FFFFFFF - degree) << 32 |
 // id; beyond, a stable radix sort by degree that starts in id order.
 #include <algorithm>
@@ -12,6 +12,10 @@ namespace {
 
 constexpr int kSortTile = 2048;
 constexpr int kSortThreads = 1024;
+// The radix sort's 15 launches take 60 to 70 us however few the vertices; the
+// bitonic network pads to a power of two: 2,049 to 4,096 vertices 41-43 us (radix
+// 60-66), up to 8,192 59 us (62-70), up to 16,384 80 us (62-70).
+constexpr int64_t kBitonicMax = 8192;
 
 __global__ void k_deg_keys(const int64_t* row_ptr, int64_t n, int64_t n2, uint64_t* keys) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n2; i += (int64_t)gridDim.x * blockDim.x) {
@@ -274,7 +278,7 @@ extern "C" int plb_degree_order(const plb_csr* g, int32_t* order_out, plb_stream
     cudaStream_t s = (cudaStream_t)stream;
     int64_t n2 = 1;
     while (n2 < g->n) n2 <<= 1;
-    const bool radix = g->n > plb::kSortTile;
+    const bool radix = g->n > plb::kBitonicMax;
     uint64_t* keys = nullptr;
     if (plb::dev_alloc((void**)&keys, sizeof(uint64_t) * (radix ? plb::radix_scratch_words(g->n) : n2), s) !=
         cudaSuccess) {
