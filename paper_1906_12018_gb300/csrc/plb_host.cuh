@@ -156,6 +156,14 @@ inline bool tiers_fit(int warps, int w_log_s, int w_log_m, size_t b_smem) {
 // 90.7 | 90.9 | 91.8 | 92.1; R-MAT 2^22 532 | 534 | 535 | 535 | 535.  What a wider
 // bound costs: receivers whose candidates do not fit after all are gathered
 // twice, the second time beside nothing else (see launch_tiers).
+// In dense graphs few candidates come in very many messages, 8 us per thousand for
+// a warp: receivers with more than warp_msgs are gathered by a block.  Complete
+// graphs of 600 | 900 | 1,500 vertices took 2.4 | 6.2 | 13.7 ms without this limit
+// (warps with half a million messages each, crowded into the SMs that the block tier
+// left first), 1.0 | 1.2 | 2.3 with it (262,144: 2.4 | 1.2 | 2.3; counting the rows as
+// they are cut at v: 1.4 | 2.2 | 3.1); directed R-MAT 2^20 90.8 ms without, 88.9 with
+// it, the other builds equal.  16,384 is up to 2% faster still, but then graphs from
+// 182 vertices instead of 363 have columns (warp_only_vertices).
 inline TierLimits tier_limits(int warp_cand, int warp_label) {
     TierLimits lim;
     lim.warp_bound = 5 * (int64_t)warp_cand / 2;
@@ -163,17 +171,23 @@ inline TierLimits tier_limits(int warp_cand, int warp_label) {
     lim.short_label = 128;
     lim.warp_label = warp_label;
     lim.warp_deg = (int64_t)32 * 64;
+    lim.warp_msgs = 65536;
     return lim;
 }
 
 // The most vertices of a graph whose receivers all stay in the warp tier: arcs,
 // label row, candidate bound and candidates are each at most the vertex count,
 // and the tier's limits on them are no smaller than these (tier_limits; the set
-// holds warp_cand entries, the candidate list as many).  Only a CSR with repeated
-// arcs, which the input check refuses, can take such a receiver to the block tier.
+// holds warp_cand entries, the candidate list as many); a neighbour of rank a
+// sends at most a hubs, so the messages are at most n (n - 1) / 2.  Only a CSR
+// with repeated arcs, which the input check refuses, can take such a receiver to
+// the block tier.
 inline int64_t warp_only_vertices(const plb_options& o) {
     const int warp_cand = pow2_at_least(std::max(32, o.warp_cand_cap)), warp_label = std::max(16, o.warp_label_cap);
-    return std::min<int64_t>({warp_cand, warp_label, tier_limits(warp_cand, warp_label).warp_deg});
+    const TierLimits lim = tier_limits(warp_cand, warp_label);
+    int64_t n = std::min<int64_t>({warp_cand, warp_label, lim.warp_deg});
+    while (n * (n - 1) / 2 > lim.warp_msgs) --n;
+    return n;
 }
 
 // Lists and bitmaps of the split receivers of a build over n vertices (the

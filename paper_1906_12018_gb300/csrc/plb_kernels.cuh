@@ -249,6 +249,7 @@ struct TierLimits {
     int64_t short_label;
     int64_t warp_label;   // largest |L(v)| of the warp tier
     int64_t warp_deg;     // largest degree of the warp tier
+    int64_t warp_msgs;    // most messages of the warp tier (rows of the neighbours, not cut at v)
 };
 
 struct WarpSync {

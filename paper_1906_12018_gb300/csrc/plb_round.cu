@@ -218,7 +218,7 @@ __global__ void k_mark(const int64_t* roff, const int32_t* rcol, const uint64_t*
 // Receivers (recv[v] > 0) with many arcs are split (SplitLists), the others
 // are routed by the candidate bound min(v, recv[v])
 // (v counted from the first rank of its graph in a disjoint union),
-// |L(v)| and degree: warp tier (R) or block tier (O1); the bound is kept in
+// messages, |L(v)| and degree: warp tier (R) or block tier (O1); the bound is kept in
 // rbound[v] (it sizes the warp tier's tables) and, when obound is given, in
 // obound[v] for every v (0 for non-receivers: its scan places each row of the
 // new frontier).  Also clears recv and the new frontier descriptors, and sums
@@ -244,7 +244,7 @@ __global__ void k_collect(unsigned long long* recv, const int64_t* roff, const i
             const int64_t ll = loff[v + 1] - loff[v];
             const int64_t deg = roff[v + 1] - roff[v];
             tier = ((int64_t)bound <= (ll <= lim.short_label ? lim.short_bound : lim.warp_bound) &&
-                    ll <= lim.warp_label && deg <= lim.warp_deg) ? 0 : 1;
+                    ll <= lim.warp_label && deg <= lim.warp_deg && (int64_t)c <= lim.warp_msgs) ? 0 : 1;
             if (deg > kSplitArcs && below <= (unsigned long long)kMapHubs && split.max > 0) {
                 const int np = (int)((deg + kSplitPart - 1) / kSplitPart);
                 const int g = atomicAdd(&ctr->nG, 1);
