@@ -144,18 +144,22 @@ inline bool tiers_fit(int warps, int w_log_s, int w_log_m, size_t b_smem) {
 
 // Tier of a receiver.  The bound counts messages; the candidates, which have to
 // fit the warp tier's list (968 for the default 512), are fewer, by 2 to 5 times
-// on power-law graphs, and a receiver with more goes on to the block tier.  With
-// the bound at 2 x warp_cand the block tier took receivers that a warp finishes
-// sooner than a block starts; with long rows L(v) a warp does less well (staging
-// them, and no pruning by columns).  2 | 3 | 4 | 8 x warp_cand | the rule below, ms:
-// Chung-Lu 2^20 23.4 | 22.2 | 21.9 | 22.0 | 21.8; batch of 200 graphs 47.7 |
+// on power-law graphs in degree order, and a receiver with more goes on to the
+// block tier.  With the bound at 2 x warp_cand for all, the block tier took
+// receivers that a warp finishes sooner than a block starts; with long rows L(v) a
+// warp does less well (staging them, and no pruning by columns) and keeps that
+// bound.  All rows 2 | 3 | 4 | 8 x warp_cand | 4 x up to 128 entries and 2.5 x beyond,
+// ms: Chung-Lu 2^20 23.4 | 22.2 | 21.9 | 22.0 | 21.8; batch of 200 graphs 47.7 |
 // 46.2 | 45.5 | 45.6 | 45.6; directed R-MAT 2^20 95.8 | 93.4 | 94.4 | 98.7 | 93.4;
 // R-MAT 2^22 535.6 | 536 | 538 | 545 | 537; 1.5 x: 25.1, 49.3, 100.6, 547.  Rows up
 // to which the larger bound holds, none | 64 | 128 | 256 | any: Chung-Lu 22.8 |
 // 22.1 | 22.1 | 22.1 | 22.2; batch 45.5 | 44.5 | 44.5 | 44.5 | 44.6; directed 91.6 |
-// 90.7 | 90.9 | 91.8 | 92.1; R-MAT 2^22 532 | 534 | 535 | 535 | 535.  What a wider
-// bound costs: receivers whose candidates do not fit after all are gathered
-// twice, the second time beside nothing else (see launch_tiers).
+// 90.7 | 90.9 | 91.8 | 92.1; R-MAT 2^22 532 | 534 | 535 | 535 | 535.  Longer rows 1.5 |
+// 2 | 2.5 x: Chung-Lu 22.0 | 22.2 | 22.3, directed 89.7 | 89.2 | 89.3, batch, weighted
+// and R-MAT 2^22 equal; in random order, where rows are long and few messages
+// repeat, Chung-Lu with 5,000 vertices 9.6 | 10.1 | 10.5, R-MAT 2^13 10.4 | 10.9 |
+// 11.3.  What a wider bound costs: receivers whose candidates do not fit after all
+// are gathered twice, the second time beside nothing else (see launch_tiers).
 // In dense graphs few candidates come in very many messages, 8 us per thousand for
 // a warp: receivers with more than warp_msgs are gathered by a block.  Complete
 // graphs of 600 | 900 | 1,500 vertices took 2.4 | 6.2 | 13.7 ms without this limit
@@ -166,7 +170,7 @@ inline bool tiers_fit(int warps, int w_log_s, int w_log_m, size_t b_smem) {
 // 182 vertices instead of 363 have columns (warp_only_vertices).
 inline TierLimits tier_limits(int warp_cand, int warp_label) {
     TierLimits lim;
-    lim.warp_bound = 5 * (int64_t)warp_cand / 2;
+    lim.warp_bound = 2 * (int64_t)warp_cand;
     lim.short_bound = 4 * (int64_t)warp_cand;
     lim.short_label = 128;
     lim.warp_label = warp_label;
